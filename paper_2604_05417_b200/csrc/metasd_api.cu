@@ -303,6 +303,7 @@ int metasd_verify(metasd_ctx *ctx, int32_t batch, int32_t k, const void *target_
     p.st = ctx->st; p.stats = ctx->stats; p.status = ctx->status;
     {
         const long long nvec = (long long)cfg.vocab * (long long)logit_size(cfg.logit_dtype) / 16;
+        p.keep_permille = ctx->keep_permille;
         p.keep_from_vec = (int32_t)(nvec - nvec * ctx->keep_permille / 1000);
     }
     p.poll_limit = cfg.wait_poll_limit > 0 ? (uint32_t)cfg.wait_poll_limit : (1u << 18);

@@ -51,6 +51,60 @@ __device__ __forceinline__ float ex2(float x)
 }
 
 // ---------------------------------------------------------------------------------------------
+// Pairs of fp32 values in one 64-bit register (sm_100a: one instruction works on both halves)
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ uint64_t pack2(float both) { return pack2(both, both); }
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t v;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t v;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ float sum2(uint64_t v)
+{
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return lo + hi;
+}
+// acc + 2^y, half by half
+__device__ __forceinline__ uint64_t add_ex2(uint64_t acc, uint64_t y)
+{
+    float lo, hi;
+    unpack2(y, lo, hi);
+    return add2(acc, pack2(ex2(lo), ex2(hi)));
+}
+// acc + 2^min(ya, yb), half by half
+__device__ __forceinline__ uint64_t add_ex2_min(uint64_t acc, uint64_t ya, uint64_t yb)
+{
+    float alo, ahi, blo, bhi;
+    unpack2(ya, alo, ahi);
+    unpack2(yb, blo, bhi);
+    return add2(acc, pack2(ex2(fminf(alo, blo)), ex2(fminf(ahi, bhi))));
+}
+
+// ---------------------------------------------------------------------------------------------
 // Logit element types: 16-byte vectors of bf16 (8 per vector) or fp32 (4 per vector)
 // ---------------------------------------------------------------------------------------------
 template <typename LT> struct Logit;
@@ -70,6 +124,55 @@ template <> struct Logit<__nv_bfloat16> {
     {
         return __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(p)[i] << 16);
     }
+    // the two logits of a 32-bit word
+    __device__ static __forceinline__ uint64_t pair_of(uint32_t w)
+    {
+        return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+    }
+    // A logit in the form vectors are compared with it (both halves of a word), and whether any of a vector's eight is
+    // larger: four instructions, two logits each.  NaN entries are not larger than anything.
+    using Best = uint32_t;
+    __device__ static __forceinline__ Best best_of(float x) { return __byte_perm(__float_as_uint(x), 0u, 0x3232); }
+    __device__ static __forceinline__ uint32_t max_word(uint32_t a, uint32_t b)
+    {
+        uint32_t m;
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(b));
+        return m;
+    }
+    __device__ static __forceinline__ uint32_t max_word(const uint4 &raw)
+    {
+        return max_word(max_word(raw.x, raw.y), max_word(raw.z, raw.w));
+    }
+    __device__ static __forceinline__ bool any_above(const uint4 &raw, Best best)
+    {
+        uint32_t any;
+        asm("{\n\t.reg .pred p, q;\n\t"
+            "setp.gt.bf16x2 p|q, %1, %2;\n\t"
+            "or.pred p, p, q;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(any) : "r"(max_word(raw)), "r"(best));
+        return any != 0;
+    }
+    __device__ static __forceinline__ float max_of(const uint4 &raw)
+    {
+        const uint32_t m = max_word(raw);
+        return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
+    }
+    // acc + sum 2^(x c + nm) over a vector; acc + sum 2^min(a c + na, b c + nb) over a pair of vectors
+    __device__ static __forceinline__ uint64_t add_exp(uint64_t acc, const uint4 &r, uint64_t c, uint64_t nm)
+    {
+        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc = add_ex2(acc, fma2(pair_of(w[i]), c, nm));
+        return acc;
+    }
+    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb)
+    {
+        const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc = add_ex2_min(acc, fma2(pair_of(wa[i]), c, na), fma2(pair_of(wb[i]), c, nb));
+        return acc;
+    }
 };
 
 template <> struct Logit<float> {
@@ -82,6 +185,25 @@ template <> struct Logit<float> {
         x[3] = __uint_as_float(raw.w);
     }
     __device__ static __forceinline__ float scalar(const float *p, size_t i) { return p[i]; }
+    using Best = float;
+    __device__ static __forceinline__ Best best_of(float x) { return x; }
+    __device__ static __forceinline__ float max_of(const uint4 &raw)
+    {
+        return fmaxf(fmaxf(__uint_as_float(raw.x), __uint_as_float(raw.y)), fmaxf(__uint_as_float(raw.z), __uint_as_float(raw.w)));
+    }
+    __device__ static __forceinline__ bool any_above(const uint4 &raw, Best best) { return max_of(raw) > best; }
+    __device__ static __forceinline__ uint64_t add_exp(uint64_t acc, const uint4 &r, uint64_t c, uint64_t nm)
+    {
+        acc = add_ex2(acc, fma2(pack2(__uint_as_float(r.x), __uint_as_float(r.y)), c, nm));
+        return add_ex2(acc, fma2(pack2(__uint_as_float(r.z), __uint_as_float(r.w)), c, nm));
+    }
+    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb)
+    {
+        acc = add_ex2_min(acc, fma2(pack2(__uint_as_float(a.x), __uint_as_float(a.y)), c, na),
+                          fma2(pack2(__uint_as_float(b.x), __uint_as_float(b.y)), c, nb));
+        return add_ex2_min(acc, fma2(pack2(__uint_as_float(a.z), __uint_as_float(a.w)), c, na),
+                           fma2(pack2(__uint_as_float(b.z), __uint_as_float(b.w)), c, nb));
+    }
 };
 
 // Tokens sequence b drafted this round: the call's k unless the caller registered per-sequence lengths, which are
@@ -182,6 +304,13 @@ __device__ __forceinline__ void second_sweep_offsets(MaxSum a, MaxSum b, float c
 struct ArgMax {
     float v;
     int32_t i;
+};
+
+// What a warp of the staged row-statistics kernel found in its part of a row pair: the reference m of both sums, the
+// sums, the largest target logit and its first index.
+struct WarpRecord {
+    float m, sum_a, sum_b, best;
+    int32_t best_i;
 };
 
 __device__ __forceinline__ ArgMax better(ArgMax a, ArgMax b)

@@ -66,12 +66,14 @@ struct VerifyParams {
     RowStats *stats;   // [batch, k+1]
     uint32_t *status;
     int32_t vector_ok; // rows are 16-byte aligned and a whole number of 16-byte vectors
-    int32_t keep_from_vec;   // first 16-byte vector of a row in the share that the first sweep asks L2 to keep
+    int32_t keep_permille;   // share (its end) of every row that the first sweep asks L2 to keep for the second
+    int32_t keep_from_vec;   // the same as the first 16-byte vector of that share
     uint32_t poll_limit;     // polls after which a wait on an asynchronous copy gives up
     uint32_t table_mask;     // pointer-table mode: low address bits that must be clear in every entry
 };
 
 // streaming path (metasd_streaming.cu, metasd_bulk.cu)
+bool long_row(int dtype, int vocab);   // selects the launch shape: see streaming_prepare
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo);
 cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches);
 cudaError_t bulk_prepare(int dtype, RowGeometry *geo);

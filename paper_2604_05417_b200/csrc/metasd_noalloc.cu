@@ -58,8 +58,8 @@ __global__ void noalloc_prepare_kernel(int batch, int32_t round)
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_lock;
 StaticScratch *g_scratch_ptr[MAX_DEVICES];   // device address of the array on each device, once known
-RowGeometry g_geometry[MAX_DEVICES][2];      // launch shape of the row-statistics kernel per device and logit type
-bool g_geometry_ready[MAX_DEVICES][2];
+RowGeometry g_geometry[MAX_DEVICES][2][2];   // launch shape of the row-statistics kernel per device, logit type, long rows
+bool g_geometry_ready[MAX_DEVICES][2][2];
 
 // Once per device, with that device current: ask the runtime where the array lives there.
 cudaError_t scratch_address(int device, StaticScratch **out)
@@ -75,19 +75,21 @@ cudaError_t scratch_address(int device, StaticScratch **out)
     return cudaSuccess;
 }
 
-// Once per device and logit type: the default launch shape and the function attribute (a larger dynamic
+// Once per device, logit type and class of row length: the default launch shape and the function attribute (a larger dynamic
 // shared-memory window) its kernel needs.  Neither allocates device memory.
-cudaError_t default_geometry(int device, int dtype, RowGeometry *out)
+cudaError_t default_geometry(int device, int dtype, int vocab, RowGeometry *out)
 {
     std::lock_guard<std::mutex> guard(g_setup_lock);
-    if (!g_geometry_ready[device][dtype]) {
+    const int lng = long_row(dtype, vocab) ? 1 : 0;
+    if (!g_geometry_ready[device][dtype][lng]) {
         metasd_config cfg;
         metasd_default_config(&cfg);
-        cudaError_t e = streaming_prepare(device, dtype, cfg, &g_geometry[device][dtype]);
+        cfg.vocab = vocab;
+        cudaError_t e = streaming_prepare(device, dtype, cfg, &g_geometry[device][dtype][lng]);
         if (e != cudaSuccess) return e;
-        g_geometry_ready[device][dtype] = true;
+        g_geometry_ready[device][dtype][lng] = true;
     }
-    *out = g_geometry[device][dtype];
+    *out = g_geometry[device][dtype][lng];
     return cudaSuccess;
 }
 
@@ -116,7 +118,7 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     StaticScratch *scratch = nullptr;
     if (scratch_address(device, &scratch) != cudaSuccess) return METASD_ERR_CUDA;
     RowGeometry geo;
-    if (default_geometry(device, logit_dtype, &geo) != cudaSuccess) return METASD_ERR_CUDA;
+    if (default_geometry(device, logit_dtype, vocab, &geo) != cudaSuccess) return METASD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
     VerifyParams p = {};
@@ -138,7 +140,8 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     p.vector_ok = row_bytes % 16 == 0 && ((uintptr_t)target_logits % 16) == 0 && ((uintptr_t)draft_logits % 16) == 0;
     {   // the share of every row that L2 is asked to keep between the sweeps: as in a default context
         const long long nvec = (long long)row_bytes / 16;
-        p.keep_from_vec = (int32_t)(nvec - nvec * (logit_dtype == METASD_BF16 ? 750 : 900) / 1000);
+        p.keep_permille = logit_dtype == METASD_BF16 ? 750 : 900;
+        p.keep_from_vec = (int32_t)(nvec - nvec * p.keep_permille / 1000);
     }
     p.poll_limit = 1u << 18;
 

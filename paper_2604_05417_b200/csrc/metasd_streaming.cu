@@ -13,6 +13,8 @@
 //                          accept step), first rejection, inverse-CDF draw of the correction token from
 //                          max(0, p - q) or of the bonus token from p (its resampling step), the reward, the
 //                          bandit update and the next round's arm (Algorithm 2, update and selection steps).
+#include <type_traits>
+
 #include "metasd_device.cuh"
 
 namespace metasd {
@@ -157,12 +159,12 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // -------------------------------------------------------------------------------------------
 // K1p
 // -------------------------------------------------------------------------------------------
-// K1 with its loads staged through shared memory.  Every thread copies its own vectors D - 1 trips ahead with
-// cp.async and reads them back when their group has landed; a slot is written and read by the same thread only, so
-// there is no barrier and no register cost.  The second sweep visits the thread's trips in reverse: the last D trips
-// of the first sweep are still in their slots and are not read from memory again, and each slot is refilled with the
-// trip D further down as soon as it has been used.  Vectors and their order per thread in sweep 1 are K1's; in
-// sweep 2 the partition of the row among threads differs from K1's, which only regroups an fp32 sum.
+// K1 with its loads staged through shared memory.  A row is cut into trips of 32 vectors (512 bytes); every warp owns a
+// contiguous range of trips of the row pair and copies its own vectors D - 1 trips ahead with cp.async, one slot per
+// lane and stage; a slot is written and read by the same thread only, so there is no barrier and no register cost.  The
+// second sweep visits the warp's trips in reverse: the last D trips of the first sweep are still in their slots and are
+// not read from memory again, and each slot is refilled with the trip D further down as soon as it has been used.  Lanes
+// behind the end of the row hold -Inf in their slot, which adds nothing to any sum: the loops carry no lane predicate.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t policy)
 {
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
@@ -170,19 +172,77 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// 16 bytes of -Inf logits.
+template <typename LT> __device__ __forceinline__ void fill_neg_inf(uint32_t slot)
+{
+    const uint32_t w = sizeof(LT) == 2 ? 0xFF80FF80u : 0xFF800000u;
+    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(slot), "r"(w) : "memory");
+}
+
+// One warp's running statistics of a row pair.  All lanes share the reference `m` that both rows' sums are relative to and
+// the best target logit `best` (its first index in `best_i`); the sums are the lane's own, two partial sums each.
+template <typename LT> struct WarpSums {
+    uint64_t a, b;        // packed fp32 pairs: sum 2^((x - m) c) of the target and the draft row
+    float m, best;
+    uint64_t nm;          // -m c, twice
+    typename Logit<LT>::Best cmp;   // `best` as the vectors are compared with it
+    int32_t best_i;
+};
+
+// A vector of the target row that holds a larger logit than any before it in the warp's range: rare (a warp's n-th trip
+// brings a new maximum with probability about 1/n), so the whole warp takes this branch together.
+template <typename LT>
+__device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int vec, float c)
+{
+    constexpr int VEC = Logit<LT>::VEC;
+    float x[VEC];
+    Logit<LT>::unpack(raw, x);
+    float cm = x[0];
+#pragma unroll
+    for (int e = 1; e < VEC; ++e) cm = fmaxf(cm, x[e]);
+    const float top = warp_max_f(cm);
+    const bool first_finite = w.best == -INFINITY;   // the reference may still be a stand-in, on either side of `top`
+    if (top > w.m || first_finite) {
+        const uint64_t shrink = pack2(ex2((w.m - top) * c));
+        if (!first_finite) w.a = mul2(w.a, shrink);
+        w.b = mul2(w.b, shrink);
+        w.m = top;
+        w.nm = pack2(-top * c);
+    }
+    int first = 0;
+#pragma unroll
+    for (int e = VEC - 1; e >= 0; --e)
+        if (x[e] == top) first = e;
+    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, cm == top)) - 1;   // lanes are in token order
+    w.best_i = __shfl_sync(0xFFFFFFFFu, vec * VEC + first, src & 31);
+    w.best = top;
+    w.cmp = Logit<LT>::best_of(top);
+}
+
+// What bounds it (bf16, B = 512, k = 8, V = 152064; 2.65 GB): the special-function unit (three exponentials a pair, 80 %
+// busy) and, in a long run, the board's power limit, so instructions and re-read bytes both cost time.  Against one vector
+// per thread and trip strided over the CTA: the warp-wide reference and the packed fp32 pairs take the maximum search, the
+// lane predicates and half the arithmetic instructions out of the loop (109.5 M warp instructions instead of 141.8 M on
+// B = 148), contiguous ranges make a range's pages and its second sweep its own, and six stages at two CTAs per SM keep a
+// third more of a pair on chip between the sweeps than four stages at three CTAs (3.17 GB read instead of 3.39 GB).  A
+// round of that size takes 630 us instead of 664 in a long run on one box; fp32, B = 1024, k = 5, V = 128256 1164 instead of
+// 1261; V = 262144, B = 40, k = 16 218 instead of 232.
 //
-// CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of it.  The CTAs
-// exchange their sweep-1 records through distributed shared memory (every CTA gets every record and merges them in
-// rank order, so all hold the same normalisers), sweep their own part again, and rank 0 adds up the parts of
-// sum min(p, q).  The same number of threads then holds a CL-th of the row pairs in flight.
+// CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
+// of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
+// order, so all hold the same normalisers; each sweeps its part again, and rank 0 adds up the parts of sum min(p, q).
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
     static_assert(D >= 2, "at least two stages");
     constexpr int VEC = Logit<LT>::VEC;
-    constexpr int NWARP = THREADS / 32;
+    constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
     constexpr uint32_t ROW_STRIDE = THREADS * 16, STAGE_STRIDE = 2 * ROW_STRIDE;
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
     extern __shared__ __align__(16) unsigned char stage_mem[];   // [D][2 rows][THREADS] 16-byte slots
+    __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
+    __shared__ MaxSum sh_redo[NREC];
+    __shared__ double sh_min[NREC];
     launch_dependents();   // the epilogue may be set up while this kernel runs; it waits for the whole grid before it reads
     // Blocks are dispatched in index order.  BONUS_LAST: the row pairs come first and the bonus rows (one row, half
     // the work) last, so that the launch ends on its shortest items (measured: better for the bf16 geometry, worse
@@ -193,7 +253,8 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     const int b = BONUS_LAST ? (unit < first_bonus ? unit / p.k : unit - first_bonus) : unit / (p.k + 1);
     const int kb = drafted(p.draft_len, b, p.k);
     const int j = BONUS_LAST ? (unit < first_bonus ? unit - b * p.k : kb) : unit - b * (p.k + 1);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(FULL, tid >> 5, 0);              // the same in every lane, and known to be
     const float c = p.c;
     // nothing to do behind the sequence's bonus row; with BONUS_LAST the bonus row belongs to its own late block
     // (the same for every CTA of a cluster: none of them reaches a cluster barrier)
@@ -202,153 +263,149 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // a peer's shared memory may be written once that peer is running: every CTA says so here and checks it after sweep 1
     if (CL > 1) cluster_arrive();
 
-    const int nvec_row = p.V / VEC;
-    const int v_lo = (int)((long long)nvec_row * rank / CL), v_hi = (int)((long long)nvec_row * (rank + 1) / CL);
-    const uint4 *a4 = reinterpret_cast<const uint4 *>(reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V) + v_lo;
-    const uint4 *d4 = pair ? reinterpret_cast<const uint4 *>(draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V) + v_lo : nullptr;
-    const int nvec = v_hi - v_lo;   // vectors of this CTA, numbered from 0
-    const int n_trip = tid < nvec ? (nvec - tid + THREADS - 1) / THREADS : 0;   // vectors of this thread
+    const int nvec = p.V / VEC;
+    const int trips_row = (nvec + 31) >> 5;
+    const int part = rank * NWARP + warp;                         // this warp's part of the row's trips
+    const int g0 = (int)((long long)trips_row * part / NREC), n_trip = (int)((long long)trips_row * (part + 1) / NREC) - g0;
+    const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
+    const uint4 *a4 = reinterpret_cast<const uint4 *>(reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V) + v0;
+    const uint4 *d4 = pair ? reinterpret_cast<const uint4 *>(draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V) + v0 : a4;
     const uint32_t slot0 = smem_addr(stage_mem) + (uint32_t)tid * 16u;
+    // trips in which this lane is inside the row, and in which every lane is: only the row's last trip may be ragged
+    const int lane_trips = v0 + 32 * (n_trip - 1) < nvec ? n_trip : n_trip - 1;
+    const int n_full = (g0 + n_trip) * 32 <= nvec ? n_trip : n_trip - 1;
 
-    // ---- sweep 1: online (max, sum) of the target row and its arg-max; the draft row's sum is taken relative to
+    // ---- sweep 1: sums of both rows and the arg-max of the target row.  The draft row's sum is taken relative to
     // the SAME running reference (the target's maximum so far): a softmax sum may be taken relative to any
     // reference that neither overflows nor underflows it, and sharing one spares the draft row its own maximum
-    // search (the kernel is bound by instruction issue).  Whether the reference suited the draft row is checked
-    // after the sweep; if not, that row's statistics are redone relative to its own maximum.
-    MaxSum sa = {METASD_NEG_BIG, 0.f}, sb = {METASD_NEG_BIG, 0.f};
-    ArgMax am = {METASD_NEG_BIG, 0x7FFFFFFF};
+    // search.  Whether the reference suited the draft row is checked after the sweep; if not, that row's statistics are
+    // redone relative to its own maximum.
     // a bonus row is read once: nothing of it is worth keeping in L2
     const uint64_t drop = l2_policy_evict_first(), keep = pair ? l2_policy_evict_last() : drop;
-    const int keep_from = p.keep_from_vec / CL;   // first 16-byte vector of this CTA's part that L2 is asked to keep
-    // One group of copies per call, empty past the end: the group count stays in step with the trips.
-    auto request1 = [&](int m, int slot, uint64_t pol) {
-        if (m < n_trip) {
-            const int i = tid + m * THREADS;
-            const uint32_t dst = slot0 + (uint32_t)slot * STAGE_STRIDE;
-            cp_async16(dst, a4 + i, pol);
-            if (pair) cp_async16(dst + ROW_STRIDE, d4 + i, pol);
-        }
-        cp_async_commit();
-    };
-    // Trip n of sweep 1 (its vectors sit in slot n mod D): first ask for the trip D - 1 ahead.
-    auto trip1 = [&](int n, int slot, uint64_t pol) {
-        request1(n + D - 1, (slot + D - 1) % D, pol);
-        cp_async_wait<D - 1>();   // all but the D - 1 youngest groups have landed: trip n's is among them
-        const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
-        const int i = tid + n * THREADS;
-        float xa[VEC];
-        Logit<LT>::unpack(lds16(src), xa);
-        float cm = xa[0];
-#pragma unroll
-        for (int e = 1; e < VEC; ++e) cm = fmaxf(cm, xa[e]);
-        if (cm > sa.m) {
-            const float shrink = ex2((sa.m - cm) * c);
-            sa.s *= shrink;
-            sb.s *= shrink;
-            sa.m = cm;
-            int first = 0;
-#pragma unroll
-            for (int e = VEC - 1; e >= 0; --e)
-                if (xa[e] == cm) first = e;
-            am.v = cm;
-            am.i = (v_lo + i) * VEC + first;
-        }
-        const float nma = -sa.m * c;
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) sa.s += ex2(fmaf(xa[e], c, nma));
-        if (pair) {
-            float xb[VEC];
-            Logit<LT>::unpack(lds16(src + ROW_STRIDE), xb);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) sb.s += ex2(fmaf(xb[e], c, nma));
-        }
-    };
-    // The trips run in groups of D so that the slot of every copy and read is a constant, and in two phases so that
-    // the L2 policy is one too: requests below the kept share of the row ask L2 to drop the line, the rest to keep it
-    // (the boundary is rounded down to a whole group: a few vectors more are kept).
-    const int m_keep = keep_from > tid ? (keep_from - tid + THREADS - 1) / THREADS : 0;   // first request that is kept
-    const int groups = n_trip / D;
-    int groups_drop = (m_keep - (D - 1)) / D;
-    groups_drop = groups_drop < 0 ? 0 : (groups_drop > groups ? groups : groups_drop);
-#pragma unroll
-    for (int m = 0; m < D - 1; ++m) request1(m, m, m >= m_keep ? keep : drop);
-    int n = 0;
-    for (int g = 0; g < groups_drop; ++g, n += D) {
-#pragma unroll
-        for (int u = 0; u < D; ++u) trip1(n + u, u, drop);
-    }
-    for (int g = groups_drop; g < groups; ++g, n += D) {
-#pragma unroll
-        for (int u = 0; u < D; ++u) trip1(n + u, u, keep);
-    }
-#pragma unroll
-    for (int u = 0; u < D - 1; ++u)
-        if (n + u < n_trip) trip1(n + u, u, keep);
-    cp_async_wait<0>();
-    if (CL > 1) cluster_wait();
-    sb.m = sa.m;   // the draft row's sum is relative to the target row's maximum
-
-    __shared__ MaxSum sh_a[NWARP], sh_b[NWARP];
-    __shared__ ArgMax sh_am[NWARP];
-    __shared__ double sh_min[NWARP];
-    __shared__ float sh_bcast[7];
-
-    // records of the cluster's CTAs, written by their owners: of sweep 1, of a redone draft row, of sweep 2
-    __shared__ float sh_xrec[CL][6];
-    __shared__ float sh_xredo[CL][2];
-    __shared__ double sh_xmin[CL];
-
-    sa = warp_merge(sa, c);
-    sb = warp_merge(sb, c);
-    am = warp_argmax(am);
-    if (lane == 0) { sh_a[warp] = sa; sh_b[warp] = sb; sh_am[warp] = am; }
-    __syncthreads();
-    if (warp == 0) {
-        MaxSum ra = lane < NWARP ? sh_a[lane] : MaxSum{METASD_NEG_BIG, 0.f};
-        MaxSum rb = lane < NWARP ? sh_b[lane] : MaxSum{METASD_NEG_BIG, 0.f};
-        ArgMax rm = lane < NWARP ? sh_am[lane] : ArgMax{METASD_NEG_BIG, 0x7FFFFFFF};
-        ra = warp_merge(ra, c);
-        rb = warp_merge(rb, c);
-        rm = warp_argmax(rm);
-        if (CL > 1) {
-            // lane r hands this CTA's record to the CTA of rank r (every lane holds the merged values)
-            if (lane < CL) {
-                const uint32_t dst = map_to_rank(smem_addr(&sh_xrec[rank][0]), (uint32_t)lane);
-                st_cluster(dst, __float_as_int(ra.m));      st_cluster(dst + 4, __float_as_int(ra.s));
-                st_cluster(dst + 8, __float_as_int(rb.m));  st_cluster(dst + 12, __float_as_int(rb.s));
-                st_cluster(dst + 16, __float_as_int(rm.v)); st_cluster(dst + 20, rm.i);
+    WarpSums<LT> w;
+    w.a = w.b = 0ull;
+    w.m = 0.f;
+    w.nm = 0ull;
+    w.best = -INFINITY;
+    w.cmp = Logit<LT>::best_of(-INFINITY);
+    w.best_i = 0x7FFFFFFF;
+    const uint64_t c2 = pack2(c);
+    // Requests below the kept share of the warp's range ask L2 to drop the line, the rest to keep it for sweep 2.
+    const int m_keep = n_trip - (int)((long long)n_trip * p.keep_permille / 1000);
+    // BOTH: a row pair; else a bonus row.
+    auto sweep1 = [&](auto both_tag) {
+        constexpr bool BOTH = decltype(both_tag)::value;
+        // One group of copies per trip, empty past the end: the group count stays in step with the trips.
+        auto request = [&](uint32_t dst, const uint4 *a, const uint4 *d, uint64_t pol) {
+            cp_async16(dst, a, pol);
+            if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
+            cp_async_commit();
+        };
+        auto request_checked = [&](int m, uint32_t dst) {
+            if (m < lane_trips) {
+                request(dst, a4 + 32 * m, d4 + 32 * m, m >= m_keep ? keep : drop);
+            } else {
+                if (m < n_trip) {
+                    fill_neg_inf<LT>(dst);
+                    fill_neg_inf<LT>(dst + ROW_STRIDE);
+                }
+                cp_async_commit();
             }
-        } else if (lane == 0) {
-            sh_bcast[0] = ra.m; sh_bcast[1] = ra.s; sh_bcast[2] = rb.m; sh_bcast[3] = rb.s;
-            second_sweep_offsets(ra, rb, c, sh_bcast + 4);
-            sh_am[0] = rm;
+        };
+        auto consume = [&](int n, uint32_t src) {
+            cp_async_wait<D - 1>();   // all but the D - 1 youngest groups have landed: trip n's is among them
+            const uint4 ra = lds16(src);
+            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT>(w, ra, v0 + 32 * n, c);
+            w.a = Logit<LT>::add_exp(w.a, ra, c2, w.nm);
+            if (BOTH) w.b = Logit<LT>::add_exp(w.b, lds16(src + ROW_STRIDE), c2, w.nm);
+        };
+#pragma unroll
+        for (int m = 0; m < D - 1; ++m) request_checked(m, slot0 + (uint32_t)m * STAGE_STRIDE);
+        // The first reference: the maximum of the warp's first trip.  Where the target's logits are all masked there, the
+        // draft row's (or 0) stands in, so that the draft row's sum does not overflow.
+        if (n_trip > 0) {
+            cp_async_wait<D - 2>();
+            w.m = warp_max_f(Logit<LT>::max_of(lds16(slot0)));
+            if (!(w.m > METASD_NEG_BIG)) {
+                w.m = BOTH ? warp_max_f(Logit<LT>::max_of(lds16(slot0 + ROW_STRIDE))) : 0.f;
+                if (!(w.m > METASD_NEG_BIG)) w.m = 0.f;
+            }
+            w.nm = pack2(-w.m * c);
         }
-    }
+        // Trip n asks for the trip D - 1 ahead, then works on its own vectors (slot n mod D).  Groups of D trips whose
+        // requests all lie inside the row carry no checks, and their slots and their L2 policy are constants (the boundary
+        // of the kept share is rounded down to a whole group: a few vectors more are kept).
+        int n = 0;
+        const uint4 *a_next = a4 + 32 * (D - 1), *d_next = d4 + 32 * (D - 1);
+        auto group = [&](uint64_t pol) {
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                request(slot0 + (uint32_t)((u + D - 1) % D) * STAGE_STRIDE, a_next + 32 * u, d_next + 32 * u, pol);
+                consume(n + u, slot0 + (uint32_t)u * STAGE_STRIDE);
+            }
+            n += D;
+            a_next += 32 * D;
+            d_next += 32 * D;
+        };
+        while (n + 2 * D - 2 < min(m_keep, n_full)) group(drop);
+        while (n + 2 * D - 2 < n_full) group(keep);
+        for (int slot = 0, ask = D - 1; n < n_trip; ++n) {
+            request_checked(n + D - 1, slot0 + (uint32_t)ask * STAGE_STRIDE);
+            consume(n, slot0 + (uint32_t)slot * STAGE_STRIDE);
+            ask = slot;
+            slot = slot + 1 == D ? 0 : slot + 1;
+        }
+        cp_async_wait<0>();
+    };
+    if (pair) sweep1(std::true_type{});
+    else sweep1(std::false_type{});
+
+    // ---- the warps' records, merged by every warp for itself (no second barrier)
+    const float sum_aw = warp_sum_f(sum2(w.a)), sum_bw = warp_sum_f(sum2(w.b));
     if (CL > 1) {
-        cluster_sync_all();   // every CTA's record has arrived in every CTA
-        if (tid == 0) {
-            MaxSum ra = {sh_xrec[0][0], sh_xrec[0][1]}, rb = {sh_xrec[0][2], sh_xrec[0][3]};
-            ArgMax rm = {sh_xrec[0][4], __float_as_int(sh_xrec[0][5])};
-            for (int r = 1; r < CL; ++r) {
-                ra = merge(ra, MaxSum{sh_xrec[r][0], sh_xrec[r][1]}, c);
-                rb = merge(rb, MaxSum{sh_xrec[r][2], sh_xrec[r][3]}, c);
-                rm = better(rm, ArgMax{sh_xrec[r][4], __float_as_int(sh_xrec[r][5])});
-            }
-            sh_bcast[0] = ra.m; sh_bcast[1] = ra.s; sh_bcast[2] = rb.m; sh_bcast[3] = rb.s;
-            second_sweep_offsets(ra, rb, c, sh_bcast + 4);
-            sh_am[0] = rm;
+        cluster_wait();   // every CTA of the cluster is running
+        if (lane < CL) {
+            const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane);
+            st_cluster(dst, __float_as_int(w.m));           st_cluster(dst + 4, __float_as_int(sum_aw));
+            st_cluster(dst + 8, __float_as_int(sum_bw));    st_cluster(dst + 12, __float_as_int(w.best));
+            st_cluster(dst + 16, w.best_i);
+        }
+        cluster_sync_all();
+    } else {
+        if (lane == 0) sh_rec[warp] = WarpRecord{w.m, sum_aw, sum_bw, w.best, w.best_i};
+        __syncthreads();
+    }
+    MaxSum ra = {METASD_NEG_BIG, 0.f}, rb = {METASD_NEG_BIG, 0.f};
+    ArgMax rm = {-INFINITY, 0x7FFFFFFF};
+#pragma unroll
+    for (int r0 = 0; r0 < NREC; r0 += 32) {
+        if (NREC - r0 >= 32 || lane < NREC - r0) {
+            const WarpRecord r = sh_rec[r0 + lane];
+            // a part whose target logits are all masked has a stand-in for its reference and nothing in sum_a
+            const MaxSum pa = {r.best > -INFINITY ? r.m : METASD_NEG_BIG, r.sum_a};
+            const MaxSum pb = {r.sum_b == 0.f ? METASD_NEG_BIG : r.m, r.sum_b};
+            ra = r0 ? merge(ra, pa, c) : pa;
+            rb = r0 ? merge(rb, pb, c) : pb;
+            rm = better(rm, ArgMax{r.best, r.best_i});
         }
     }
-    __syncthreads();
+    {
+        const float top = warp_max_f(ra.m);     // both sums end up relative to the target row's maximum
+        ra.s = warp_sum_f(ra.s * ex2((ra.m - top) * c));
+        rb.s = warp_sum_f(rb.s * ex2((rb.m - top) * c));
+        ra.m = rb.m = top;
+        const float best = warp_max_f(rm.v);
+        rm.i = __reduce_min_sync(FULL, rm.v == best ? rm.i : 0x7FFFFFFF);
+        rm.v = best;
+    }
     // The shared reference suits the draft row when its sum is neither flushed nor overflowed: 2^-60 .. finite
     // leaves every term that matters in fp32 range.  Otherwise (draft logits far from the target's, or a row
     // that is not finite) the draft row is swept again relative to its own running maximum.
-    if (pair && !(sh_bcast[3] >= 0x1p-60f && sh_bcast[3] < INFINITY)) {
-        __syncthreads();   // everybody has read the first verdict
+    if (pair && !(rb.s >= 0x1p-60f && rb.s < INFINITY)) {
         MaxSum own = {METASD_NEG_BIG, 0.f};
-        for (int i = tid; i < nvec; i += THREADS) {
+        for (int n = 0; n < lane_trips; ++n) {
             float xb[VEC];
-            Logit<LT>::unpack(ld_stream(d4 + i), xb);
+            Logit<LT>::unpack(ld_stream(d4 + 32 * n), xb);
             float bm = xb[0];
 #pragma unroll
             for (int e = 1; e < VEC; ++e) bm = fmaxf(bm, xb[e]);
@@ -361,94 +418,89 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             for (int e = 0; e < VEC; ++e) own.s += ex2(fmaf(xb[e], c, nmb));
         }
         own = warp_merge(own, c);
-        if (lane == 0) sh_b[warp] = own;
-        __syncthreads();
-        if (warp == 0) {
-            MaxSum rb = lane < NWARP ? sh_b[lane] : MaxSum{METASD_NEG_BIG, 0.f};
-            rb = warp_merge(rb, c);
-            if (CL > 1) {
-                if (lane < CL) {
-                    const uint32_t dst = map_to_rank(smem_addr(&sh_xredo[rank][0]), (uint32_t)lane);
-                    st_cluster(dst, __float_as_int(rb.m));
-                    st_cluster(dst + 4, __float_as_int(rb.s));
-                }
-            } else if (lane == 0) {
-                sh_bcast[2] = rb.m; sh_bcast[3] = rb.s;
-                second_sweep_offsets(MaxSum{sh_bcast[0], sh_bcast[1]}, rb, c, sh_bcast + 4);
-            }
-        }
         if (CL > 1) {
-            cluster_sync_all();   // the verdict above came from the merged records: every CTA of the cluster is here
-            if (tid == 0) {
-                MaxSum rb = {sh_xredo[0][0], sh_xredo[0][1]};
-                for (int r = 1; r < CL; ++r) rb = merge(rb, MaxSum{sh_xredo[r][0], sh_xredo[r][1]}, c);
-                sh_bcast[2] = rb.m; sh_bcast[3] = rb.s;
-                second_sweep_offsets(MaxSum{sh_bcast[0], sh_bcast[1]}, rb, c, sh_bcast + 4);
+            if (lane < CL) {
+                const uint32_t dst = map_to_rank(smem_addr(&sh_redo[part]), (uint32_t)lane);
+                st_cluster(dst, __float_as_int(own.m));
+                st_cluster(dst + 4, __float_as_int(own.s));
             }
+            cluster_sync_all();   // the verdict above came from the merged records: every CTA of the cluster is here
+        } else {
+            if (lane == 0) sh_redo[warp] = own;
+            __syncthreads();
         }
-        __syncthreads();
+        rb = MaxSum{METASD_NEG_BIG, 0.f};
+        for (int r = lane; r < NREC; r += 32) rb = merge(rb, sh_redo[r], c);
+        rb = warp_merge(rb, c);
     }
-    const float max_a = sh_bcast[0], sum_a = sh_bcast[1], max_b = sh_bcast[2], sum_b = sh_bcast[3];
 
-    // ---- sweep 2, this thread's trips in reverse: sum_v 2^min(ya_v, yb_v), one exponential per pair
+    // ---- sweep 2, this warp's trips in reverse: sum_v 2^min(ya_v, yb_v), one exponential per pair
     double total_min = 0.0;
     if (pair) {
-        const float nma = sh_bcast[4], nmb = sh_bcast[5], ia = sh_bcast[6];
-        float acc = 0.f;
-        // Trip n of sweep 2 from its slot; the slot is then refilled with the trip D further down.
-        auto trip2 = [&](int n, int slot) {
+        float offs[3];
+        second_sweep_offsets(ra, rb, c, offs);
+        const uint64_t nma = pack2(offs[0]), nmb = pack2(offs[1]);
+        uint64_t acc = 0ull;
+        // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
+        // every lane: the ragged trip is the row's last).
+        auto consume = [&](uint32_t src) {
             // the first D trips are still in their slots from sweep 1; the group of a later one was committed D trips
             // ago, so at most D - 1 younger groups may still be pending
             cp_async_wait<D - 1>();
-            const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
-            float xa[VEC], xb[VEC];
-            Logit<LT>::unpack(lds16(src), xa);
-            Logit<LT>::unpack(lds16(src + ROW_STRIDE), xb);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e)
-                acc += ex2(fminf(fmaf(xa[e], c, nma), fmaf(xb[e], c, nmb)));
-            if (n >= D) {   // refill the slot just used with the trip D further down
-                const int i = tid + (n - D) * THREADS;
-                cp_async16(src, a4 + i, drop);
-                cp_async16(src + ROW_STRIDE, d4 + i, drop);
-            }
-            cp_async_commit();
+            acc = Logit<LT>::add_exp_min(acc, lds16(src), lds16(src + ROW_STRIDE), c2, nma, nmb);
+        };
+        auto refill = [&](uint32_t dst, const uint4 *a, const uint4 *d) {
+            cp_async16(dst, a, drop);
+            cp_async16(dst + ROW_STRIDE, d, drop);
         };
         // the ragged top first, then whole groups downwards with constant slots
         int n = n_trip - 1;
-        for (; n >= 0 && (n + 1) % D != 0; --n) trip2(n, n % D);
+        for (int slot = n % D; n >= 0 && slot != D - 1; --n) {
+            const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
+            consume(src);
+            if (n >= D) refill(src, a4 + 32 * (n - D), d4 + 32 * (n - D));
+            cp_async_commit();
+            slot = slot == 0 ? D - 1 : slot - 1;
+        }
+        const uint4 *a_next = a4 + 32 * (n - D), *d_next = d4 + 32 * (n - D);
         for (; n >= D; n -= D) {   // n + 1 is a multiple of D and a whole group lies below: every refill is real
 #pragma unroll
-            for (int u = 0; u < D; ++u) trip2(n - u, D - 1 - u);
+            for (int u = 0; u < D; ++u) {
+                const uint32_t src = slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE;
+                consume(src);
+                refill(src, a_next - 32 * u, d_next - 32 * u);
+                cp_async_commit();
+            }
+            a_next -= 32 * D;
+            d_next -= 32 * D;
         }
         if (n >= 0) {
 #pragma unroll
-            for (int u = 0; u < D; ++u) trip2(n - u, D - 1 - u);
-        }
-        cp_async_wait<0>();
-        double w = warp_sum((double)(acc * ia));
-        if (lane == 0) sh_min[warp] = w;
-        __syncthreads();
-        if (tid == 0) {
-            for (int i = 0; i < NWARP; ++i) total_min += sh_min[i];
-            if (CL > 1) st_cluster(map_to_rank(smem_addr(&sh_xmin[rank]), 0u), total_min);
-        }
-        if (CL > 1) {
-            cluster_sync_all();   // rank 0 holds every part; no CTA leaves while a peer may still write to it
-            if (tid == 0) {
-                total_min = 0.0;
-                for (int r = 0; r < CL; ++r) total_min += sh_xmin[r];
+            for (int u = 0; u < D; ++u) {
+                consume(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
+                cp_async_commit();
             }
         }
+        cp_async_wait<0>();
+        const double part_min = warp_sum((double)(sum2(acc) * offs[2]));
+        if (CL > 1) {
+            if (lane == 0) st_cluster(map_to_rank(smem_addr(&sh_min[part]), 0u), part_min);
+            cluster_sync_all();   // rank 0 holds every part; no CTA leaves while a peer may still write to it
+        } else {
+            if (lane == 0) sh_min[warp] = part_min;
+            __syncthreads();
+        }
+        if (tid == 0)
+            for (int i = 0; i < NREC; ++i) total_min += sh_min[i];
     }
 
     if (tid == 0 && rank == 0) {
         RowStats r;
-        r.max_a = max_a; r.sum_a = sum_a; r.max_b = max_b; r.sum_b = sum_b;
-        r.argmax_a = sh_am[0].i;
+        r.max_a = ra.m; r.sum_a = ra.s; r.max_b = rb.m; r.sum_b = rb.s;
+        r.argmax_a = rm.i;
         uint32_t flags = 0;
-        const bool bad_a = !(sum_a > 0.f) || !(sum_a < INFINITY) || !(max_a < INFINITY);
-        const bool bad_b = pair && (!(sum_b > 0.f) || !(sum_b < INFINITY) || !(max_b < INFINITY));
+        const bool bad_a = !(ra.s > 0.f) || !(ra.s < INFINITY) || !(rm.v < INFINITY);
+        const bool bad_b = pair && (!(rb.s > 0.f) || !(rb.s < INFINITY) || !(rb.m < INFINITY));
         if (bad_a || bad_b) flags |= METASD_STATUS_NONFINITE;
         r.sum_min = flags ? 0.0 : total_min;
         r.flags = flags;
@@ -902,7 +954,7 @@ __global__ void __launch_bounds__(K2_THREADS, 1024 / K2_THREADS) epilogue_kernel
 // -------------------------------------------------------------------------------------------
 // The built shapes of the staged kernel, per logit type: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).
 #define METASD_STAGED_SHAPES(X) \
-    X(512, 4, 3, true, 1) X(1024, 6, 1, false, 1) X(1024, 4, 1, true, 1) X(768, 4, 2, true, 1) X(384, 4, 4, true, 1) \
+    X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(1024, 6, 1, false, 1) X(1024, 4, 1, true, 1) X(768, 4, 2, true, 1) X(384, 4, 4, true, 1) \
     X(512, 4, 3, true, 3) X(512, 4, 3, true, 2) X(768, 4, 2, true, 2)
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
@@ -931,9 +983,15 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
     return cudaErrorNotSupported;
 }
 
+// Whether a row is so long that a larger share of the pair kept on chip pays for fewer row pairs in flight.  Measured on
+// B200, us a round at k = 5 (bf16: 512 threads with 4 stages at 3 CTAs per SM / 6 stages at 2 CTAs; fp32: 512 threads with
+// 6 stages at 2 CTAs per SM / 1024 threads with 6 stages at 1):
+//   bf16, B = 256: V = 32000 71 / 74, 50264 95 / 100, 64000 110 / 112, 80000 132 / 131, 96000 152 / 149, 112000 174 / 169
+//   fp32: B = 256, V = 32000 89 / 107, 64000 167 / 168; B = 64, V = 128256 130 / 121
+// Short rows want more of them in flight: the fixed part of a CTA's life is what they cost.
+bool long_row(int dtype, int vocab) { return dtype == METASD_BF16 ? vocab >= 80000 : vocab >= 64000; }
+
 // Resolves the row-statistics shape for a context and sets the launch attributes its kernels need, once.
-// Measured on B200: bf16 rows (8 logits per 16 bytes) are bound by arithmetic as much as by memory, fp32 rows (4 logits
-// per 16 bytes) by memory: they want few row pairs in flight and a large share of each kept in shared memory.
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo)
 {
     cudaError_t e = cudaDeviceGetAttribute(&geo->n_sm, cudaDevAttrMultiProcessorCount, device);
@@ -957,8 +1015,9 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         return bulk_prepare(dtype, geo);
     }
     if (geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;
-    if (!geo->threads) geo->threads = dtype == METASD_BF16 ? 512 : 1024;
-    if (!geo->stages) geo->stages = dtype == METASD_BF16 ? 4 : 6;
+    const bool lng = long_row(dtype, cfg.vocab);
+    if (!geo->threads) geo->threads = dtype == METASD_FP32 && lng ? 1024 : 512;
+    if (!geo->stages) geo->stages = dtype == METASD_BF16 && !lng && geo->threads == 512 ? 4 : 6;
     geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, &geo->per_sm)
                                 : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, &geo->per_sm);

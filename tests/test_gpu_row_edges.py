@@ -1,0 +1,52 @@
+"""Row-statistics kernels at the edges of their tiles: lengths around whole trips and whole groups of trips per warp, and
+masked stretches that leave a warp without a finite logit.  Oracle: the float64 CPU implementation.  The 1e-5 bound on
+every probability is the lock-step harness's (2^-22 exponentials, fp32 sums of at most a few hundred terms per lane)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_05417_b200 import binding as M
+from paper_2604_05417_b200.workloads import RoundGenerator, Workload
+
+pytestmark = pytest.mark.gpu
+
+
+def workload(**kw):
+    d = dict(name="t", B=3, N=2, k=2, V=1024, rounds=2, temperature=1.0, dtype="bf16", bandit="ucb", sigmas=(0.5, 2.0))
+    d.update(kw)
+    return Workload(**d)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [8, 248, 256, 264, 4088, 4096, 4104, 6 * 4096, 6 * 4096 + 8, 11 * 4096, 12 * 4096 - 8, 12 * 4096 + 264])
+def test_row_lengths_at_the_edges_of_trips_and_groups(dtype, V):
+    from _harness import run_lockstep
+    c = run_lockstep(workload(V=V, dtype=dtype), rounds=3, seed=V % 83, path=M.PATH_STREAMING)
+    assert c["rounds"] == 3 and c["status"] == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("shift", [0.0, 120.0, -120.0])
+def test_masked_stretches_cover_whole_warps(dtype, shift):
+    """Target and / or draft logits of whole ranges of the vocabulary are -inf, the draft row on another scale."""
+    from _harness import make_pair, compare_round
+    V = 3 * 4096 + 40
+    wl = workload(V=V, dtype=dtype, B=6)
+    rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=9).gathered_round(0, np.zeros(6, dtype=np.int64))
+    target, draft = rd["target"].clone(), (rd["draft"].float() + shift).to(rd["draft"].dtype)
+    ninf = float("-inf")
+    target[0, :, : V // 2] = ninf
+    target[1, :, V // 2:] = ninf
+    draft[1, :, : V // 4] = ninf
+    target[2, :, :-3] = ninf
+    draft[3, :, : V - 9] = ninf
+    target[4, :, 3:] = ninf
+    draft[4, :, : V // 3] = ninf
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    try:
+        res = gpu.verify(target, draft, rd["tokens"], 1.0, 3, want_diag=True)
+        out = orc.verify(target, draft, rd["tokens"].cpu().numpy(), 1.0, 3)
+        compare_round(res, out, target, draft, 1.0, 1.0, {})
+        assert gpu.last_status() & M.STATUS_NONFINITE == 0
+    finally:
+        gpu.close()
