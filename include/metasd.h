@@ -13,9 +13,9 @@
  *
  * Conventions
  *   - Every pointer is a DEVICE pointer unless the parameter name starts with host_.
- *   - Logit tensors are dense, row-major, innermost dimension V (the vocabulary).  Rows whose
- *     byte length and base address are multiples of 16 take the vectorised path; anything else
- *     is still correct through a scalar path.
+ *   - Logit tensors are dense, row-major, innermost dimension V (the vocabulary), aligned to their
+ *     element size.  Rows may start anywhere: where they start off a 16-byte boundary (an odd
+ *     vocabulary) the row-statistics kernel realigns them on chip.
  *   - The caller owns every input and output buffer.  The library owns the context, the bandit
  *     state and its scratch; nothing is allocated after metasd_init.
  *   - Calls are asynchronous on the CUDA stream passed as `stream` (a cudaStream_t, typed void*
@@ -68,8 +68,8 @@ enum metasd_bandit {
 };
 enum metasd_reward { METASD_REWARD_BD = 0, METASD_REWARD_BE = 1 };
 
-/* How the row-statistics kernel of the streaming path brings logit rows on chip (16-byte aligned rows; rows
- * that are not take plain scalar loads whatever is asked for). */
+/* How the row-statistics kernel of the streaming path brings logit rows on chip (rows off a
+ * 16-byte boundary: the staged variant, else plain scalar loads). */
 enum metasd_row_kernel {
     METASD_ROWS_AUTO = 0,    /* the fastest measured variant for the dtype */
     METASD_ROWS_PLAIN = 1,   /* ld.global straight into registers */
@@ -250,8 +250,8 @@ int metasd_resolved_row_kernel(const metasd_ctx *ctx);
  * latency-critical thread that must stay clear of the allocator.  Such callers cannot create a
  * context, so there is no bandit here and nothing persists between calls.)
  *
- * It launches the kernels of a default streaming context (the staged row-statistics kernel for 16-byte aligned
- * rows, the plain-load one otherwise, then the epilogue).  Their scratch lives in a fixed array inside the library image (about 0.7 MB, held
+ * It launches the kernels of a default streaming context (the staged row-statistics kernel, then the
+ * epilogue).  Their scratch lives in a fixed array inside the library image (about 0.7 MB, held
  * by every GPU that loads the library until the process exits), which bounds the sizes:
  * batch <= METASD_NOALLOC_MAX_BATCH and batch * (k + 1) <= METASD_NOALLOC_MAX_ROWS; beyond that the
  * call returns METASD_ERR_UNSUPPORTED and launches nothing.  The call makes no cudaMalloc / cudaFree

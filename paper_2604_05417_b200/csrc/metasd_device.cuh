@@ -124,6 +124,34 @@ template <> struct Logit<__nv_bfloat16> {
     {
         return __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(p)[i] << 16);
     }
+    // The vector of tokens tok0 .. tok0 + 7 with -Inf in the place of tokens outside [0, V).
+    __device__ static __forceinline__ uint4 masked(const uint4 &r, int tok0, int V)
+    {
+        uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (tok0 + 2 * i < 0 || tok0 + 2 * i >= V) w[i] = (w[i] & 0xFFFF0000u) | 0xFF80u;
+            if (tok0 + 2 * i + 1 < 0 || tok0 + 2 * i + 1 >= V) w[i] = (w[i] & 0xFFFFu) | 0xFF800000u;
+        }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __device__ static __forceinline__ void put_scalar(uint32_t addr, const __nv_bfloat16 *row, int i)
+    {
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(reinterpret_cast<const uint16_t *>(row)[i]) : "memory");
+    }
+    // The eight logits that start `shift` (0 .. 7) logits into lo, hi laid end to end.
+    __device__ static __forceinline__ uint4 shifted(const uint4 &lo, const uint4 &hi, int shift)
+    {
+        uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = shift & 4 ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = shift & 2 ? w[i + 1] : w[i];
+        const uint32_t sel = shift & 1 ? 0x5432u : 0x3210u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = __byte_perm(w[i], w[i + 1], sel);
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
     // the two logits of a 32-bit word
     __device__ static __forceinline__ uint64_t pair_of(uint32_t w)
     {
@@ -185,6 +213,27 @@ template <> struct Logit<float> {
         x[3] = __uint_as_float(raw.w);
     }
     __device__ static __forceinline__ float scalar(const float *p, size_t i) { return p[i]; }
+    __device__ static __forceinline__ uint4 masked(const uint4 &r, int tok0, int V)
+    {
+        uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (tok0 + i < 0 || tok0 + i >= V) w[i] = 0xFF800000u;
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __device__ static __forceinline__ void put_scalar(uint32_t addr, const float *row, int i)
+    {
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(row[i]) : "memory");
+    }
+    __device__ static __forceinline__ uint4 shifted(const uint4 &lo, const uint4 &hi, int shift)
+    {
+        uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = shift & 2 ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = shift & 1 ? w[i + 1] : w[i];
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
     using Best = float;
     __device__ static __forceinline__ Best best_of(float x) { return x; }
     __device__ static __forceinline__ float max_of(const uint4 &raw)
@@ -430,6 +479,11 @@ __device__ __forceinline__ uint4 lds16(uint32_t addr)
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void sts16(uint32_t addr, const uint4 &v)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
 // Programmatic dependent launch: lets the next kernel in the stream be set up while this grid still runs.  That

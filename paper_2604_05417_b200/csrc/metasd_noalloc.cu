@@ -9,8 +9,8 @@
 //
 // The round it runs is the stateless part of metasd_verify: softmax statistics, accept tests, first
 // rejection, correction/bonus draw and the reward, launched as the two streaming kernels a context
-// with the default configuration launches for the same logit type (the staged row-statistics kernel
-// for 16-byte aligned rows, the plain-load one otherwise, then the epilogue).  There is no bandit here
+// with the default configuration launches for the same logit type (the staged row-statistics kernel,
+// then the epilogue).  There is no bandit here
 // (nothing persists between calls); the caller passes the round counter that keys the random numbers.
 #include <mutex>
 

@@ -4,7 +4,7 @@
 //                          row and the draft row with an online maximum, the target arg-max, then
 //                          sum_v min(p_v, q_v) = 1 - d_TV(p_j, q_j) (Definition 2) in a second
 //                          sweep over the same rows.  Writes one RowStats record.  Plain loads: any alignment.
-//   K1p row_stats_staged_kernel  K1 for 16-byte aligned rows: every thread stages its own
+//   K1p row_stats_staged_kernel  the default, any alignment: every thread stages its own
 //                          vectors through shared memory with cp.async, several trips ahead, and the second
 //                          sweep starts on the trips that are still staged instead of reading them again.
 //   K1t row_stats_bulk_kernel    (metasd_bulk.cu) the same two sweeps by persistent CTAs whose rows arrive as TMA
@@ -165,9 +165,21 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // second sweep visits the warp's trips in reverse: the last D trips of the first sweep are still in their slots and are
 // not read from memory again, and each slot is refilled with the trip D further down as soon as it has been used.  Lanes
 // behind the end of the row hold -Inf in their slot, which adds nothing to any sum: the loops carry no lane predicate.
+//
+// SHIFTED: rows that start off a 16-byte boundary (an odd vocabulary), each row at its own offset.  Copies are of the
+// aligned 16-byte vectors that the row overlaps, of which those that reach over an end of the row have the tokens outside
+// replaced by -Inf once they have landed (nothing outside the row's tensor is read).  A lane's vectors of the two rows then hold tokens `shift` apart.  The first sweep does not
+// care (its sums are over one row each); the second takes the draft row's tokens from the lane's vector and the next one
+// (a 33rd vector per trip is copied for the last lane).  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96, k = 5
+// 115.5 -> 81.5 us a round, V = 128257, B = 256 590 -> 270, V = 32001, fp32, B = 256 226 -> 126.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t policy)
 {
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
+}
+// The first `bytes` (0 .. 16) bytes of the vector, zeros behind them.
+__device__ __forceinline__ void cp_async16_part(uint32_t dst, const void *src, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -231,15 +243,17 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
 // CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
 // of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
 // order, so all hold the same normalisers; each sweeps its part again, and rank 0 adds up the parts of sum min(p, q).
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
+template <int D, int THREADS, bool SHIFTED> constexpr uint32_t STAGED_SMEM = D * (THREADS * 32u + (SHIFTED ? THREADS / 32 * 16u : 0u));
+
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
     static_assert(D >= 2, "at least two stages");
     constexpr int VEC = Logit<LT>::VEC;
     constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
-    constexpr uint32_t ROW_STRIDE = THREADS * 16, STAGE_STRIDE = 2 * ROW_STRIDE;
+    constexpr uint32_t STAGE_STRIDE = STAGED_SMEM<D, THREADS, SHIFTED> / D;
     constexpr uint32_t FULL = 0xFFFFFFFFu;
-    extern __shared__ __align__(16) unsigned char stage_mem[];   // [D][2 rows][THREADS] 16-byte slots
+    extern __shared__ __align__(16) unsigned char stage_mem[];   // [D][2 rows][THREADS] 16-byte slots (SHIFTED: one more per warp)
     __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
     __shared__ double sh_min[NREC];
@@ -263,17 +277,59 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // a peer's shared memory may be written once that peer is running: every CTA says so here and checks it after sweep 1
     if (CL > 1) cluster_arrive();
 
-    const int nvec = p.V / VEC;
+    const LT *a_row = reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V;
+    const LT *d_row = pair ? draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V : a_row;
+    // Vector i of the target row holds tokens VEC i - lead .., of the draft row VEC i - lead - shift .. (0 <= shift < VEC).
+    int lead = 0, shift = 0;
+    if (SHIFTED) {
+        lead = (int)((reinterpret_cast<uintptr_t>(a_row) & 15) / sizeof(LT));
+        shift = pair ? (int)((reinterpret_cast<uintptr_t>(d_row) & 15) / sizeof(LT)) - lead : 0;
+        if (shift < 0) shift += VEC;
+    }
+    const int nvec = SHIFTED ? (p.V + lead + shift + VEC - 1) / VEC : p.V / VEC;
     const int trips_row = (nvec + 31) >> 5;
     const int part = rank * NWARP + warp;                         // this warp's part of the row's trips
     const int g0 = (int)((long long)trips_row * part / NREC), n_trip = (int)((long long)trips_row * (part + 1) / NREC) - g0;
     const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
-    const uint4 *a4 = reinterpret_cast<const uint4 *>(reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V) + v0;
-    const uint4 *d4 = pair ? reinterpret_cast<const uint4 *>(draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V) + v0 : a4;
+    const uint4 *a4 = reinterpret_cast<const uint4 *>(a_row - lead) + v0;
+    const uint4 *d4 = reinterpret_cast<const uint4 *>(d_row - lead - shift) + v0;
+    // this thread's slots of stage 0: of the target row, and of the draft row behind them
     const uint32_t slot0 = smem_addr(stage_mem) + (uint32_t)tid * 16u;
-    // trips in which this lane is inside the row, and in which every lane is: only the row's last trip may be ragged
+    const uint32_t ROW_STRIDE = THREADS * 16u + (SHIFTED ? (uint32_t)warp * 16u : 0u);
+    // Trips in which this lane is inside the row, and in which every lane (SHIFTED: with whole vectors, the 33rd included)
+    // is: only the row's last trip (SHIFTED: its last two, and its first) may be ragged.
     const int lane_trips = v0 + 32 * (n_trip - 1) < nvec ? n_trip : n_trip - 1;
-    const int n_full = (g0 + n_trip) * 32 <= nvec ? n_trip : n_trip - 1;
+    const int n_full = SHIFTED ? min(n_trip, ((p.V + lead) / VEC - 1) / 32 - g0) : (g0 + n_trip) * 32 <= nvec ? n_trip : n_trip - 1;
+    // SHIFTED, a trip that may reach over an end of the row: the part of a vector in front of the row's end.  What it takes
+    // from in front of the row's start belongs to the tensor's row before, where there is one (`room`).
+    auto copy_part = [&](uint32_t dst, const uint4 *src, const LT *row, int tok0, bool room) {
+        int bytes = min(max((p.V - tok0) * (int)sizeof(LT), 0), 16);
+        if (tok0 + VEC <= 0) bytes = 0;
+        if (tok0 < 0 && bytes > 0 && !room) {
+#pragma unroll 1
+            for (int e = -tok0; e < VEC && tok0 + e < p.V; ++e) Logit<LT>::put_scalar(dst + e * (uint32_t)sizeof(LT), row, tok0 + e);
+        } else {
+            cp_async16_part(dst, src, bytes);
+        }
+    };
+    const bool a_room = ((size_t)b * (p.k + 1) + j) * p.V >= 16, d_room = ((size_t)b * p.k + j) * p.V >= 16;
+    auto copy_ragged = [&](int m, uint32_t dst, bool both) {
+        const int tok0 = (v0 + 32 * m) * VEC - lead;
+        copy_part(dst, a4 + 32 * m, a_row, tok0, a_room);
+        if (both) {
+            copy_part(dst + ROW_STRIDE, d4 + 32 * m, d_row, tok0 - shift, d_room);
+            if (lane == 0) copy_part(dst + ROW_STRIDE + 512u, d4 + 32 * m + 32, d_row, tok0 - shift + 32 * VEC, true);
+        }
+    };
+    // and, when it has landed, -Inf for the tokens outside the row
+    auto mask_ragged = [&](int m, uint32_t src, bool both) {
+        const int tok0 = (v0 + 32 * m) * VEC - lead;
+        sts16(src, Logit<LT>::masked(lds16(src), tok0, p.V));
+        if (both) {
+            sts16(src + ROW_STRIDE, Logit<LT>::masked(lds16(src + ROW_STRIDE), tok0 - shift, p.V));
+            if (lane == 0) sts16(src + ROW_STRIDE + 512u, Logit<LT>::masked(lds16(src + ROW_STRIDE + 512u), tok0 - shift + 32 * VEC, p.V));
+        }
+    };
 
     // ---- sweep 1: sums of both rows and the arg-max of the target row.  The draft row's sum is taken relative to
     // the SAME running reference (the target's maximum so far): a softmax sum may be taken relative to any
@@ -299,10 +355,14 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         auto request = [&](uint32_t dst, const uint4 *a, const uint4 *d, uint64_t pol) {
             cp_async16(dst, a, pol);
             if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
+            if (SHIFTED && BOTH && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32, pol);
             cp_async_commit();
         };
         auto request_checked = [&](int m, uint32_t dst) {
-            if (m < lane_trips) {
+            if (SHIFTED) {
+                if (m < n_trip) copy_ragged(m, dst, BOTH);
+                cp_async_commit();
+            } else if (m < lane_trips) {
                 request(dst, a4 + 32 * m, d4 + 32 * m, m >= m_keep ? keep : drop);
             } else {
                 if (m < n_trip) {
@@ -325,6 +385,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         // draft row's (or 0) stands in, so that the draft row's sum does not overflow.
         if (n_trip > 0) {
             cp_async_wait<D - 2>();
+            if (SHIFTED) mask_ragged(0, slot0, BOTH);
             w.m = warp_max_f(Logit<LT>::max_of(lds16(slot0)));
             if (!(w.m > METASD_NEG_BIG)) {
                 w.m = BOTH ? warp_max_f(Logit<LT>::max_of(lds16(slot0 + ROW_STRIDE))) : 0.f;
@@ -351,6 +412,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         while (n + 2 * D - 2 < n_full) group(keep);
         for (int slot = 0, ask = D - 1; n < n_trip; ++n) {
             request_checked(n + D - 1, slot0 + (uint32_t)ask * STAGE_STRIDE);
+            if (SHIFTED && n >= n_full) {
+                cp_async_wait<D - 1>();
+                mask_ragged(n, slot0 + (uint32_t)slot * STAGE_STRIDE, BOTH);
+            }
             consume(n, slot0 + (uint32_t)slot * STAGE_STRIDE);
             ask = slot;
             slot = slot + 1 == D ? 0 : slot + 1;
@@ -368,11 +433,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane);
             st_cluster(dst, __float_as_int(w.m));           st_cluster(dst + 4, __float_as_int(sum_aw));
             st_cluster(dst + 8, __float_as_int(sum_bw));    st_cluster(dst + 12, __float_as_int(w.best));
-            st_cluster(dst + 16, w.best_i);
+            st_cluster(dst + 16, w.best_i - lead);
         }
         cluster_sync_all();
     } else {
-        if (lane == 0) sh_rec[warp] = WarpRecord{w.m, sum_aw, sum_bw, w.best, w.best_i};
+        if (lane == 0) sh_rec[warp] = WarpRecord{w.m, sum_aw, sum_bw, w.best, w.best_i - lead};
         __syncthreads();
     }
     MaxSum ra = {METASD_NEG_BIG, 0.f}, rb = {METASD_NEG_BIG, 0.f};
@@ -405,7 +470,13 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         MaxSum own = {METASD_NEG_BIG, 0.f};
         for (int n = 0; n < lane_trips; ++n) {
             float xb[VEC];
-            Logit<LT>::unpack(ld_stream(d4 + 32 * n), xb);
+            const int tok0 = (v0 + 32 * n) * VEC - lead - shift;
+            if (!SHIFTED || (tok0 >= 0 && tok0 + VEC <= p.V)) {
+                Logit<LT>::unpack(ld_stream(d4 + 32 * n), xb);
+            } else {
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) xb[e] = tok0 + e >= 0 && tok0 + e < p.V ? Logit<LT>::scalar(d_row, tok0 + e) : -INFINITY;
+            }
             float bm = xb[0];
 #pragma unroll
             for (int e = 1; e < VEC; ++e) bm = fmaxf(bm, xb[e]);
@@ -442,23 +513,35 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         const uint64_t nma = pack2(offs[0]), nmb = pack2(offs[1]);
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
-        // every lane: the ragged trip is the row's last).
-        auto consume = [&](uint32_t src) {
+        // every lane: the ragged trips are the row's last; SHIFTED: and its first).
+        auto consume = [&](int m, uint32_t src) {
             // the first D trips are still in their slots from sweep 1; the group of a later one was committed D trips
             // ago, so at most D - 1 younger groups may still be pending
             cp_async_wait<D - 1>();
-            acc = Logit<LT>::add_exp_min(acc, lds16(src), lds16(src + ROW_STRIDE), c2, nma, nmb);
+            if (SHIFTED) {
+                if (m == 0) mask_ragged(0, src, true);
+                __syncwarp();   // the next lane's vector has landed too
+            }
+            uint4 d = lds16(src + ROW_STRIDE);
+            if (SHIFTED) d = Logit<LT>::shifted(d, lds16(src + ROW_STRIDE + 16u), shift);
+            acc = Logit<LT>::add_exp_min(acc, lds16(src), d, c2, nma, nmb);
+            if (SHIFTED) __syncwarp();   // and has been read before its lane refills the slot
         };
-        auto refill = [&](uint32_t dst, const uint4 *a, const uint4 *d) {
+        auto refill = [&](uint32_t dst, int m, const uint4 *a, const uint4 *d) {
+            if (SHIFTED && m == 0) {
+                copy_ragged(0, dst, true);
+                return;
+            }
             cp_async16(dst, a, drop);
             cp_async16(dst + ROW_STRIDE, d, drop);
+            if (SHIFTED && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32, drop);
         };
         // the ragged top first, then whole groups downwards with constant slots
         int n = n_trip - 1;
         for (int slot = n % D; n >= 0 && slot != D - 1; --n) {
             const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
-            consume(src);
-            if (n >= D) refill(src, a4 + 32 * (n - D), d4 + 32 * (n - D));
+            consume(n, src);
+            if (n >= D) refill(src, n - D, a4 + 32 * (n - D), d4 + 32 * (n - D));
             cp_async_commit();
             slot = slot == 0 ? D - 1 : slot - 1;
         }
@@ -467,8 +550,8 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
 #pragma unroll
             for (int u = 0; u < D; ++u) {
                 const uint32_t src = slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE;
-                consume(src);
-                refill(src, a_next - 32 * u, d_next - 32 * u);
+                consume(n - u, src);
+                refill(src, n - u - D, a_next - 32 * u, d_next - 32 * u);
                 cp_async_commit();
             }
             a_next -= 32 * D;
@@ -477,7 +560,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         if (n >= 0) {
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                consume(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
+                consume(n - u, slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
                 cp_async_commit();
             }
         }
@@ -508,12 +591,12 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     }
 }
 
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 static cudaError_t launch_staged(const VerifyParams &p, unsigned units, cudaStream_t stream)
 {
-    const size_t smem = (size_t)D * 2 * THREADS * 16;   // the attribute that allows it was set by streaming_prepare
+    constexpr uint32_t smem = STAGED_SMEM<D, THREADS, SHIFTED>;   // the attribute that allows it was set by streaming_prepare
     if (CL == 1) {
-        row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL><<<units, THREADS, smem, stream>>>(p);
+        row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED><<<units, THREADS, smem, stream>>>(p);
         return cudaSuccess;
     }
     cudaLaunchConfig_t cfg = {};
@@ -526,7 +609,7 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, cudaStre
     at.val.clusterDim.x = CL; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL>, p);
+    return cudaLaunchKernelEx(&cfg, row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, p);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -960,8 +1043,12 @@ __global__ void __launch_bounds__(K2_THREADS, 1024 / K2_THREADS) epilogue_kernel
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
 static cudaError_t prepare_staged()
 {
-    return cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, D * 2 * THREADS * 16);
+    cudaError_t e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM<D, THREADS, false>);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, true>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM<D, THREADS, true>);
+    return e;
 }
 
 template <typename LT>
@@ -977,7 +1064,8 @@ template <typename LT>
 static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo, cudaStream_t stream)
 {
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
-#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) return launch_staged<LT, D, T, M, BL, C>(p, units, stream);
+#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
+        return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, stream);
     METASD_STAGED_SHAPES(X)
 #undef X
     return cudaErrorNotSupported;
@@ -1027,12 +1115,12 @@ template <typename LT>
 static cudaError_t launch_streaming_t(const VerifyParams &p, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches)
 {
     cudaError_t e = cudaSuccess;
-    if (!p.vector_ok) {
+    if (geo.kernel == METASD_ROWS_STAGED) {
+        e = launch_staged_t<LT>(p, geo, stream);
+    } else if (!p.vector_ok) {
         row_stats_kernel<LT, false><<<dim3(p.k + 1, p.batch), K1_THREADS, 0, stream>>>(p);
     } else if (geo.kernel == METASD_ROWS_BULK) {
         e = launch_row_stats_bulk(p, sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32, geo, stream);
-    } else if (geo.kernel == METASD_ROWS_STAGED) {
-        e = launch_staged_t<LT>(p, geo, stream);
     } else {
         row_stats_kernel<LT, true><<<dim3(p.k + 1, p.batch), K1_THREADS, 0, stream>>>(p);
     }

@@ -50,3 +50,45 @@ def test_masked_stretches_cover_whole_warps(dtype, shift):
         assert gpu.last_status() & M.STATUS_NONFINITE == 0
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [1, 2, 7, 9, 250, 255, 257, 4085, 4095, 4097, 6 * 4096 + 3, 12 * 4096 - 1, 50257])
+def test_rows_off_a_16_byte_boundary(dtype, V):
+    """Odd vocabularies: every row starts at an offset of its own, target and draft rows at different ones."""
+    from _harness import run_lockstep
+    c = run_lockstep(workload(V=V, dtype=dtype, k=3), rounds=3, seed=V % 83, path=M.PATH_STREAMING)
+    assert c["rounds"] == 3 and c["status"] == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [40, 8200, 33003])
+def test_tensors_that_start_anywhere(dtype, V):
+    """Target, and each drafter's tensor, as views that start 0 .. 9 logits into a buffer; what surrounds them is NaN."""
+    from _harness import make_pair, compare_round, gather_by_arm
+    wl = workload(V=V, dtype=dtype, B=4, N=3, k=3, sigmas=(0.4, 1.0, 2.5))
+    dev = torch.device("cuda", 0)
+    gen = RoundGenerator(wl, device=dev, seed=5)
+
+    def moved(t, off):
+        back = torch.full((t.numel() + 32,), float("nan"), dtype=t.dtype, device=dev)
+        view = back[off:off + t.numel()].view(t.shape)
+        view.copy_(t)
+        return view
+
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    try:
+        for t in range(4):
+            arm = orc.select()
+            assert np.array_equal(gpu.select().cpu().numpy(), arm)
+            rd = gen.table_round(t)
+            target = moved(rd["target"], 1 + 2 * t)
+            drafts = [moved(d, (3 * i + t) % 10) for i, d in enumerate(rd["drafts"])]
+            res = gpu.verify(target, None, rd["tokens"], 1.0, 7, drafter_table=M.pointer_table(drafts),
+                             token_arm_stride=wl.B * wl.k, want_diag=True)
+            draft, tokens = gather_by_arm(rd["drafts"], rd["tokens"], arm, dev)
+            out = orc.verify(rd["target"], draft, tokens.cpu().numpy(), 1.0, 7)
+            compare_round(res, out, rd["target"], draft, 1.0, 1.0, {})
+            assert gpu.last_status() == 0
+    finally:
+        gpu.close()
