@@ -170,8 +170,9 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // aligned 16-byte vectors that the row overlaps, of which those that reach over an end of the row have the tokens outside
 // replaced by -Inf once they have landed (nothing outside the row's tensor is read).  A lane's vectors of the two rows then hold tokens `shift` apart.  The first sweep does not
 // care (its sums are over one row each); the second takes the draft row's tokens from the lane's vector and the next one
-// (a 33rd vector per trip is copied for the last lane).  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96, k = 5
-// 115.5 -> 81.5 us a round, V = 128257, B = 256 590 -> 270, V = 32001, fp32, B = 256 226 -> 126.
+// (a 33rd vector per trip is copied for the last lane).  These copies carry no L2 policy: with one, some builds of this
+// form ended in an illegal instruction at the first such copy.  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96,
+// k = 5 115.5 -> 81.5 us a round, V = 128257, B = 256 590 -> 270, V = 32001, fp32, B = 256 226 -> 126.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t policy)
 {
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
@@ -180,6 +181,10 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64
 __device__ __forceinline__ void cp_async16_part(uint32_t dst, const void *src, int bytes)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -252,8 +257,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     constexpr int VEC = Logit<LT>::VEC;
     constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
     constexpr uint32_t STAGE_STRIDE = STAGED_SMEM<D, THREADS, SHIFTED> / D;
+    constexpr uint32_t ROW_STRIDE = SHIFTED ? 512u : THREADS * 16u;
     constexpr uint32_t FULL = 0xFFFFFFFFu;
-    extern __shared__ __align__(16) unsigned char stage_mem[];   // [D][2 rows][THREADS] 16-byte slots (SHIFTED: one more per warp)
+    // 16-byte slots: [D][2 rows][THREADS]; SHIFTED: [D][NWARP][32 of the target row, 33 of the draft row]
+    extern __shared__ __align__(16) unsigned char stage_mem[];
     __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
     __shared__ double sh_min[NREC];
@@ -293,9 +300,8 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
     const uint4 *a4 = reinterpret_cast<const uint4 *>(a_row - lead) + v0;
     const uint4 *d4 = reinterpret_cast<const uint4 *>(d_row - lead - shift) + v0;
-    // this thread's slots of stage 0: of the target row, and of the draft row behind them
-    const uint32_t slot0 = smem_addr(stage_mem) + (uint32_t)tid * 16u;
-    const uint32_t ROW_STRIDE = THREADS * 16u + (SHIFTED ? (uint32_t)warp * 16u : 0u);
+    // this thread's slot of stage 0 for the target row; the draft row's lies ROW_STRIDE behind it
+    const uint32_t slot0 = smem_addr(stage_mem) + (SHIFTED ? (uint32_t)warp * (65u * 16u) + (uint32_t)lane * 16u : (uint32_t)tid * 16u);
     // Trips in which this lane is inside the row, and in which every lane (SHIFTED: with whole vectors, the 33rd included)
     // is: only the row's last trip (SHIFTED: its last two, and its first) may be ragged.
     const int lane_trips = v0 + 32 * (n_trip - 1) < nvec ? n_trip : n_trip - 1;
@@ -353,9 +359,14 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         constexpr bool BOTH = decltype(both_tag)::value;
         // One group of copies per trip, empty past the end: the group count stays in step with the trips.
         auto request = [&](uint32_t dst, const uint4 *a, const uint4 *d, uint64_t pol) {
-            cp_async16(dst, a, pol);
-            if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
-            if (SHIFTED && BOTH && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32, pol);
+            if (SHIFTED) {
+                cp_async16(dst, a);
+                if (BOTH) cp_async16(dst + ROW_STRIDE, d);
+                if (BOTH && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32);
+            } else {
+                cp_async16(dst, a, pol);
+                if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
+            }
             cp_async_commit();
         };
         auto request_checked = [&](int m, uint32_t dst) {
@@ -532,9 +543,14 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
                 copy_ragged(0, dst, true);
                 return;
             }
-            cp_async16(dst, a, drop);
-            cp_async16(dst + ROW_STRIDE, d, drop);
-            if (SHIFTED && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32, drop);
+            if (SHIFTED) {
+                cp_async16(dst, a);
+                cp_async16(dst + ROW_STRIDE, d);
+                if (lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32);
+            } else {
+                cp_async16(dst, a, drop);
+                cp_async16(dst + ROW_STRIDE, d, drop);
+            }
         };
         // the ragged top first, then whole groups downwards with constant slots
         int n = n_trip - 1;
