@@ -14,6 +14,7 @@ struct metasd_ctx {
     metasd_config cfg;
     BanditState st;
     RowStats *stats;     // scratch of the streaming path: [max_batch, max_draft + 1]
+    RowSegment *segments;   // and [max_batch, max_draft + 1, geo.n_seg]
     uint32_t *status;    // device status word
     const int32_t *draft_len;   // the caller's per-sequence draft lengths (device), or nullptr
     uint64_t launches;
@@ -99,7 +100,8 @@ int validate_config(const metasd_config *c)
 void free_all(metasd_ctx *c)
 {
     cudaFree(c->st.t); cudaFree(c->st.arm); cudaFree(c->st.stat_a); cudaFree(c->st.stat_b);
-    cudaFree(c->st.win_arm); cudaFree(c->st.win_reward); cudaFree(c->stats); cudaFree(c->status);
+    cudaFree(c->st.win_arm); cudaFree(c->st.win_reward); cudaFree(c->stats); cudaFree(c->segments);
+    cudaFree(c->status);
     cudaFree(c->stage_target); cudaFree(c->stage_draft); cudaFree(c->stage_tokens);
     cudaFree(c->stage_acc); cudaFree(c->stage_tok); cudaFree(c->stage_reward);
 }
@@ -212,6 +214,7 @@ int metasd_init(metasd_ctx **out, const metasd_config *cfg)
         e = streaming_prepare(cfg->device, cfg->logit_dtype, *cfg, &c->geo);
         if (e == cudaErrorNotSupported) { unsupported = true; (void)cudaGetLastError(); }
     }
+    alloc((void **)&c->segments, B * kp1 * c->geo.n_seg * sizeof(RowSegment));
     if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(uint32_t));
     if (e == cudaSuccess) e = launch_reset(c->st, cfg->max_batch, cfg->n_drafters, cfg->window, cfg->bandit, cfg->gamma,
                                             cfg->sequence_base, nullptr, cfg->max_batch, 0);
@@ -300,7 +303,7 @@ int metasd_verify(metasd_ctx *ctx, int32_t batch, int32_t k, const void *target_
     p.c = (float)(1.4426950408889634 / T);
     p.seed = seed; p.beta = cfg.beta; p.gamma = cfg.gamma;
     p.accepted_len = accepted_len; p.next_token = next_token; p.reward = reward; p.diag = diag;
-    p.st = ctx->st; p.stats = ctx->stats; p.status = ctx->status;
+    p.st = ctx->st; p.stats = ctx->stats; p.segments = ctx->segments; p.status = ctx->status;
     {
         const long long nvec = (long long)cfg.vocab * (long long)logit_size(cfg.logit_dtype) / 16;
         p.keep_permille = ctx->keep_permille;

@@ -310,9 +310,9 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) row_stats_bulk_kernel(co
             RowStats r;
             r.max_a = max_a; r.sum_a = sum_a; r.max_b = max_b; r.sum_b = sum_b;
             r.argmax_a = rm.i;
-            r.sum_min = flags ? 0.0 : total_min;
             r.flags = flags;
             p.stats[(size_t)b * (p.k + 1) + j] = r;
+            p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{1.f, (float)total_min};
         };
         if (!pair) {
             if (tid == 0) write_stats(0.0);

@@ -14,10 +14,19 @@ struct RowStats {
     float max_a, sum_a;   // target row
     float max_b, sum_b;   // draft row (unused at the bonus position); max_b is the reference sum_b is relative to:
                           // the row's maximum, or the target row's where the staged kernels could share it
-    double sum_min;       // sum_v min(p_v, q_v) = 1 - d_TV(p, q)
     int32_t argmax_a;     // first index of the target row's maximum
     uint32_t flags;       // METASD_STATUS_* of this row pair
 };
+
+// What the row-statistics pass says about a contiguous part of a row: its share of the target's probability, and (row
+// pairs) of sum_v min(p_v, q_v) = 1 - d_TV(p, q).  A row has n_seg parts of nearly equal length (segment_begin); the
+// residual max(0, p - q) of a part has mass p - min.
+struct RowSegment {
+    float p, min;
+};
+// First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
+__host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }
+constexpr int MAX_SEGMENTS = 128;   // most parts of a row
 
 // Bandit state of all sequences, structure of arrays in device memory.
 struct BanditState {
@@ -37,6 +46,7 @@ struct RowGeometry {
     int32_t per_sm;     // CTAs per SM the shape is built for
     int32_t n_sm;       // SMs of the device (persistent kernels size their grid with it)
     int32_t cluster;    // CTAs that share one row pair (1: none)
+    int32_t n_seg;      // parts of a row that the kernel reports on (RowSegment)
 };
 
 struct VerifyParams {
@@ -64,6 +74,8 @@ struct VerifyParams {
     // state + scratch
     BanditState st;
     RowStats *stats;   // [batch, k+1]
+    RowSegment *segments;    // [batch, k+1, n_seg]
+    int32_t n_seg;           // parts per row, set by the launcher
     uint32_t *status;
     int32_t vector_ok; // rows are 16-byte aligned and a whole number of 16-byte vectors
     int32_t keep_permille;   // share (its end) of every row that the first sweep asks L2 to keep for the second

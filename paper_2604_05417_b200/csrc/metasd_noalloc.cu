@@ -22,10 +22,12 @@ namespace {
 
 constexpr int NOALLOC_MAX_ROWS = METASD_NOALLOC_MAX_ROWS;    // batch * (k + 1)
 constexpr int NOALLOC_MAX_BATCH = METASD_NOALLOC_MAX_BATCH;
+constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row of the default launch shapes, at most
 
 // Everything the two kernels keep in global memory besides the caller's inputs and outputs.
 struct StaticScratch {
     RowStats rows[NOALLOC_MAX_ROWS];       // written by the row-statistics kernel, read by the epilogue
+    RowSegment segments[NOALLOC_MAX_ROWS * NOALLOC_MAX_SEGMENTS];
     double stat_a[NOALLOC_MAX_BATCH];      // a one-armed dummy bandit per sequence: the epilogue kernel
     double stat_b[NOALLOC_MAX_BATCH];      // updates it and nobody reads it
     double win_reward[NOALLOC_MAX_BATCH];
@@ -118,7 +120,7 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     StaticScratch *scratch = nullptr;
     if (scratch_address(device, &scratch) != cudaSuccess) return METASD_ERR_CUDA;
     RowGeometry geo;
-    if (default_geometry(device, logit_dtype, vocab, &geo) != cudaSuccess) return METASD_ERR_CUDA;
+    if (default_geometry(device, logit_dtype, vocab, &geo) != cudaSuccess || geo.n_seg > NOALLOC_MAX_SEGMENTS) return METASD_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
     VerifyParams p = {};
@@ -134,7 +136,7 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     p.st.t = scratch->t; p.st.arm = scratch->arm;
     p.st.stat_a = scratch->stat_a; p.st.stat_b = scratch->stat_b;
     p.st.win_arm = scratch->win_arm; p.st.win_reward = scratch->win_reward;
-    p.stats = scratch->rows;
+    p.stats = scratch->rows; p.segments = scratch->segments;
     p.status = &scratch->status;
     const size_t row_bytes = (size_t)vocab * (logit_dtype == METASD_BF16 ? 2 : 4);
     p.vector_ok = row_bytes % 16 == 0 && ((uintptr_t)target_logits % 16) == 0 && ((uintptr_t)draft_logits % 16) == 0;

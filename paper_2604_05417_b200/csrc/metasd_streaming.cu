@@ -150,9 +150,9 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
         const bool bad_a = !(sum_a > 0.f) || !(sum_a < INFINITY) || !(max_a < INFINITY);
         const bool bad_b = pair && (!(sum_b > 0.f) || !(sum_b < INFINITY) || !(max_b < INFINITY));
         if (bad_a || bad_b) flags |= METASD_STATUS_NONFINITE;
-        r.sum_min = flags ? 0.0 : total_min;
         r.flags = flags;
         p.stats[(size_t)b * (p.k + 1) + j] = r;
+        p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{1.f, (float)total_min};
     }
 }
 
@@ -247,13 +247,14 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
 //
 // CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
 // of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
-// order, so all hold the same normalisers; each sweeps its part again, and rank 0 adds up the parts of sum min(p, q).
+// order, so all hold the same normalisers; each sweeps its part again.
 template <int D, int THREADS, bool SHIFTED> constexpr uint32_t STAGED_SMEM = D * (THREADS * 32u + (SHIFTED ? THREADS / 32 * 16u : 0u));
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
     static_assert(D >= 2, "at least two stages");
+    static_assert(THREADS / 32 * CL <= MAX_SEGMENTS, "the epilogue holds four parts per lane");
     constexpr int VEC = Logit<LT>::VEC;
     constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
     constexpr uint32_t STAGE_STRIDE = STAGED_SMEM<D, THREADS, SHIFTED> / D;
@@ -263,7 +264,6 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     extern __shared__ __align__(16) unsigned char stage_mem[];
     __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
-    __shared__ double sh_min[NREC];
     launch_dependents();   // the epilogue may be set up while this kernel runs; it waits for the whole grid before it reads
     // Blocks are dispatched in index order.  BONUS_LAST: the row pairs come first and the bonus rows (one row, half
     // the work) last, so that the launch ends on its shortest items (measured: better for the bf16 geometry, worse
@@ -286,17 +286,12 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
 
     const LT *a_row = reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V;
     const LT *d_row = pair ? draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V : a_row;
-    // Vector i of the target row holds tokens VEC i - lead .., of the draft row VEC i - lead - shift .. (0 <= shift < VEC).
     int lead = 0, shift = 0;
-    if (SHIFTED) {
-        lead = (int)((reinterpret_cast<uintptr_t>(a_row) & 15) / sizeof(LT));
-        shift = pair ? (int)((reinterpret_cast<uintptr_t>(d_row) & 15) / sizeof(LT)) - lead : 0;
-        if (shift < 0) shift += VEC;
-    }
+    if (SHIFTED) row_alignment(a_row, pair ? d_row : nullptr, lead, shift);
     const int nvec = SHIFTED ? (p.V + lead + shift + VEC - 1) / VEC : p.V / VEC;
     const int trips_row = (nvec + 31) >> 5;
     const int part = rank * NWARP + warp;                         // this warp's part of the row's trips
-    const int g0 = (int)((long long)trips_row * part / NREC), n_trip = (int)((long long)trips_row * (part + 1) / NREC) - g0;
+    const int g0 = segment_begin(trips_row, part, NREC), n_trip = segment_begin(trips_row, part + 1, NREC) - g0;
     const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
     const uint4 *a4 = reinterpret_cast<const uint4 *>(a_row - lead) + v0;
     const uint4 *d4 = reinterpret_cast<const uint4 *>(d_row - lead - shift) + v0;
@@ -326,6 +321,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             copy_part(dst + ROW_STRIDE, d4 + 32 * m, d_row, tok0 - shift, d_room);
             if (lane == 0) copy_part(dst + ROW_STRIDE + 512u, d4 + 32 * m + 32, d_row, tok0 - shift + 32 * VEC, true);
         }
+        __syncwarp();
     };
     // and, when it has landed, -Inf for the tokens outside the row
     auto mask_ragged = [&](int m, uint32_t src, bool both) {
@@ -335,6 +331,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             sts16(src + ROW_STRIDE, Logit<LT>::masked(lds16(src + ROW_STRIDE), tok0 - shift, p.V));
             if (lane == 0) sts16(src + ROW_STRIDE + 512u, Logit<LT>::masked(lds16(src + ROW_STRIDE + 512u), tok0 - shift + 32 * VEC, p.V));
         }
+        __syncwarp();
     };
 
     // ---- sweep 1: sums of both rows and the arg-max of the target row.  The draft row's sum is taken relative to
@@ -516,8 +513,19 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         rb = warp_merge(rb, c);
     }
 
+    const size_t row = (size_t)b * (p.k + 1) + j;
+    if (tid == 0 && rank == 0) {
+        RowStats r;
+        r.max_a = ra.m; r.sum_a = ra.s; r.max_b = rb.m; r.sum_b = rb.s;
+        r.argmax_a = rm.i;
+        const bool bad_a = !(ra.s > 0.f) || !(ra.s < INFINITY) || !(rm.v < INFINITY);
+        const bool bad_b = pair && (!(rb.s > 0.f) || !(rb.s < INFINITY) || !(rb.m < INFINITY));
+        r.flags = bad_a || bad_b ? METASD_STATUS_NONFINITE : 0u;
+        p.stats[row] = r;
+    }
+
     // ---- sweep 2, this warp's trips in reverse: sum_v 2^min(ya_v, yb_v), one exponential per pair
-    double total_min = 0.0;
+    float part_min = 0.f;
     if (pair) {
         float offs[3];
         second_sweep_offsets(ra, rb, c, offs);
@@ -581,30 +589,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             }
         }
         cp_async_wait<0>();
-        const double part_min = warp_sum((double)(sum2(acc) * offs[2]));
-        if (CL > 1) {
-            if (lane == 0) st_cluster(map_to_rank(smem_addr(&sh_min[part]), 0u), part_min);
-            cluster_sync_all();   // rank 0 holds every part; no CTA leaves while a peer may still write to it
-        } else {
-            if (lane == 0) sh_min[warp] = part_min;
-            __syncthreads();
-        }
-        if (tid == 0)
-            for (int i = 0; i < NREC; ++i) total_min += sh_min[i];
+        part_min = (float)warp_sum((double)(sum2(acc) * offs[2]));
     }
-
-    if (tid == 0 && rank == 0) {
-        RowStats r;
-        r.max_a = ra.m; r.sum_a = ra.s; r.max_b = rb.m; r.sum_b = rb.s;
-        r.argmax_a = rm.i;
-        uint32_t flags = 0;
-        const bool bad_a = !(ra.s > 0.f) || !(ra.s < INFINITY) || !(rm.v < INFINITY);
-        const bool bad_b = pair && (!(rb.s > 0.f) || !(rb.s < INFINITY) || !(rb.m < INFINITY));
-        if (bad_a || bad_b) flags |= METASD_STATUS_NONFINITE;
-        r.sum_min = flags ? 0.0 : total_min;
-        r.flags = flags;
-        p.stats[(size_t)b * (p.k + 1) + j] = r;
-    }
+    if (lane == 0)   // the warp's trips are part `part` of the row
+        p.segments[row * NREC + part] = RowSegment{sum_aw * ex2((w.m - ra.m) * c) / ra.s, part_min};
 }
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
@@ -668,384 +656,365 @@ __device__ __forceinline__ void unpack_raw(const RawVec<LT, VEC> &r, float (&x)[
     else x[0] = r.v;
 }
 
+// The row (pair) a draw is made from: weights max(0, p - q) (mode 1) or p (mode 2) of its tokens, in vectors of VEC.
+template <typename LT> struct DrawRow {
+    const LT *a, *d;
+    int mode, nvec;
+    float c, nma, ia, nmb, ib;
+};
+
 template <typename LT, int VEC>
-__device__ __forceinline__ void draw_weights(const LT *a, const LT *d, int i, int mode, float c, float nma,
-                                             float ia, float nmb, float ib, float (&w)[VEC])
+__device__ __forceinline__ void draw_weights(const DrawRow<LT> &row, const RawVec<LT, VEC> &ra, const RawVec<LT, VEC> &rb, float (&w)[VEC])
 {
     float xa[VEC], xb[VEC];
-    unpack_raw<LT, VEC>(load_raw<LT, VEC>(a, i), xa);
-    if (mode == 1) {
-        unpack_raw<LT, VEC>(load_raw<LT, VEC>(d, i), xb);
-        weights_of<LT, VEC, 1>(xa, xb, c, nma, ia, nmb, ib, w);
+    unpack_raw<LT, VEC>(ra, xa);
+    if (row.mode == 1) {
+        unpack_raw<LT, VEC>(rb, xb);
+        weights_of<LT, VEC, 1>(xa, xb, row.c, row.nma, row.ia, row.nmb, row.ib, w);
     } else {
-        weights_of<LT, VEC, 2>(xa, xa, c, nma, ia, nmb, ib, w);
+        weights_of<LT, VEC, 2>(xa, xa, row.c, row.nma, row.ia, row.nmb, row.ib, w);
     }
 }
 
-// Sum of the draw's weights over the vectors [lo, hi), by one warp: lane l takes lo + l, lo + l + 32, ... and adds
-// each vector's fp32 sum to its fp64 total in that order.  U vectors' loads are issued before the first is used.
-template <typename LT, int VEC, int MODE, int U>
-__device__ __forceinline__ double warp_range_sum_m(const LT *a, const LT *d, int lo, int hi, float c, float nma,
-                                                   float ia, float nmb, float ib)
-{
-    const int lane = threadIdx.x & 31;
-    double acc = 0.0;
-    for (int i0 = lo + lane; i0 < hi; i0 += 32 * U) {
-        RawVec<LT, VEC> ra[U], rb[U];
+// U vectors of the row (pair) per lane, 32 apart: all loads are issued before the first is used.  Behind `hi`: nothing.
+template <typename LT, int VEC, int U> struct DrawBatch {
+    RawVec<LT, VEC> ra[U], rb[U];
+    __device__ __forceinline__ void load(const DrawRow<LT> &row, int i0, int hi)
+    {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + 32 * u;
-            if (i < hi) {
-                ra[u] = load_raw<LT, VEC>(a, i);
-                if (MODE == 1) rb[u] = load_raw<LT, VEC>(d, i);
+        for (int u = 0; u < U; ++u)
+            if (i0 + 32 * u < hi) {
+                ra[u] = load_raw<LT, VEC>(row.a, i0 + 32 * u);
+                if (row.mode == 1) rb[u] = load_raw<LT, VEC>(row.d, i0 + 32 * u);
             }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + 32 * u;
-            if (i < hi) {
-                float xa[VEC], xb[VEC], w[VEC];
-                unpack_raw<LT, VEC>(ra[u], xa);
-                if (MODE == 1) unpack_raw<LT, VEC>(rb[u], xb);
-                weights_of<LT, VEC, MODE>(xa, MODE == 1 ? xb : xa, c, nma, ia, nmb, ib, w);
-                float s = 0.f;
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) s += w[e];
-                acc += (double)s;
-            }
-        }
     }
-    return warp_sum(acc);
-}
+};
 
-template <typename LT, int VEC, int U = 4>
-__device__ __forceinline__ double warp_range_sum(const LT *a, const LT *d, int lo, int hi, int mode, float c,
-                                                 float nma, float ia, float nmb, float ib)
-{
-    return mode == 1 ? warp_range_sum_m<LT, VEC, 1, U>(a, d, lo, hi, c, nma, ia, nmb, ib)
-                     : warp_range_sum_m<LT, VEC, 2, U>(a, d, lo, hi, c, nma, ia, nmb, ib);
-}
-
-// Given n <= 64 non-negative parts x[0..n) laid end to end after base0, finds the first part whose end lies beyond
-// the threshold; rounding may leave none, then the last part with mass (-1 if there is none).  FRACTION: the
-// threshold comes in as a fraction of the parts' sum and goes out absolute.  Returns the part, the sum of the parts
-// before it plus base0 in `base`, and the sum of all parts in `total`.  Every lane of the calling warp takes part
-// and gets the same answers.
+// Parts laid end to end after base0, lane l holding parts 4 l .. 4 l + 3 (0 where there is none): finds the first part
+// whose end lies beyond the threshold; rounding may leave none, then the last part with mass (-1 if there is none).
+// FRACTION: the threshold comes in as a fraction of the parts' sum and goes out absolute.  Returns the part, the sum of
+// the parts before it plus base0 in `base`, and the sum of all parts in `total`.  Every lane of the calling warp takes
+// part and gets the same answers.
 template <bool FRACTION>
-__device__ __forceinline__ int warp_find_part(const double *x, int n, double base0, double &threshold, double &base,
-                                              double &total)
+__device__ __forceinline__ int warp_find_part(const double (&x)[4], double base0, double &threshold, double &base, double &total)
 {
     const unsigned FULL = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
-    const double x0 = lane < n ? x[lane] : 0.0, x1 = lane + 32 < n ? x[lane + 32] : 0.0;
-    double i0 = x0, i1 = x1;
+    double incl = (x[0] + x[1]) + (x[2] + x[3]);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const double t0 = __shfl_up_sync(FULL, i0, o), t1 = __shfl_up_sync(FULL, i1, o);
-        if (lane >= o) { i0 += t0; i1 += t1; }
+        const double t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
     }
-    const double tot0 = __shfl_sync(FULL, i0, 31);
-    i1 += tot0;
-    total = __shfl_sync(FULL, i1, 31);
+    total = __shfl_sync(FULL, incl, 31);
     if (FRACTION) threshold *= total;
-    double e0 = __shfl_up_sync(FULL, i0, 1), e1 = __shfl_up_sync(FULL, i1, 1);
-    if (lane == 0) { e0 = 0.0; e1 = tot0; }
-    const unsigned c0 = __ballot_sync(FULL, lane < n && base0 + i0 > threshold);
-    const unsigned c1 = __ballot_sync(FULL, lane + 32 < n && base0 + i1 > threshold);
-    const unsigned m0 = __ballot_sync(FULL, x0 > 0.0), m1 = __ballot_sync(FULL, x1 > 0.0);
-    int part, src;
-    bool upper;
-    if (c0)      { src = __ffs(c0) - 1;    upper = false; }
-    else if (c1) { src = __ffs(c1) - 1;    upper = true; }
-    else if (m1) { src = 31 - __clz(m1);   upper = true; }
-    else if (m0) { src = 31 - __clz(m0);   upper = false; }
-    else { base = base0; return -1; }
-    part = src + (upper ? 32 : 0);
-    const double b0 = __shfl_sync(FULL, e0, src), b1 = __shfl_sync(FULL, e1, src);
-    base = base0 + (upper ? b1 : b0);
-    return part;
+    double before = __shfl_up_sync(FULL, incl, 1);
+    if (lane == 0) before = 0.0;
+    // the lane's first part that crosses, else its last one with mass
+    int hit = -1, mass = -1;
+    double hit_base = 0.0, mass_base = 0.0, cum = base0 + before;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (x[i] > 0.0) { mass = i; mass_base = cum; }
+        if (hit < 0 && x[i] > 0.0 && cum + x[i] > threshold) { hit = i; hit_base = cum; }
+        cum += x[i];
+    }
+    const unsigned hits = __ballot_sync(FULL, hit >= 0), masses = __ballot_sync(FULL, mass >= 0);
+    if (!masses) { base = base0; return -1; }
+    const int src = hits ? __ffs(hits) - 1 : 31 - __clz(masses);
+    base = __shfl_sync(FULL, hits ? hit_base : mass_base, src);
+    return src * 4 + __shfl_sync(FULL, hits ? hit : mass, src);
+}
+
+// The token of one vector per lane (lane order is token order) where the running weight, `run` before the first lane,
+// exceeds the threshold: the same answer in every lane, -1 if it does not in these 32 vectors.  `last` collects the last
+// token with mass seen so far.
+template <int VEC>
+__device__ __forceinline__ int warp_find_token(const float (&w)[VEC], int vec, double &run, double threshold, int &last)
+{
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    float s = 0.f;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) s += w[e];
+    double incl = (double)s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const unsigned hits = __ballot_sync(FULL, run + incl > threshold);
+    int mine = -1, tok = -1;
+    double cum = run + incl - (double)s;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+        if (w[e] > 0.f) mine = vec * VEC + e;
+        cum += (double)w[e];
+        if (tok < 0 && w[e] > 0.f && cum > threshold) tok = vec * VEC + e;
+    }
+    if (tok < 0) tok = mine;
+    last = max(last, __reduce_max_sync(FULL, mine));
+    run += __shfl_sync(FULL, incl, 31);
+    return hits ? __shfl_sync(FULL, tok, __ffs(hits) - 1) : -1;
 }
 
 // Shared-memory work space of the draw.
 template <int NWARP> struct DrawShared {
-    double tot[NWARP], sub[NWARP];   // warp totals of the two search levels
-    double before;                   // weight in front of the token that was found
+    double tot[NWARP];
     int tok;
 };
 
-// Inverse CDF in token order over the vectors [0, v_end) of one row (pair): the smallest token v with
-// sum_{w <= v} weight_w > threshold.  Every warp owns a contiguous range of vectors and sums it (fp32 weights, fp64
-// sums); one warp-parallel scan finds the range that holds the crossing, the same two steps repeat inside that range,
-// and the owning warp finishes with a lane scan.  FRACTION: the threshold comes in as a fraction of the range's total
-// (the walk's own total, when the range is the whole row) and rounding may leave no crossing: then the last token
-// with mass.  Otherwise it is absolute, and -2 says that the crossing lies behind the range.  Returns the token (-1:
-// the range has no mass), the weight in front of it in `before` and the weight of the range in `total`.
+// Barrier among the draw's warps only: the control warp goes its own way.
+template <int THREADS> __device__ __forceinline__ void draw_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
+
+// Inverse CDF in token order over the vectors [lo, hi) of one row (pair), of which `base` is the weight in front: the
+// smallest token v with sum_{w <= v} weight_w > threshold.  Every warp owns a contiguous range of vectors and sums it
+// (fp32 a vector, fp64 across); one warp-parallel scan finds the range that holds the crossing, and so on down to a range
+// of a few vectors per lane, which one warp searches vector by vector.  FRACTION: the threshold comes in as a fraction of
+// the range's own total.  Rounding may leave no crossing: then the last token with mass.  -1: no mass.
 template <typename LT, int VEC, int NWARP, bool FRACTION>
-__device__ __forceinline__ int range_inverse_cdf(const LT *a, const LT *d, int v_end, int mode, double threshold, float c,
-                                                 float nma, float ia, float nmb, float ib, DrawShared<NWARP> &sh,
-                                                 double &before, double &total)
+__device__ __forceinline__ int range_inverse_cdf(const DrawRow<LT> &row, int lo, int hi, double base, double threshold, DrawShared<NWARP> &sh)
 {
+    constexpr int U = 4, DIRECT = 32 * U * (VEC == 1 ? 1 : 2);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per_warp = (v_end + NWARP - 1) / NWARP;
-    const int v0 = min(warp * per_warp, v_end), v1 = min(v0 + per_warp, v_end);
-    const double acc = warp_range_sum<LT, VEC>(a, d, v0, v1, mode, c, nma, ia, nmb, ib);
-    if (lane == 0) sh.tot[warp] = acc;
-    if (tid == 0) { sh.tok = -1; sh.before = 0.0; }
-    __syncthreads();
-    double base;
-    const int wstar = warp_find_part<FRACTION>(sh.tot, NWARP, 0.0, threshold, base, total);
-    if (!(total > 0.0) || wstar < 0) { before = 0.0; return -1; }
-    if (!FRACTION && !(total > threshold)) { before = total; return -2; }   // the crossing is not inside the range
-    const int r0 = min(wstar * per_warp, v_end), r1 = min(r0 + per_warp, v_end);
-    const int per_sub = (r1 - r0 + NWARP - 1) / NWARP;
-    const int s0 = min(r0 + warp * per_sub, r1), s1 = min(s0 + per_sub, r1);
-    {
-        const double acc2 = warp_range_sum<LT, VEC>(a, d, s0, s1, mode, c, nma, ia, nmb, ib);
-        if (lane == 0) sh.sub[warp] = acc2;
-    }
-    __syncthreads();
-    double total2;
-    const int sstar = warp_find_part<false>(sh.sub, NWARP, base, threshold, base, total2);
-    if (warp == sstar) {
-        int found = -1, last_pos = -1;
-        double found_before = base, last_before = base;
-        double run_base = base;
-        for (int i0 = s0; i0 < s1 && found < 0; i0 += 32) {
-            const int i = i0 + lane;
-            float w[VEC];
+    bool fraction = FRACTION;
+    for (;;) {
+        const int per_warp = (hi - lo + NWARP - 1) / NWARP;
+        const int v0 = min(lo + warp * per_warp, hi), v1 = min(v0 + per_warp, hi);
+        double acc = 0.0;
+        for (int i0 = v0 + lane; i0 < v1; i0 += 32 * U) {
+            DrawBatch<LT, VEC, U> batch;
+            batch.load(row, i0, v1);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) w[e] = 0.f;
-            if (i < s1) draw_weights<LT, VEC>(a, d, i, mode, c, nma, ia, nmb, ib, w);
-            float s = 0.f;
+            for (int u = 0; u < U; ++u)
+                if (i0 + 32 * u < v1) {
+                    float w[VEC], s = 0.f;
+                    draw_weights<LT, VEC>(row, batch.ra[u], batch.rb[u], w);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) s += w[e];
-            double incl = (double)s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                double t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const bool crosses = run_base + incl > threshold;
-            const unsigned ballot = __ballot_sync(0xFFFFFFFFu, crosses);
-            {
-                double cum = run_base + incl - (double)s;
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) {
-                    if (w[e] > 0.f) { last_pos = i * VEC + e; last_before = cum; }
-                    cum += (double)w[e];
+                    for (int e = 0; e < VEC; ++e) s += w[e];
+                    acc += (double)s;
                 }
-            }
-            if (ballot) {
-                const int src = __ffs(ballot) - 1;
-                if (lane == src) {
-                    double cum = run_base + incl - (double)s;
-                    int tok = -1;
+        }
+        acc = warp_sum(acc);
+        if (lane == 0) sh.tot[warp] = acc;
+        draw_sync<NWARP * 32>();
+        double x[4], total;
 #pragma unroll
-                    for (int e = 0; e < VEC; ++e) {
-                        if (tok < 0 && cum + (double)w[e] > threshold) { tok = i * VEC + e; found_before = cum; }
-                        cum += (double)w[e];
+        for (int i = 0; i < 4; ++i) x[i] = lane * 4 + i < NWARP ? sh.tot[lane * 4 + i] : 0.0;
+        const int part = fraction ? warp_find_part<true>(x, base, threshold, base, total)
+                                  : warp_find_part<false>(x, base, threshold, base, total);
+        fraction = false;
+        if (part < 0) return -1;         // the same in every warp
+        lo = min(lo + part * per_warp, hi);
+        hi = min(lo + per_warp, hi);
+        if (hi - lo > DIRECT) {
+            draw_sync<NWARP * 32>();     // every warp has read the totals before the next level writes them
+            continue;
+        }
+        if (warp == part) {
+            int found = -1, last = -1;
+            double run = base;
+            for (int i0 = lo; i0 < hi && found < 0; i0 += 32 * U) {
+                DrawBatch<LT, VEC, U> batch;
+                batch.load(row, i0 + lane, hi);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + lane + 32 * u;
+                    if (i0 + 32 * u < hi && found < 0) {
+                        float w[VEC];
+                        if (i < hi) {
+                            draw_weights<LT, VEC>(row, batch.ra[u], batch.rb[u], w);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < VEC; ++e) w[e] = 0.f;
+                        }
+                        found = warp_find_token<VEC>(w, i, run, threshold, last);
                     }
-                    if (tok < 0) { tok = last_pos; found_before = last_before; }
-                    found = tok;
                 }
-                found = __shfl_sync(0xFFFFFFFFu, found, src);
-                found_before = __shfl_sync(0xFFFFFFFFu, found_before, src);
             }
-            run_base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+            if (lane == 0) sh.tok = found >= 0 ? found : last;
         }
-        if (found < 0) {
-            int best = last_pos;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
-            const unsigned who = __ballot_sync(0xFFFFFFFFu, best >= 0 && last_pos == best);
-            found = best;
-            if (who) found_before = __shfl_sync(0xFFFFFFFFu, last_before, __ffs(who) - 1);
-        }
-        if (lane == 0) { sh.tok = found; sh.before = found_before; }
+        draw_sync<NWARP * 32>();
+        return sh.tok;
     }
-    __syncthreads();
-    before = sh.before;
-    return sh.tok;
 }
 
-// The draw of one sequence: the smallest v with sum_{w<=v} weight_w > u * total, total being the sum of all the weights
-// as the walk over the whole row adds them up.  `approx_total` is the same total as the row statistics already give
-// it (1 - sum_v min(p_v, q_v) for the residual, 1 for the bonus row); the two are fp32 evaluations of one sum and
-// agree to within `guard` (they were never seen further apart than 2e-6, typically 2e-7, over millions of rows).
-// So the first eighth of the vocabulary is searched first, with the upper end of the band u * (approx_total +- guard)
-// as the threshold: a token found there whose weight in front does not reach the lower end of the band is the answer
-// for every total in the band, hence the full walk's answer, and the rest of the row is never read.  Otherwise (the
-// crossing lies further back, a CDF edge falls inside the band, or the total is too small for the band to mean
-// anything) the whole row is walked and its own total decides.  With a frequency-sorted vocabulary most draws end in
-// the probe; with the likely tokens at the end of the vocabulary none does, and the probe costs an eighth more.
-template <typename LT, bool VECTOR, int K2_THREADS>
-__device__ __forceinline__ int block_inverse_cdf(const LT *a, const LT *d, int V, int mode, float u, float c, float max_a, float sum_a,
-                                 float max_b, float sum_b, double approx_total, DrawShared<K2_THREADS / 32> &sh)
+// The draw over a whole row with the walk's own total, for the cases that the parts of the row statistics do not settle
+// (a residual with next to no mass; row-statistics kernels that report on whole rows).  A call and not another inlined copy.
+template <typename LT, int VEC, int NWARP>
+__device__ __noinline__ int draw_whole_row(const DrawRow<LT> &row, float u, DrawShared<NWARP> &sh)
 {
-    constexpr int VEC = VECTOR ? Logit<LT>::VEC : 1;
-    constexpr int NWARP = K2_THREADS / 32;
-    constexpr double guard = 5.0e-6;
-    const int nvec = V / VEC;
-    const float nma = -max_a * c, nmb = -max_b * c;
-    const float ia = 1.0f / sum_a, ib = 1.0f / sum_b;
-    const double lo = (double)u * (approx_total - guard), hi = (double)u * (approx_total + guard);
-    double before, total;
-    const int probe = (nvec / 8 + 31) & ~31;
-    if (approx_total > 16.0 * guard && probe >= NWARP * 32 && probe < nvec) {
-        const int tok = range_inverse_cdf<LT, VEC, NWARP, false>(a, d, probe, mode, hi, c, nma, ia, nmb, ib, sh, before, total);
-        if (tok >= 0 && before <= lo) return tok;
-        __syncthreads();
-    }
-    return range_inverse_cdf<LT, VEC, NWARP, true>(a, d, nvec, mode, (double)u, c, nma, ia, nmb, ib, sh, before, total);
-}
-
-// The draw from p alone over the whole row, for the one case that needs a second draw: the residual of a rejected
-// position has no mass in fp32 (p == q to rounding).  Rare, so it is a call and not a second inlined copy.
-template <typename LT, bool VECTOR, int K2_THREADS>
-__device__ __noinline__ int draw_from_target(const LT *a, int V, float u, float c, float max_a, float sum_a,
-                                             DrawShared<K2_THREADS / 32> &sh)
-{
-    constexpr int VEC = VECTOR ? Logit<LT>::VEC : 1;
-    double before, total;
-    return range_inverse_cdf<LT, VEC, K2_THREADS / 32, true>(a, nullptr, V / VEC, 2, (double)u, c, -max_a * c, 1.0f / sum_a, 0.f,
-                                                             0.f, sh, before, total);
+    draw_sync<NWARP * 32>();   // every thread has read what the last search left in the work space
+    return range_inverse_cdf<LT, VEC, NWARP, true>(row, 0, row.nvec, 0.0, (double)u, sh);
 }
 
 // Blocks until the kernel launched before this one in the stream has finished and its writes are visible (a no-op
 // when this kernel was launched without programmatic stream serialisation).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// K2_THREADS: the draw walks (part of) one row pair per sequence, so a small batch wants large CTAs (many warps keep the
-// load chains short) and a large batch wants many small ones.  512 threads per SM in either shape: the draw keeps a
-// dozen fp64 running values next to its loads in flight and wants about 100 registers per thread.
-template <typename LT, bool VECTOR, int K2_THREADS>
-__global__ void __launch_bounds__(K2_THREADS, 1024 / K2_THREADS) epilogue_kernel(const VerifyParams p)
+// One CTA per sequence: DRAW_THREADS threads for the draw (GREEDY: there is none, they only add up the parts of
+// sum min(p, q)) and one control warp for the accept tests, the first rejection, the reward and the bandit, which runs
+// while the other warps search for the token.  What bounds it is the chain of dependent reads of its slowest sequence.
+//
+// The draw: the smallest v with sum_{w <= v} weight_w > u * total.  The row-statistics kernel leaves the mass of every
+// part of the row, so the part that holds the crossing is known without reading a logit, and only that part is walked
+// (a sixteenth of the row or less).  Where the mass sits in the vocabulary does not matter.  Against walking the row (its
+// first eighth first), kernel alone from cold caches: B = 256, V = 128256 bf16 31..40 -> 20 us; B = 1024, V = 128256 fp32
+// 90 -> 34; B = 40, V = 262144 bf16 (no frequency order) 43 -> 22; B = 96, V = 50257 bf16 36 -> 18; B = 64, V = 32000 17 -> 14.5.
+template <typename LT, bool VECTOR, int DRAW_THREADS, bool GREEDY>
+__global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_kernel(const VerifyParams p)
 {
-    const int b = blockIdx.x, tid = threadIdx.x;
+    constexpr int NWARP = DRAW_THREADS / 32, VEC = VECTOR ? Logit<LT>::VEC : 1;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k_slots = p.k, V = p.V, K = p.K;   // rows and tokens are laid out for k_slots positions per sequence
     const float c = p.c;
 
-    __shared__ int sh_nacc, sh_mode, sh_tok;
+    __shared__ int sh_nacc, sh_mode;
     __shared__ float sh_u;
-    __shared__ uint32_t sh_flags;
-    __shared__ double sh_reward;
-    __shared__ DrawShared<K2_THREADS / 32> sh_draw;
-    __shared__ int sh_accept[16];
     __shared__ double sh_align[16];
+    __shared__ DrawShared<NWARP> sh_draw;
 
-    // The row-statistics kernel may still be running when this kernel starts (programmatic stream serialisation):
-    // nothing it writes is read, and nothing it reads is written, before this wait.
-    grid_dependency_wait();
-
+    // The row-statistics kernel may still be running when this kernel starts (programmatic stream serialisation).  What it
+    // writes (stats, segments) is read, and what it reads is written, behind grid_dependency_wait() only; everything else
+    // was there before it began and is fetched meanwhile.
     const int k = drafted(p.draft_len, b, k_slots);   // positions this sequence drafted this round
     const LT *target = reinterpret_cast<const LT *>(p.target) + (size_t)b * (k_slots + 1) * V;
     const LT *draft = draft_rows<LT>(p, b) + (size_t)b * k_slots * V;
     const RowStats *stats = p.stats + (size_t)b * (k_slots + 1);
+    const RowSegment *segments = p.segments + (size_t)b * (k_slots + 1) * p.n_seg;
 
-    if (tid == 0) sh_flags = (p.draft_len && p.draft_len[b] != k) ? METASD_STATUS_BAD_LENGTH : 0u;
-    __syncthreads();
-    // pointer-table mode: an entry that must not be dereferenced is flagged once per call, played or not
-    if (b == 0 && p.drafter_ptrs && tid < K) {
-        const void *q = p.drafter_ptrs[tid];
-        if (q == nullptr || (reinterpret_cast<uintptr_t>(q) & p.table_mask) != 0) atomicOr(&sh_flags, METASD_STATUS_BAD_POINTER);
-    }
-    const int t = p.st.t[b];
-    const int arm = p.st.arm[b];
-    if (tid < k) {
-        // position j = tid: the accept test of Algorithm 4
-        const int j = tid;
-        const int32_t *tokens = p.tokens + (p.token_arm_stride ? (size_t)arm * p.token_arm_stride : 0) + (size_t)b * k_slots;
-        const RowStats r = stats[j];
+    if (warp == NWARP) {
+        uint32_t flags = lane == 0 && p.draft_len && p.draft_len[b] != k ? METASD_STATUS_BAD_LENGTH : 0u;
+        // pointer-table mode: an entry that must not be dereferenced is flagged once per call, played or not
+        if (b == 0 && p.drafter_ptrs && lane < K) {
+            const void *q = p.drafter_ptrs[lane];
+            if (q == nullptr || (reinterpret_cast<uintptr_t>(q) & p.table_mask) != 0) flags |= METASD_STATUS_BAD_POINTER;
+        }
+        const int t = p.st.t[b], arm = p.st.arm[b];
+        // lane j < k: the accept test of Algorithm 4 at position j; lane j = k only brings the bonus row's words and flags
+        const int j = min(lane, k);
         const uint4 words = round_words(p.seed, p.sequence_base + (uint32_t)b, (uint32_t)t, (uint32_t)j);
         const float u = uniform24(words.x);
-        const int x = tokens[j];
+        int x = -1;
+        if (lane < k) x = p.tokens[(p.token_arm_stride ? (size_t)arm * p.token_arm_stride : 0) + (size_t)b * k_slots + j];
         const bool in_range = x >= 0 && x < V;
-        float p_x = 0.f, q_x = 0.f, D = 1.f;
+        float a_x = 0.f, d_x = 0.f;
+        if (in_range) {
+            a_x = Logit<LT>::scalar(target + (size_t)j * V, x);
+            d_x = Logit<LT>::scalar(draft + (size_t)j * V, x);
+        }
+        grid_dependency_wait();
+        const RowStats r = stats[j];
+        float p_x = 0.f, q_x = 0.f;
         bool accepted = false;
-        uint32_t flags = r.flags;
-        double align = 0.0;
-        if (!r.flags) {
-            D = (float)(1.0 - r.sum_min);
-            align = r.sum_min;
-            if (!in_range) {
-                flags |= METASD_STATUS_TOKEN_OOR;
-            } else {
-                p_x = ex2(fmaf(Logit<LT>::scalar(target + (size_t)j * V, x), c, -r.max_a * c)) / r.sum_a;
-                q_x = ex2(fmaf(Logit<LT>::scalar(draft + (size_t)j * V, x), c, -r.max_b * c)) / r.sum_b;
-                if (p.greedy) {
-                    accepted = x == r.argmax_a;
+        if (lane < k) {
+            flags |= r.flags;
+            if (!r.flags) {
+                if (!in_range) {
+                    flags |= METASD_STATUS_TOKEN_OOR;
                 } else {
-                    if (q_x == 0.f) flags |= METASD_STATUS_Q_ZERO;
-                    accepted = u * q_x < p_x;  // u < min(1, p/q) without the division
+                    p_x = ex2(fmaf(a_x, c, -r.max_a * c)) / r.sum_a;
+                    q_x = ex2(fmaf(d_x, c, -r.max_b * c)) / r.sum_b;
+                    if (GREEDY) {
+                        accepted = x == r.argmax_a;
+                    } else {
+                        if (q_x == 0.f) flags |= METASD_STATUS_Q_ZERO;
+                        accepted = u * q_x < p_x;  // u < min(1, p/q) without the division
+                    }
                 }
             }
         }
-        sh_accept[j] = accepted ? 1 : 0;
-        sh_align[j] = align;
-        if (flags) atomicOr(&sh_flags, flags);
-        if (p.diag) {
+        // first rejection (Algorithm 4, the rejection step ends the loop): what to draw, and from which row
+        const int n_acc = __ffs(__ballot_sync(FULL, !accepted)) - 1;   // lanes >= k never accept
+        const uint32_t row_flags = __shfl_sync(FULL, r.flags, n_acc);
+        const int argmax = __shfl_sync(FULL, r.argmax_a, n_acc);
+        if (n_acc == k) flags |= row_flags;
+        if (!GREEDY) {
+            if (lane == 0) {
+                sh_nacc = n_acc;
+                sh_mode = row_flags ? 0 : n_acc == k ? 2 : 1;   // 2: bonus token from p_k, 1: correction from the residual
+            }
+            if (lane == n_acc) sh_u = uniform24(words.y);
+        }
+        __syncthreads();   // the draw may start; the positions' sums of min(p, q) are there
+        const double align = lane < k && !r.flags ? sh_align[lane] : 0.0;
+        if (lane < k && p.diag) {
             metasd_diag dg;
-            dg.p_x = p_x; dg.q_x = q_x; dg.D = D; dg.u = u; dg.accept = accepted ? 1 : 0;
+            dg.p_x = p_x; dg.q_x = q_x; dg.D = (float)(1.0 - align); dg.u = u; dg.accept = accepted ? 1 : 0;
             p.diag[(size_t)b * k_slots + j] = dg;
         }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        // first rejection (Algorithm 4, the rejection step ends the loop), reward (Definition 2), what to draw
-        int n_acc = k;
-        double sum_align = 0.0;
-        for (int j = k - 1; j >= 0; --j)
-            if (!sh_accept[j]) n_acc = j;
-        for (int j = 0; j < k; ++j) sum_align += sh_align[j];
-        int mode = n_acc == k ? 2 : 1;  // 2: bonus token from p_k, 1: correction from the residual
-        int tok = -1;
-        const RowStats rs = stats[n_acc];
-        if (n_acc == k && rs.flags) sh_flags |= rs.flags;
-        if (rs.flags) {
-            mode = 0;
-        } else if (p.greedy) {
-            mode = 0;
-            tok = rs.argmax_a;
-        }
-        sh_nacc = n_acc;
-        sh_mode = mode;
-        sh_tok = tok;
-        sh_u = uniform24(round_words(p.seed, p.sequence_base + (uint32_t)b, (uint32_t)t, (uint32_t)n_acc).y);
-        sh_reward = p.reward_kind == METASD_REWARD_BE ? (double)n_acc / (double)k : sum_align / (double)k;
-    }
-    __syncthreads();
-
-    int token = sh_tok;
-    const int mode = sh_mode, n_acc = sh_nacc;
-    if (mode != 0) {
-        const RowStats rs = stats[n_acc];
-        const LT *a = target + (size_t)n_acc * V;
-        const LT *d = mode == 1 ? draft + (size_t)n_acc * V : nullptr;
-        // the total of the draw's weights as the row statistics give it: sum max(0, p - q) = 1 - sum min(p, q); sum p = 1
-        const double known = mode == 1 ? 1.0 - rs.sum_min : 1.0;
-        token = block_inverse_cdf<LT, VECTOR, K2_THREADS>(a, d, V, mode, sh_u, c, rs.max_a, rs.sum_a, rs.max_b, rs.sum_b,
-                                                          known, sh_draw);
-        if (token < 0 && mode == 1) {  // p == q in fp32 yet rejected (the residual has no mass): draw from p
-            __syncthreads();   // every thread has read the first draw's answer before the work space is reused
-            token = draw_from_target<LT, VECTOR, K2_THREADS>(a, V, sh_u, c, rs.max_a, rs.sum_a, sh_draw);
-        }
-    }
-
-    if (tid < 32) {
-        // the bandit of this sequence: update with the reward, then the next round's arm (one lane per drafter)
-        const double r = sh_reward;
-        double *sa = p.st.stat_a + (size_t)b * K, *sb = p.st.stat_b + (size_t)b * K;
-        int32_t *wa = p.st.win_arm + (size_t)b * p.tau;
-        double *wr = p.st.win_reward + (size_t)b * p.tau;
-        warp_bandit_step(p.bandit, K, p.beta, p.gamma, p.tau, &p.st.t[b], &p.st.arm[b], sa, sb, wa, wr, arm, r, p.seed,
-                         p.sequence_base + (uint32_t)b);
-        if (tid == 0) {
+        // the reward (Definition 2), then the bandit of this sequence: update, and the next round's arm
+        const double reward = p.reward_kind == METASD_REWARD_BE ? (double)n_acc / (double)k : warp_sum(align) / (double)k;
+        warp_bandit_step(p.bandit, K, p.beta, p.gamma, p.tau, &p.st.t[b], &p.st.arm[b], p.st.stat_a + (size_t)b * K,
+                         p.st.stat_b + (size_t)b * K, p.st.win_arm + (size_t)b * p.tau, p.st.win_reward + (size_t)b * p.tau, arm,
+                         reward, p.seed, p.sequence_base + (uint32_t)b);
+        flags = __reduce_or_sync(FULL, flags);
+        if (lane == 0) {
             p.accepted_len[b] = n_acc;
-            p.next_token[b] = token;
-            p.reward[b] = (float)r;
-            if (sh_flags) atomicOr(p.status, sh_flags);
+            p.reward[b] = (float)reward;
+            if (GREEDY || row_flags) p.next_token[b] = row_flags ? -1 : argmax;
+            if (flags) atomicOr(p.status, flags);
+        }
+        return;
+    }
+
+    grid_dependency_wait();
+    // sum_v min(p_v, q_v) of every drafted position (16 at most), two positions per warp at a time
+    static_assert(NWARP >= 8, "two positions per warp cover the largest draft length");
+    double m[2] = {0.0, 0.0};
+    for (int s = lane; s < p.n_seg; s += 32) {
+        if (warp < k) m[0] += (double)segments[warp * p.n_seg + s].min;
+        if (warp + NWARP < k) m[1] += (double)segments[(warp + NWARP) * p.n_seg + s].min;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        m[i] = warp_sum(m[i]);
+        if (lane == 0 && warp + i * NWARP < k) sh_align[warp + i * NWARP] = m[i];
+    }
+    __syncthreads();
+    if (GREEDY || sh_mode == 0) return;   // greedy, or the row it needs is not finite: the control warp has the token
+    const int n_acc = sh_nacc;
+    const RowStats rs = stats[n_acc];
+    DrawRow<LT> row;
+    row.mode = sh_mode;
+    row.a = target + (size_t)n_acc * V;
+    row.d = row.mode == 1 ? draft + (size_t)n_acc * V : row.a;
+    row.nvec = V / VEC;
+    row.c = c;
+    row.nma = -rs.max_a * c; row.ia = 1.0f / rs.sum_a;
+    row.nmb = -rs.max_b * c; row.ib = 1.0f / rs.sum_b;
+    const float u = sh_u;
+    int token = -1;
+    if (p.n_seg > 1) {
+        // the part of the row with the crossing, found by every warp for itself
+        double x[4], threshold = (double)u, base, total;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[i] = 0.0;
+            if (lane * 4 + i < p.n_seg) {
+                const RowSegment g = segments[n_acc * p.n_seg + lane * 4 + i];
+                x[i] = row.mode == 1 ? fmax((double)g.p - (double)g.min, 0.0) : (double)g.p;
+            }
+        }
+        const int part = warp_find_part<true>(x, 0.0, threshold, base, total);
+        // Below a thousandth the parts' masses p - min are differences of numbers that far above them: the walk over
+        // the row, which takes the difference token by token, decides instead (such a rejection is rare by its own measure).
+        if (total > 1.0e-3) {
+            int lead = 0, shift = 0;
+            if (!VECTOR) row_alignment(row.a, row.mode == 1 ? row.d : nullptr, lead, shift);
+            const int trip = 32 * Logit<LT>::VEC, trips = (V + lead + shift + trip - 1) / trip;
+            const int lo = max(trip * segment_begin(trips, part, p.n_seg) - lead, 0);
+            const int hi = min(trip * segment_begin(trips, part + 1, p.n_seg) - lead, V);
+            token = range_inverse_cdf<LT, VEC, NWARP, false>(row, lo / VEC, hi / VEC, base, threshold, sh_draw);
         }
     }
+    if (token < 0) token = draw_whole_row<LT, VEC, NWARP>(row, u, sh_draw);
+    if (token < 0 && row.mode == 1) {   // p == q in fp32 yet rejected (the residual has no mass): draw from p
+        row.mode = 2;
+        token = draw_whole_row<LT, VEC, NWARP>(row, u, sh_draw);
+    }
+    if (tid == 0) p.next_token[b] = token;
 }
 
 // -------------------------------------------------------------------------------------------
@@ -1105,6 +1074,7 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
     geo->stages = cfg.row_stages;
     geo->per_sm = 1;
     geo->cluster = 1;
+    geo->n_seg = 1;
     if (cfg.row_cluster > 1 && geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;   // only the staged kernel has a cluster form
     if (geo->kernel == METASD_ROWS_PLAIN) {
         if (geo->threads && geo->threads != K1_THREADS) return cudaErrorNotSupported;
@@ -1123,14 +1093,18 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
     if (!geo->threads) geo->threads = dtype == METASD_FP32 && lng ? 1024 : 512;
     if (!geo->stages) geo->stages = dtype == METASD_BF16 && !lng && geo->threads == 512 ? 4 : 6;
     geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
+    geo->n_seg = geo->threads / 32 * geo->cluster;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, &geo->per_sm)
                                 : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, &geo->per_sm);
 }
 
+constexpr int DRAW_THREADS = 256;   // of an epilogue CTA besides its control warp
+
 template <typename LT>
-static cudaError_t launch_streaming_t(const VerifyParams &p, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches)
+static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches)
 {
     cudaError_t e = cudaSuccess;
+    p.n_seg = geo.n_seg;
     if (geo.kernel == METASD_ROWS_STAGED) {
         e = launch_staged_t<LT>(p, geo, stream);
     } else if (!p.vector_ok) {
@@ -1144,10 +1118,9 @@ static cudaError_t launch_streaming_t(const VerifyParams &p, const RowGeometry &
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // The epilogue is launched with programmatic stream serialisation: its blocks may be set up while the
     // row-statistics kernel drains, and wait (griddepcontrol.wait) for its completion before they read anything.
-    const bool big_ctas = p.batch <= 320;   // up to about one sequence per SM
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.batch);
-    cfg.blockDim = dim3(big_ctas ? 512u : 256u);
+    cfg.blockDim = dim3(DRAW_THREADS + 32u);   // and the control warp
     cfg.dynamicSmemBytes = 0;
     cfg.stream = stream;
     cudaLaunchAttribute at;
@@ -1155,13 +1128,9 @@ static cudaError_t launch_streaming_t(const VerifyParams &p, const RowGeometry &
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    if (!p.vector_ok) {
-        if (big_ctas) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, false, 512>, p);
-        else e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, false, 256>, p);
-    } else {
-        if (big_ctas) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, 512>, p);
-        else e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, 256>, p);
-    }
+    if (p.greedy) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, DRAW_THREADS, true>, p);
+    else if (p.vector_ok) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, DRAW_THREADS, false>, p);
+    else e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, false, DRAW_THREADS, false>, p);
     *launches += 2;
     return e;
 }
