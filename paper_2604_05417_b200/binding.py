@@ -122,12 +122,15 @@ def _check(code: int, what: str):
         raise MetasdError(code, what)
 
 
+# Plain integers: the signatures' c_void_p converts them, and a c_void_p object per argument and a torch.cuda.Stream object
+# per call were a third of the host time of a small round (19.5 us, of which the stream lookups 4.8).
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(device) -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _stream(device: torch.device) -> int:
+    """The current stream of the device, as the address of its cudaStream_t."""
+    return torch._C._cuda_getCurrentRawStream(device.index)
 
 
 @dataclass
@@ -210,7 +213,7 @@ class MetaSD:
             out.diag = torch.zeros((B, k, 5), dtype=torch.float32, device=self.device)
         rc = self.lib.metasd_verify(
             self._ctx, B, k, _ptr(target_logits), _ptr(draft_logits), _ptr(drafter_table),
-            _ptr(draft_tokens), token_arm_stride, C.c_float(temperature), C.c_uint64(seed),
+            _ptr(draft_tokens), token_arm_stride, temperature, seed,
             _ptr(out.accepted_len), _ptr(out.next_token), _ptr(out.reward), _ptr(out.diag),
             _stream(self.device))
         _check(rc, "metasd_verify")
@@ -224,7 +227,7 @@ class MetaSD:
         B, kp1, V = target_logits.shape
         rc = self.lib.metasd_verify_host(
             self._ctx, B, kp1 - 1, _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens),
-            C.c_float(temperature), C.c_uint64(seed), _ptr(accepted_len), _ptr(next_token),
+            temperature, seed, _ptr(accepted_len), _ptr(next_token),
             _ptr(reward), _ptr(arm_next), _stream(self.device))
         _check(rc, "metasd_verify_host")
 
@@ -274,8 +277,8 @@ def verify_noalloc(target_logits: torch.Tensor, draft_logits: torch.Tensor, draf
     dev = target_logits.device
     return load_library().metasd_verify_noalloc(
         B, kp1 - 1, V, DTYPES[target_logits.dtype], _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens),
-        C.c_float(temperature), C.c_float(reward_temperature), reward_kind, C.c_uint64(seed),
-        C.c_uint32(sequence_base), C.c_uint32(round_), _ptr(accepted_len), _ptr(next_token), _ptr(reward),
+        temperature, reward_temperature, reward_kind, seed,
+        sequence_base, round_, _ptr(accepted_len), _ptr(next_token), _ptr(reward),
         _ptr(status), _stream(dev))
 
 
