@@ -14,7 +14,7 @@ struct metasd_ctx {
     metasd_config cfg;
     BanditState st;
     RowStats *stats;     // scratch of the streaming path: [max_batch, max_draft + 1]
-    RowSegment *segments;   // and [max_batch, max_draft + 1, geo.n_seg]
+    RowSegment *segments;   // and the parts of their rows
     uint32_t *status;    // device status word
     const int32_t *draft_len;   // the caller's per-sequence draft lengths (device), or nullptr
     uint64_t launches;
@@ -214,7 +214,7 @@ int metasd_init(metasd_ctx **out, const metasd_config *cfg)
         e = streaming_prepare(cfg->device, cfg->logit_dtype, *cfg, &c->geo);
         if (e == cudaErrorNotSupported) { unsupported = true; (void)cudaGetLastError(); }
     }
-    alloc((void **)&c->segments, B * kp1 * c->geo.n_seg * sizeof(RowSegment));
+    alloc((void **)&c->segments, segment_capacity(c->geo, B * kp1) * sizeof(RowSegment));
     if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(uint32_t));
     if (e == cudaSuccess) e = launch_reset(c->st, cfg->max_batch, cfg->n_drafters, cfg->window, cfg->bandit, cfg->gamma,
                                             cfg->sequence_base, nullptr, cfg->max_batch, 0);

@@ -38,7 +38,8 @@ struct BanditState {
     double *win_reward;  // [B, tau]
 };
 
-// Shape of the row-statistics launch, resolved from the configuration once per context.
+// Shape of the row-statistics launch: what a context's configuration pins, resolved once; threads == 0 (staged kernel):
+// the shape follows the size of each launch.
 struct RowGeometry {
     int32_t kernel;     // metasd_row_kernel, never AUTO
     int32_t threads;    // threads per CTA
@@ -85,7 +86,7 @@ struct VerifyParams {
 };
 
 // streaming path (metasd_streaming.cu, metasd_bulk.cu)
-bool long_row(int dtype, int vocab);   // selects the launch shape: see streaming_prepare
+size_t segment_capacity(const RowGeometry &geo, size_t units);
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo);
 cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches);
 cudaError_t bulk_prepare(int dtype, RowGeometry *geo);

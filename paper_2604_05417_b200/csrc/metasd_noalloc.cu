@@ -22,7 +22,7 @@ namespace {
 
 constexpr int NOALLOC_MAX_ROWS = METASD_NOALLOC_MAX_ROWS;    // batch * (k + 1)
 constexpr int NOALLOC_MAX_BATCH = METASD_NOALLOC_MAX_BATCH;
-constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row of the default launch shapes, at most
+constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row where there are many rows (few rows have more: segment_capacity)
 
 // Everything the two kernels keep in global memory besides the caller's inputs and outputs.
 struct StaticScratch {
@@ -60,8 +60,8 @@ __global__ void noalloc_prepare_kernel(int batch, int32_t round)
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_lock;
 StaticScratch *g_scratch_ptr[MAX_DEVICES];   // device address of the array on each device, once known
-RowGeometry g_geometry[MAX_DEVICES][2][2];   // launch shape of the row-statistics kernel per device, logit type, long rows
-bool g_geometry_ready[MAX_DEVICES][2][2];
+RowGeometry g_geometry[MAX_DEVICES][2];      // of the row-statistics kernel per device and logit type
+bool g_geometry_ready[MAX_DEVICES][2];
 
 // Once per device, with that device current: ask the runtime where the array lives there.
 cudaError_t scratch_address(int device, StaticScratch **out)
@@ -77,21 +77,19 @@ cudaError_t scratch_address(int device, StaticScratch **out)
     return cudaSuccess;
 }
 
-// Once per device, logit type and class of row length: the default launch shape and the function attribute (a larger dynamic
-// shared-memory window) its kernel needs.  Neither allocates device memory.
-cudaError_t default_geometry(int device, int dtype, int vocab, RowGeometry *out)
+// Once per device and logit type: the default geometry and the function attribute (a larger dynamic
+// shared-memory window) its kernels need.  Neither allocates device memory.
+cudaError_t default_geometry(int device, int dtype, RowGeometry *out)
 {
     std::lock_guard<std::mutex> guard(g_setup_lock);
-    const int lng = long_row(dtype, vocab) ? 1 : 0;
-    if (!g_geometry_ready[device][dtype][lng]) {
+    if (!g_geometry_ready[device][dtype]) {
         metasd_config cfg;
         metasd_default_config(&cfg);
-        cfg.vocab = vocab;
-        cudaError_t e = streaming_prepare(device, dtype, cfg, &g_geometry[device][dtype][lng]);
+        cudaError_t e = streaming_prepare(device, dtype, cfg, &g_geometry[device][dtype]);
         if (e != cudaSuccess) return e;
-        g_geometry_ready[device][dtype][lng] = true;
+        g_geometry_ready[device][dtype] = true;
     }
-    *out = g_geometry[device][dtype][lng];
+    *out = g_geometry[device][dtype];
     return cudaSuccess;
 }
 
@@ -120,7 +118,8 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     StaticScratch *scratch = nullptr;
     if (scratch_address(device, &scratch) != cudaSuccess) return METASD_ERR_CUDA;
     RowGeometry geo;
-    if (default_geometry(device, logit_dtype, vocab, &geo) != cudaSuccess || geo.n_seg > NOALLOC_MAX_SEGMENTS) return METASD_ERR_CUDA;
+    if (default_geometry(device, logit_dtype, &geo) != cudaSuccess) return METASD_ERR_CUDA;
+    if (segment_capacity(geo, (size_t)batch * (k + 1)) > sizeof(scratch->segments) / sizeof(RowSegment)) return METASD_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
 
     VerifyParams p = {};

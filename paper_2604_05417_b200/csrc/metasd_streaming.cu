@@ -1021,7 +1021,11 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
 // launchers
 // -------------------------------------------------------------------------------------------
 // The built shapes of the staged kernel, per logit type: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).
-#define METASD_STAGED_SHAPES(X) \
+// Those that staged_shape() picks, and those that a configuration can ask for.
+#define METASD_STAGED_AUTO_SHAPES(X) \
+    X(512, 4, 3, true, 8) X(512, 4, 3, true, 4) X(512, 4, 3, true, 2) X(512, 4, 3, true, 1) X(512, 6, 2, true, 1) \
+    X(512, 6, 2, true, 2) X(256, 6, 4, true, 2) X(256, 6, 4, true, 1) X(256, 4, 6, true, 1) X(128, 4, 12, true, 1) X(1024, 6, 1, false, 1)
+#define METASD_STAGED_PINNED_SHAPES(X) \
     X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(1024, 6, 1, false, 1) X(1024, 4, 1, true, 1) X(768, 4, 2, true, 1) X(384, 4, 4, true, 1) \
     X(512, 4, 3, true, 3) X(512, 4, 3, true, 2) X(768, 4, 2, true, 2)
 
@@ -1036,13 +1040,18 @@ static cudaError_t prepare_staged()
     return e;
 }
 
+// threads == 0: every shape that staged_shape() may pick.
 template <typename LT>
-static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int *per_sm)
+static cudaError_t prepare_staged_t(int threads, int stages, int cluster)
 {
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) { *per_sm = M; return prepare_staged<LT, D, T, M, BL, C>(); }
-    METASD_STAGED_SHAPES(X)
+    cudaError_t e = threads == 0 ? cudaSuccess : cudaErrorNotSupported;
+#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C>();
+    METASD_STAGED_PINNED_SHAPES(X)
 #undef X
-    return cudaErrorNotSupported;
+#define X(T, D, M, BL, C) if (e == cudaSuccess) e = prepare_staged<LT, D, T, M, BL, C>();
+    METASD_STAGED_AUTO_SHAPES(X)
+#undef X
+    return e;
 }
 
 template <typename LT>
@@ -1051,20 +1060,80 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
 #define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
         return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, stream);
-    METASD_STAGED_SHAPES(X)
+    METASD_STAGED_AUTO_SHAPES(X)
+    METASD_STAGED_PINNED_SHAPES(X)
 #undef X
     return cudaErrorNotSupported;
 }
 
-// Whether a row is so long that a larger share of the pair kept on chip pays for fewer row pairs in flight.  Measured on
-// B200, us a round at k = 5 (bf16: 512 threads with 4 stages at 3 CTAs per SM / 6 stages at 2 CTAs; fp32: 512 threads with
-// 6 stages at 2 CTAs per SM / 1024 threads with 6 stages at 1):
-//   bf16, B = 256: V = 32000 71 / 74, 50264 95 / 100, 64000 110 / 112, 80000 132 / 131, 96000 152 / 149, 112000 174 / 169
-//   fp32: B = 256, V = 32000 89 / 107, 64000 167 / 168; B = 64, V = 128256 130 / 121
-// Short rows want more of them in flight: the fixed part of a CTA's life is what they cost.
-bool long_row(int dtype, int vocab) { return dtype == METASD_BF16 ? vocab >= 80000 : vocab >= 64000; }
+// Launches of at most this many rows (row pairs) may take the cluster shapes with more than 32 parts per row.
+constexpr int FEW_ROWS = 148;
 
-// Resolves the row-statistics shape for a context and sets the launch attributes its kernels need, once.
+// The shape for rows of `row_bytes` bytes in a launch of `units` rows (row pairs and bonus rows).  Measured on B200, us a
+// round (threads / stages / CTAs per row; units = B (k + 1)):
+//   bf16, few rows: a row is split until every SM has a CTA.
+//     5 rows, V = 32000: 512/4/1 19.4, /4 16.8, /8 16.5.  36, V = 152064: 34.3, /4 21.7, /8 23.0.  72, V = 128256: 31.6, /2 23.5, /4 25.2.
+//   bf16, many short rows: small CTAs, because the fixed part of a CTA's life is what a short row costs.
+//     V = 8000, 5120 rows: 512/4 108, 256/4 85, 128/4 74.  V = 16000, 9216 rows: 218, 174, 161; 1536 rows: 44, 37, 38.
+//     V = 32000, 1536 rows: 65.6, 60.0; 5120 rows: 182, 164.  V = 48000, 5120 rows: 258, 238.  V = 50257, 5120 rows: 324, 347.
+//   bf16, long rows in a few waves of CTAs: two small CTAs share a row, so that the last wave is finer.
+//     V = 152064, 576 rows: 512/6/1 102, 512/4/2 96.5, 256/6/2 96.4.  V = 128256, 768 rows: 108, 102, 101.  V = 80000, 384 rows: 48, 49, 44.
+//     Off 16-byte boundaries: V = 152065, 680 rows: 165, 145, 161.  V = 80001, 384 rows: 67, 64, 71, 512/4/1 63.
+//   bf16, medium rows: V = 60000, 5120 rows: 512/4/1 302, 256/6/1 283; 1536 rows: 94.5, 94.6.  V = 72000, 1536 rows: 112.5, 111.7.
+//     Off 16-byte boundaries (V = 50257, 5120 rows): 324, 349.
+//   bf16, long rows: a larger share of the pair kept on chip pays for fewer of them in flight from 80000 tokens on
+//     (B = 256, k = 5, 512/4 / 512/6: V = 64000 110 / 112, 80000 132 / 131, 112000 174 / 169).
+//   fp32 (half as many exponentials per byte) wants more of a row in flight and on chip.
+//     24 rows, V = 128256: split until the slots of all SMs are taken: 96 rows 512/4/1 37, /4 31.4.  V = 8000, 5120 rows: 512/4 111, 256/4 91.
+//     V = 32000: 5120 rows 512/6 265, 256/6 255; 1536 rows 88, 90; 384 rows 31.8, 29.0.
+//     V = 128256: 192 rows 1024/6/1 69, 512/6/2 63; 384 rows 98, 97; 768 rows 161, 167.
+struct StagedShape {
+    int threads, stages, cluster;
+};
+static StagedShape staged_shape(int dtype, long long row_bytes, long long units, bool aligned)
+{
+    const bool fp32 = dtype == METASD_FP32;
+    const long long trips = (row_bytes + 511) / 512;
+    // few rows: as many CTAs per row as there is room for, each warp with a trip or two left
+    for (int cl = 8; cl > 1; cl /= 2)
+        if (units <= FEW_ROWS && units * cl <= (fp32 ? 3 * FEW_ROWS : FEW_ROWS) && trips >= (fp32 ? 3 : 2) * 16 * cl) return {512, 4, cl};
+    if (fp32) {
+        if (row_bytes <= 32 * 1024) return {256, 4, 1};
+        if (row_bytes < 250 * 1024) return {256, 6, 1};
+        return units <= 500 ? StagedShape{512, 6, 2} : StagedShape{1024, 6, 1};
+    }
+    if (units <= FEW_ROWS) return {512, 4, 1};
+    if (row_bytes <= 32 * 1024) return {128, 4, 1};
+    if (row_bytes < 100 * 1000) return {256, 4, 1};
+    if (units <= 1000) return aligned ? StagedShape{256, 6, 2} : StagedShape{512, 4, row_bytes >= 200 * 1000 ? 2 : 1};
+    if (row_bytes < 160 * 1000) return aligned ? StagedShape{256, 6, 1} : StagedShape{512, 4, 1};
+    return {512, 6, 1};
+}
+
+// The shape of a launch: what the configuration pinned, else by the size of the launch.
+static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units, bool aligned)
+{
+    RowGeometry g = geo;
+    if (g.kernel == METASD_ROWS_STAGED && g.threads == 0) {
+        const StagedShape s = staged_shape(dtype, (long long)vocab * (dtype == METASD_BF16 ? 2 : 4), units, aligned);
+        g.threads = s.threads;
+        g.stages = s.stages;
+        g.cluster = s.cluster;
+    }
+    g.n_seg = g.kernel == METASD_ROWS_STAGED ? g.threads / 32 * g.cluster : 1;
+    return g;
+}
+
+// Parts of rows that launches of up to `units` rows report on, at most.
+size_t segment_capacity(const RowGeometry &geo, size_t units)
+{
+    if (geo.kernel != METASD_ROWS_STAGED) return units;
+    if (geo.threads) return units * (size_t)(geo.threads / 32 * geo.cluster);
+    const size_t few = (units < FEW_ROWS ? units : FEW_ROWS) * MAX_SEGMENTS, many = units * 32;
+    return few > many ? few : many;
+}
+
+// Resolves the row-statistics variant of a context and sets the launch attributes its kernels need, once.
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo)
 {
     cudaError_t e = cudaDeviceGetAttribute(&geo->n_sm, cudaDevAttrMultiProcessorCount, device);
@@ -1074,7 +1143,6 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
     geo->stages = cfg.row_stages;
     geo->per_sm = 1;
     geo->cluster = 1;
-    geo->n_seg = 1;
     if (cfg.row_cluster > 1 && geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;   // only the staged kernel has a cluster form
     if (geo->kernel == METASD_ROWS_PLAIN) {
         if (geo->threads && geo->threads != K1_THREADS) return cudaErrorNotSupported;
@@ -1089,21 +1157,24 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         return bulk_prepare(dtype, geo);
     }
     if (geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;
-    const bool lng = long_row(dtype, cfg.vocab);
-    if (!geo->threads) geo->threads = dtype == METASD_FP32 && lng ? 1024 : 512;
-    if (!geo->stages) geo->stages = dtype == METASD_BF16 && !lng && geo->threads == 512 ? 4 : 6;
-    geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
-    geo->n_seg = geo->threads / 32 * geo->cluster;
-    return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, &geo->per_sm)
-                                : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, &geo->per_sm);
+    // a configuration that names any of the three pins the shape: the others take the values of a long row of the type
+    if (geo->threads || geo->stages || cfg.row_cluster > 0) {
+        if (!geo->threads) geo->threads = dtype == METASD_BF16 ? 512 : 1024;
+        if (!geo->stages) geo->stages = dtype == METASD_BF16 && geo->threads == 512 ? 4 : 6;
+        geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
+    }
+    return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster)
+                                : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster);
 }
 
 constexpr int DRAW_THREADS = 256;   // of an epilogue CTA besides its control warp
 
 template <typename LT>
-static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches)
+static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context_geo, cudaStream_t stream, uint64_t *launches)
 {
     cudaError_t e = cudaSuccess;
+    const RowGeometry geo = resolve_geometry(context_geo, sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32, p.V, (long long)p.batch * (p.k + 1),
+                                             p.vector_ok != 0);
     p.n_seg = geo.n_seg;
     if (geo.kernel == METASD_ROWS_STAGED) {
         e = launch_staged_t<LT>(p, geo, stream);

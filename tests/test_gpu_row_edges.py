@@ -92,3 +92,17 @@ def test_tensors_that_start_anywhere(dtype, V):
             assert gpu.last_status() == 0
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("dtype,V,B,k", [
+    ("bf16", 65536, 1, 2), ("bf16", 65543, 6, 2), ("bf16", 33000, 12, 2), ("bf16", 17001, 49, 2),        # few rows, split over CTAs
+    ("bf16", 4104, 60, 2), ("bf16", 4101, 60, 2), ("bf16", 17008, 60, 2), ("bf16", 17003, 60, 2),        # short rows
+    ("bf16", 50008, 60, 2), ("bf16", 50011, 60, 2), ("bf16", 100003, 60, 2),                             # a few waves of long rows
+    ("bf16", 50008, 340, 2), ("bf16", 50003, 340, 2), ("bf16", 80008, 340, 2),                           # many of them
+    ("fp32", 16384, 1, 2), ("fp32", 49155, 12, 2), ("fp32", 8192, 60, 2), ("fp32", 9001, 60, 2), ("fp32", 64008, 60, 2),
+    ("fp32", 64009, 170, 2)])
+def test_every_shape_that_a_launch_size_selects(dtype, V, B, k):
+    """The row-statistics shape follows the row length, the number of rows and their alignment: one launch of each."""
+    from _harness import run_lockstep
+    c = run_lockstep(workload(V=V, dtype=dtype, B=B, k=k, temperature=0.9), rounds=2, seed=V % 83, path=M.PATH_STREAMING)
+    assert c["rounds"] == 2 and c["status"] == 0
