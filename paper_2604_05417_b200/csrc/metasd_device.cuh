@@ -124,6 +124,10 @@ template <> struct Logit<__nv_bfloat16> {
     {
         return __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(p)[i] << 16);
     }
+    __device__ static __forceinline__ float scalar_l2(const __nv_bfloat16 *p, size_t i)
+    {
+        return __uint_as_float((uint32_t)__ldcg(reinterpret_cast<const unsigned short *>(p) + i) << 16);
+    }
     // The vector of tokens tok0 .. tok0 + 7 with -Inf in the place of tokens outside [0, V).
     __device__ static __forceinline__ uint4 masked(const uint4 &r, int tok0, int V)
     {
@@ -213,6 +217,7 @@ template <> struct Logit<float> {
         x[3] = __uint_as_float(raw.w);
     }
     __device__ static __forceinline__ float scalar(const float *p, size_t i) { return p[i]; }
+    __device__ static __forceinline__ float scalar_l2(const float *p, size_t i) { return __ldcg(p + i); }
     __device__ static __forceinline__ uint4 masked(const uint4 &r, int tok0, int V)
     {
         uint32_t w[4] = {r.x, r.y, r.z, r.w};
@@ -255,13 +260,21 @@ template <> struct Logit<float> {
     }
 };
 
+// What a kernel reads before its grid_dependency_wait() is read from L2 (__ldcg): the kernels that wrote it are complete,
+// but nothing has yet made their writes visible to a line that this SM's L1 may still hold.
+
 // Tokens sequence b drafted this round: the call's k unless the caller registered per-sequence lengths, which are
 // clamped to 1 .. k (the epilogue flags a length outside that range).
 __device__ __forceinline__ int drafted(const int32_t *draft_len, int b, int k)
 {
     if (!draft_len) return k;
-    const int kb = draft_len[b];
+    const int kb = __ldcg(draft_len + b);
     return kb < 1 ? 1 : (kb > k ? k : kb);
+}
+
+__device__ __forceinline__ const void *table_entry(const void *const *table, int i)
+{
+    return reinterpret_cast<const void *>(__ldcg(reinterpret_cast<const unsigned long long *>(table) + i));
 }
 
 // Rows of the drafter sequence b plays: the gathered tensor, or the entry of the caller's pointer table for the
@@ -272,7 +285,7 @@ template <typename LT>
 __device__ __forceinline__ const LT *draft_rows(const VerifyParams &p, int b)
 {
     if (p.draft) return reinterpret_cast<const LT *>(p.draft);
-    const void *q = p.drafter_ptrs[p.st.arm[b]];
+    const void *q = table_entry(p.drafter_ptrs, __ldcg(p.st.arm + b));
     if (q == nullptr || (reinterpret_cast<uintptr_t>(q) & p.table_mask) != 0) q = p.target;
     return reinterpret_cast<const LT *>(q);
 }
@@ -496,8 +509,11 @@ __device__ __forceinline__ void sts16(uint32_t addr, const uint4 &v)
     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// Programmatic dependent launch: lets the next kernel in the stream be set up while this grid still runs.  That
-// kernel waits for this whole grid (griddepcontrol.wait) before it touches anything this one reads or writes.
+// Programmatic dependent launch.  launch_dependents lets the next kernel in the stream be set up while this grid still runs;
+// grid_dependency_wait blocks until the kernel launched before this one has finished and its writes are visible (a no-op
+// when this kernel was launched without programmatic stream serialisation).  Every kernel that is launched that way waits
+// before it ends, so the completion of one means the completion of all before it.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float warp_sum_f(float v)

@@ -78,6 +78,8 @@ struct VerifyParams {
     RowSegment *segments;    // [batch, k+1, n_seg]
     int32_t n_seg;           // parts per row, set by the launcher
     uint32_t *status;
+    int32_t stateless;       // no bandit: the round counter is `round`, `st` is not touched, *status is this call's alone
+    int32_t round;
     int32_t vector_ok; // rows are 16-byte aligned and a whole number of 16-byte vectors
     int32_t keep_permille;   // share (its end) of every row that the first sweep asks L2 to keep for the second
     int32_t keep_from_vec;   // the same as the first 16-byte vector of that share

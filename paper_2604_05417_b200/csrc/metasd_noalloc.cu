@@ -28,34 +28,12 @@ constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row where there are many
 struct StaticScratch {
     RowStats rows[NOALLOC_MAX_ROWS];       // written by the row-statistics kernel, read by the epilogue
     RowSegment segments[NOALLOC_MAX_ROWS * NOALLOC_MAX_SEGMENTS];
-    double stat_a[NOALLOC_MAX_BATCH];      // a one-armed dummy bandit per sequence: the epilogue kernel
-    double stat_b[NOALLOC_MAX_BATCH];      // updates it and nobody reads it
-    double win_reward[NOALLOC_MAX_BATCH];
-    int32_t t[NOALLOC_MAX_BATCH];          // round counter the epilogue keys the uniforms with
-    int32_t arm[NOALLOC_MAX_BATCH];
-    int32_t win_arm[NOALLOC_MAX_BATCH];
-    uint32_t status;
+    uint32_t status;                       // where the status bits go that the caller does not ask for
 };
 
 // The scratch itself.  In host code this name is only a handle for cudaGetSymbolAddress: it is not a
 // device address and must never be passed to a kernel.
 static __device__ __align__(256) StaticScratch g_noalloc_scratch[1];
-
-// Device code may name the array directly: start every call from a clean dummy-bandit block.
-__global__ void noalloc_prepare_kernel(int batch, int32_t round)
-{
-    StaticScratch &s = g_noalloc_scratch[0];
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b == 0) s.status = 0u;
-    if (b < batch) {
-        s.t[b] = round;
-        s.arm[b] = 0;
-        s.stat_a[b] = 0.0;
-        s.stat_b[b] = 0.0;
-        s.win_arm[b] = 0;
-        s.win_reward[b] = 0.0;
-    }
-}
 
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_lock;
@@ -132,11 +110,10 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     p.c = (float)(1.4426950408889634 / (p.greedy ? (double)reward_temperature : (double)temperature));
     p.seed = seed; p.beta = 0.0; p.gamma = 1.0;
     p.accepted_len = accepted_len; p.next_token = next_token; p.reward = reward; p.diag = nullptr;
-    p.st.t = scratch->t; p.st.arm = scratch->arm;
-    p.st.stat_a = scratch->stat_a; p.st.stat_b = scratch->stat_b;
-    p.st.win_arm = scratch->win_arm; p.st.win_reward = scratch->win_reward;
+    p.stateless = 1;
+    p.round = (int32_t)round;
     p.stats = scratch->rows; p.segments = scratch->segments;
-    p.status = &scratch->status;
+    p.status = status_out ? status_out : &scratch->status;   // zeroed by the row-statistics kernel
     const size_t row_bytes = (size_t)vocab * (logit_dtype == METASD_BF16 ? 2 : 4);
     p.vector_ok = row_bytes % 16 == 0 && ((uintptr_t)target_logits % 16) == 0 && ((uintptr_t)draft_logits % 16) == 0;
     {   // the share of every row that L2 is asked to keep between the sweeps: as in a default context
@@ -146,11 +123,7 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     }
     p.poll_limit = 1u << 18;
 
-    noalloc_prepare_kernel<<<(batch + 255) / 256, 256, 0, s>>>(batch, (int32_t)round);
-    cudaError_t e = cudaGetLastError();
     uint64_t launches = 0;
-    if (e == cudaSuccess) e = launch_streaming(p, logit_dtype, geo, s, &launches);
-    if (e == cudaSuccess && status_out)
-        e = cudaMemcpyAsync(status_out, &scratch->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
+    const cudaError_t e = launch_streaming(p, logit_dtype, geo, s, &launches);
     return e == cudaSuccess ? METASD_OK : METASD_ERR_CUDA;
 }

@@ -264,7 +264,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     extern __shared__ __align__(16) unsigned char stage_mem[];
     __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
-    launch_dependents();   // the epilogue may be set up while this kernel runs; it waits for the whole grid before it reads
+    // The rows, the arms and what the last epilogue read of the scratch belong to the kernels before.  The epilogue may be
+    // set up behind that wait only: what this kernel does not write, it reads before its own.
+    grid_dependency_wait();
+    launch_dependents();
+    if (p.stateless && blockIdx.x == 0 && threadIdx.x == 0) *p.status = 0u;
     // Blocks are dispatched in index order.  BONUS_LAST: the row pairs come first and the bonus rows (one row, half
     // the work) last, so that the launch ends on its shortest items (measured: better for the bf16 geometry, worse
     // for the fp32 one, which keeps the bonus rows interleaved).
@@ -595,25 +599,43 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         p.segments[row * NREC + part] = RowSegment{sum_aw * ex2((w.m - ra.m) * c) / ra.s, part_min};
 }
 
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
-static cudaError_t launch_staged(const VerifyParams &p, unsigned units, cudaStream_t stream)
+// Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it
+// in the stream drains, and wait (grid_dependency_wait) before they touch what that one does.
+template <typename... Params, typename... Args>
+static cudaError_t launch_kernel(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, int cluster, bool chained,
+                                 cudaStream_t stream, const Args &...args)
 {
-    constexpr uint32_t smem = STAGED_SMEM<D, THREADS, SHIFTED>;   // the attribute that allows it was set by streaming_prepare
-    if (CL == 1) {
-        row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED><<<units, THREADS, smem, stream>>>(p);
-        return cudaSuccess;
-    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(units * CL);
-    cfg.blockDim = dim3(THREADS);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = CL; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, p);
+    cudaLaunchAttribute at[2];
+    cfg.attrs = at;
+    if (chained) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        cudaLaunchAttribute &a = at[cfg.numAttrs++];
+        a.val.clusterDim.x = (unsigned)cluster; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
+static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm, cudaStream_t stream)
+{
+    // A launch of about one wave wants its blocks spread evenly over idle SMs: set up while the last epilogue still holds some
+    // of them, they crowd on the others and stay there (us a round, chained / not: B = 64, k = 5, V = 32000 34.9 / 26.7; B = 4,
+    // k = 8, V = 152064 in clusters, 144 CTAs, 23.5 / 20.5; several waves gain: B = 96, k = 5, V = 50257 56.7 / 62.0, B = 192,
+    // k = 8 ragged, V = 50264 61.9 / 69.8).
+    const unsigned ctas = units * CL;
+    const bool chained = ctas <= (unsigned)n_sm / 2 || ctas > (unsigned)n_sm * MINB;
+    // the attribute that allows the shared memory was set by streaming_prepare
+    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, ctas, THREADS,
+                         STAGED_SMEM<D, THREADS, SHIFTED>, CL, chained, stream, p);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -848,10 +870,6 @@ __device__ __noinline__ int draw_whole_row(const DrawRow<LT> &row, float u, Draw
     return range_inverse_cdf<LT, VEC, NWARP, true>(row, 0, row.nvec, 0.0, (double)u, sh);
 }
 
-// Blocks until the kernel launched before this one in the stream has finished and its writes are visible (a no-op
-// when this kernel was launched without programmatic stream serialisation).
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // One CTA per sequence: DRAW_THREADS threads for the draw (GREEDY: there is none, they only add up the parts of
 // sum min(p, q)) and one control warp for the accept tests, the first rejection, the reward and the bandit, which runs
 // while the other warps search for the token.  What bounds it is the chain of dependent reads of its slowest sequence.
@@ -875,9 +893,10 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     __shared__ double sh_align[16];
     __shared__ DrawShared<NWARP> sh_draw;
 
-    // The row-statistics kernel may still be running when this kernel starts (programmatic stream serialisation).  What it
-    // writes (stats, segments) is read, and what it reads is written, behind grid_dependency_wait() only; everything else
-    // was there before it began and is fetched meanwhile.
+    // The row-statistics kernel may still be running when this kernel starts.  What it writes (stats, segments) is read,
+    // and what it reads is written, behind grid_dependency_wait() only; everything else was there before that kernel let
+    // this one start, and is fetched meanwhile.
+    launch_dependents();
     const int k = drafted(p.draft_len, b, k_slots);   // positions this sequence drafted this round
     const LT *target = reinterpret_cast<const LT *>(p.target) + (size_t)b * (k_slots + 1) * V;
     const LT *draft = draft_rows<LT>(p, b) + (size_t)b * k_slots * V;
@@ -885,24 +904,24 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     const RowSegment *segments = p.segments + (size_t)b * (k_slots + 1) * p.n_seg;
 
     if (warp == NWARP) {
-        uint32_t flags = lane == 0 && p.draft_len && p.draft_len[b] != k ? METASD_STATUS_BAD_LENGTH : 0u;
+        uint32_t flags = lane == 0 && p.draft_len && __ldcg(p.draft_len + b) != k ? METASD_STATUS_BAD_LENGTH : 0u;
         // pointer-table mode: an entry that must not be dereferenced is flagged once per call, played or not
         if (b == 0 && p.drafter_ptrs && lane < K) {
-            const void *q = p.drafter_ptrs[lane];
+            const void *q = table_entry(p.drafter_ptrs, lane);
             if (q == nullptr || (reinterpret_cast<uintptr_t>(q) & p.table_mask) != 0) flags |= METASD_STATUS_BAD_POINTER;
         }
-        const int t = p.st.t[b], arm = p.st.arm[b];
+        const int t = p.stateless ? p.round : __ldcg(p.st.t + b), arm = p.stateless ? 0 : __ldcg(p.st.arm + b);
         // lane j < k: the accept test of Algorithm 4 at position j; lane j = k only brings the bonus row's words and flags
         const int j = min(lane, k);
         const uint4 words = round_words(p.seed, p.sequence_base + (uint32_t)b, (uint32_t)t, (uint32_t)j);
         const float u = uniform24(words.x);
         int x = -1;
-        if (lane < k) x = p.tokens[(p.token_arm_stride ? (size_t)arm * p.token_arm_stride : 0) + (size_t)b * k_slots + j];
+        if (lane < k) x = __ldcg(p.tokens + (p.token_arm_stride ? (size_t)arm * p.token_arm_stride : 0) + (size_t)b * k_slots + j);
         const bool in_range = x >= 0 && x < V;
         float a_x = 0.f, d_x = 0.f;
         if (in_range) {
-            a_x = Logit<LT>::scalar(target + (size_t)j * V, x);
-            d_x = Logit<LT>::scalar(draft + (size_t)j * V, x);
+            a_x = Logit<LT>::scalar_l2(target + (size_t)j * V, x);
+            d_x = Logit<LT>::scalar_l2(draft + (size_t)j * V, x);
         }
         grid_dependency_wait();
         const RowStats r = stats[j];
@@ -946,9 +965,10 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         }
         // the reward (Definition 2), then the bandit of this sequence: update, and the next round's arm
         const double reward = p.reward_kind == METASD_REWARD_BE ? (double)n_acc / (double)k : warp_sum(align) / (double)k;
-        warp_bandit_step(p.bandit, K, p.beta, p.gamma, p.tau, &p.st.t[b], &p.st.arm[b], p.st.stat_a + (size_t)b * K,
-                         p.st.stat_b + (size_t)b * K, p.st.win_arm + (size_t)b * p.tau, p.st.win_reward + (size_t)b * p.tau, arm,
-                         reward, p.seed, p.sequence_base + (uint32_t)b);
+        if (!p.stateless)
+            warp_bandit_step(p.bandit, K, p.beta, p.gamma, p.tau, &p.st.t[b], &p.st.arm[b], p.st.stat_a + (size_t)b * K,
+                             p.st.stat_b + (size_t)b * K, p.st.win_arm + (size_t)b * p.tau, p.st.win_reward + (size_t)b * p.tau,
+                             arm, reward, p.seed, p.sequence_base + (uint32_t)b);
         flags = __reduce_or_sync(FULL, flags);
         if (lane == 0) {
             p.accepted_len[b] = n_acc;
@@ -1020,6 +1040,8 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
 // -------------------------------------------------------------------------------------------
 // launchers
 // -------------------------------------------------------------------------------------------
+constexpr int DRAW_THREADS = 256;   // of an epilogue CTA besides its control warp
+
 // The built shapes of the staged kernel, per logit type: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).
 // Those that staged_shape() picks, and those that a configuration can ask for.
 #define METASD_STAGED_AUTO_SHAPES(X) \
@@ -1059,7 +1081,7 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
 {
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
 #define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
-        return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, stream);
+        return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, geo.n_sm, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
     METASD_STAGED_AUTO_SHAPES(X)
     METASD_STAGED_PINNED_SHAPES(X)
 #undef X
@@ -1133,6 +1155,25 @@ size_t segment_capacity(const RowGeometry &geo, size_t units)
     return few > many ? few : many;
 }
 
+__global__ void select_kernel(const int32_t *arm, int batch, int32_t *arm_out);
+
+// The kernels between two row-statistics launches leave the SMs set to the large shared memory that those need: an SM
+// changes the split between L1 and shared memory only when it is idle, and the blocks of the next launch arrive before
+// (B = 64, k = 5, V = 32000: 35.7 us a round without this).
+template <typename LT>
+static cudaError_t prepare_small_kernels()
+{
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void *kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    };
+    set((const void *)epilogue_kernel<LT, true, DRAW_THREADS, true>);
+    set((const void *)epilogue_kernel<LT, true, DRAW_THREADS, false>);
+    set((const void *)epilogue_kernel<LT, false, DRAW_THREADS, false>);
+    set((const void *)select_kernel);
+    return e;
+}
+
 // Resolves the row-statistics variant of a context and sets the launch attributes its kernels need, once.
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo)
 {
@@ -1163,11 +1204,10 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         if (!geo->stages) geo->stages = dtype == METASD_BF16 && geo->threads == 512 ? 4 : 6;
         geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
     }
+    if ((e = dtype == METASD_BF16 ? prepare_small_kernels<__nv_bfloat16>() : prepare_small_kernels<float>()) != cudaSuccess) return e;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster)
                                 : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster);
 }
-
-constexpr int DRAW_THREADS = 256;   // of an epilogue CTA besides its control warp
 
 template <typename LT>
 static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context_geo, cudaStream_t stream, uint64_t *launches)
@@ -1187,21 +1227,10 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
     }
     if (e != cudaSuccess) return e;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // The epilogue is launched with programmatic stream serialisation: its blocks may be set up while the
-    // row-statistics kernel drains, and wait (griddepcontrol.wait) for its completion before they read anything.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.batch);
-    cfg.blockDim = dim3(DRAW_THREADS + 32u);   // and the control warp
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    if (p.greedy) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, DRAW_THREADS, true>, p);
-    else if (p.vector_ok) e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, true, DRAW_THREADS, false>, p);
-    else e = cudaLaunchKernelEx(&cfg, epilogue_kernel<LT, false, DRAW_THREADS, false>, p);
+    const unsigned grid = (unsigned)p.batch, threads = DRAW_THREADS + 32;   // and the control warp
+    if (p.greedy) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, true>, grid, threads, 0, 1, true, stream, p);
+    else if (p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
+    else e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
     *launches += 2;
     return e;
 }
@@ -1219,14 +1248,15 @@ cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry
 // device-to-device cudaMemcpyAsync: measured on the launch-bound configurations the copy-engine hop cost more.)
 __global__ void select_kernel(const int32_t *arm, int batch, int32_t *arm_out)
 {
+    launch_dependents();
+    grid_dependency_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < batch) arm_out[b] = arm[b];
 }
 
 cudaError_t launch_select(const BanditState &st, int batch, int32_t *arm_out, cudaStream_t stream)
 {
-    select_kernel<<<(batch + 255) / 256, 256, 0, stream>>>(st.arm, batch, arm_out);
-    return cudaGetLastError();
+    return launch_kernel(select_kernel, (unsigned)(batch + 255) / 256, 256, 0, 1, true, stream, (const int *)st.arm, batch, arm_out);
 }
 
 __global__ void reset_kernel(BanditState st, int max_batch, int K, int tau, int variant, double gamma,
