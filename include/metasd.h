@@ -205,8 +205,8 @@ int metasd_verify(metasd_ctx *ctx, int32_t batch, int32_t k, const void *target_
 int metasd_set_draft_lengths(metasd_ctx *ctx, const int32_t *draft_len);
 
 /* The same round with HOST buffers (gathered draft logits only): copies the inputs to the context's
- * staging memory, runs metasd_verify, copies the three outputs (and host_arm_next, optional: the
- * next round's selection) back, and synchronises the stream.  Needs cfg.host_staging != 0.
+ * staging memory, runs metasd_verify with outputs in pinned host memory, hands those (and host_arm_next, optional: the
+ * next round's selection) to the caller, and synchronises the stream.  Needs cfg.host_staging != 0.
  * Pinned host memory makes the copies asynchronous. */
 int metasd_verify_host(metasd_ctx *ctx, int32_t batch, int32_t k, const void *host_target_logits,
                        const void *host_draft_logits, const int32_t *host_draft_tokens,

@@ -76,3 +76,27 @@ def test_no_allocation_calls_back_to_back():
     for i, (x, y) in enumerate(zip(one, many)):
         assert all(torch.equal(p, q) for p, q in zip(x, y))
         assert int(x[3]) == (M.STATUS_TOKEN_OOR if i & 1 else 0)
+
+
+@pytest.mark.parametrize("B,V,k,bandit", [(10, 152064, 3, "swucb"), (7, 100003, 4, "ucb"), (3, 300000, 2, "exp3")])
+@pytest.mark.parametrize("T", [0.0, 0.8])
+def test_host_buffers_give_the_device_calls_round(B, V, k, bandit, T):
+    """Results that the kernels write to host memory: outputs, next arms and bandit state of the device call, bit for bit."""
+    wl = Workload("t", B=B, N=2, k=k, V=V, rounds=3, temperature=T, dtype="bf16", bandit="ucb", sigmas=(0.4, 2.0))
+    gen = RoundGenerator(wl, device=torch.device("cuda", 0), seed=V % 71)
+    a = M.MetaSD(B + 2, 2, k + 1, V, bandit=bandit, window=4, sequence_base=5)
+    b = M.MetaSD(B + 2, 2, k + 1, V, bandit=bandit, window=4, sequence_base=5, host_staging=True)
+    lengths = torch.tensor([1 + i % k for i in range(B + 2)], dtype=torch.int32, device="cuda")
+    for t in range(3):
+        rd = gen.gathered_round(t, np.zeros(B, dtype=np.int64))
+        for m in (a, b):
+            m.set_draft_lengths(lengths if t == 1 else None)
+        ra = a.verify(rd["target"], rd["draft"], rd["tokens"], T, 3)
+        host = [rd[n].cpu().pin_memory() for n in ("target", "draft", "tokens")]
+        acc, tok, nxt = (torch.zeros(B, dtype=torch.int32) for _ in range(3))
+        rew = torch.zeros(B)
+        b.verify_host(*host, T, 3, acc, tok, rew, nxt)
+        assert torch.equal(ra.accepted_len.cpu(), acc) and torch.equal(ra.next_token.cpu(), tok) and torch.equal(ra.reward.cpu(), rew)
+        assert torch.equal(a.select(B).cpu(), nxt)
+    assert a.state_export() == b.state_export()
+    a.close(); b.close()
