@@ -676,90 +676,124 @@ __device__ inline void bandit_update(int variant, int K, double gamma, int tau, 
     *t = *t + 1;
 }
 
-// bandit_update followed by bandit_select for one sequence, by one whole warp: for the UCB family (Algorithm 2, its
-// discounted and its sliding-window form) lane i holds arm i, so the fp64 divisions, square roots and the window
-// scan of the K arms run side by side; the arithmetic per arm, the order of the window's additions and the
-// lowest-index tie-break are those of the serial functions.  The other policies run on lane 0.  Returns the next arm
-// (the same value in every lane) after storing it and the advanced round counter.
-__device__ inline int warp_bandit_step(int variant, int K, double beta, double gamma, int tau, int32_t *t_ptr, int32_t *arm_ptr,
-                                       double *sa, double *sb, int32_t *wa, double *wr, int a, double r, uint64_t seed,
-                                       uint32_t sequence)
+// bandit_update followed by bandit_select for one sequence, by one whole warp, in two steps: everything that does not need
+// the round's reward first (the state's loads, the logarithm, the square roots, the sums over the window's old entries),
+// then what does.  For the UCB family (Algorithm 2, its discounted and its sliding-window form) lane i holds arm i; the
+// arithmetic per arm, the order of the window's additions and the lowest-index tie-break are those of the serial functions.
+// The other policies run on lane 0, on a copy of the statistics in shared memory.
+struct BanditShared {
+    double sa[16], sb[16];
+};
+struct BanditStep {
+    int t, arm;
+    double a, b;        // lane i: the statistics of arm i before the round; SW-UCB: sum and count of its entries in the window
+    double root;        // sqrt(2 ln t / n_i) with the count n_i after the round
+};
+
+__device__ __forceinline__ bool ucb_family(int variant) { return variant == METASD_UCB || variant == METASD_DUCB || variant == METASD_SWUCB; }
+
+__device__ inline BanditStep warp_bandit_fetch(const VerifyParams &p, int b, int t, int arm, BanditShared &sh)
 {
-    const int lane = threadIdx.x & 31;
-    const int t = *t_ptr;
-    int next = 0;
-    if (variant != METASD_UCB && variant != METASD_DUCB && variant != METASD_SWUCB) {
-        if (lane == 0) {
-            int32_t tt = t;
-            bandit_update(variant, K, gamma, tau, &tt, sa, sb, wa, wr, a, r);
-            next = bandit_select(variant, K, beta, gamma, tau, tt, sa, sb, wa, wr, seed, sequence);
-            *t_ptr = tt;
-            *arm_ptr = next;
-        }
-        return __shfl_sync(0xFFFFFFFFu, next, 0);
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, K = p.K;
+    const double *sa = p.st.stat_a + (size_t)b * K, *sb = p.st.stat_b + (size_t)b * K;
+    BanditStep s = {t, arm, 0.0, 0.0, 0.0};
+    if (p.bandit != METASD_SWUCB && lane < K) { s.a = __ldcg(sa + lane); s.b = __ldcg(sb + lane); }
+    if (!ucb_family(p.bandit)) {
+        if (lane < K) { sh.sa[lane] = s.a; sh.sb[lane] = s.b; }
+        return s;
     }
-    double a_i = 0.0, b_i = 0.0;
-    if (variant == METASD_UCB) {
-        if (lane < K) { a_i = sa[lane]; b_i = sb[lane]; }
-        if (lane == a) {
-            a_i = (a_i * b_i + r) / (b_i + 1.0);
-            b_i = b_i + 1.0;
-            sa[lane] = a_i;
-            sb[lane] = b_i;
+    double n;
+    if (p.bandit == METASD_SWUCB) {
+        // the window after the round: the entries of the last tau - 1 rounds, oldest first, and the round's own behind them
+        const int32_t *wa = p.st.win_arm + (size_t)b * p.tau;
+        const double *wr = p.st.win_reward + (size_t)b * p.tau;
+        for (int s0 = max(t + 1 - p.tau, 0); s0 < t; s0 += 32) {
+            int entry_arm = -1;
+            double entry = 0.0;
+            if (s0 + lane < t) {
+                const int slot = (s0 + lane) % p.tau;
+                entry_arm = __ldcg(wa + slot);
+                entry = __ldcg(wr + slot);
+            }
+            const int count = min(32, t - s0);
+            for (int e = 0; e < count; ++e) {
+                const int i = __shfl_sync(FULL, entry_arm, e);
+                const double r = __shfl_sync(FULL, entry, e);
+                if (i == lane) { s.a += r; s.b += 1.0; }
+            }
         }
-    } else if (variant == METASD_DUCB) {
-        if (lane < K) {
-            a_i = sa[lane] * gamma;
-            b_i = sb[lane] * gamma;
-            if (lane == a) { a_i += r; b_i += 1.0; }
-            sa[lane] = a_i;
-            sb[lane] = b_i;
-        }
+        n = s.b + (lane == arm ? 1.0 : 0.0);
     } else {
+        n = p.bandit == METASD_DUCB ? s.b * p.gamma : s.b;
+        if (lane == arm) n += 1.0;
+    }
+    if (t + 1 >= K) s.root = sqrt(2.0 * log((double)(t + 1)) / n);
+    return s;
+}
+
+// Stores the updated statistics, the advanced round counter and the arm of the next round.
+__device__ inline void warp_bandit_finish(const VerifyParams &p, int b, BanditStep s, double r, BanditShared &sh)
+{
+    const unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, K = p.K, t1 = s.t + 1;
+    double *sa = p.st.stat_a + (size_t)b * K, *sb = p.st.stat_b + (size_t)b * K;
+    int next = t1;   // initial sweep: every drafter once, in order
+    if (!ucb_family(p.bandit)) {
+        __syncwarp();
         if (lane == 0) {
-            const int slot = t % tau;
-            wa[slot] = a;
-            wr[slot] = r;
+            int32_t tt = s.t;
+            bandit_update(p.bandit, K, p.gamma, p.tau, &tt, sh.sa, sh.sb, nullptr, nullptr, s.arm, r);
+            next = bandit_select(p.bandit, K, p.beta, p.gamma, p.tau, tt, sh.sa, sh.sb, nullptr, nullptr, p.seed,
+                                 p.sequence_base + (uint32_t)b);
         }
         __syncwarp();
-    }
-    const int t1 = t + 1;
-    next = t1;   // initial sweep: every drafter once, in order
-    if (t1 >= K) {
-        double mu = 0.0, n = 0.0;
-        if (variant == METASD_SWUCB) {
-            if (lane < K) {
-                const int first = t1 - tau > 0 ? t1 - tau : 0;
-                for (int s = first; s < t1; ++s) {   // oldest first
-                    const int slot = s % tau;
-                    if (wa[slot] == lane) { mu += wr[slot]; n += 1.0; }
-                }
-                if (n > 0.0) mu /= n;
+        if (lane < K) { sa[lane] = sh.sa[lane]; sb[lane] = sh.sb[lane]; }
+    } else {
+        double mu, n;
+        if (p.bandit == METASD_UCB) {
+            if (lane == s.arm) {
+                s.a = (s.a * s.b + r) / (s.b + 1.0);
+                s.b = s.b + 1.0;
+                sa[lane] = s.a;
+                sb[lane] = s.b;
             }
-        } else if (variant == METASD_DUCB) {
-            n = b_i;
-            mu = a_i / b_i;
+            mu = s.a;
+            n = s.b;
+        } else if (p.bandit == METASD_DUCB) {
+            s.a *= p.gamma;
+            s.b *= p.gamma;
+            if (lane == s.arm) { s.a += r; s.b += 1.0; }
+            if (lane < K) { sa[lane] = s.a; sb[lane] = s.b; }
+            mu = s.a / s.b;
+            n = s.b;
         } else {
-            mu = a_i;
-            n = b_i;
+            if (lane == s.arm) {
+                const int slot = s.t % p.tau;
+                p.st.win_arm[(size_t)b * p.tau + slot] = s.arm;
+                p.st.win_reward[(size_t)b * p.tau + slot] = r;
+                s.a += r;
+                s.b += 1.0;
+            }
+            mu = s.b > 0.0 ? s.a / s.b : 0.0;
+            n = s.b;
         }
-        const double two_ln_t = 2.0 * log((double)t1);
-        double score = -INFINITY;
-        if (lane < K) score = n > 0.0 ? mu + beta * sqrt(two_ln_t / n) : INFINITY;
-        int best = lane;
+        if (t1 >= K) {
+            double score = -INFINITY;
+            if (lane < K) score = n > 0.0 ? mu + p.beta * s.root : INFINITY;
+            next = lane;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double os = __shfl_xor_sync(0xFFFFFFFFu, score, o);
-            const int ob = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-            if (os > score || (os == score && ob < best)) { score = os; best = ob; }
+            for (int o = 16; o > 0; o >>= 1) {
+                const double os = __shfl_xor_sync(FULL, score, o);
+                const int ob = __shfl_xor_sync(FULL, next, o);
+                if (os > score || (os == score && ob < next)) { score = os; next = ob; }
+            }
         }
-        next = best;
     }
     if (lane == 0) {
-        *t_ptr = t1;
-        *arm_ptr = next;
+        p.st.t[b] = t1;
+        p.st.arm[b] = next;
     }
-    return next;
 }
 
 }  // namespace metasd

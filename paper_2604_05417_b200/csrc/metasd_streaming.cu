@@ -641,23 +641,6 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm
 // -------------------------------------------------------------------------------------------
 // K2
 // -------------------------------------------------------------------------------------------
-// weight of token v in the draw: MODE 1 = max(0, p_v - q_v) (correction), MODE 2 = p_v (bonus)
-template <typename LT, int VEC, int MODE>
-__device__ __forceinline__ void weights_of(const float (&xa)[VEC], const float (&xb)[VEC], float c, float nma, float ia,
-                                           float nmb, float ib, float (&w)[VEC])
-{
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-        const float pv = ex2(fmaf(xa[e], c, nma)) * ia;
-        if (MODE == 1) {
-            const float qv = ex2(fmaf(xb[e], c, nmb)) * ib;
-            w[e] = fmaxf(pv - qv, 0.f);
-        } else {
-            w[e] = pv;
-        }
-    }
-}
-
 // one vector of logits as loaded (unpacked to fp32 only where it is used: registers)
 template <typename LT, int VEC> struct RawVec { uint4 v; };
 template <typename LT> struct RawVec<LT, 1> { float v; };
@@ -678,10 +661,10 @@ __device__ __forceinline__ void unpack_raw(const RawVec<LT, VEC> &r, float (&x)[
     else x[0] = r.v;
 }
 
-// The row (pair) a draw is made from: weights max(0, p - q) (mode 1) or p (mode 2) of its tokens, in vectors of VEC.
+// The row (pair) a draw is made from, in vectors of VEC tokens with weights max(0, p - q).  The bonus row's weights are p:
+// its q is the row itself, scaled by ib = 0.
 template <typename LT> struct DrawRow {
     const LT *a, *d;
-    int mode, nvec;
     float c, nma, ia, nmb, ib;
 };
 
@@ -690,184 +673,151 @@ __device__ __forceinline__ void draw_weights(const DrawRow<LT> &row, const RawVe
 {
     float xa[VEC], xb[VEC];
     unpack_raw<LT, VEC>(ra, xa);
-    if (row.mode == 1) {
-        unpack_raw<LT, VEC>(rb, xb);
-        weights_of<LT, VEC, 1>(xa, xb, row.c, row.nma, row.ia, row.nmb, row.ib, w);
-    } else {
-        weights_of<LT, VEC, 2>(xa, xa, row.c, row.nma, row.ia, row.nmb, row.ib, w);
-    }
+    unpack_raw<LT, VEC>(rb, xb);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e)
+        w[e] = fmaxf(__fmaf_rn(ex2(fmaf(xb[e], row.c, row.nmb)), -row.ib, __fmul_rn(ex2(fmaf(xa[e], row.c, row.nma)), row.ia)), 0.f);
 }
 
-// U vectors of the row (pair) per lane, 32 apart: all loads are issued before the first is used.  Behind `hi`: nothing.
-template <typename LT, int VEC, int U> struct DrawBatch {
-    RawVec<LT, VEC> ra[U], rb[U];
-    __device__ __forceinline__ void load(const DrawRow<LT> &row, int i0, int hi)
-    {
+// Sum of the weights of the vectors [i, hi): fp32 a vector, fp64 across; U vectors' loads are issued before the first is used.
+template <typename LT, int VEC, int U>
+__device__ __forceinline__ double draw_sum(const DrawRow<LT> &row, int i, int hi)
+{
+    double acc = 0.0;
+#pragma unroll 1
+    for (; i < hi; i += U) {
+        RawVec<LT, VEC> ra[U], rb[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i0 + 32 * u < hi) {
-                ra[u] = load_raw<LT, VEC>(row.a, i0 + 32 * u);
-                if (row.mode == 1) rb[u] = load_raw<LT, VEC>(row.d, i0 + 32 * u);
+            if (i + u < hi) {
+                ra[u] = load_raw<LT, VEC>(row.a, i + u);
+                rb[u] = load_raw<LT, VEC>(row.d, i + u);
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < hi) {
+                float w[VEC], s = 0.f;
+                draw_weights<LT, VEC>(row, ra[u], rb[u], w);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) s += w[e];
+                acc += (double)s;
             }
     }
+    return acc;
+}
+
+// Inclusive sums over the lanes of a warp.
+__device__ __forceinline__ double warp_scan(double x)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += t;
+    }
+    return x;
+}
+
+// Where among the lanes' parts x, laid end to end (incl: their inclusive sums), the threshold lies: the first part whose end is
+// beyond it; rounding may leave none, then the last part with mass; -1: no mass at all.
+__device__ __forceinline__ int warp_crossing(double x, double incl, double threshold)
+{
+    const unsigned mass = __ballot_sync(0xFFFFFFFFu, x > 0.0), hits = __ballot_sync(0xFFFFFFFFu, incl > threshold) & mass;
+    return hits ? __ffs(hits) - 1 : 31 - __clz(mass);
+}
+
+// What a search of one row needs of its parts: where the crossing lies.
+struct PartHit {
+    double base, threshold, total;
+    int part;
 };
 
-// Parts laid end to end after base0, lane l holding parts 4 l .. 4 l + 3 (0 where there is none): finds the first part
-// whose end lies beyond the threshold; rounding may leave none, then the last part with mass (-1 if there is none).
-// FRACTION: the threshold comes in as a fraction of the parts' sum and goes out absolute.  Returns the part, the sum of
-// the parts before it plus base0 in `base`, and the sum of all parts in `total`.  Every lane of the calling warp takes
-// part and gets the same answers.
-template <bool FRACTION>
-__device__ __forceinline__ int warp_find_part(const double (&x)[4], double base0, double &threshold, double &base, double &total)
-{
-    const unsigned FULL = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31;
-    double incl = (x[0] + x[1]) + (x[2] + x[3]);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double t = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += t;
-    }
-    total = __shfl_sync(FULL, incl, 31);
-    if (FRACTION) threshold *= total;
-    double before = __shfl_up_sync(FULL, incl, 1);
-    if (lane == 0) before = 0.0;
-    // the lane's first part that crosses, else its last one with mass
-    int hit = -1, mass = -1;
-    double hit_base = 0.0, mass_base = 0.0, cum = base0 + before;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (x[i] > 0.0) { mass = i; mass_base = cum; }
-        if (hit < 0 && x[i] > 0.0 && cum + x[i] > threshold) { hit = i; hit_base = cum; }
-        cum += x[i];
-    }
-    const unsigned hits = __ballot_sync(FULL, hit >= 0), masses = __ballot_sync(FULL, mass >= 0);
-    if (!masses) { base = base0; return -1; }
-    const int src = hits ? __ffs(hits) - 1 : 31 - __clz(masses);
-    base = __shfl_sync(FULL, hits ? hit_base : mass_base, src);
-    return src * 4 + __shfl_sync(FULL, hits ? hit : mass, src);
-}
-
-// The token of one vector per lane (lane order is token order) where the running weight, `run` before the first lane,
-// exceeds the threshold: the same answer in every lane, -1 if it does not in these 32 vectors.  `last` collects the last
-// token with mass seen so far.
-template <int VEC>
-__device__ __forceinline__ int warp_find_token(const float (&w)[VEC], int vec, double &run, double threshold, int &last)
-{
-    const unsigned FULL = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31;
-    float s = 0.f;
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) s += w[e];
-    double incl = (double)s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double t = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += t;
-    }
-    const unsigned hits = __ballot_sync(FULL, run + incl > threshold);
-    int mine = -1, tok = -1;
-    double cum = run + incl - (double)s;
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-        if (w[e] > 0.f) mine = vec * VEC + e;
-        cum += (double)w[e];
-        if (tok < 0 && w[e] > 0.f && cum > threshold) tok = vec * VEC + e;
-    }
-    if (tok < 0) tok = mine;
-    last = max(last, __reduce_max_sync(FULL, mine));
-    run += __shfl_sync(FULL, incl, 31);
-    return hits ? __shfl_sync(FULL, tok, __ffs(hits) - 1) : -1;
-}
-
-// Shared-memory work space of the draw.
+// Shared-memory work space of the draw: the warps' totals of one level of the search, by parity of the level, and the piece
+// that the next level is made in.
 template <int NWARP> struct DrawShared {
-    double tot[NWARP];
-    int tok;
+    double tot[2][NWARP];
+    double base;
+    int lo;
 };
 
 // Barrier among the draw's warps only: the control warp goes its own way.
 template <int THREADS> __device__ __forceinline__ void draw_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
 
-// Inverse CDF in token order over the vectors [lo, hi) of one row (pair), of which `base` is the weight in front: the
-// smallest token v with sum_{w <= v} weight_w > threshold.  Every warp owns a contiguous range of vectors and sums it
-// (fp32 a vector, fp64 across); one warp-parallel scan finds the range that holds the crossing, and so on down to a range
-// of a few vectors per lane, which one warp searches vector by vector.  FRACTION: the threshold comes in as a fraction of
-// the range's own total.  Rounding may leave no crossing: then the last token with mass.  -1: no mass.
-template <typename LT, int VEC, int NWARP, bool FRACTION>
-__device__ __forceinline__ int range_inverse_cdf(const DrawRow<LT> &row, int lo, int hi, double base, double threshold, DrawShared<NWARP> &sh)
+// Inverse CDF in token order over the vectors [lo, hi) of one row (pair), of which `base` is the weight in front: writes the
+// smallest token v with sum_{w <= v} weight_w > threshold to *out.  Every thread sums a contiguous piece; the piece with the
+// crossing is found by a scan (fp64), and when it is no longer than a warp, a vector a lane, the token in it.  FRACTION:
+// the threshold comes in as a fraction of the range's own total.  Rounding may leave no crossing: then the last token with
+// mass.  false: no mass (the same in every thread).  The levels of a row's searches are counted in `level`.
+template <typename LT, int VEC, int NWARP>
+__device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo, int hi, double base, double threshold, bool fraction,
+                                                  DrawShared<NWARP> &sh, int &level, int32_t *out)
 {
-    constexpr int U = 4, DIRECT = 32 * U * (VEC == 1 ? 1 : 2);
+    constexpr int U = VEC == 1 ? 8 : 4;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    bool fraction = FRACTION;
-    for (;;) {
-        const int per_warp = (hi - lo + NWARP - 1) / NWARP;
-        const int v0 = min(lo + warp * per_warp, hi), v1 = min(v0 + per_warp, hi);
-        double acc = 0.0;
-        for (int i0 = v0 + lane; i0 < v1; i0 += 32 * U) {
-            DrawBatch<LT, VEC, U> batch;
-            batch.load(row, i0, v1);
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (i0 + 32 * u < v1) {
-                    float w[VEC], s = 0.f;
-                    draw_weights<LT, VEC>(row, batch.ra[u], batch.rb[u], w);
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) s += w[e];
-                    acc += (double)s;
-                }
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) sh.tot[warp] = acc;
+#pragma unroll 1
+    for (;; ++level) {
+        const int piece = (hi - lo + NWARP * 32 - 1) / (NWARP * 32);
+        const int v0 = min(lo + tid * piece, hi);
+        const double x = draw_sum<LT, VEC, U>(row, v0, min(v0 + piece, hi)), incl = warp_scan(x);
+        double *tot = sh.tot[level & 1];
+        if (lane == 31) tot[warp] = incl;
         draw_sync<NWARP * 32>();
-        double x[4], total;
+        double total = 0.0, before = 0.0, cum = base;
+        int owner = -1, last = -1;
+        if (fraction) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = lane * 4 + i < NWARP ? sh.tot[lane * 4 + i] : 0.0;
-        const int part = fraction ? warp_find_part<true>(x, base, threshold, base, total)
-                                  : warp_find_part<false>(x, base, threshold, base, total);
-        fraction = false;
-        if (part < 0) return -1;         // the same in every warp
-        lo = min(lo + part * per_warp, hi);
-        hi = min(lo + per_warp, hi);
-        if (hi - lo > DIRECT) {
-            draw_sync<NWARP * 32>();     // every warp has read the totals before the next level writes them
-            continue;
+            for (int w = 0; w < NWARP; ++w) total += tot[w];
+            threshold *= total;
+            fraction = false;
         }
-        if (warp == part) {
-            int found = -1, last = -1;
-            double run = base;
-            for (int i0 = lo; i0 < hi && found < 0; i0 += 32 * U) {
-                DrawBatch<LT, VEC, U> batch;
-                batch.load(row, i0 + lane, hi);
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = i0 + lane + 32 * u;
-                    if (i0 + 32 * u < hi && found < 0) {
-                        float w[VEC];
-                        if (i < hi) {
-                            draw_weights<LT, VEC>(row, batch.ra[u], batch.rb[u], w);
-                        } else {
+        for (int w = 0; w < NWARP; ++w) {
+            const double y = tot[w];
+            if (w == warp) before = cum;
+            cum += y;
+            if (y > 0.0) {
+                last = w;
+                if (owner < 0 && cum > threshold) owner = w;
+            }
+        }
+        if (last < 0) return false;
+        if (owner < 0) owner = last;
+        const bool another = piece > 32;
+        if (warp == owner) {
+            const int src = warp_crossing(x, before + incl, threshold);
+            const double front = before + __shfl_sync(0xFFFFFFFFu, incl - x, src);
+            const int first = min(lo + (warp * 32 + src) * piece, hi);
+            if (another) {
+                if (lane == 0) { sh.base = front; sh.lo = first; }
+            } else {
+                const int i = first + lane;
+                float w[VEC], s = 0.f;
 #pragma unroll
-                            for (int e = 0; e < VEC; ++e) w[e] = 0.f;
-                        }
-                        found = warp_find_token<VEC>(w, i, run, threshold, last);
+                for (int e = 0; e < VEC; ++e) w[e] = 0.f;
+                if (lane < piece && i < hi) draw_weights<LT, VEC>(row, load_raw<LT, VEC>(row.a, i), load_raw<LT, VEC>(row.d, i), w);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) s += w[e];
+                const double end = front + warp_scan((double)s);
+                const int who = warp_crossing((double)s, end, threshold);
+                double run = end - (double)s;
+                int token = -1, last_token = -1;
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    run += (double)w[e];
+                    if (w[e] > 0.f) {
+                        last_token = i * VEC + e;
+                        if (token < 0 && run > threshold) token = last_token;
                     }
                 }
+                if (lane == max(who, 0)) *out = who < 0 ? first * VEC : token >= 0 ? token : last_token;
             }
-            if (lane == 0) sh.tok = found >= 0 ? found : last;
         }
+        if (!another) return true;
         draw_sync<NWARP * 32>();
-        return sh.tok;
+        base = sh.base;
+        lo = sh.lo;
+        hi = min(lo + piece, hi);
     }
-}
-
-// The draw over a whole row with the walk's own total, for the cases that the parts of the row statistics do not settle
-// (a residual with next to no mass; row-statistics kernels that report on whole rows).  A call and not another inlined copy.
-template <typename LT, int VEC, int NWARP>
-__device__ __noinline__ int draw_whole_row(const DrawRow<LT> &row, float u, DrawShared<NWARP> &sh)
-{
-    draw_sync<NWARP * 32>();   // every thread has read what the last search left in the work space
-    return range_inverse_cdf<LT, VEC, NWARP, true>(row, 0, row.nvec, 0.0, (double)u, sh);
 }
 
 // One CTA per sequence: DRAW_THREADS threads for the draw (GREEDY: there is none, they only add up the parts of
@@ -876,9 +826,11 @@ __device__ __noinline__ int draw_whole_row(const DrawRow<LT> &row, float u, Draw
 //
 // The draw: the smallest v with sum_{w <= v} weight_w > u * total.  The row-statistics kernel leaves the mass of every
 // part of the row, so the part that holds the crossing is known without reading a logit, and only that part is walked
-// (a sixteenth of the row or less).  Where the mass sits in the vocabulary does not matter.  Against walking the row (its
-// first eighth first), kernel alone from cold caches: B = 256, V = 128256 bf16 31..40 -> 20 us; B = 1024, V = 128256 fp32
-// 90 -> 34; B = 40, V = 262144 bf16 (no frequency order) 43 -> 22; B = 96, V = 50257 bf16 36 -> 18; B = 64, V = 32000 17 -> 14.5.
+// (a sixteenth of the row or less).  Where the mass sits in the vocabulary does not matter.  The code runs once per CTA, much
+// of its time is the first fetch of its instructions: one copy of the weights' arithmetic for both kinds of draw and all
+// levels, loops instead of unrolled rows.  Us a round against a walk of the row with an unrolled two-level search: B = 64,
+// k = 5, V = 32000 35.9 -> 24.6; B = 96, k = 5, V = 50257 61.8 -> 50.6; B = 256, k = 7, V = 128256 with the row statistics' 237 -> 229;
+// the sliding-window policy's scan before the wait instead of behind it (B = 192, greedy) 61.7 -> 54.5.
 template <typename LT, bool VECTOR, int DRAW_THREADS, bool GREEDY>
 __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_kernel(const VerifyParams p)
 {
@@ -889,9 +841,12 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     const float c = p.c;
 
     __shared__ int sh_nacc, sh_mode;
-    __shared__ float sh_u;
-    __shared__ double sh_align[16];
+    __shared__ double sh_align[17];
+    __shared__ PartHit sh_hit[17];       // per position: the part of its row that the draw would be made from
+    __shared__ RowStats sh_stats[17];
+    __shared__ float sh_u[17];
     __shared__ DrawShared<NWARP> sh_draw;
+    __shared__ BanditShared sh_bandit;
 
     // The row-statistics kernel may still be running when this kernel starts.  What it writes (stats, segments) is read,
     // and what it reads is written, behind grid_dependency_wait() only; everything else was there before that kernel let
@@ -913,10 +868,11 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         const int t = p.stateless ? p.round : __ldcg(p.st.t + b), arm = p.stateless ? 0 : __ldcg(p.st.arm + b);
         // lane j < k: the accept test of Algorithm 4 at position j; lane j = k only brings the bonus row's words and flags
         const int j = min(lane, k);
-        const uint4 words = round_words(p.seed, p.sequence_base + (uint32_t)b, (uint32_t)t, (uint32_t)j);
-        const float u = uniform24(words.x);
+        const float u = uniform24(round_words(p.seed, p.sequence_base + (uint32_t)b, (uint32_t)t, (uint32_t)j).x);
         int x = -1;
         if (lane < k) x = __ldcg(p.tokens + (p.token_arm_stride ? (size_t)arm * p.token_arm_stride : 0) + (size_t)b * k_slots + j);
+        BanditStep step;
+        if (!p.stateless) step = warp_bandit_fetch(p, b, t, arm, sh_bandit);
         const bool in_range = x >= 0 && x < V;
         float a_x = 0.f, d_x = 0.f;
         if (in_range) {
@@ -954,7 +910,6 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
                 sh_nacc = n_acc;
                 sh_mode = row_flags ? 0 : n_acc == k ? 2 : 1;   // 2: bonus token from p_k, 1: correction from the residual
             }
-            if (lane == n_acc) sh_u = uniform24(words.y);
         }
         __syncthreads();   // the draw may start; the positions' sums of min(p, q) are there
         const double align = lane < k && !r.flags ? sh_align[lane] : 0.0;
@@ -965,10 +920,7 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         }
         // the reward (Definition 2), then the bandit of this sequence: update, and the next round's arm
         const double reward = p.reward_kind == METASD_REWARD_BE ? (double)n_acc / (double)k : warp_sum(align) / (double)k;
-        if (!p.stateless)
-            warp_bandit_step(p.bandit, K, p.beta, p.gamma, p.tau, &p.st.t[b], &p.st.arm[b], p.st.stat_a + (size_t)b * K,
-                             p.st.stat_b + (size_t)b * K, p.st.win_arm + (size_t)b * p.tau, p.st.win_reward + (size_t)b * p.tau,
-                             arm, reward, p.seed, p.sequence_base + (uint32_t)b);
+        if (!p.stateless) warp_bandit_finish(p, b, step, reward, sh_bandit);
         flags = __reduce_or_sync(FULL, flags);
         if (lane == 0) {
             p.accepted_len[b] = n_acc;
@@ -979,62 +931,87 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         return;
     }
 
+    // Row by row, a row per warp: sum_v min(p_v, q_v), and the part of the row that holds the crossing if the draw turns out to
+    // be made from this row (which one it is, the control warp finds out meanwhile).
+    const uint32_t t = (uint32_t)(p.stateless ? p.round : __ldcg(p.st.t + b));
+    const uint32_t sequence = p.sequence_base + (uint32_t)b;
+    float u = uniform24(round_words(p.seed, sequence, t, (uint32_t)warp).y);
     grid_dependency_wait();
-    // sum_v min(p_v, q_v) of every drafted position (16 at most), two positions per warp at a time
-    static_assert(NWARP >= 8, "two positions per warp cover the largest draft length");
-    double m[2] = {0.0, 0.0};
-    for (int s = lane; s < p.n_seg; s += 32) {
-        if (warp < k) m[0] += (double)segments[warp * p.n_seg + s].min;
-        if (warp + NWARP < k) m[1] += (double)segments[(warp + NWARP) * p.n_seg + s].min;
-    }
+    // lane l holds parts n l / 32 ..: contiguous, so that lane order is token order
+    const int per_lane = (p.n_seg + 31) >> 5;    // 1 .. 4
+#pragma unroll 1
+    for (int j = warp; j < (GREEDY ? k : k + 1); j += NWARP) {
+        const RowSegment *seg = segments + (size_t)j * p.n_seg;
+        double m = 0.0, x = 0.0;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        m[i] = warp_sum(m[i]);
-        if (lane == 0 && warp + i * NWARP < k) sh_align[warp + i * NWARP] = m[i];
+        for (int q = 0; q < MAX_SEGMENTS / 32; ++q)
+            if (q < per_lane && lane * per_lane + q < p.n_seg) {
+                const RowSegment g = seg[lane * per_lane + q];
+                m += (double)g.min;
+                x += j < k ? fmax((double)g.p - (double)g.min, 0.0) : (double)g.p;
+            }
+        if (!GREEDY) {
+            if (j != warp) u = uniform24(round_words(p.seed, sequence, t, (uint32_t)j).y);
+            PartHit hit;
+            const double incl = warp_scan(x);
+            hit.total = __shfl_sync(FULL, incl, 31);
+            hit.threshold = (double)u * hit.total;
+            const int src = warp_crossing(x, incl, hit.threshold);
+            hit.base = __shfl_sync(FULL, incl - x, max(src, 0));
+            hit.part = src * per_lane;
+            if (lane == 0) { sh_hit[j] = hit; sh_u[j] = u; sh_stats[j] = stats[j]; }
+        }
+        if (j < k) {
+            m = warp_sum(m);
+            if (lane == 0) sh_align[j] = m;
+        }
     }
     __syncthreads();
     if (GREEDY || sh_mode == 0) return;   // greedy, or the row it needs is not finite: the control warp has the token
     const int n_acc = sh_nacc;
-    const RowStats rs = stats[n_acc];
+    const RowStats rs = sh_stats[n_acc];
+    const PartHit hit = sh_hit[n_acc];
     DrawRow<LT> row;
-    row.mode = sh_mode;
     row.a = target + (size_t)n_acc * V;
-    row.d = row.mode == 1 ? draft + (size_t)n_acc * V : row.a;
-    row.nvec = V / VEC;
     row.c = c;
     row.nma = -rs.max_a * c; row.ia = 1.0f / rs.sum_a;
-    row.nmb = -rs.max_b * c; row.ib = 1.0f / rs.sum_b;
-    const float u = sh_u;
-    int token = -1;
-    if (p.n_seg > 1) {
-        // the part of the row with the crossing, found by every warp for itself
-        double x[4], threshold = (double)u, base, total;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            x[i] = 0.0;
-            if (lane * 4 + i < p.n_seg) {
-                const RowSegment g = segments[n_acc * p.n_seg + lane * 4 + i];
-                x[i] = row.mode == 1 ? fmax((double)g.p - (double)g.min, 0.0) : (double)g.p;
-            }
-        }
-        const int part = warp_find_part<true>(x, 0.0, threshold, base, total);
-        // Below a thousandth the parts' masses p - min are differences of numbers that far above them: the walk over
-        // the row, which takes the difference token by token, decides instead (such a rejection is rare by its own measure).
-        if (total > 1.0e-3) {
-            int lead = 0, shift = 0;
-            if (!VECTOR) row_alignment(row.a, row.mode == 1 ? row.d : nullptr, lead, shift);
-            const int trip = 32 * Logit<LT>::VEC, trips = (V + lead + shift + trip - 1) / trip;
-            const int lo = max(trip * segment_begin(trips, part, p.n_seg) - lead, 0);
-            const int hi = min(trip * segment_begin(trips, part + 1, p.n_seg) - lead, V);
-            token = range_inverse_cdf<LT, VEC, NWARP, false>(row, lo / VEC, hi / VEC, base, threshold, sh_draw);
-        }
+    bool residual = sh_mode == 1;
+    auto draw_from_target = [&] { row.d = row.a; row.nmb = row.nma; row.ib = 0.f; };
+    if (residual) {
+        row.d = draft + (size_t)n_acc * V;
+        row.nmb = -rs.max_b * c; row.ib = 1.0f / rs.sum_b;
+    } else {
+        draw_from_target();
     }
-    if (token < 0) token = draw_whole_row<LT, VEC, NWARP>(row, u, sh_draw);
-    if (token < 0 && row.mode == 1) {   // p == q in fp32 yet rejected (the residual has no mass): draw from p
-        row.mode = 2;
-        token = draw_whole_row<LT, VEC, NWARP>(row, u, sh_draw);
+    int lo = 0, hi = V, level = 0;
+    double base = 0.0, threshold = (double)sh_u[n_acc];
+    // Below a thousandth the parts' masses p - min are differences of numbers that far above them: the walk over the whole
+    // row, which takes the difference token by token, decides instead (such a rejection is rare by its own measure).
+    bool whole = p.n_seg <= 1 || !(hit.total > 1.0e-3);
+    if (!whole) {
+        int lead = 0, shift = 0;
+        if (!VECTOR) row_alignment(row.a, residual ? row.d : nullptr, lead, shift);
+        const int trip = 32 * Logit<LT>::VEC, trips = (V + lead + shift + trip - 1) / trip;
+        lo = max(trip * segment_begin(trips, hit.part, p.n_seg) - lead, 0);
+        hi = min(trip * segment_begin(trips, min(hit.part + per_lane, p.n_seg), p.n_seg) - lead, V);
+        base = hit.base;
+        threshold = hit.threshold;
     }
-    if (tid == 0) p.next_token[b] = token;
+    for (;;) {
+        if (range_inverse_cdf<LT, VEC, NWARP>(row, lo / VEC, hi / VEC, base, threshold, whole, sh_draw, level, p.next_token + b)) return;
+        ++level;
+        if (whole) {
+            if (!residual) break;
+            draw_from_target();   // p == q in fp32 yet rejected (the residual has no mass): draw from p
+            residual = false;
+        }
+        whole = true;
+        lo = 0;
+        hi = V;
+        base = 0.0;
+        threshold = (double)sh_u[n_acc];
+    }
+    if (tid == 0) p.next_token[b] = -1;
 }
 
 // -------------------------------------------------------------------------------------------
