@@ -372,6 +372,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         };
         auto request_checked = [&](int m, uint32_t dst) {
             if (SHIFTED) {
+                if (m < n_full && m + g0 > 0) {   // whole vectors: most of a short range is asked for here
+                    request(dst, a4 + 32 * m, d4 + 32 * m, drop);
+                    return;
+                }
                 if (m < n_trip) copy_ragged(m, dst, BOTH);
                 cp_async_commit();
             } else if (m < lane_trips) {
