@@ -13,6 +13,7 @@
 //                          accept step), first rejection, inverse-CDF draw of the correction token from
 //                          max(0, p - q) or of the bonus token from p (its resampling step), the reward, the
 //                          bandit update and the next round's arm (Algorithm 2, update and selection steps).
+#include <algorithm>
 #include <type_traits>
 
 #include "metasd_device.cuh"
@@ -628,18 +629,25 @@ static cudaError_t launch_kernel(void (*kernel)(Params...), unsigned grid, unsig
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Dynamic shared memory that one CTA alone on its SM asks for: leaves room for an epilogue CTA beside it.
+constexpr unsigned STAGED_SMEM_MAX = 216 * 1024;
+
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm, cudaStream_t stream)
 {
-    // A launch of about one wave wants its blocks spread evenly over idle SMs: set up while the last epilogue still holds some
-    // of them, they crowd on the others and stay there (us a round, chained / not: B = 64, k = 5, V = 32000 34.9 / 26.7; B = 4,
-    // k = 8, V = 152064 in clusters, 144 CTAs, 23.5 / 20.5; several waves gain: B = 96, k = 5, V = 50257 56.7 / 62.0, B = 192,
-    // k = 8 ragged, V = 50264 61.9 / 69.8).
-    const unsigned ctas = units * CL;
-    const bool chained = ctas <= (unsigned)n_sm / 2 || ctas > (unsigned)n_sm * MINB;
-    // the attribute that allows the shared memory was set by streaming_prepare
-    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, ctas, THREADS,
-                         STAGED_SMEM<D, THREADS, SHIFTED>, CL, chained, stream, p);
+    // A launch of up to one wave wants its blocks spread evenly over the SMs: set up while the last epilogue still holds some of
+    // them, they would crowd on the others and stay there.  So such a launch is chained only where the last layer of blocks
+    // is nearly full (or, of clusters, which are placed within groups of SMs, where every one finds free SMs), and asks for
+    // so much shared memory that an SM takes no more blocks than an even spread puts there.  Us a round, chained so / not:
+    // 384 blocks (B = 64, k = 5, V = 32000) 22.8 / 24.6, 240 18.5 / 20.5, 144 (V = 128256) 28.1 / 28.7, 96 14.0 / 16.1;
+    // 320 blocks 22.2 / 20.5, 480 26.5 / 24.6; 32 clusters of 4 13.5 / 14.4, 36 21.8 / 19.8.  Several waves are always chained
+    // (B = 192, k = 8 ragged, V = 50264 61.9 / 69.8).
+    const unsigned ctas = units * CL, sms = (unsigned)n_sm, layers = (ctas + sms - 1) / sms, spare = layers * sms - ctas;
+    const bool one_wave = layers <= MINB;
+    const bool chained = !one_wave || ctas <= sms / 2 || (CL == 1 ? spare <= sms / 2 : layers == 1 && spare >= sms / 8);
+    constexpr unsigned needed = STAGED_SMEM<D, THREADS, SHIFTED>;   // the attribute that allows it, and more, was set by streaming_prepare
+    const unsigned smem = one_wave && chained ? std::max(needed, STAGED_SMEM_MAX / layers - 4096u) : needed;
+    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, ctas, THREADS, smem, CL, chained, stream, p);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -1036,10 +1044,10 @@ template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
 static cudaError_t prepare_staged()
 {
     cudaError_t e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM<D, THREADS, false>);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM<D, THREADS, true>);
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
     return e;
 }
 
