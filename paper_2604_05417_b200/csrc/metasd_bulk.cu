@@ -308,11 +308,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) row_stats_bulk_kernel(co
         const uint32_t flags = (bad_a || bad_b) ? METASD_STATUS_NONFINITE : 0u;
         auto write_stats = [&](double total_min) {
             RowStats r;
-            r.max_a = max_a; r.sum_a = sum_a; r.max_b = max_b; r.sum_b = sum_b;
+            r.ref_a = -max_a * c; r.sum_a = sum_a; r.ref_b = -max_b * c; r.sum_b = sum_b;
             r.argmax_a = rm.i;
             r.flags = flags;
             p.stats[(size_t)b * (p.k + 1) + j] = r;
-            p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{1.f, (float)total_min};
+            p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{(float)(pair ? 1.0 - total_min : 1.0)};
         };
         if (!pair) {
             if (tid == 0) write_stats(0.0);

@@ -88,20 +88,20 @@ __device__ __forceinline__ float sum2(uint64_t v)
     unpack2(v, lo, hi);
     return lo + hi;
 }
-// acc + 2^y, half by half
-__device__ __forceinline__ uint64_t add_ex2(uint64_t acc, uint64_t y)
+// 2^y, half by half
+__device__ __forceinline__ uint64_t ex2_2(uint64_t y)
 {
     float lo, hi;
     unpack2(y, lo, hi);
-    return add2(acc, pack2(ex2(lo), ex2(hi)));
+    return pack2(ex2(lo), ex2(hi));
 }
-// acc + 2^min(ya, yb), half by half
-__device__ __forceinline__ uint64_t add_ex2_min(uint64_t acc, uint64_t ya, uint64_t yb)
+// 2^min(ya, yb), half by half
+__device__ __forceinline__ uint64_t ex2_min2(uint64_t ya, uint64_t yb)
 {
     float alo, ahi, blo, bhi;
     unpack2(ya, alo, ahi);
     unpack2(yb, blo, bhi);
-    return add2(acc, pack2(ex2(fminf(alo, blo)), ex2(fminf(ahi, bhi))));
+    return pack2(ex2(fminf(alo, blo)), ex2(fminf(ahi, bhi)));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -190,20 +190,23 @@ template <> struct Logit<__nv_bfloat16> {
         const uint32_t m = max_word(raw);
         return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
     }
-    // acc + sum 2^(x c + nm) over a vector; acc + sum 2^min(a c + na, b c + nb) over a pair of vectors
+    // The vector is summed before it joins the accumulator, which a large term is in for long: a rounding at its size per vector.
+    // acc + sum 2^(x c + nm) over a vector; acc + sum 2^min(a c + na, (b c + nb) + lg) over a pair of vectors
     __device__ static __forceinline__ uint64_t add_exp(uint64_t acc, const uint4 &r, uint64_t c, uint64_t nm)
     {
         const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+        uint64_t s = ex2_2(fma2(pair_of(w[0]), c, nm));
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc = add_ex2(acc, fma2(pair_of(w[i]), c, nm));
-        return acc;
+        for (int i = 1; i < 4; ++i) s = add2(s, ex2_2(fma2(pair_of(w[i]), c, nm)));
+        return add2(acc, s);
     }
-    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb)
+    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb, uint64_t lg)
     {
         const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
+        uint64_t s = ex2_min2(fma2(pair_of(wa[0]), c, na), add2(fma2(pair_of(wb[0]), c, nb), lg));
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc = add_ex2_min(acc, fma2(pair_of(wa[i]), c, na), fma2(pair_of(wb[i]), c, nb));
-        return acc;
+        for (int i = 1; i < 4; ++i) s = add2(s, ex2_min2(fma2(pair_of(wa[i]), c, na), add2(fma2(pair_of(wb[i]), c, nb), lg)));
+        return add2(acc, s);
     }
 };
 
@@ -248,15 +251,15 @@ template <> struct Logit<float> {
     __device__ static __forceinline__ bool any_above(const uint4 &raw, Best best) { return max_of(raw) > best; }
     __device__ static __forceinline__ uint64_t add_exp(uint64_t acc, const uint4 &r, uint64_t c, uint64_t nm)
     {
-        acc = add_ex2(acc, fma2(pack2(__uint_as_float(r.x), __uint_as_float(r.y)), c, nm));
-        return add_ex2(acc, fma2(pack2(__uint_as_float(r.z), __uint_as_float(r.w)), c, nm));
+        const uint64_t s = ex2_2(fma2(pack2(__uint_as_float(r.x), __uint_as_float(r.y)), c, nm));
+        return add2(acc, add2(s, ex2_2(fma2(pack2(__uint_as_float(r.z), __uint_as_float(r.w)), c, nm))));
     }
-    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb)
+    __device__ static __forceinline__ uint64_t add_exp_min(uint64_t acc, const uint4 &a, const uint4 &b, uint64_t c, uint64_t na, uint64_t nb, uint64_t lg)
     {
-        acc = add_ex2_min(acc, fma2(pack2(__uint_as_float(a.x), __uint_as_float(a.y)), c, na),
-                          fma2(pack2(__uint_as_float(b.x), __uint_as_float(b.y)), c, nb));
-        return add_ex2_min(acc, fma2(pack2(__uint_as_float(a.z), __uint_as_float(a.w)), c, na),
-                           fma2(pack2(__uint_as_float(b.z), __uint_as_float(b.w)), c, nb));
+        const uint64_t s = ex2_min2(fma2(pack2(__uint_as_float(a.x), __uint_as_float(a.y)), c, na),
+                                    add2(fma2(pack2(__uint_as_float(b.x), __uint_as_float(b.y)), c, nb), lg));
+        return add2(acc, add2(s, ex2_min2(fma2(pack2(__uint_as_float(a.z), __uint_as_float(a.w)), c, na),
+                                          add2(fma2(pack2(__uint_as_float(b.z), __uint_as_float(b.w)), c, nb), lg))));
     }
 };
 
@@ -378,10 +381,17 @@ struct ArgMax {
     int32_t i;
 };
 
-// What a warp of the staged row-statistics kernel found in its part of a row pair: the reference m of both sums, the
-// sums, the largest target logit and its first index.
+// 2^d for a whole number d (any float); 0 below the normal range, infinity above it, 0 for NaN.
+__device__ __forceinline__ float exp2i(float d)
+{
+    const int e = (int)fminf(fmaxf(d, -150.f), 128.f);
+    return e < -126 ? 0.f : __int_as_float((e + 127) << 23);
+}
+
+// What a warp of the staged row-statistics kernel found in its part of a row pair: the reference of both sums, the sums,
+// the largest target logit and its first index.
 struct WarpRecord {
-    float m, sum_a, sum_b, best;
+    float ref, sum_a, sum_b, best;
     int32_t best_i;
 };
 

@@ -9,20 +9,20 @@ namespace metasd {
 
 // Per-(sequence, position) result of the row-statistics pass; the scratch the streaming path keeps
 // between its two kernels.  Softmax terms are held relative to the raw row maximum:
-//   p_v = 2^((x_v - max_a) * c) / sum_a,  c = log2(e) / T.
+//   p_v = 2^(x_v * c + ref_a) / sum_a,  c = log2(e) / T.
 struct RowStats {
-    float max_a, sum_a;   // target row
-    float max_b, sum_b;   // draft row (unused at the bonus position); max_b is the reference sum_b is relative to:
-                          // the row's maximum, or the target row's where the staged kernels could share it
+    float ref_a, sum_a;   // target row; ref_a is about -(its largest logit) c
+    float ref_b, sum_b;   // draft row (unused at the bonus position); the staged kernel shares the target row's reference
+                          // where it can
     int32_t argmax_a;     // first index of the target row's maximum
     uint32_t flags;       // METASD_STATUS_* of this row pair
 };
 
-// What the row-statistics pass says about a contiguous part of a row: its share of the target's probability, and (row
-// pairs) of sum_v min(p_v, q_v) = 1 - d_TV(p, q).  A row has n_seg parts of nearly equal length (segment_begin); the
-// residual max(0, p - q) of a part has mass p - min.
+// What the row-statistics pass says about a contiguous part of a row: of a row pair the mass sum_v max(0, p_v - q_v) =
+// sum_v p_v - min(p_v, q_v), which adds up to d_TV(p, q) over the row; of a bonus row its share of p.  A row has n_seg parts of
+// nearly equal length (segment_begin).
 struct RowSegment {
-    float p, min;
+    float weight;
 };
 // First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
 __host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 
     if (tid == 0) {
         RowStats r;
-        r.max_a = max_a; r.sum_a = sum_a; r.max_b = max_b; r.sum_b = sum_b;
+        r.ref_a = -max_a * c; r.sum_a = sum_a; r.ref_b = -max_b * c; r.sum_b = sum_b;
         r.argmax_a = sh_am[0].i;
         uint32_t flags = 0;
         // NaN or +Inf anywhere makes the sum NaN; an all -Inf row leaves it 0
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
         if (bad_a || bad_b) flags |= METASD_STATUS_NONFINITE;
         r.flags = flags;
         p.stats[(size_t)b * (p.k + 1) + j] = r;
-        p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{1.f, (float)total_min};
+        p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{(float)(pair ? 1.0 - total_min : 1.0)};
     }
 }
 
@@ -197,12 +197,14 @@ template <typename LT> __device__ __forceinline__ void fill_neg_inf(uint32_t slo
     asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(slot), "r"(w) : "memory");
 }
 
-// One warp's running statistics of a row pair.  All lanes share the reference `m` that both rows' sums are relative to and
-// the best target logit `best` (its first index in `best_i`); the sums are the lane's own, two partial sums each.
+// One warp's running statistics of a row pair.  All lanes share the reference `ref` that both rows' sums are relative to and
+// the best target logit `best` (its first index in `best_i`); the sums are the lane's own, two partial sums each.  The
+// reference is a whole number, the best logit's exponent with its sign changed and rounded: a change of reference is then
+// an exact scaling by a power of two, and sums of different warps are merged without an error of their own.
 template <typename LT> struct WarpSums {
-    uint64_t a, b;        // packed fp32 pairs: sum 2^((x - m) c) of the target and the draft row
-    float m, best;
-    uint64_t nm;          // -m c, twice
+    uint64_t a, b;        // packed fp32 pairs: sum 2^(x c + ref) of the target and the draft row
+    float ref, best;
+    uint64_t nm;          // ref, twice
     typename Logit<LT>::Best cmp;   // `best` as the vectors are compared with it
     int32_t best_i;
 };
@@ -220,12 +222,13 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
     for (int e = 1; e < VEC; ++e) cm = fmaxf(cm, x[e]);
     const float top = warp_max_f(cm);
     const bool first_finite = w.best == -INFINITY;   // the reference may still be a stand-in, on either side of `top`
-    if (top > w.m || first_finite) {
-        const uint64_t shrink = pack2(ex2((w.m - top) * c));
+    const float ref = -rintf(top * c);
+    if (ref < w.ref || first_finite) {
+        const uint64_t shrink = pack2(exp2i(ref - w.ref));
         if (!first_finite) w.a = mul2(w.a, shrink);
         w.b = mul2(w.b, shrink);
-        w.m = top;
-        w.nm = pack2(-top * c);
+        w.ref = ref;
+        w.nm = pack2(ref);
     }
     int first = 0;
 #pragma unroll
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     const uint64_t drop = l2_policy_evict_first(), keep = pair ? l2_policy_evict_last() : drop;
     WarpSums<LT> w;
     w.a = w.b = 0ull;
-    w.m = 0.f;
+    w.ref = 0.f;
     w.nm = 0ull;
     w.best = -INFINITY;
     w.cmp = Logit<LT>::best_of(-INFINITY);
@@ -403,12 +406,13 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         if (n_trip > 0) {
             cp_async_wait<D - 2>();
             if (SHIFTED) mask_ragged(0, slot0, BOTH);
-            w.m = warp_max_f(Logit<LT>::max_of(lds16(slot0)));
-            if (!(w.m > METASD_NEG_BIG)) {
-                w.m = BOTH ? warp_max_f(Logit<LT>::max_of(lds16(slot0 + ROW_STRIDE))) : 0.f;
-                if (!(w.m > METASD_NEG_BIG)) w.m = 0.f;
+            float top = warp_max_f(Logit<LT>::max_of(lds16(slot0)));
+            if (!(top > METASD_NEG_BIG)) {
+                top = BOTH ? warp_max_f(Logit<LT>::max_of(lds16(slot0 + ROW_STRIDE))) : 0.f;
+                if (!(top > METASD_NEG_BIG)) top = 0.f;
             }
-            w.nm = pack2(-w.m * c);
+            w.ref = -rintf(top * c);
+            w.nm = pack2(w.ref);
         }
         // Trip n asks for the trip D - 1 ahead, then works on its own vectors (slot n mod D).  Groups of D trips whose
         // requests all lie inside the row carry no checks, and their slots and their L2 policy are constants (the boundary
@@ -448,43 +452,48 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         cluster_wait();   // every CTA of the cluster is running
         if (lane < CL) {
             const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane);
-            st_cluster(dst, __float_as_int(w.m));           st_cluster(dst + 4, __float_as_int(sum_aw));
+            st_cluster(dst, __float_as_int(w.ref));          st_cluster(dst + 4, __float_as_int(sum_aw));
             st_cluster(dst + 8, __float_as_int(sum_bw));    st_cluster(dst + 12, __float_as_int(w.best));
             st_cluster(dst + 16, w.best_i - lead);
         }
         cluster_sync_all();
     } else {
-        if (lane == 0) sh_rec[warp] = WarpRecord{w.m, sum_aw, sum_bw, w.best, w.best_i - lead};
+        if (lane == 0) sh_rec[warp] = WarpRecord{w.ref, sum_aw, sum_bw, w.best, w.best_i - lead};
         __syncthreads();
     }
-    MaxSum ra = {METASD_NEG_BIG, 0.f}, rb = {METASD_NEG_BIG, 0.f};
+    float ref_a = INFINITY, sum_a = 0.f, sum_b = 0.f;   // both sums end up relative to the target row's largest logit
     ArgMax rm = {-INFINITY, 0x7FFFFFFF};
 #pragma unroll
-    for (int r0 = 0; r0 < NREC; r0 += 32) {
+    for (int r0 = 0; r0 < NREC; r0 += 32)
         if (NREC - r0 >= 32 || lane < NREC - r0) {
             const WarpRecord r = sh_rec[r0 + lane];
-            // a part whose target logits are all masked has a stand-in for its reference and nothing in sum_a
-            const MaxSum pa = {r.best > -INFINITY ? r.m : METASD_NEG_BIG, r.sum_a};
-            const MaxSum pb = {r.sum_b == 0.f ? METASD_NEG_BIG : r.m, r.sum_b};
-            ra = r0 ? merge(ra, pa, c) : pa;
-            rb = r0 ? merge(rb, pb, c) : pb;
+            if (r.best > METASD_NEG_BIG) ref_a = fminf(ref_a, r.ref);   // a part without a finite target logit has a stand-in
             rm = better(rm, ArgMax{r.best, r.best_i});
         }
-    }
+    ref_a = -warp_max_f(-ref_a);
+    if (!(ref_a < INFINITY)) ref_a = 0.f;
+#pragma unroll
+    for (int r0 = 0; r0 < NREC; r0 += 32)
+        if (NREC - r0 >= 32 || lane < NREC - r0) {
+            const WarpRecord r = sh_rec[r0 + lane];
+            const float d = ref_a - r.ref;   // above zero for stand-ins alone, whose sum_a is zero
+            sum_a = fmaf(r.sum_a, exp2i(fminf(d, 0.f)), sum_a);
+            sum_b = fmaf(r.sum_b, exp2i(d), sum_b);
+        }
+    sum_a = warp_sum_f(sum_a);
+    sum_b = warp_sum_f(sum_b);
     {
-        const float top = warp_max_f(ra.m);     // both sums end up relative to the target row's maximum
-        ra.s = warp_sum_f(ra.s * ex2((ra.m - top) * c));
-        rb.s = warp_sum_f(rb.s * ex2((rb.m - top) * c));
-        ra.m = rb.m = top;
         const float best = warp_max_f(rm.v);
         rm.i = __reduce_min_sync(FULL, rm.v == best ? rm.i : 0x7FFFFFFF);
         rm.v = best;
     }
+    float ref_b = ref_a;
+    bool bad_b = false;
     // The shared reference suits the draft row when its sum is neither flushed nor overflowed: 2^-60 .. finite
     // leaves every term that matters in fp32 range.  Otherwise (draft logits far from the target's, or a row
     // that is not finite) the draft row is swept again relative to its own running maximum.
-    if (pair && !(rb.s >= 0x1p-60f && rb.s < INFINITY)) {
-        MaxSum own = {METASD_NEG_BIG, 0.f};
+    if (pair && !(sum_b >= 0x1p-60f && sum_b < INFINITY)) {
+        MaxSum own = {METASD_NEG_BIG, 0.f};   // m: the running maximum's exponent, a whole number here too
         for (int n = 0; n < lane_trips; ++n) {
             float xb[VEC];
             const int tok0 = (v0 + 32 * n) * VEC - lead - shift;
@@ -497,15 +506,19 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             float bm = xb[0];
 #pragma unroll
             for (int e = 1; e < VEC; ++e) bm = fmaxf(bm, xb[e]);
-            if (bm > own.m) {
-                own.s *= ex2((own.m - bm) * c);
-                own.m = bm;
+            const float top = rintf(bm * c);
+            if (top > own.m) {
+                own.s *= exp2i(own.m - top);
+                own.m = top;
             }
-            const float nmb = -own.m * c;
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) own.s += ex2(fmaf(xb[e], c, nmb));
+            for (int e = 0; e < VEC; ++e) own.s += ex2(fmaf(xb[e], c, -own.m));
         }
-        own = warp_merge(own, c);
+        auto merge_warp = [](MaxSum v) {
+            const float top = warp_max_f(v.m);
+            return MaxSum{top, warp_sum_f(v.s * exp2i(v.m - top))};
+        };
+        own = merge_warp(own);
         if (CL > 1) {
             if (lane < CL) {
                 const uint32_t dst = map_to_rank(smem_addr(&sh_redo[part]), (uint32_t)lane);
@@ -517,28 +530,36 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             if (lane == 0) sh_redo[warp] = own;
             __syncthreads();
         }
-        rb = MaxSum{METASD_NEG_BIG, 0.f};
-        for (int r = lane; r < NREC; r += 32) rb = merge(rb, sh_redo[r], c);
-        rb = warp_merge(rb, c);
+        MaxSum rb = {METASD_NEG_BIG, 0.f};
+        for (int r = lane; r < NREC; r += 32) {
+            const MaxSum q = sh_redo[r];
+            const float top = fmaxf(rb.m, q.m);
+            rb = MaxSum{top, rb.s * exp2i(rb.m - top) + q.s * exp2i(q.m - top)};
+        }
+        rb = merge_warp(rb);
+        ref_b = -rb.m;
+        sum_b = rb.s;
+        bad_b = !(sum_b > 0.f) || !(sum_b < INFINITY);
     }
 
     const size_t row = (size_t)b * (p.k + 1) + j;
     if (tid == 0 && rank == 0) {
         RowStats r;
-        r.max_a = ra.m; r.sum_a = ra.s; r.max_b = rb.m; r.sum_b = rb.s;
+        r.ref_a = ref_a; r.sum_a = sum_a; r.ref_b = ref_b; r.sum_b = sum_b;
         r.argmax_a = rm.i;
-        const bool bad_a = !(ra.s > 0.f) || !(ra.s < INFINITY) || !(rm.v < INFINITY);
-        const bool bad_b = pair && (!(rb.s > 0.f) || !(rb.s < INFINITY) || !(rb.m < INFINITY));
+        const bool bad_a = !(sum_a > 0.f) || !(sum_a < INFINITY) || !(rm.v < INFINITY);
         r.flags = bad_a || bad_b ? METASD_STATUS_NONFINITE : 0u;
         p.stats[row] = r;
     }
 
     // ---- sweep 2, this warp's trips in reverse: sum_v 2^min(ya_v, yb_v), one exponential per pair
-    float part_min = 0.f;
+    // With rho = sum_a / sum_b: min(p, q) = 2^min(a c + ref_a, b c + ref_b + log2 rho) / sum_a.  The logarithm's whole part joins
+    // the reference, which stays exact; its fraction is added to the exponents on its own (folded into a reference of 20 it
+    // would be rounded at that size, and every term of the draft row scaled by the error, up to 7e-7).
+    float weight = sum2(w.a) * exp2i(fminf(ref_a - w.ref, 0.f));
     if (pair) {
-        float offs[3];
-        second_sweep_offsets(ra, rb, c, offs);
-        const uint64_t nma = pack2(offs[0]), nmb = pack2(offs[1]);
+        const float rho = sum_a / sum_b, whole = rintf(log2f(rho));
+        const uint64_t nma = pack2(ref_a), nmb = pack2(ref_b + whole), lg = pack2(log2f(rho * exp2i(-whole)));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last; SHIFTED: and its first).
@@ -552,7 +573,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             }
             uint4 d = lds16(src + ROW_STRIDE);
             if (SHIFTED) d = Logit<LT>::shifted(d, lds16(src + ROW_STRIDE + 16u), shift);
-            acc = Logit<LT>::add_exp_min(acc, lds16(src), d, c2, nma, nmb);
+            acc = Logit<LT>::add_exp_min(acc, lds16(src), d, c2, nma, nmb, lg);
             if (SHIFTED) __syncwarp();   // and has been read before its lane refills the slot
         };
         auto refill = [&](uint32_t dst, int m, const uint4 *a, const uint4 *d) {
@@ -598,10 +619,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             }
         }
         cp_async_wait<0>();
-        part_min = (float)warp_sum((double)(sum2(acc) * offs[2]));
+        weight -= sum2(acc);   // lane by lane: the difference of two large sums would lose it
     }
+    weight = warp_sum_f(weight);
     if (lane == 0)   // the warp's trips are part `part` of the row
-        p.segments[row * NREC + part] = RowSegment{sum_aw * ex2((w.m - ra.m) * c) / ra.s, part_min};
+        p.segments[row * NREC + part] = RowSegment{weight / sum_a};
 }
 
 // Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it
@@ -832,8 +854,8 @@ __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo
     }
 }
 
-// One CTA per sequence: DRAW_THREADS threads for the draw (GREEDY: there is none, they only add up the parts of
-// sum min(p, q)) and one control warp for the accept tests, the first rejection, the reward and the bandit, which runs
+// One CTA per sequence: DRAW_THREADS threads for the draw (GREEDY: there is none, they only add up the parts'
+// weights) and one control warp for the accept tests, the first rejection, the reward and the bandit, which runs
 // while the other warps search for the token.  What bounds it is the chain of dependent reads of its slowest sequence.
 //
 // The draw: the smallest v with sum_{w <= v} weight_w > u * total.  The row-statistics kernel leaves the mass of every
@@ -901,8 +923,8 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
                 if (!in_range) {
                     flags |= METASD_STATUS_TOKEN_OOR;
                 } else {
-                    p_x = ex2(fmaf(a_x, c, -r.max_a * c)) / r.sum_a;
-                    q_x = ex2(fmaf(d_x, c, -r.max_b * c)) / r.sum_b;
+                    p_x = ex2(fmaf(a_x, c, r.ref_a)) / r.sum_a;
+                    q_x = ex2(fmaf(d_x, c, r.ref_b)) / r.sum_b;
                     if (GREEDY) {
                         accepted = x == r.argmax_a;
                     } else {
@@ -954,13 +976,13 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
 #pragma unroll 1
     for (int j = warp; j < (GREEDY ? k : k + 1); j += NWARP) {
         const RowSegment *seg = segments + (size_t)j * p.n_seg;
-        double m = 0.0, x = 0.0;
+        double m = 0.0, x = 0.0;     // the parts' weights, as they are and without what rounding left below zero
 #pragma unroll
         for (int q = 0; q < MAX_SEGMENTS / 32; ++q)
             if (q < per_lane && lane * per_lane + q < p.n_seg) {
-                const RowSegment g = seg[lane * per_lane + q];
-                m += (double)g.min;
-                x += j < k ? fmax((double)g.p - (double)g.min, 0.0) : (double)g.p;
+                const double weight = (double)seg[lane * per_lane + q].weight;
+                m += weight;
+                x += fmax(weight, 0.0);
             }
         if (!GREEDY) {
             if (j != warp) u = uniform24(round_words(p.seed, sequence, t, (uint32_t)j).y);
@@ -975,7 +997,7 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         }
         if (j < k) {
             m = warp_sum(m);
-            if (lane == 0) sh_align[j] = m;
+            if (lane == 0) sh_align[j] = 1.0 - m;
         }
     }
     __syncthreads();
@@ -986,19 +1008,19 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     DrawRow<LT> row;
     row.a = target + (size_t)n_acc * V;
     row.c = c;
-    row.nma = -rs.max_a * c; row.ia = 1.0f / rs.sum_a;
+    row.nma = rs.ref_a; row.ia = 1.0f / rs.sum_a;
     bool residual = sh_mode == 1;
     auto draw_from_target = [&] { row.d = row.a; row.nmb = row.nma; row.ib = 0.f; };
     if (residual) {
         row.d = draft + (size_t)n_acc * V;
-        row.nmb = -rs.max_b * c; row.ib = 1.0f / rs.sum_b;
+        row.nmb = rs.ref_b; row.ib = 1.0f / rs.sum_b;
     } else {
         draw_from_target();
     }
     int lo = 0, hi = V, level = 0;
     double base = 0.0, threshold = (double)sh_u[n_acc];
-    // Below a thousandth the parts' masses p - min are differences of numbers that far above them: the walk over the whole
-    // row, which takes the difference token by token, decides instead (such a rejection is rare by its own measure).
+    // Below a thousandth the parts' masses are what is left of numbers that far above them: the walk over the whole row,
+    // which takes the difference token by token, decides instead (such a rejection is rare by its own measure).
     bool whole = p.n_seg <= 1 || !(hit.total > 1.0e-3);
     if (!whole) {
         int lead = 0, shift = 0;
