@@ -22,7 +22,7 @@ struct RowStats {
 // sum_v p_v - min(p_v, q_v), which adds up to d_TV(p, q) over the row; of a bonus row its share of p.  A row has n_seg parts of
 // nearly equal length (segment_begin).
 struct RowSegment {
-    float weight;
+    double weight;
 };
 // First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
 __host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }
