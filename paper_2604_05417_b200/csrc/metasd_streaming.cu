@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         cp_async_wait<0>();
         weight -= sum2(acc);   // lane by lane: the difference of two large sums would lose it
     }
-    // fp64 across lanes: a rounding here would move the draw by itself.  Tokens drawn unlike the oracle's (all next
+    // fp64 across lanes: a rounding here would move the draw by itself.  Tokens unlike a float64 evaluation's (all next
     // to an edge), of 49450 rejections at V = 32000: 28 with references per row and fp32 here, 20 with the warp's reference.
     const double total = warp_sum((double)weight);
     if (lane == 0)   // the warp's trips are part `part` of the row
@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     // Below a thousandth the parts' masses are what is left of numbers that far above them: the walk over the whole row,
     // which takes the difference token by token, decides instead.  The line lies low because one such walk in a batch is
     // what the launch waits for: at a sixteenth B = 64, V = 32000 takes 28.2 us a round instead of 23.8, B = 256, V = 128256
-    // 283 instead of 247, and no fewer tokens differ from the oracle's.
+    // 283 instead of 247, and no fewer tokens differ from a float64 evaluation's.
     bool whole = p.n_seg <= 1 || !(hit.total > 1.0e-3);
     if (!whole) {
         int lead = 0, shift = 0;
