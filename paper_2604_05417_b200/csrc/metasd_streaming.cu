@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     w.ref = 0.f;
     w.nm = 0ull;
     w.best = -INFINITY;
-    w.cmp = Logit<LT>::best_of(-INFINITY);
+    // Logits at the type's lowest value are masks as -Inf is: as a reference they would overflow.
+    w.cmp = Logit<LT>::best_of(METASD_NEG_BIG);
     w.best_i = 0x7FFFFFFF;
     const uint64_t c2 = pack2(c);
     // Requests below the kept share of the warp's range ask L2 to drop the line, the rest to keep it for sweep 2.

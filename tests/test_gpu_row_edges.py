@@ -53,6 +53,34 @@ def test_masked_stretches_cover_whole_warps(dtype, shift):
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [3 * 4096 + 40, 3 * 4096 + 41])
+@pytest.mark.parametrize("T", [1.0, 2.0])
+def test_masks_of_the_types_lowest_value(dtype, V, T):
+    """Masks written as torch.finfo(dtype).min (and as -1e38) over stretches that hold the first trips of some warps: they
+    weigh nothing, as -inf does, although their product with log2(e) / T leaves the range of fp32."""
+    from _harness import make_pair, compare_round
+    wl = workload(V=V, dtype=dtype, B=6, temperature=T)
+    rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=9).gathered_round(0, np.zeros(6, dtype=np.int64))
+    target, draft = rd["target"].clone(), rd["draft"].clone()
+    low = torch.finfo(target.dtype).min
+    target[0, :, : V // 2] = low
+    target[1, :, V // 2:] = low
+    draft[1, :, : V // 4] = low
+    target[2, :, :-3] = low
+    draft[3, :, : V - 9] = low
+    target[4, :, 3:] = -1e38
+    draft[4, :, : V // 3] = low
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    try:
+        res = gpu.verify(target, draft, rd["tokens"], T, 3, want_diag=True)
+        out = orc.verify(target, draft, rd["tokens"].cpu().numpy(), T, 3)
+        compare_round(res, out, target, draft, T, 1.0, {})
+        assert gpu.last_status() & M.STATUS_NONFINITE == 0
+    finally:
+        gpu.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [1, 2, 7, 9, 250, 255, 257, 4085, 4095, 4097, 6 * 4096 + 3, 12 * 4096 - 1, 50257])
 def test_rows_off_a_16_byte_boundary(dtype, V):
     """Odd vocabularies: every row starts at an offset of its own, target and draft rows at different ones."""
