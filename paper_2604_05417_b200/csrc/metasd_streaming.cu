@@ -490,10 +490,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     }
     float ref_b = ref_a;
     bool bad_b = false;
-    // The shared reference suits the draft row when its sum is neither flushed nor overflowed: 2^-60 .. finite
-    // leaves every term that matters in fp32 range.  Otherwise (draft logits far from the target's, or a row
-    // that is not finite) the draft row is swept again relative to its own running maximum.
-    if (pair && !(sum_b >= 0x1p-60f && sum_b < INFINITY)) {
+    // The shared reference suits the draft row when its sum is neither flushed nor near overflow: 2^-60 .. 2^100
+    // leaves every term that matters, and 2^+-(the whole part of log2(sum_a / sum_b)), in fp32 range.  Otherwise (draft
+    // logits far from the target's, or a row that is not finite) the draft row is swept again relative to its own
+    // running maximum.
+    if (pair && !(sum_b >= 0x1p-60f && sum_b < 0x1p100f)) {
         MaxSum own = {METASD_NEG_BIG, 0.f};   // m: the running maximum's exponent, a whole number here too
         for (int n = 0; n < lane_trips; ++n) {
             float xb[VEC];

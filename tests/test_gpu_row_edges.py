@@ -81,6 +81,32 @@ def test_masks_of_the_types_lowest_value(dtype, V, T):
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("V", [4096, 4099])
+def test_draft_sums_next_to_the_end_of_the_fp32_range(dtype, V):
+    """Draft rows whose sum, relative to the target row's maximum (0 here), is 2^99 .. 2^128: 2^127.6 is a finite fp32
+    number, and its inverse's whole exponent, 128, is not one that an fp32 power of two can have."""
+    from _harness import make_pair, compare_round
+    wl = workload(V=V, dtype=dtype, B=8, N=1, k=2)
+    dev = torch.device("cuda", 0)
+    target = torch.full((8, 3, V), -30.0, dtype=torch.float32, device=dev)
+    target[:, :, 0] = 0.0
+    draft = torch.full((8, 2, V), -30.0, dtype=torch.float32, device=dev)
+    for b, (low, high) in enumerate([(68.0, 68.5), (69.0, 69.5), (70.0, 70.0), (87.0, 87.0), (87.5, 87.5), (87.5, 88.0), (88.0, 87.5),
+                                     (88.5, 88.5)]):
+        draft[b, :, 0], draft[b, :, 5] = low, high
+    target, draft = (x.to({"bf16": torch.bfloat16, "fp32": torch.float32}[dtype]) for x in (target, draft))
+    tokens = torch.zeros((8, 2), dtype=torch.int32, device=dev)
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    try:
+        res = gpu.verify(target, draft, tokens, 1.0, 3, want_diag=True)
+        out = orc.verify(target, draft, tokens.cpu().numpy(), 1.0, 3)
+        compare_round(res, out, target, draft, 1.0, 1.0, {})
+        assert gpu.last_status() == 0
+    finally:
+        gpu.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [1, 2, 7, 9, 250, 255, 257, 4085, 4095, 4097, 6 * 4096 + 3, 12 * 4096 - 1, 50257])
 def test_rows_off_a_16_byte_boundary(dtype, V):
     """Odd vocabularies: every row starts at an offset of its own, target and draft rows at different ones."""
