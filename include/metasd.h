@@ -251,7 +251,7 @@ int metasd_resolved_row_kernel(const metasd_ctx *ctx);
  * context, so there is no bandit here and nothing persists between calls.)
  *
  * It launches the kernels of a default streaming context (the staged row-statistics kernel, then the
- * epilogue).  Their scratch lives in a fixed array inside the library image (about 5 MB, held
+ * epilogue).  Their scratch lives in a fixed array inside the library image (about 9 MB, held
  * by every GPU that loads the library until the process exits), which bounds the sizes:
  * batch <= METASD_NOALLOC_MAX_BATCH and batch * (k + 1) <= METASD_NOALLOC_MAX_ROWS; beyond that the
  * call returns METASD_ERR_UNSUPPORTED and launches nothing.  The call makes no cudaMalloc / cudaFree

@@ -312,7 +312,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, MINB) row_stats_bulk_kernel(co
             r.argmax_a = rm.i;
             r.flags = flags;
             p.stats[(size_t)b * (p.k + 1) + j] = r;
-            p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{pair ? 1.0 - total_min : 1.0};
+            p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{pair ? 1.0 - total_min : 1.0, total_min};
         };
         if (!pair) {
             if (tid == 0) write_stats(0.0);

@@ -18,11 +18,12 @@ struct RowStats {
     uint32_t flags;       // METASD_STATUS_* of this row pair
 };
 
-// What the row-statistics pass says about a contiguous part of a row: of a row pair the mass sum_v max(0, p_v - q_v) =
-// sum_v p_v - min(p_v, q_v), which adds up to d_TV(p, q) over the row; of a bonus row its share of p.  A row has n_seg parts of
-// nearly equal length (segment_begin).
+// What the row-statistics pass says about a contiguous part of a row.  Of a row pair the mass sum_v max(0, p_v - q_v) =
+// sum_v p_v - min(p_v, q_v), which the draw is made from, and sum_v min(p_v, q_v) itself: over the row it adds up to
+// 1 - d_TV(p, q), which a difference would lose where the rows hardly overlap.  Of a bonus row its share of p, and 0.  A row
+// has n_seg parts of nearly equal length (segment_begin).
 struct RowSegment {
-    double weight;
+    double weight, shared;
 };
 // First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
 __host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
         if (bad_a || bad_b) flags |= METASD_STATUS_NONFINITE;
         r.flags = flags;
         p.stats[(size_t)b * (p.k + 1) + j] = r;
-        p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{pair ? 1.0 - total_min : 1.0};
+        p.segments[(size_t)b * (p.k + 1) + j] = RowSegment{pair ? 1.0 - total_min : 1.0, total_min};
     }
 }
 
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // With rho = sum_a / sum_b: min(p, q) = 2^min(a c + ref_a, b c + ref_b + log2 rho) / sum_a.  The logarithm's whole part joins
     // the reference, which stays exact; its fraction is added to the exponents on its own (folded into a reference of 20 it
     // would be rounded at that size, and every term of the draft row scaled by the error, up to 7e-7).
-    float weight = sum2(w.a);
+    float weight = sum2(w.a), shared = 0.f;
     if (pair) {
         const float rho = sum_a / sum_b, whole = rintf(log2f(rho));
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
@@ -622,13 +622,16 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             }
         }
         cp_async_wait<0>();
-        weight -= sum2(acc);   // lane by lane: the difference of two large sums would lose it
+        shared = sum2(acc);
+        weight -= shared;   // lane by lane: the difference of two large sums would lose it
     }
     // fp64 across lanes: a rounding here would move the draw by itself.  Tokens unlike a float64 evaluation's (all next
     // to an edge), of 49450 rejections at V = 32000: 28 with references per row and fp32 here, 20 with the warp's reference.
-    const double total = warp_sum((double)weight);
-    if (lane == 0)   // the warp's trips are part `part` of the row
-        p.segments[row * NREC + part] = RowSegment{total * (double)(exp2i(fminf(ref_a - w.ref, 0.f)) / sum_a)};
+    const double total = warp_sum((double)weight), total_min = warp_sum((double)shared);
+    if (lane == 0) {   // the warp's trips are part `part` of the row
+        const double scale = (double)(exp2i(fminf(ref_a - w.ref, 0.f)) / sum_a);
+        p.segments[row * NREC + part] = RowSegment{total * scale, total_min * scale};
+    }
 }
 
 // Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it
@@ -981,13 +984,13 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
 #pragma unroll 1
     for (int j = warp; j < (GREEDY ? k : k + 1); j += NWARP) {
         const RowSegment *seg = segments + (size_t)j * p.n_seg;
-        double m = 0.0, x = 0.0;     // the parts' weights, as they are and without what rounding left below zero
+        double m = 0.0, x = 0.0;     // the parts' sums of min(p, q), and their weights without what rounding left below zero
 #pragma unroll
         for (int q = 0; q < MAX_SEGMENTS / 32; ++q)
             if (q < per_lane && lane * per_lane + q < p.n_seg) {
-                const double weight = seg[lane * per_lane + q].weight;
-                m += weight;
-                x += fmax(weight, 0.0);
+                const RowSegment part = seg[lane * per_lane + q];
+                m += part.shared;
+                x += fmax(part.weight, 0.0);
             }
         if (!GREEDY) {
             if (j != warp) u = uniform24(round_words(p.seed, sequence, t, (uint32_t)j).y);
@@ -1002,7 +1005,7 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         }
         if (j < k) {
             m = warp_sum(m);
-            if (lane == 0) sh_align[j] = 1.0 - m;
+            if (lane == 0) sh_align[j] = m;
         }
     }
     __syncthreads();

@@ -160,3 +160,28 @@ def test_every_shape_that_a_launch_size_selects(dtype, V, B, k):
     from _harness import run_lockstep
     c = run_lockstep(workload(V=V, dtype=dtype, B=B, k=k, temperature=0.9), rounds=2, seed=V % 83, path=M.PATH_STREAMING)
     assert c["rounds"] == 2 and c["status"] == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("kernel", [M.ROWS_AUTO, M.ROWS_PLAIN, M.ROWS_BULK])
+def test_alignment_of_rows_that_hardly_overlap(dtype, kernel):
+    """Target and draft mass in different halves of the vocabulary: the alignment 1 - d_TV is a small sum of positive terms,
+    each a 2^-22 exponential of an fp32 exponent of up to 130 (off by 2^-18 at most) over an fp32 normaliser, never a
+    difference: 1e-5 of itself."""
+    B, V = 12, 8200
+    wl = workload(V=V, dtype=dtype, B=B, N=1, k=1)
+    rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=2).gathered_round(0, np.zeros(B, dtype=np.int64))
+    gap = torch.linspace(2.0, 60.0, B, device="cuda").view(B, 1, 1)
+    target, draft = rd["target"].float(), rd["draft"].float()
+    target[..., V // 2:] -= gap
+    draft[..., : V // 2] -= gap
+    target, draft = target.to(rd["target"].dtype), draft.to(rd["draft"].dtype)
+    gpu = M.MetaSD(B, 1, 1, V, dtype=dtype, path=M.PATH_STREAMING, row_kernel=kernel)
+    try:
+        res = gpu.verify(target, draft, rd["tokens"], 1.0, 3, want_diag=True)
+        p, q = (torch.softmax(x[:, 0].double(), -1) for x in (target, draft))
+        want = torch.minimum(p, q).sum(-1)
+        assert float(want.min()) < 1e-20 and float(res.reward.min()) > 0 and float(res.diag_fields()[2].max()) <= 1.0
+        torch.testing.assert_close(res.reward.double(), want, rtol=1e-5, atol=0)
+    finally:
+        gpu.close()
