@@ -780,6 +780,7 @@ template <int NWARP> struct DrawShared {
     double tot[2][NWARP];
     double base;
     int lo;
+    bool sure;
 };
 
 // Barrier among the draw's warps only: the control warp goes its own way.
@@ -789,10 +790,11 @@ template <int THREADS> __device__ __forceinline__ void draw_sync() { asm volatil
 // smallest token v with sum_{w <= v} weight_w > threshold to *out.  Every thread sums a contiguous piece; the piece with the
 // crossing is found by a scan (fp64), and when it is no longer than a warp, a vector a lane, the token in it.  FRACTION:
 // the threshold comes in as a fraction of the range's own total.  Rounding may leave no crossing: then the last token with
-// mass.  false: no mass (the same in every thread).  The levels of a row's searches are counted in `level`.
+// mass.  A token whose ends are not `guard` away from the threshold is not written (guard < 0: any token is).  false: no mass,
+// or no token written (the same in every thread).  The levels of a row's searches are counted in `level`.
 template <typename LT, int VEC, int NWARP>
 __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo, int hi, double base, double threshold, bool fraction,
-                                                  DrawShared<NWARP> &sh, int &level, int32_t *out)
+                                                  double guard, DrawShared<NWARP> &sh, int &level, int32_t *out)
 {
     constexpr int U = VEC == 1 ? 8 : 4;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -843,18 +845,30 @@ __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo
                 const int who = warp_crossing((double)s, end, threshold);
                 double run = end - (double)s;
                 int token = -1, last_token = -1;
+                bool sure = guard < 0.0;
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) {
+                    const double front_e = run;
                     run += (double)w[e];
                     if (w[e] > 0.f) {
                         last_token = i * VEC + e;
-                        if (token < 0 && run > threshold) token = last_token;
+                        if (token < 0 && run > threshold) {
+                            token = last_token;
+                            sure = sure || (front_e < threshold - guard && run > threshold + guard);
+                        }
                     }
                 }
-                if (lane == max(who, 0)) *out = who < 0 ? first * VEC : token >= 0 ? token : last_token;
+                if (lane == max(who, 0)) {
+                    if (sure) *out = who < 0 ? first * VEC : token >= 0 ? token : last_token;
+                    sh.sure = sure;
+                }
             }
         }
-        if (!another) return true;
+        if (!another) {
+            if (guard < 0.0) return true;
+            draw_sync<NWARP * 32>();
+            return sh.sure;
+        }
         draw_sync<NWARP * 32>();
         base = sh.base;
         lo = sh.lo;
@@ -1032,6 +1046,12 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
     // what the launch waits for: at a sixteenth B = 64, V = 32000 takes 28.2 us a round instead of 23.8, B = 256, V = 128256
     // 283 instead of 247, and no fewer tokens differ from a float64 evaluation's.
     bool whole = p.n_seg <= 1 || !(hit.total > 1.0e-3);
+    // Up to a sixteenth the row is walked where the parts leave a doubt.  A part's weight is off by what its lanes' fp32 sums
+    // were rounded by, which follows the heaviest of them (a token of about 1 / sum_a): 3e-8 of the row's mass rms, 1.4e-7 at
+    // most, in 460000 draws of seven kinds, and next to a small residual that counts for more.  Doubted wherever it is (every
+    // residual, and bonus rows) tokens unlike a float64 evaluation's are 63 of these draws instead of 143 (58 with every row
+    // walked), but moving batches of V = 32000 take 26.4 us instead of 23.9, and odd vocabularies 64 instead of 52.
+    const double guard = hit.total < 0.0625 ? (double)(1.0e-7f * __fsqrt_rn(__fdividef(1.f, rs.sum_a) + 0.01f)) : -1.0;
     if (!whole) {
         int lead = 0, shift = 0;
         if (!VECTOR) row_alignment(row.a, residual ? row.d : nullptr, lead, shift);
@@ -1042,7 +1062,9 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
         threshold = hit.threshold;
     }
     for (;;) {
-        if (range_inverse_cdf<LT, VEC, NWARP>(row, lo / VEC, hi / VEC, base, threshold, whole, sh_draw, level, p.next_token + b)) return;
+        if (range_inverse_cdf<LT, VEC, NWARP>(row, lo / VEC, hi / VEC, base, threshold, whole, whole ? -1.0 : guard, sh_draw, level,
+                                              p.next_token + b))
+            return;
         ++level;
         if (whole) {
             if (!residual) break;

@@ -54,6 +54,35 @@ def test_a_residual_with_next_to_no_mass_is_drawn_from_token_by_token(V):
     assert drawn > 5
 
 
+@pytest.mark.parametrize("sigma", [0.15, 0.03])
+def test_draws_from_small_residuals_are_those_of_the_whole_row(sigma):
+    """Good drafters: residuals of a thousandth to a sixteenth of the row's mass, whose parts are differences of numbers up
+    to 1e3 times larger.  A token taken from the parts alone was up to 9e-8 of the row's mass away from its interval of the
+    float64 CDF; a walk over the row, which takes the differences token by token, each off by 2^-25 of the heaviest token at
+    most, stays within 2^-24 of it."""
+    B, k, V, dev = 256, 4, 32000, torch.device("cuda", 0)
+    wl = workload(B=B, N=1, k=k, V=V, sigmas=(sigma,), order="rank")
+    acc, tok = (torch.zeros(B, dtype=torch.int32, device=dev) for _ in range(2))
+    reward = torch.zeros(B, device=dev)
+    draws = 0
+    for s in range(4):
+        rd = RoundGenerator(wl, device=dev, seed=100 + s).gathered_round(0, np.zeros(B, dtype=np.int64))
+        p, q = torch.softmax(rd["target"].double(), -1), torch.softmax(rd["draft"].double(), -1)
+        cdf = (p[:, :k] - q).clamp_min(0).cumsum(-1)
+        for i in range(100):
+            assert M.verify_noalloc(rd["target"], rd["draft"], rd["tokens"], 1.0, 7 + i, i, acc, tok, reward) == M.OK
+            n = acc.cpu().numpy()
+            u = torch.tensor([O.round_uniforms(7 + i, b, i, int(n[b]))[1] for b in range(B)], dtype=torch.float64, device=dev)
+            row = cdf[torch.arange(B, device=dev), acc.long().clamp_max(k - 1)]
+            band = (acc < k) & (row[:, -1] > 1e-3) & (row[:, -1] < 1 / 16)
+            at, end = u * row[:, -1], row.gather(1, tok.long()[:, None])[:, 0]
+            front = torch.where(tok > 0, row.gather(1, (tok.long() - 1).clamp_min(0)[:, None])[:, 0], torch.zeros_like(end))
+            off = torch.maximum(front - at, at - end)[band]
+            assert off.numel() == 0 or float(off.max()) < 2.0 ** -24
+            draws += int(band.sum())
+    assert draws > 2000
+
+
 @pytest.mark.parametrize("window", [1, 2, 31, 32, 33, 64, 65])
 def test_sliding_windows_around_a_warp(window):
     from _harness import run_lockstep
