@@ -721,23 +721,24 @@ __device__ __forceinline__ void draw_weights(const DrawRow<LT> &row, const RawVe
         w[e] = fmaxf(__fmaf_rn(ex2(fmaf(xb[e], row.c, row.nmb)), -row.ib, __fmul_rn(ex2(fmaf(xa[e], row.c, row.nma)), row.ia)), 0.f);
 }
 
-// Sum of the weights of the vectors [i, hi): fp32 a vector, fp64 across; U vectors' loads are issued before the first is used.
+// Sum of the weights of every `step`-th vector of [i, hi): fp32 a vector, fp64 across; U vectors' loads are issued before
+// the first is used.
 template <typename LT, int VEC, int U>
-__device__ __forceinline__ double draw_sum(const DrawRow<LT> &row, int i, int hi)
+__device__ __forceinline__ double draw_sum(const DrawRow<LT> &row, int i, int hi, int step)
 {
     double acc = 0.0;
 #pragma unroll 1
-    for (; i < hi; i += U) {
+    for (; i < hi; i += U * step) {
         RawVec<LT, VEC> ra[U], rb[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i + u < hi) {
-                ra[u] = load_raw<LT, VEC>(row.a, i + u);
-                rb[u] = load_raw<LT, VEC>(row.d, i + u);
+            if (i + u * step < hi) {
+                ra[u] = load_raw<LT, VEC>(row.a, i + u * step);
+                rb[u] = load_raw<LT, VEC>(row.d, i + u * step);
             }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i + u < hi) {
+            if (i + u * step < hi) {
                 float w[VEC], s = 0.f;
                 draw_weights<LT, VEC>(row, ra[u], rb[u], w);
 #pragma unroll
@@ -800,9 +801,21 @@ __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll 1
     for (;; ++level) {
-        const int piece = (hi - lo + NWARP * 32 - 1) / (NWARP * 32);
-        const int v0 = min(lo + tid * piece, hi);
-        const double x = draw_sum<LT, VEC, U>(row, v0, min(v0 + piece, hi)), incl = warp_scan(x);
+        // A lane reads a piece of its own.  Where that would be long, a whole row, a warp's range is in eight pieces that its
+        // lanes read together, neighbouring vectors by neighbouring lanes, one piece after another (lane t keeps piece t's).
+        int piece = (hi - lo + NWARP * 32 - 1) / (NWARP * 32);
+        const bool another = piece > 32;
+        const int pieces = another ? 8 : 32;
+        if (another) piece = (hi - lo + NWARP * 8 - 1) / (NWARP * 8);
+        double x = 0.0;
+#pragma unroll 1
+        for (int t = 0; t < (another ? 8 : 1); ++t) {
+            const int v0 = min(lo + (warp * pieces + (another ? t : lane)) * piece, hi);
+            double sum = draw_sum<LT, VEC, U>(row, another ? v0 + lane : v0, min(v0 + piece, hi), another ? 32 : 1);
+            if (another) sum = warp_sum(sum);
+            if (!another || lane == t) x = sum;
+        }
+        const double incl = warp_scan(x);
         double *tot = sh.tot[level & 1];
         if (lane == 31) tot[warp] = incl;
         draw_sync<NWARP * 32>();
@@ -826,11 +839,10 @@ __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo
         }
         if (last < 0) return false;
         if (owner < 0) owner = last;
-        const bool another = piece > 32;
         if (warp == owner) {
             const int src = warp_crossing(x, before + incl, threshold);
             const double front = before + __shfl_sync(0xFFFFFFFFu, incl - x, src);
-            const int first = min(lo + (warp * 32 + src) * piece, hi);
+            const int first = min(lo + (warp * pieces + src) * piece, hi);
             if (another) {
                 if (lane == 0) { sh.base = front; sh.lo = first; }
             } else {
@@ -888,7 +900,7 @@ __device__ __forceinline__ bool range_inverse_cdf(const DrawRow<LT> &row, int lo
 // k = 5, V = 32000 35.9 -> 24.6; B = 96, k = 5, V = 50257 61.8 -> 50.6; B = 256, k = 7, V = 128256 with the row statistics' 237 -> 229;
 // the sliding-window policy's scan before the wait instead of behind it (B = 192, greedy) 61.7 -> 54.5.
 template <typename LT, bool VECTOR, int DRAW_THREADS, bool GREEDY>
-__global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_kernel(const VerifyParams p)
+__global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS == 256 ? 2 : 1) epilogue_kernel(const VerifyParams p)
 {
     constexpr int NWARP = DRAW_THREADS / 32, VEC = VECTOR ? Logit<LT>::VEC : 1;
     constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -1083,7 +1095,10 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : 2) epilogue_ke
 // -------------------------------------------------------------------------------------------
 // launchers
 // -------------------------------------------------------------------------------------------
-constexpr int DRAW_THREADS = 256;   // of an epilogue CTA besides its control warp
+// Threads of an epilogue CTA besides its control warp.  Rows in one part (the plain and the bulk kernel) are walked whole, by
+// twice the threads where every sequence has an SM: B = 64, k = 4, V = 152064, plain 125 -> 107 us a round, bulk (whose rows are
+// not in L2) 169 -> 96, with the coalesced pieces of range_inverse_cdf; B = 300, k = 2, V = 128256 205 -> 196 and 256 -> 188.
+constexpr int DRAW_THREADS = 256, DRAW_THREADS_ROW = 512;
 
 // The built shapes of the staged kernel, per logit type: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).
 // Those that staged_shape() picks, and those that a configuration can ask for.
@@ -1270,8 +1285,11 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
     }
     if (e != cudaSuccess) return e;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const unsigned grid = (unsigned)p.batch, threads = DRAW_THREADS + 32;   // and the control warp
+    const unsigned grid = (unsigned)p.batch, threads = DRAW_THREADS + 32, threads_row = DRAW_THREADS_ROW + 32;   // and the control warp
+    const bool row = p.n_seg <= 1 && p.batch <= geo.n_sm;
     if (p.greedy) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, true>, grid, threads, 0, 1, true, stream, p);
+    else if (row && p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS_ROW, false>, grid, threads_row, 0, 1, true, stream, p);
+    else if (row) e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS_ROW, false>, grid, threads_row, 0, 1, true, stream, p);
     else if (p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
     else e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
     *launches += 2;
