@@ -212,7 +212,7 @@ int metasd_init(metasd_ctx **out, const metasd_config *cfg)
         e = streaming_prepare(cfg->device, cfg->logit_dtype, *cfg, &c->geo);
         if (e == cudaErrorNotSupported) { unsupported = true; (void)cudaGetLastError(); }
     }
-    alloc((void **)&c->segments, segment_capacity(c->geo, B * kp1) * sizeof(RowSegment));
+    alloc((void **)&c->segments, B * kp1 * (size_t)row_parts(c->geo, cfg->logit_dtype, cfg->vocab) * sizeof(RowSegment));
     if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(uint32_t));
     if (e == cudaSuccess) e = launch_reset(c->st, cfg->max_batch, cfg->n_drafters, cfg->window, cfg->bandit, cfg->gamma,
                                             cfg->sequence_base, nullptr, cfg->max_batch, 0);

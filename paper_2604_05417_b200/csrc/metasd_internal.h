@@ -27,7 +27,7 @@ struct RowSegment {
 };
 // First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
 __host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }
-constexpr int MAX_SEGMENTS = 128;   // most parts of a row
+constexpr int MAX_SEGMENTS = 64;   // most parts of a row
 
 // Bandit state of all sequences, structure of arrays in device memory.
 struct BanditState {
@@ -40,7 +40,7 @@ struct BanditState {
 };
 
 // Shape of the row-statistics launch: what a context's configuration pins, resolved once; threads == 0 (staged kernel):
-// the shape follows the size of each launch.
+// the shape follows the size of each launch, the warps per row (and with them all arithmetic) the row's length alone.
 struct RowGeometry {
     int32_t kernel;     // metasd_row_kernel, never AUTO
     int32_t threads;    // threads per CTA
@@ -48,7 +48,6 @@ struct RowGeometry {
     int32_t per_sm;     // CTAs per SM the shape is built for
     int32_t n_sm;       // SMs of the device (persistent kernels size their grid with it)
     int32_t cluster;    // CTAs that share one row pair (1: none)
-    int32_t n_seg;      // parts of a row that the kernel reports on (RowSegment)
 };
 
 struct VerifyParams {
@@ -89,7 +88,7 @@ struct VerifyParams {
 };
 
 // streaming path (metasd_streaming.cu, metasd_bulk.cu)
-size_t segment_capacity(const RowGeometry &geo, size_t units);
+int row_parts(const RowGeometry &geo, int dtype, int vocab);   // parts of a row that a launch reports on
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo);
 cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches);
 cudaError_t bulk_prepare(int dtype, RowGeometry *geo);

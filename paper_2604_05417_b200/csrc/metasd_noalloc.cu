@@ -22,7 +22,7 @@ namespace {
 
 constexpr int NOALLOC_MAX_ROWS = METASD_NOALLOC_MAX_ROWS;    // batch * (k + 1)
 constexpr int NOALLOC_MAX_BATCH = METASD_NOALLOC_MAX_BATCH;
-constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row where there are many rows (few rows have more: segment_capacity)
+constexpr int NOALLOC_MAX_SEGMENTS = 32;   // parts per row, at most (row_parts)
 
 // Everything the two kernels keep in global memory besides the caller's inputs and outputs.
 struct StaticScratch {
@@ -63,6 +63,7 @@ cudaError_t default_geometry(int device, int dtype, RowGeometry *out)
     if (!g_geometry_ready[device][dtype]) {
         metasd_config cfg;
         metasd_default_config(&cfg);
+        cfg.vocab = 0;   // calls bring vocabularies of any size
         cudaError_t e = streaming_prepare(device, dtype, cfg, &g_geometry[device][dtype]);
         if (e != cudaSuccess) return e;
         g_geometry_ready[device][dtype] = true;
@@ -97,7 +98,7 @@ extern "C" int metasd_verify_noalloc(int32_t batch, int32_t k, int32_t vocab, in
     if (scratch_address(device, &scratch) != cudaSuccess) return METASD_ERR_CUDA;
     RowGeometry geo;
     if (default_geometry(device, logit_dtype, &geo) != cudaSuccess) return METASD_ERR_CUDA;
-    if (segment_capacity(geo, (size_t)batch * (k + 1)) > sizeof(scratch->segments) / sizeof(RowSegment)) return METASD_ERR_UNSUPPORTED;
+    if (row_parts(geo, logit_dtype, vocab) > NOALLOC_MAX_SEGMENTS) return METASD_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
 
     VerifyParams p = {};

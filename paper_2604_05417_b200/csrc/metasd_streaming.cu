@@ -258,7 +258,7 @@ template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bo
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
     static_assert(D >= 2, "at least two stages");
-    static_assert(THREADS / 32 * CL <= MAX_SEGMENTS, "the epilogue holds four parts per lane");
+    static_assert(THREADS / 32 * CL <= MAX_SEGMENTS, "the epilogue holds two parts per lane");
     constexpr int VEC = Logit<LT>::VEC;
     constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
     constexpr uint32_t STAGE_STRIDE = STAGED_SMEM<D, THREADS, SHIFTED> / D;
@@ -1006,7 +1006,7 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
     float u = uniform24(round_words(p.seed, sequence, t, (uint32_t)warp).y);
     grid_dependency_wait();
     // lane l holds parts n l / 32 ..: contiguous, so that lane order is token order
-    const int per_lane = (p.n_seg + 31) >> 5;    // 1 .. 4
+    const int per_lane = (p.n_seg + 31) >> 5;    // 1 or 2
 #pragma unroll 1
     for (int j = warp; j < (GREEDY ? k : k + 1); j += NWARP) {
         const RowSegment *seg = segments + (size_t)j * p.n_seg;
@@ -1100,36 +1100,44 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
 // not in L2) 169 -> 96, with the coalesced pieces of range_inverse_cdf; B = 300, k = 2, V = 128256 205 -> 196 and 256 -> 188.
 constexpr int DRAW_THREADS = 256, DRAW_THREADS_ROW = 512;
 
-// The built shapes of the staged kernel, per logit type: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).
-// Those that staged_shape() picks, and those that a configuration can ask for.
-#define METASD_STAGED_AUTO_SHAPES(X) \
-    X(512, 4, 3, true, 8) X(512, 4, 3, true, 4) X(512, 4, 3, true, 2) X(512, 4, 3, true, 1) X(512, 6, 2, true, 1) \
-    X(512, 6, 2, true, 2) X(256, 6, 4, true, 2) X(256, 6, 4, true, 1) X(256, 4, 6, true, 1) X(128, 4, 12, true, 1) X(1024, 6, 1, false, 1)
+// The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).  Those that
+// staged_shape() picks, by logit type, and those that a configuration can ask for.
+#define METASD_STAGED_BF16_SHAPES(X) \
+    X(128, 4, 12, true, 1) X(256, 4, 6, true, 1) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) \
+    X(256, 6, 4, true, 2) X(128, 6, 6, true, 4)
+#define METASD_STAGED_FP32_SHAPES(X) \
+    X(256, 4, 6, true, 1) X(256, 6, 4, true, 2) X(128, 6, 6, true, 4) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
 #define METASD_STAGED_PINNED_SHAPES(X) \
     X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(1024, 6, 1, false, 1) X(1024, 4, 1, true, 1) X(768, 4, 2, true, 1) X(384, 4, 4, true, 1) \
     X(512, 4, 3, true, 3) X(512, 4, 3, true, 2) X(768, 4, 2, true, 2)
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
-static cudaError_t prepare_staged()
+static cudaError_t prepare_staged(bool aligned)
 {
-    cudaError_t e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
-    if (e == cudaSuccess)
+    cudaError_t e = cudaSuccess;
+    if (aligned)
+        e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
+    if (e == cudaSuccess)   // a tensor may start off a 16-byte boundary whatever its rows' length
         e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
     return e;
 }
 
-// threads == 0: every shape that staged_shape() may pick.
+// The pinned shape; threads == 0: every shape that staged_shape() may pick for rows of `warps` warps (0: for any row).
 template <typename LT>
-static cudaError_t prepare_staged_t(int threads, int stages, int cluster)
+static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int warps, bool aligned)
 {
-    cudaError_t e = threads == 0 ? cudaSuccess : cudaErrorNotSupported;
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C>();
-    METASD_STAGED_PINNED_SHAPES(X)
+    if (threads) {
+#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C>(aligned);
+        METASD_STAGED_PINNED_SHAPES(X)
 #undef X
-#define X(T, D, M, BL, C) if (e == cudaSuccess) e = prepare_staged<LT, D, T, M, BL, C>();
-    METASD_STAGED_AUTO_SHAPES(X)
+        return cudaErrorNotSupported;
+    }
+    cudaError_t e = cudaSuccess;
+#define X(T, D, M, BL, C) if (e == cudaSuccess && (warps == 0 || warps == T / 32 * C)) e = prepare_staged<LT, D, T, M, BL, C>(aligned);
+    if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
+    else { METASD_STAGED_FP32_SHAPES(X) }
 #undef X
     return e;
 }
@@ -1140,77 +1148,75 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
 #define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
         return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, geo.n_sm, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
-    METASD_STAGED_AUTO_SHAPES(X)
+    if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
+    else { METASD_STAGED_FP32_SHAPES(X) }
     METASD_STAGED_PINNED_SHAPES(X)
 #undef X
     return cudaErrorNotSupported;
 }
 
-// Launches of at most this many rows (row pairs) may take the cluster shapes with more than 32 parts per row.
-constexpr int FEW_ROWS = 148;
+static long long row_bytes(int dtype, int vocab) { return (long long)vocab * (dtype == METASD_BF16 ? 2 : 4); }
 
-// The shape for rows of `row_bytes` bytes in a launch of `units` rows (row pairs and bonus rows).  Measured on B200, us a
-// round (threads / stages / CTAs per row; units = B (k + 1)):
-//   bf16, few rows: a row is split until every SM has a CTA.
-//     5 rows, V = 32000: 512/4/1 19.4, /4 16.8, /8 16.5.  36, V = 152064: 34.3, /4 21.7, /8 23.0.  72, V = 128256: 31.6, /2 23.5, /4 25.2.
-//   bf16, many short rows: small CTAs, because the fixed part of a CTA's life is what a short row costs.
-//     V = 8000, 5120 rows: 512/4 108, 256/4 85, 128/4 74.  V = 16000, 9216 rows: 218, 174, 161; 1536 rows: 44, 37, 38.
-//     V = 32000, 1536 rows: 65.6, 60.0; 5120 rows: 182, 164.  V = 48000, 5120 rows: 258, 238.  V = 50257, 5120 rows: 324, 347.
-//   bf16, long rows in a few waves of CTAs: two small CTAs share a row, so that the last wave is finer.
-//     V = 152064, 576 rows: 512/6/1 102, 512/4/2 96.5, 256/6/2 96.4.  V = 128256, 768 rows: 108, 102, 101.  V = 80000, 384 rows: 48, 49, 44.
-//     Off 16-byte boundaries: V = 152065, 680 rows: 165, 145, 161.  V = 80001, 384 rows: 67, 64, 71, 512/4/1 63.
-//   bf16, medium rows: V = 60000, 5120 rows: 512/4/1 302, 256/6/1 283; 1536 rows: 94.5, 94.6.  V = 72000, 1536 rows: 112.5, 111.7.
-//     Off 16-byte boundaries (V = 50257, 5120 rows): 324, 349.
-//   bf16, long rows: a larger share of the pair kept on chip pays for fewer of them in flight from 80000 tokens on
-//     (B = 256, k = 5, 512/4 / 512/6: V = 64000 110 / 112, 80000 132 / 131, 112000 174 / 169).
-//   fp32 (half as many exponentials per byte) wants more of a row in flight and on chip.
-//     24 rows, V = 128256: split until the slots of all SMs are taken: 96 rows 512/4/1 37, /4 31.4.  V = 8000, 5120 rows: 512/4 111, 256/4 91.
-//     V = 32000: 5120 rows 512/6 265, 256/6 255; 1536 rows 88, 90; 384 rows 31.8, 29.0.
-//     V = 128256: 192 rows 1024/6/1 69, 512/6/2 63; 384 rows 98, 97; 768 rows 161, 167.
+// Warps that share a row, by its length and type alone: which tokens a warp adds up, relative to what and in which order,
+// and the parts that a draw is made from, are then the same whatever else is in the launch, and a sequence's results do not
+// depend on its batch.  Measured on B200, us a round (a graph of rounds; threads / stages / CTAs per row; units = B (k + 1)):
+//   bf16, V = 8000: 4 warps 65.4 (5120 units) and 10.5 (5), 8 warps 74.1 and 9.0.  V = 16000: 95.0 and 12.1, 101.2 and 11.2.
+//     V = 32000: 8 warps 143 (4800), 51.3 (1536), 22.7 (384), 14.7 (96) and 13.6 (6), 16 warps 163, 57.2, 23.4, 12.2 and 10.7.
+//     V = 50264: 212 (4800), 75.4 (1536), 30.6 (384) and 15.0 (6), 234, 79.6, 30.3 and 12.5.  V = 80000: 107.6 (1536), 42.6 and 19.0, 109.6,
+//     39.7 and 14.3.  The line lies where a few sequences gain more than many lose.
+//     V = 152064: 16 warps 215 (1728), 85.9 (576) and 19.6 (9), 32 warps 231, 88.7 and 15.8.
+//   fp32, V = 8000: 8 warps 81.5 (5120).  V = 32000: 8 warps 82.9 (1536), 27.9 (384) and 12.6 (4), 16 warps 81.8, 28.1 and 10.4.
+//     V = 64000: 16 warps 80.3 (768), 48.6 (384) and 12.7 (6), 32 warps 80.5, 48.3 and 10.4.  V = 128256: 162 and 18.7, 137 and 12.6.
+static int row_warps(int dtype, long long bytes)
+{
+    if (dtype == METASD_FP32) return bytes < 80 * 1024 ? 8 : bytes < 250 * 1024 ? 16 : 32;
+    return bytes <= 20 * 1024 ? 4 : bytes < 56 * 1024 ? 8 : 16;
+}
+
+// The shape of a launch: how many CTAs a row's warps are spread over, and the stages.  Us a round as above:
+//   bf16, 16 warps: V = 32000: 128/6/4 11.0 (24 units), 12.2 (96), 23.9 (384), 31.5 (576), 71.7 (1536), 256/6/2 11.8, 13.5, 23.4,
+//     29.0, 64.3, 512/4/1 12.9, 13.3, 24.4, 28.1, 57.2.  V = 80000: 128/6/4 16.6 (72), 39.8 (384), 121 (1536), 256/6/2 16.5, 39.7, 112, 512/4/1
+//     19.3, 42.8, 110, 512/6/1 19.3, 41.6, 113.  V = 152064: 128/6/4 19.8 (36), 24.3 (72), 88.1 (576), 223 (1728), 256/6/2 22.5, 23.6, 85.9,
+//     215, 512/6/1 28.9, 29.4, 91.5, 218 (4608: 527, 256/6/2 590).
+//   fp32, 16 warps, V = 32000: 128/6/4 11.1 (32 units), 15.2 (128), 29.2 (384), 86.9 (1536), 256/6/2 11.8, 15.5, 28.1, 81.8.
+//   fp32, 32 warps: V = 64000: 128/6/8 11.8 (24 units), 50.8 (384), 180 (1728), 614 (6144), 256/6/4 12.1, 48.3, 157, 574, 1024/6/1
+//     17.5, 51.7, 168, 525; V = 128256: 15.8, 79.7, 292 and 1062, 16.0, 86.0, 302 and 1094, 26.5, 91.0, 302 and 1029.
 struct StagedShape {
     int threads, stages, cluster;
 };
-static StagedShape staged_shape(int dtype, long long row_bytes, long long units, bool aligned)
+static StagedShape staged_shape(int dtype, long long bytes, long long units, int n_sm)
 {
     const bool fp32 = dtype == METASD_FP32;
-    const long long trips = (row_bytes + 511) / 512;
-    // few rows: as many CTAs per row as there is room for, each warp with a trip or two left
-    for (int cl = 8; cl > 1; cl /= 2)
-        if (units <= FEW_ROWS && units * cl <= (fp32 ? 3 * FEW_ROWS : FEW_ROWS) && trips >= (fp32 ? 3 : 2) * 16 * cl) return {512, 4, cl};
-    if (fp32) {
-        if (row_bytes <= 32 * 1024) return {256, 4, 1};
-        if (row_bytes < 250 * 1024) return {256, 6, 1};
-        return units <= 500 ? StagedShape{512, 6, 2} : StagedShape{1024, 6, 1};
+    switch (row_warps(dtype, bytes)) {
+    case 4: return {128, 4, 1};
+    case 8: return {256, 4, 1};
+    case 16:
+        if (units * 4 <= n_sm || (units <= n_sm && bytes < 140 * 1000)) return {128, 6, 4};
+        if (fp32 || units <= (bytes < 100 * 1000 ? 3 : 7) * n_sm) return {256, 6, 2};
+        return bytes < 180 * 1000 ? StagedShape{512, 4, 1} : StagedShape{512, 6, 1};
+    default:
+        if (units > 20 * n_sm) return {1024, 6, 1};
+        return bytes >= 400 * 1000 || units <= n_sm ? StagedShape{128, 6, 8} : StagedShape{256, 6, 4};
     }
-    if (units <= FEW_ROWS) return {512, 4, 1};
-    if (row_bytes <= 32 * 1024) return {128, 4, 1};
-    if (row_bytes < 100 * 1000) return {256, 4, 1};
-    if (units <= 1000) return aligned ? StagedShape{256, 6, 2} : StagedShape{512, 4, row_bytes >= 200 * 1000 ? 2 : 1};
-    if (row_bytes < 160 * 1000) return aligned ? StagedShape{256, 6, 1} : StagedShape{512, 4, 1};
-    return {512, 6, 1};
 }
 
 // The shape of a launch: what the configuration pinned, else by the size of the launch.
-static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units, bool aligned)
+static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units)
 {
     RowGeometry g = geo;
     if (g.kernel == METASD_ROWS_STAGED && g.threads == 0) {
-        const StagedShape s = staged_shape(dtype, (long long)vocab * (dtype == METASD_BF16 ? 2 : 4), units, aligned);
+        const StagedShape s = staged_shape(dtype, row_bytes(dtype, vocab), units, geo.n_sm);
         g.threads = s.threads;
         g.stages = s.stages;
         g.cluster = s.cluster;
     }
-    g.n_seg = g.kernel == METASD_ROWS_STAGED ? g.threads / 32 * g.cluster : 1;
     return g;
 }
 
-// Parts of rows that launches of up to `units` rows report on, at most.
-size_t segment_capacity(const RowGeometry &geo, size_t units)
+int row_parts(const RowGeometry &geo, int dtype, int vocab)
 {
-    if (geo.kernel != METASD_ROWS_STAGED) return units;
-    if (geo.threads) return units * (size_t)(geo.threads / 32 * geo.cluster);
-    const size_t few = (units < FEW_ROWS ? units : FEW_ROWS) * MAX_SEGMENTS, many = units * 32;
-    return few > many ? few : many;
+    if (geo.kernel != METASD_ROWS_STAGED) return 1;
+    return geo.threads ? geo.threads / 32 * geo.cluster : row_warps(dtype, row_bytes(dtype, vocab));
 }
 
 __global__ void select_kernel(const int32_t *arm, int batch, int32_t *arm_out);
@@ -1263,23 +1269,25 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
     }
     if ((e = dtype == METASD_BF16 ? prepare_small_kernels<__nv_bfloat16>() : prepare_small_kernels<float>()) != cudaSuccess) return e;
-    return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster)
-                                : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster);
+    const int warps = cfg.vocab > 0 ? row_warps(dtype, row_bytes(dtype, cfg.vocab)) : 0;
+    const bool aligned = row_bytes(dtype, cfg.vocab) % 16 == 0;
+    return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, warps, aligned)
+                                : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, warps, aligned);
 }
 
 template <typename LT>
 static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context_geo, cudaStream_t stream, uint64_t *launches)
 {
     cudaError_t e = cudaSuccess;
-    const RowGeometry geo = resolve_geometry(context_geo, sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32, p.V, (long long)p.batch * (p.k + 1),
-                                             p.vector_ok != 0);
-    p.n_seg = geo.n_seg;
+    constexpr int dtype = sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32;
+    const RowGeometry geo = resolve_geometry(context_geo, dtype, p.V, (long long)p.batch * (p.k + 1));
+    p.n_seg = row_parts(geo, dtype, p.V);
     if (geo.kernel == METASD_ROWS_STAGED) {
         e = launch_staged_t<LT>(p, geo, stream);
     } else if (!p.vector_ok) {
         row_stats_kernel<LT, false><<<dim3(p.k + 1, p.batch), K1_THREADS, 0, stream>>>(p);
     } else if (geo.kernel == METASD_ROWS_BULK) {
-        e = launch_row_stats_bulk(p, sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32, geo, stream);
+        e = launch_row_stats_bulk(p, dtype, geo, stream);
     } else {
         row_stats_kernel<LT, true><<<dim3(p.k + 1, p.batch), K1_THREADS, 0, stream>>>(p);
     }
