@@ -16,6 +16,8 @@
  *   - Logit tensors are dense, row-major, innermost dimension V (the vocabulary), aligned to their
  *     element size.  Rows may start anywhere: where they start off a 16-byte boundary (an odd
  *     vocabulary) the row-statistics kernel realigns them on chip.
+ *   - A sequence's results depend on its own rows, tokens, state and id (sequence_base + b) alone: with the default row
+ *     kernel they are the same, bit for bit, in a batch of any size, at any place in it and in any shard of it.
  *   - The caller owns every input and output buffer.  The library owns the context, the bandit
  *     state and its scratch; nothing is allocated after metasd_init.
  *   - Calls are asynchronous on the CUDA stream passed as `stream` (a cudaStream_t, typed void*

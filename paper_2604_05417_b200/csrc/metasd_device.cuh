@@ -293,15 +293,9 @@ __device__ __forceinline__ const LT *draft_rows(const VerifyParams &p, int b)
     return reinterpret_cast<const LT *>(q);
 }
 
-// Where a row (pair) lies against 16-byte boundaries: the aligned vector i of the target row holds tokens VEC i - lead ..,
-// of the draft row (d, or nullptr) VEC i - lead - shift .. with 0 <= shift < VEC.
+// Logits between the 16-byte boundary at or in front of a row's start and the row.
 template <typename LT>
-__device__ __forceinline__ void row_alignment(const LT *a, const LT *d, int &lead, int &shift)
-{
-    lead = (int)((reinterpret_cast<uintptr_t>(a) & 15) / sizeof(LT));
-    shift = d ? (int)((reinterpret_cast<uintptr_t>(d) & 15) / sizeof(LT)) - lead : 0;
-    if (shift < 0) shift += Logit<LT>::VEC;
-}
+__device__ __forceinline__ int row_lead(const LT *row) { return (int)((reinterpret_cast<uintptr_t>(row) & 15) / sizeof(LT)); }
 
 // Streaming 16-byte load that does not allocate in L1.
 __device__ __forceinline__ uint4 ld_stream(const void *p)

@@ -167,12 +167,14 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // not read from memory again, and each slot is refilled with the trip D further down as soon as it has been used.  Lanes
 // behind the end of the row hold -Inf in their slot, which adds nothing to any sum: the loops carry no lane predicate.
 //
-// SHIFTED: rows that start off a 16-byte boundary (an odd vocabulary), each row at its own offset.  Copies are of the
-// aligned 16-byte vectors that the row overlaps, of which those that reach over an end of the row have the tokens outside
-// replaced by -Inf once they have landed (nothing outside the row's tensor is read).  A lane's vectors of the two rows then hold tokens `shift` apart.  The first sweep does not
-// care (its sums are over one row each); the second takes the draft row's tokens from the lane's vector and the next one
-// (a 33rd vector per trip is copied for the last lane).  These copies carry no L2 policy: with one, some builds of this
-// form ended in an illegal instruction at the first such copy.  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96,
+// SHIFTED: rows that start off a 16-byte boundary (an odd vocabulary), each row at its own offset.  fp32 rows are copied in
+// words, to where an aligned row has them; of bf16 rows the aligned 16-byte vectors that the row overlaps (a 33rd per trip for
+// the last lane), and a lane takes its tokens from its vector and the next one.  Lane, trip and order of a token are those of
+// an aligned row: results do not depend on where a row starts, which for an odd vocabulary is a matter of its place in the
+// batch.  Copies that reach over the end of the row have the tokens outside replaced by -Inf once they have landed (nothing
+// outside the row's tensor is read).  bf16 rows in words too: V = 50257, B = 96 69 us a round instead of 63, fp32 rows in
+// vectors: V = 32001, B = 8 17.1 instead of 14.4.  These copies carry no L2 policy: with one, some builds of this form ended in
+// an illegal instruction at the first such copy.  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96,
 // k = 5 115.5 -> 81.5 us a round, V = 128257, B = 256 590 -> 270, V = 32001, fp32, B = 256 226 -> 126.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t policy)
 {
@@ -182,6 +184,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64
 __device__ __forceinline__ void cp_async16_part(uint32_t dst, const void *src, int bytes)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4_part(uint32_t dst, const void *src, int bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 {
@@ -252,7 +262,7 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
 // CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
 // of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
 // order, so all hold the same normalisers; each sweeps its part again.
-template <int D, int THREADS, bool SHIFTED> constexpr uint32_t STAGED_SMEM = D * (THREADS * 32u + (SHIFTED ? THREADS / 32 * 16u : 0u));
+template <int D, int THREADS, bool SHIFTED> constexpr uint32_t STAGED_SMEM = D * (THREADS * 32u + (SHIFTED ? THREADS / 32 * 32u : 0u));
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
@@ -262,9 +272,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     constexpr int VEC = Logit<LT>::VEC;
     constexpr int NWARP = THREADS / 32, NREC = NWARP * CL;
     constexpr uint32_t STAGE_STRIDE = STAGED_SMEM<D, THREADS, SHIFTED> / D;
-    constexpr uint32_t ROW_STRIDE = SHIFTED ? 512u : THREADS * 16u;
+    constexpr uint32_t ROW_STRIDE = SHIFTED ? 33u * 16u : THREADS * 16u;
     constexpr uint32_t FULL = 0xFFFFFFFFu;
-    // 16-byte slots: [D][2 rows][THREADS]; SHIFTED: [D][NWARP][32 of the target row, 33 of the draft row]
+    // 16-byte slots: [D][2 rows][THREADS]; SHIFTED: [D][NWARP][2 rows][33]
     extern __shared__ __align__(16) unsigned char stage_mem[];
     __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
@@ -294,52 +304,79 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
 
     const LT *a_row = reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V;
     const LT *d_row = pair ? draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V : a_row;
-    int lead = 0, shift = 0;
-    if (SHIFTED) row_alignment(a_row, pair ? d_row : nullptr, lead, shift);
-    const int nvec = SHIFTED ? (p.V + lead + shift + VEC - 1) / VEC : p.V / VEC;
+    const int nvec = (p.V + VEC - 1) / VEC;
     const int trips_row = (nvec + 31) >> 5;
     const int part = rank * NWARP + warp;                         // this warp's part of the row's trips
     const int g0 = segment_begin(trips_row, part, NREC), n_trip = segment_begin(trips_row, part + 1, NREC) - g0;
     const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
-    const uint4 *a4 = reinterpret_cast<const uint4 *>(a_row - lead) + v0;
-    const uint4 *d4 = reinterpret_cast<const uint4 *>(d_row - lead - shift) + v0;
-    // this thread's slot of stage 0 for the target row; the draft row's lies ROW_STRIDE behind it
-    const uint32_t slot0 = smem_addr(stage_mem) + (SHIFTED ? (uint32_t)warp * (65u * 16u) + (uint32_t)lane * 16u : (uint32_t)tid * 16u);
-    // Trips in which this lane is inside the row, and in which every lane (SHIFTED: with whole vectors, the 33rd included)
-    // is: only the row's last trip (SHIFTED: its last two, and its first) may be ragged.
+    // Copies are of UNIT bytes; a lane makes those of the units lane, lane + 32, .. of a trip.  SHIFTED: a row's units start
+    // `lead` tokens in front of it (EXTRA: where they may, a trip needs one more).
+    constexpr int UNIT = SHIFTED && sizeof(LT) == 4 ? 4 : 16, COPIES = 16 / UNIT, PER_UNIT = UNIT / (int)sizeof(LT);
+    constexpr bool EXTRA = SHIFTED && PER_UNIT > 1;
+    const int lead_a = EXTRA ? row_lead(a_row) : 0, lead_d = EXTRA ? row_lead(d_row) : 0;
+    const char *a4 = reinterpret_cast<const char *>(a_row - lead_a) + g0 * 512 + lane * UNIT;
+    const char *d4 = reinterpret_cast<const char *>(d_row - lead_d) + g0 * 512 + lane * UNIT;
+    // this thread's slot of stage 0 for the target row, and from there what it copies to; the draft row's lies ROW_STRIDE behind it
+    const uint32_t slot0 = smem_addr(stage_mem) + (SHIFTED ? (uint32_t)warp * (66u * 16u) + (uint32_t)lane * 16u : (uint32_t)tid * 16u);
+    const uint32_t put = 0u - (uint32_t)lane * (16u - UNIT);
+    // Trips in which this lane is inside the row, and in which every lane (SHIFTED: with whole units, the extra one included)
+    // is: only the row's last trip (SHIFTED: its last two) may be ragged.
     const int lane_trips = v0 + 32 * (n_trip - 1) < nvec ? n_trip : n_trip - 1;
-    const int n_full = SHIFTED ? min(n_trip, ((p.V + lead) / VEC - 1) / 32 - g0) : (g0 + n_trip) * 32 <= nvec ? n_trip : n_trip - 1;
-    // SHIFTED, a trip that may reach over an end of the row: the part of a vector in front of the row's end.  What it takes
+    const int n_full = SHIFTED ? min(n_trip, (p.V / VEC - (EXTRA ? 1 : 0)) / 32 - g0) : (g0 + n_trip) * 32 <= nvec ? n_trip : n_trip - 1;
+    auto copy_unit = [&](uint32_t dst, const char *src) {
+        if (UNIT == 4) cp_async4(dst, src);
+        else cp_async16(dst, src);
+    };
+    // SHIFTED, a trip that may reach over an end of the row: the part of a unit in front of the row's end.  What it takes
     // from in front of the row's start belongs to the tensor's row before, where there is one (`room`).
-    auto copy_part = [&](uint32_t dst, const uint4 *src, const LT *row, int tok0, bool room) {
-        int bytes = min(max((p.V - tok0) * (int)sizeof(LT), 0), 16);
-        if (tok0 + VEC <= 0) bytes = 0;
-        if (tok0 < 0 && bytes > 0 && !room) {
+    auto copy_part = [&](uint32_t dst, const char *src, const LT *row, int tok0, bool room) {
+        const int bytes = min(max((p.V - tok0) * (int)sizeof(LT), 0), UNIT);
+        if (tok0 < 0 && !room) {
 #pragma unroll 1
-            for (int e = -tok0; e < VEC && tok0 + e < p.V; ++e) Logit<LT>::put_scalar(dst + e * (uint32_t)sizeof(LT), row, tok0 + e);
+            for (int e = -tok0; e < PER_UNIT && tok0 + e < p.V; ++e) Logit<LT>::put_scalar(dst + e * (uint32_t)sizeof(LT), row, tok0 + e);
+        } else if (UNIT == 4) {
+            cp_async4_part(dst, src, bytes);
         } else {
             cp_async16_part(dst, src, bytes);
         }
     };
     const bool a_room = ((size_t)b * (p.k + 1) + j) * p.V >= 16, d_room = ((size_t)b * p.k + j) * p.V >= 16;
     auto copy_ragged = [&](int m, uint32_t dst, bool both) {
-        const int tok0 = (v0 + 32 * m) * VEC - lead;
-        copy_part(dst, a4 + 32 * m, a_row, tok0, a_room);
-        if (both) {
-            copy_part(dst + ROW_STRIDE, d4 + 32 * m, d_row, tok0 - shift, d_room);
-            if (lane == 0) copy_part(dst + ROW_STRIDE + 512u, d4 + 32 * m + 32, d_row, tok0 - shift + 32 * VEC, true);
+#pragma unroll 1
+        for (int q = 0; q < (EXTRA && lane == 0 ? COPIES + 1 : COPIES); ++q) {
+            const int tok0 = ((g0 + m) * (512 / UNIT) + lane + 32 * q) * PER_UNIT;
+            copy_part(dst + q * (32u * UNIT), a4 + m * 512 + q * (32 * UNIT), a_row, tok0 - lead_a, a_room);
+            if (both) copy_part(dst + ROW_STRIDE + q * (32u * UNIT), d4 + m * 512 + q * (32 * UNIT), d_row, tok0 - lead_d, d_room);
         }
         __syncwarp();
     };
-    // and, when it has landed, -Inf for the tokens outside the row
+    auto copy_whole = [&](uint32_t dst, const char *a, const char *d, bool both) {
+#pragma unroll
+        for (int q = 0; q < COPIES; ++q) {
+            copy_unit(dst + q * (32u * UNIT), a + q * (32 * UNIT));
+            if (both) copy_unit(dst + ROW_STRIDE + q * (32u * UNIT), d + q * (32 * UNIT));
+        }
+        if (EXTRA && lane == 0) {
+            copy_unit(dst + 512u, a + 512);
+            if (both) copy_unit(dst + ROW_STRIDE + 512u, d + 512);
+        }
+    };
+    // and, when it has landed, -Inf for the tokens behind the row
     auto mask_ragged = [&](int m, uint32_t src, bool both) {
-        const int tok0 = (v0 + 32 * m) * VEC - lead;
-        sts16(src, Logit<LT>::masked(lds16(src), tok0, p.V));
-        if (both) {
-            sts16(src + ROW_STRIDE, Logit<LT>::masked(lds16(src + ROW_STRIDE), tok0 - shift, p.V));
-            if (lane == 0) sts16(src + ROW_STRIDE + 512u, Logit<LT>::masked(lds16(src + ROW_STRIDE + 512u), tok0 - shift + 32 * VEC, p.V));
+        const int tok0 = (v0 + 32 * m) * VEC;
+        auto mask = [&](uint32_t at, int tok) { sts16(at, Logit<LT>::masked(lds16(at), tok, p.V)); };
+        mask(src, tok0 - lead_a);
+        if (both) mask(src + ROW_STRIDE, tok0 - lead_d);
+        if (EXTRA && lane == 0) {
+            mask(src + 512u, tok0 - lead_a + 32 * VEC);
+            if (both) mask(src + ROW_STRIDE + 512u, tok0 - lead_d + 32 * VEC);
         }
         __syncwarp();
+    };
+    // This lane's tokens of a trip, from its slot (EXTRA: and the next one, behind a __syncwarp()).
+    auto fetch = [&](uint32_t src, int lead) {
+        const uint4 v = lds16(src);
+        return EXTRA ? Logit<LT>::shifted(v, lds16(src + 16u), lead) : v;
     };
 
     // ---- sweep 1: sums of both rows and the arg-max of the target row.  The draft row's sum is taken relative to
@@ -364,11 +401,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     auto sweep1 = [&](auto both_tag) {
         constexpr bool BOTH = decltype(both_tag)::value;
         // One group of copies per trip, empty past the end: the group count stays in step with the trips.
-        auto request = [&](uint32_t dst, const uint4 *a, const uint4 *d, uint64_t pol) {
+        auto request = [&](uint32_t dst, const char *a, const char *d, uint64_t pol) {
             if (SHIFTED) {
-                cp_async16(dst, a);
-                if (BOTH) cp_async16(dst + ROW_STRIDE, d);
-                if (BOTH && lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32);
+                copy_whole(dst, a, d, BOTH);
             } else {
                 cp_async16(dst, a, pol);
                 if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
@@ -377,14 +412,14 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         };
         auto request_checked = [&](int m, uint32_t dst) {
             if (SHIFTED) {
-                if (m < n_full && m + g0 > 0) {   // whole vectors: most of a short range is asked for here
-                    request(dst, a4 + 32 * m, d4 + 32 * m, drop);
+                if (m < n_full && m + g0 > 0) {   // whole units: most of a short range is asked for here
+                    request(dst + put, a4 + 512 * m, d4 + 512 * m, drop);
                     return;
                 }
-                if (m < n_trip) copy_ragged(m, dst, BOTH);
+                if (m < n_trip) copy_ragged(m, dst + put, BOTH);
                 cp_async_commit();
             } else if (m < lane_trips) {
-                request(dst, a4 + 32 * m, d4 + 32 * m, m >= m_keep ? keep : drop);
+                request(dst, a4 + 512 * m, d4 + 512 * m, m >= m_keep ? keep : drop);
             } else {
                 if (m < n_trip) {
                     fill_neg_inf<LT>(dst);
@@ -393,12 +428,23 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
                 cp_async_commit();
             }
         };
+        // Trip n, whose vectors have landed.
         auto consume = [&](int n, uint32_t src) {
-            cp_async_wait<D - 1>();   // all but the D - 1 youngest groups have landed: trip n's is among them
-            const uint4 ra = lds16(src);
+            const uint4 ra = fetch(src, lead_a);
             if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT>(w, ra, v0 + 32 * n, c);
             w.a = Logit<LT>::add_exp(w.a, ra, c2, w.nm);
-            if (BOTH) w.b = Logit<LT>::add_exp(w.b, lds16(src + ROW_STRIDE), c2, w.nm);
+            if (BOTH) w.b = Logit<LT>::add_exp(w.b, fetch(src + ROW_STRIDE, lead_d), c2, w.nm);
+        };
+        // Around the request for trip n + D - 1, in front of trip n.  Behind it all but the D - 1 youngest groups have
+        // landed, trip n's among them.  SHIFTED: a slot is read by the lane before its own too, so the wait (one group
+        // fewer is out) comes in front and the warp meets: trip n is there for every lane, and trip n - 1, whose slot the
+        // request takes, has been read by every lane.
+        auto landed = [&] { if (!SHIFTED) cp_async_wait<D - 1>(); };
+        auto meet = [&] {
+            if (SHIFTED) {
+                cp_async_wait<D - 2>();
+                __syncwarp();
+            }
         };
 #pragma unroll
         for (int m = 0; m < D - 1; ++m) request_checked(m, slot0 + (uint32_t)m * STAGE_STRIDE);
@@ -406,10 +452,13 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         // draft row's (or 0) stands in, so that the draft row's sum does not overflow.
         if (n_trip > 0) {
             cp_async_wait<D - 2>();
-            if (SHIFTED) mask_ragged(0, slot0, BOTH);
-            float top = warp_max_f(Logit<LT>::max_of(lds16(slot0)));
+            if (SHIFTED) {
+                __syncwarp();
+                if (n_full <= 0) mask_ragged(0, slot0, BOTH);
+            }
+            float top = warp_max_f(Logit<LT>::max_of(fetch(slot0, lead_a)));
             if (!(top > METASD_NEG_BIG)) {
-                top = BOTH ? warp_max_f(Logit<LT>::max_of(lds16(slot0 + ROW_STRIDE))) : 0.f;
+                top = BOTH ? warp_max_f(Logit<LT>::max_of(fetch(slot0 + ROW_STRIDE, lead_d))) : 0.f;
                 if (!(top > METASD_NEG_BIG)) top = 0.f;
             }
             w.ref = -rintf(top * c);
@@ -419,25 +468,27 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         // requests all lie inside the row carry no checks, and their slots and their L2 policy are constants (the boundary
         // of the kept share is rounded down to a whole group: a few vectors more are kept).
         int n = 0;
-        const uint4 *a_next = a4 + 32 * (D - 1), *d_next = d4 + 32 * (D - 1);
+        const char *a_next = a4 + 512 * (D - 1), *d_next = d4 + 512 * (D - 1);
         auto group = [&](uint64_t pol) {
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                request(slot0 + (uint32_t)((u + D - 1) % D) * STAGE_STRIDE, a_next + 32 * u, d_next + 32 * u, pol);
+                meet();
+                request(slot0 + put + (uint32_t)((u + D - 1) % D) * STAGE_STRIDE, a_next + 512 * u, d_next + 512 * u, pol);
+                landed();
                 consume(n + u, slot0 + (uint32_t)u * STAGE_STRIDE);
             }
             n += D;
-            a_next += 32 * D;
-            d_next += 32 * D;
+            a_next += 512 * D;
+            d_next += 512 * D;
         };
-        while (n + 2 * D - 2 < min(m_keep, n_full)) group(drop);
+        if (!SHIFTED)
+            while (n + 2 * D - 2 < min(m_keep, n_full)) group(drop);
         while (n + 2 * D - 2 < n_full) group(keep);
         for (int slot = 0, ask = D - 1; n < n_trip; ++n) {
+            meet();
             request_checked(n + D - 1, slot0 + (uint32_t)ask * STAGE_STRIDE);
-            if (SHIFTED && n >= n_full) {
-                cp_async_wait<D - 1>();
-                mask_ragged(n, slot0 + (uint32_t)slot * STAGE_STRIDE, BOTH);
-            }
+            landed();
+            if (SHIFTED && n >= n_full && n > 0) mask_ragged(n, slot0 + (uint32_t)slot * STAGE_STRIDE, BOTH);
             consume(n, slot0 + (uint32_t)slot * STAGE_STRIDE);
             ask = slot;
             slot = slot + 1 == D ? 0 : slot + 1;
@@ -455,11 +506,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane);
             st_cluster(dst, __float_as_int(w.ref));          st_cluster(dst + 4, __float_as_int(sum_aw));
             st_cluster(dst + 8, __float_as_int(sum_bw));    st_cluster(dst + 12, __float_as_int(w.best));
-            st_cluster(dst + 16, w.best_i - lead);
+            st_cluster(dst + 16, w.best_i);
         }
         cluster_sync_all();
     } else {
-        if (lane == 0) sh_rec[warp] = WarpRecord{w.ref, sum_aw, sum_bw, w.best, w.best_i - lead};
+        if (lane == 0) sh_rec[warp] = WarpRecord{w.ref, sum_aw, sum_bw, w.best, w.best_i};
         __syncthreads();
     }
     float ref_a = INFINITY, sum_a = 0.f, sum_b = 0.f;   // both sums end up relative to the target row's largest logit
@@ -495,15 +546,19 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // logits far from the target's, or a row that is not finite) the draft row is swept again relative to its own
     // running maximum.
     if (pair && !(sum_b >= 0x1p-60f && sum_b < 0x1p100f)) {
+        const int lead = SHIFTED ? row_lead(d_row) : 0;
+        const uint4 *d16 = reinterpret_cast<const uint4 *>(d_row - lead) + v0;
         MaxSum own = {METASD_NEG_BIG, 0.f};   // m: the running maximum's exponent, a whole number here too
         for (int n = 0; n < lane_trips; ++n) {
             float xb[VEC];
-            const int tok0 = (v0 + 32 * n) * VEC - lead - shift;
-            if (!SHIFTED || (tok0 >= 0 && tok0 + VEC <= p.V)) {
-                Logit<LT>::unpack(ld_stream(d4 + 32 * n), xb);
+            const int tok0 = (v0 + 32 * n) * VEC;
+            if (!SHIFTED) {
+                Logit<LT>::unpack(ld_stream(d16 + 32 * n), xb);
+            } else if (tok0 >= lead && tok0 - lead + 2 * VEC <= p.V) {
+                Logit<LT>::unpack(Logit<LT>::shifted(ld_stream(d16 + 32 * n), ld_stream(d16 + 32 * n + 1), lead), xb);
             } else {
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) xb[e] = tok0 + e >= 0 && tok0 + e < p.V ? Logit<LT>::scalar(d_row, tok0 + e) : -INFINITY;
+                for (int e = 0; e < VEC; ++e) xb[e] = tok0 + e < p.V ? Logit<LT>::scalar(d_row, tok0 + e) : -INFINITY;
             }
             float bm = xb[0];
 #pragma unroll
@@ -565,29 +620,19 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(log2f(rho * exp2i(-whole)));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
-        // every lane: the ragged trips are the row's last; SHIFTED: and its first).
-        auto consume = [&](int m, uint32_t src) {
+        // every lane: the ragged trips are the row's last).
+        auto consume = [&](uint32_t src) {
             // the first D trips are still in their slots from sweep 1; the group of a later one was committed D trips
             // ago, so at most D - 1 younger groups may still be pending
             cp_async_wait<D - 1>();
-            if (SHIFTED) {
-                if (m == 0) mask_ragged(0, src, true);
-                __syncwarp();   // the next lane's vector has landed too
-            }
-            uint4 d = lds16(src + ROW_STRIDE);
-            if (SHIFTED) d = Logit<LT>::shifted(d, lds16(src + ROW_STRIDE + 16u), shift);
-            acc = Logit<LT>::add_exp_min(acc, lds16(src), d, c2, nma, nmb, lg);
+            if (SHIFTED) __syncwarp();   // the next lane's vector has landed too
+            acc = Logit<LT>::add_exp_min(acc, fetch(src, lead_a), fetch(src + ROW_STRIDE, lead_d), c2, nma, nmb, lg);
             if (SHIFTED) __syncwarp();   // and has been read before its lane refills the slot
         };
-        auto refill = [&](uint32_t dst, int m, const uint4 *a, const uint4 *d) {
-            if (SHIFTED && m == 0) {
-                copy_ragged(0, dst, true);
-                return;
-            }
+        auto refill = [&](uint32_t dst, int m, const char *a, const char *d) {
             if (SHIFTED) {
-                cp_async16(dst, a);
-                cp_async16(dst + ROW_STRIDE, d);
-                if (lane == 0) cp_async16(dst + ROW_STRIDE + 512u, d + 32);
+                if (m + g0 == 0) copy_ragged(0, dst + put, true);
+                else copy_whole(dst + put, a, d, true);
             } else {
                 cp_async16(dst, a, drop);
                 cp_async16(dst + ROW_STRIDE, d, drop);
@@ -597,27 +642,27 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         int n = n_trip - 1;
         for (int slot = n % D; n >= 0 && slot != D - 1; --n) {
             const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
-            consume(n, src);
-            if (n >= D) refill(src, n - D, a4 + 32 * (n - D), d4 + 32 * (n - D));
+            consume(src);
+            if (n >= D) refill(src, n - D, a4 + 512 * (n - D), d4 + 512 * (n - D));
             cp_async_commit();
             slot = slot == 0 ? D - 1 : slot - 1;
         }
-        const uint4 *a_next = a4 + 32 * (n - D), *d_next = d4 + 32 * (n - D);
+        const char *a_next = a4 + 512 * (n - D), *d_next = d4 + 512 * (n - D);
         for (; n >= D; n -= D) {   // n + 1 is a multiple of D and a whole group lies below: every refill is real
 #pragma unroll
             for (int u = 0; u < D; ++u) {
                 const uint32_t src = slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE;
-                consume(n - u, src);
-                refill(src, n - u - D, a_next - 32 * u, d_next - 32 * u);
+                consume(src);
+                refill(src, n - u - D, a_next - 512 * u, d_next - 512 * u);
                 cp_async_commit();
             }
-            a_next -= 32 * D;
-            d_next -= 32 * D;
+            a_next -= 512 * D;
+            d_next -= 512 * D;
         }
         if (n >= 0) {
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                consume(n - u, slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
+                consume(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
                 cp_async_commit();
             }
         }
@@ -1065,11 +1110,9 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
     // walked), but moving batches of V = 32000 take 26.4 us instead of 23.9, and odd vocabularies 64 instead of 52.
     const double guard = hit.total < 0.0625 ? (double)(1.0e-7f * __fsqrt_rn(__fdividef(1.f, rs.sum_a) + 0.01f)) : -1.0;
     if (!whole) {
-        int lead = 0, shift = 0;
-        if (!VECTOR) row_alignment(row.a, residual ? row.d : nullptr, lead, shift);
-        const int trip = 32 * Logit<LT>::VEC, trips = (V + lead + shift + trip - 1) / trip;
-        lo = max(trip * segment_begin(trips, hit.part, p.n_seg) - lead, 0);
-        hi = min(trip * segment_begin(trips, min(hit.part + per_lane, p.n_seg), p.n_seg) - lead, V);
+        const int trip = 32 * Logit<LT>::VEC, trips = (V + trip - 1) / trip;
+        lo = trip * segment_begin(trips, hit.part, p.n_seg);
+        hi = min(trip * segment_begin(trips, min(hit.part + per_lane, p.n_seg), p.n_seg), V);
         base = hit.base;
         threshold = hit.threshold;
     }

@@ -1,5 +1,6 @@
 """A sequence's results do not depend on what else is in its batch: one large launch against launches of a few of its
-sequences, which take other shapes of the row-statistics kernel, bit for bit in every output."""
+sequences, which take other shapes of the row-statistics kernel, bit for bit in every output.  Of an odd vocabulary a
+sequence's rows also start at other offsets from a 16-byte boundary in another batch."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +11,8 @@ from paper_2604_05417_b200.workloads import RoundGenerator, Workload
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,V", [("bf16", 4096), ("bf16", 32000), ("bf16", 50264), ("bf16", 80008), ("bf16", 131072),
+@pytest.mark.parametrize("dtype,V", [("bf16", 4096), ("bf16", 4101), ("bf16", 20001), ("bf16", 32000), ("bf16", 50257), ("bf16", 50264),
+                                     ("bf16", 80008), ("bf16", 100003), ("bf16", 131072), ("fp32", 4099), ("fp32", 32001), ("fp32", 64009),
                                      ("fp32", 4096), ("fp32", 32000), ("fp32", 64008), ("fp32", 110000)])
 def test_results_do_not_depend_on_the_batch(dtype, V):
     """1200 row pairs and bonus rows in one launch; 3, 36, 141, 420 and 600 of them in launches of their own."""
