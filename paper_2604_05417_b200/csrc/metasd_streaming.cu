@@ -704,8 +704,8 @@ static cudaError_t launch_kernel(void (*kernel)(Params...), unsigned grid, unsig
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Dynamic shared memory that one CTA alone on its SM asks for: leaves room for an epilogue CTA beside it.
-constexpr unsigned STAGED_SMEM_MAX = 216 * 1024;
+// Shared memory of an SM, of which every block takes 1 KB besides its own, and the most that a launch below asks for.
+constexpr unsigned SM_SMEM = 228 * 1024, STAGED_SMEM_MAX = 216 * 1024;
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm, cudaStream_t stream)
@@ -713,7 +713,8 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm
     // A launch of up to one wave wants its blocks spread evenly over the SMs: set up while the last epilogue still holds some of
     // them, they would crowd on the others and stay there.  So such a launch is chained only where the last layer of blocks
     // is nearly full (or, of clusters, which are placed within groups of SMs, where every one finds free SMs), and asks for
-    // so much shared memory that an SM takes no more blocks than an even spread puts there.  Us a round, chained so / not:
+    // the shared memory that keeps one block more than an even spread off an SM, and no more: what is left there, half an SM's
+    // where there is one block, is for the kernels of other streams.  Us a round, chained so / not:
     // 384 blocks (B = 64, k = 5, V = 32000) 22.8 / 24.6, 240 18.5 / 20.5, 144 (V = 128256) 28.1 / 28.7, 96 14.0 / 16.1;
     // 320 blocks 22.2 / 20.5, 480 26.5 / 24.6; 32 clusters of 4 13.5 / 14.4, 36 21.8 / 19.8.  Several waves are always chained
     // (B = 192, k = 8 ragged, V = 50264 61.9 / 69.8).
@@ -721,7 +722,7 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm
     const bool one_wave = layers <= MINB;
     const bool chained = !one_wave || ctas <= sms / 2 || (CL == 1 ? spare <= sms / 2 : layers == 1 && spare >= sms / 8);
     constexpr unsigned needed = STAGED_SMEM<D, THREADS, SHIFTED>;   // the attribute that allows it, and more, was set by streaming_prepare
-    const unsigned smem = one_wave && chained ? std::max(needed, STAGED_SMEM_MAX / layers - 4096u) : needed;
+    const unsigned smem = one_wave && chained ? std::max(needed, (SM_SMEM / (layers + 1) + 1023u) / 1024u * 1024u) : needed;
     return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, ctas, THREADS, smem, CL, chained, stream, p);
 }
 
