@@ -128,9 +128,14 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # not a public name: a torch without it has the slower way
+
+
 def _stream(device: torch.device) -> int:
     """The current stream of the device, as the address of its cudaStream_t."""
-    return torch._C._cuda_getCurrentRawStream(device.index)
+    if _raw_stream is None or device.index is None:
+        return torch.cuda.current_stream(device).cuda_stream
+    return _raw_stream(device.index)
 
 
 @dataclass

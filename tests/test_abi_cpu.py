@@ -127,3 +127,19 @@ def test_product_code_never_touches_the_oracle():
                 assert "oracle" not in text.lower() or f == "workloads.py", f
     text = open(os.path.join(pkg, "workloads.py")).read()
     assert "import oracle" not in text and "from oracle" not in text
+
+
+def test_current_stream_without_torchs_private_lookup(monkeypatch):
+    """The raw-stream lookup is a private name of torch: without it, and for a device without an index (host tensors, which
+    torch refuses by name), the public call answers."""
+    class Stream:
+        cuda_stream = 4711
+
+    asked = []
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: asked.append(device) or Stream())
+    assert M._stream(torch.device("cpu")) == 4711
+    monkeypatch.setattr(M, "_raw_stream", None)
+    assert M._stream(torch.device("cuda", 3)) == 4711
+    assert asked == [torch.device("cpu"), torch.device("cuda", 3)]
+    monkeypatch.setattr(M, "_raw_stream", lambda index: 100 + index)
+    assert M._stream(torch.device("cuda", 3)) == 103
