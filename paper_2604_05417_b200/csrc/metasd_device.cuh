@@ -156,6 +156,14 @@ template <> struct Logit<__nv_bfloat16> {
         for (int i = 0; i < 4; ++i) w[i] = __byte_perm(w[i], w[i + 1], sel);
         return make_uint4(w[0], w[1], w[2], w[3]);
     }
+    // The eight logits that start `shift` (0 .. 3) logits into w.
+    __device__ static __forceinline__ uint4 shifted(uint32_t (&w)[6], int shift)
+    {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = shift & 2 ? w[i + 1] : w[i];
+        const uint32_t sel = shift & 1 ? 0x5432u : 0x3210u;
+        return make_uint4(__byte_perm(w[0], w[1], sel), __byte_perm(w[1], w[2], sel), __byte_perm(w[2], w[3], sel), __byte_perm(w[3], w[4], sel));
+    }
     // the two logits of a 32-bit word
     __device__ static __forceinline__ uint64_t pair_of(uint32_t w)
     {
@@ -242,6 +250,7 @@ template <> struct Logit<float> {
         for (int i = 0; i < 4; ++i) w[i] = shift & 1 ? w[i + 1] : w[i];
         return make_uint4(w[0], w[1], w[2], w[3]);
     }
+    __device__ static __forceinline__ uint4 shifted(uint32_t (&w)[6], int) { return make_uint4(w[0], w[1], w[2], w[3]); }   // not used
     using Best = float;
     __device__ static __forceinline__ Best best_of(float x) { return x; }
     __device__ static __forceinline__ float max_of(const uint4 &raw)
@@ -506,6 +515,11 @@ __device__ __forceinline__ uint4 lds16(uint32_t addr)
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void lds8(uint32_t addr, uint32_t &lo, uint32_t &hi)
+{
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(addr) : "memory");
 }
 
 __device__ __forceinline__ void sts16(uint32_t addr, const uint4 &v)

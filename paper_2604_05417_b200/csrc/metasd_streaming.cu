@@ -374,9 +374,15 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         __syncwarp();
     };
     // This lane's tokens of a trip, from its slot (EXTRA: and the next one, behind a __syncwarp()).
+    // EXTRA: three loads of 8 bytes, which halves of 8 bytes the tokens start in taken by the address: a third fewer selections
+    // than from two whole vectors (@@T@@).
     auto fetch = [&](uint32_t src, int lead) {
-        const uint4 v = lds16(src);
-        return EXTRA ? Logit<LT>::shifted(v, lds16(src + 16u), lead) : v;
+        if (!EXTRA) return lds16(src);
+        uint32_t w[6];
+        const uint32_t at = src + (uint32_t)(lead & 4) * 2u;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) lds8(at + 8u * i, w[2 * i], w[2 * i + 1]);
+        return Logit<LT>::shifted(w, lead & 3);
     };
 
     // ---- sweep 1: sums of both rows and the arg-max of the target row.  The draft row's sum is taken relative to
