@@ -25,6 +25,9 @@
  *     metasd_select, metasd_verify and metasd_reset only launch kernels: they may be captured into
  *     a CUDA graph.  A replay is the context's next round on whatever the captured buffers then
  *     hold (the round counter that keys the random numbers is device state, not a launch argument).
+ *   - The library's kernels are set up while the kernel in front of them in the stream drains and wait for it before they read
+ *     anything.  A kernel of the caller's that is itself launched with programmatic stream serialisation must wait for the
+ *     one in front of it before it ends: its end is then the end of all before it.
  *   - A context belongs to the device named in its configuration.  Every call that takes a context
  *     makes that device current for its own duration and restores the caller's current device before
  *     it returns; `stream` must be a stream of the context's device (or NULL).

@@ -253,7 +253,7 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
 // What bounds it (bf16, B = 512, k = 8, V = 152064; 2.65 GB): the special-function unit (three exponentials a pair, 80 %
 // busy) and, in a long run, the board's power limit, so instructions and re-read bytes both cost time.  Against one vector
 // per thread and trip strided over the CTA: the warp-wide reference and the packed fp32 pairs take the maximum search, the
-// lane predicates and half the arithmetic instructions out of the loop (109.5 M warp instructions instead of 141.8 M on
+// lane predicates and half the arithmetic instructions out of the loop (114.9 M warp instructions instead of 141.8 M on
 // B = 148), contiguous ranges make a range's pages and its second sweep its own, and six stages at two CTAs per SM keep a
 // third more of a pair on chip between the sweeps than four stages at three CTAs (3.17 GB read instead of 3.39 GB).  A
 // round of that size takes 630 us instead of 664 in a long run on one box; fp32, B = 1024, k = 5, V = 128256 1164 instead of
@@ -720,7 +720,8 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm
     // them, they would crowd on the others and stay there.  So such a launch is chained only where the last layer of blocks
     // is nearly full (or, of clusters, which are placed within groups of SMs, where every one finds free SMs), and asks for
     // the shared memory that keeps one block more than an even spread off an SM, and no more: what is left there, half an SM's
-    // where there is one block, is for the kernels of other streams.  Us a round, chained so / not:
+    // where there is one block, is for the kernels of other streams.  Us a round, chained so / not, in blocks
+    // of 256 and 512 threads:
     // 384 blocks (B = 64, k = 5, V = 32000) 22.8 / 24.6, 240 18.5 / 20.5, 144 (V = 128256) 28.1 / 28.7, 96 14.0 / 16.1;
     // 320 blocks 22.2 / 20.5, 480 26.5 / 24.6; 32 clusters of 4 13.5 / 14.4, 36 21.8 / 19.8.  Several waves are always chained
     // (B = 192, k = 8 ragged, V = 50264 61.9 / 69.8).
