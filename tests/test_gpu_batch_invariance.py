@@ -11,12 +11,14 @@ from paper_2604_05417_b200.workloads import RoundGenerator, Workload
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,V", [("bf16", 4096), ("bf16", 4101), ("bf16", 20001), ("bf16", 32000), ("bf16", 50257), ("bf16", 50264),
-                                     ("bf16", 80008), ("bf16", 100003), ("bf16", 131072), ("fp32", 4099), ("fp32", 32001), ("fp32", 64009),
-                                     ("fp32", 4096), ("fp32", 32000), ("fp32", 64008), ("fp32", 110000)])
-def test_results_do_not_depend_on_the_batch(dtype, V):
-    """1200 row pairs and bonus rows in one launch; 3, 36, 141, 420 and 600 of them in launches of their own."""
-    B, k, N = 400, 2, 2
+@pytest.mark.parametrize("dtype,V,B", [("bf16", 4096, 400), ("bf16", 4101, 400), ("bf16", 20001, 400), ("bf16", 32000, 400),
+                                       ("bf16", 50257, 400), ("bf16", 50264, 400), ("bf16", 80008, 400), ("bf16", 100003, 400),
+                                       ("bf16", 131072, 400), ("fp32", 4096, 400), ("fp32", 4099, 400), ("fp32", 32000, 400),
+                                       ("fp32", 32001, 400), ("fp32", 64008, 400), ("fp32", 64009, 400), ("fp32", 110000, 400),
+                                       ("fp32", 64003, 1000)])
+def test_results_do_not_depend_on_the_batch(dtype, V, B):
+    """1200 (3000) row pairs and bonus rows in one launch; 3, 36, 141, 420 and 600 of them in launches of their own."""
+    k, N = 2, 2
     wl = Workload("t", B=B, N=N, k=k, V=V, rounds=1, temperature=0.9, dtype=dtype, bandit="ucb", sigmas=(0.4, 1.5))
     rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=V % 89).table_round(0)
     drafts, tokens = rd["drafts"], rd["tokens"]
