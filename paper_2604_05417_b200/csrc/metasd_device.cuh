@@ -391,8 +391,21 @@ __device__ __forceinline__ float exp2i(float d)
     return e < -126 ? 0.f : __int_as_float((e + 127) << 23);
 }
 
-// What a warp of the staged row-statistics kernel found in its part of a row pair: the reference of both sums, the sums,
-// the largest target logit and its first index.
+// The same in fewer instructions, where there are few to spare: the sum with 1.5 2^23 has the exponent field's value in its lowest bits.
+__device__ __forceinline__ float exp2_whole(float d)
+{
+    return __int_as_float(__float_as_int(fminf(fmaxf(d, -127.f), 128.f) + 12583039.f) << 23);
+}
+
+// unit / n, given inverse_of(n) (metasd_internal.h).
+__device__ __forceinline__ int divide(int unit, int n, uint32_t inverse)
+{
+    const int q = (int)__umulhi((uint32_t)unit, inverse);   // one too small at most
+    return unit - q * n >= n ? q + 1 : q;
+}
+
+// What a warp of the row-statistics kernels found in its part of a row pair: the reference of both sums, the sums, the largest
+// target logit and its first index.
 struct WarpRecord {
     float ref, sum_a, sum_b, best;
     int32_t best_i;
@@ -413,6 +426,16 @@ __device__ __forceinline__ ArgMax warp_argmax(ArgMax a)
         a = better(a, b);
     }
     return a;
+}
+
+// Sums of two values over the lanes of a warp at once: of a in the lanes of the lower half, of b in those of the upper half.
+template <typename T> __device__ __forceinline__ T half_warp_sums(T a, T b)
+{
+    const bool upper = threadIdx.x & 16;
+    T v = (upper ? b : a) + __shfl_xor_sync(0xFFFFFFFFu, upper ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -470,6 +493,10 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t local, uint32_t rank)
 __device__ __forceinline__ void st_cluster(uint32_t addr, int32_t v)
 {
     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, const uint4 &v)
+{
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ void st_cluster(uint32_t addr, double v)
 {

@@ -25,6 +25,8 @@ struct RowStats {
 struct RowSegment {
     double weight, shared;
 };
+// 2^32 / n, rounded down (n = 1: below it): the high word of its product with a whole number is that number over n, or one less.
+inline uint32_t inverse_of(uint32_t n) { return n <= 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / n); }
 // First trip (32 vectors of 16 bytes) of part s of n in a row of `trips` trips.
 __host__ __device__ inline int segment_begin(int trips, int s, int n) { return (int)((long long)trips * s / n); }
 constexpr int MAX_SEGMENTS = 64;   // most parts of a row
@@ -48,6 +50,7 @@ struct RowGeometry {
     int32_t per_sm;     // CTAs per SM the shape is built for
     int32_t n_sm;       // SMs of the device (persistent kernels size their grid with it)
     int32_t cluster;    // CTAs that share one row pair (1: none)
+    int32_t hinted;     // aligned rows by the staged kernel with L2 policies
 };
 
 struct VerifyParams {
@@ -85,12 +88,16 @@ struct VerifyParams {
     int32_t keep_from_vec;   // the same as the first 16-byte vector of that share
     uint32_t poll_limit;     // polls after which a wait on an asynchronous copy gives up
     uint32_t table_mask;     // pointer-table mode: low address bits that must be clear in every entry
+    uint32_t k_inverse, k1_inverse;   // inverse_of(k), inverse_of(k + 1), set by the launcher
 };
 
 // streaming path (metasd_streaming.cu, metasd_bulk.cu)
 int row_parts(const RowGeometry &geo, int dtype, int vocab);   // parts of a row that a launch reports on
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo);
 cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches);
+// the staged kernel with L2 policies (metasd_hinted.cu); threads == 0: every shape that may be picked
+cudaError_t hinted_prepare(int dtype, int threads, int stages, int cluster);
+cudaError_t launch_row_stats_hinted(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream);
 cudaError_t bulk_prepare(int dtype, RowGeometry *geo);
 cudaError_t launch_row_stats_bulk(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream);
 // fused cluster path (metasd_fused.cu)

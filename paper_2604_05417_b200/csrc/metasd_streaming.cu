@@ -7,6 +7,7 @@
 //   K1p row_stats_staged_kernel  the default, any alignment: every thread stages its own
 //                          vectors through shared memory with cp.async, several trips ahead, and the second
 //                          sweep starts on the trips that are still staged instead of reading them again.
+//   K1h row_stats_hinted_kernel  (metasd_hinted.cu) the same with L2 policies, for more rows in flight than L2 holds.
 //   K1t row_stats_bulk_kernel    (metasd_bulk.cu) the same two sweeps by persistent CTAs whose rows arrive as TMA
 //                          bulk copies issued by one warp into a shared-memory ring.
 //   K2  epilogue_kernel    one CTA per sequence: accept tests with the Philox uniforms (Algorithm 4,
@@ -16,7 +17,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "metasd_device.cuh"
+#include "metasd_staged.cuh"
 
 namespace metasd {
 
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // second sweep visits the warp's trips in reverse: the last D trips of the first sweep are still in their slots and are
 // not read from memory again, and each slot is refilled with the trip D further down as soon as it has been used.  Lanes
 // behind the end of the row hold -Inf in their slot, which adds nothing to any sum: the loops carry no lane predicate.
+// Launches of more rows in flight than L2 keeps between the sweeps are the hinted kernel's (metasd_hinted.cu).
 //
 // SHIFTED: rows that start off a 16-byte boundary (an odd vocabulary), each row at its own offset.  fp32 rows are copied in
 // words, to where an aligned row has them; of bf16 rows the aligned 16-byte vectors that the row overlaps (a 33rd per trip for
@@ -173,97 +175,57 @@ __global__ void __launch_bounds__(K1_THREADS) row_stats_kernel(const VerifyParam
 // an aligned row: results do not depend on where a row starts, which for an odd vocabulary is a matter of its place in the
 // batch.  Copies that reach over the end of the row have the tokens outside replaced by -Inf once they have landed (nothing
 // outside the row's tensor is read).  bf16 rows in words too: V = 50257, B = 96 69 us a round instead of 63, fp32 rows in
-// vectors: V = 32001, B = 8 17.1 instead of 14.4.  These copies carry no L2 policy: with one, some builds of this form ended in
-// an illegal instruction at the first such copy.  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96,
+// vectors: V = 32001, B = 8 17.1 instead of 14.4.  Against plain 2- or 4-byte loads: V = 50257, bf16, B = 96,
 // k = 5 115.5 -> 81.5 us a round, V = 128257, B = 256 590 -> 270, V = 32001, fp32, B = 256 226 -> 126.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t policy)
-{
-    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
-}
-// The first `bytes` (0 .. 16) bytes of the vector, zeros behind them.
-__device__ __forceinline__ void cp_async16_part(uint32_t dst, const void *src, int bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4_part(uint32_t dst, const void *src, int bytes)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// 16 bytes of -Inf logits.
-template <typename LT> __device__ __forceinline__ void fill_neg_inf(uint32_t slot)
-{
-    const uint32_t w = sizeof(LT) == 2 ? 0xFF80FF80u : 0xFF800000u;
-    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(slot), "r"(w) : "memory");
-}
-
-// One warp's running statistics of a row pair.  All lanes share the reference `ref` that both rows' sums are relative to and
-// the best target logit `best` (its first index in `best_i`); the sums are the lane's own, two partial sums each.  The
-// reference is a whole number, the best logit's exponent with its sign changed and rounded: a change of reference is then
-// an exact scaling by a power of two, and sums of different warps are merged without an error of their own.
-template <typename LT> struct WarpSums {
-    uint64_t a, b;        // packed fp32 pairs: sum 2^(x c + ref) of the target and the draft row
-    float ref, best;
-    uint64_t nm;          // ref, twice
-    typename Logit<LT>::Best cmp;   // `best` as the vectors are compared with it
+// What a warp found in its part of a row pair: the reference of both sums, the sums, the largest target logit and its first
+// index; the first 16 bytes are sent as one.
+struct __align__(16) PartRecord {
+    float ref, sum_a, best;
     int32_t best_i;
+    float sum_b;
 };
 
 // A vector of the target row that holds a larger logit than any before it in the warp's range: rare (a warp's n-th trip
-// brings a new maximum with probability about 1/n), so the whole warp takes this branch together.
+// brings a new maximum with probability about 1/n), so the whole warp takes this branch together.  Where the largest logit
+// is, greedy rounds alone need to know.
 template <typename LT>
-__device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int vec, float c)
+__device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int vec, float c, bool index)
 {
     constexpr int VEC = Logit<LT>::VEC;
-    float x[VEC];
-    Logit<LT>::unpack(raw, x);
-    float cm = x[0];
-#pragma unroll
-    for (int e = 1; e < VEC; ++e) cm = fmaxf(cm, x[e]);
-    const float top = warp_max_f(cm);
+    const float cm = Logit<LT>::max_of(raw), top = warp_max_f(cm);
     const bool first_finite = w.best == -INFINITY;   // the reference may still be a stand-in, on either side of `top`
     const float ref = -rintf(top * c);
     if (ref < w.ref || first_finite) {
-        const uint64_t shrink = pack2(exp2i(ref - w.ref));
+        const uint64_t shrink = pack2(exp2_whole(ref - w.ref));
         if (!first_finite) w.a = mul2(w.a, shrink);
         w.b = mul2(w.b, shrink);
         w.ref = ref;
         w.nm = pack2(ref);
     }
-    int first = 0;
-#pragma unroll
-    for (int e = VEC - 1; e >= 0; --e)
-        if (x[e] == top) first = e;
-    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, cm == top)) - 1;   // lanes are in token order
-    w.best_i = __shfl_sync(0xFFFFFFFFu, vec * VEC + first, src & 31);
     w.best = top;
     w.cmp = Logit<LT>::best_of(top);
+    if (index) {
+        float x[VEC];
+        Logit<LT>::unpack(raw, x);
+        int first = 0;
+#pragma unroll
+        for (int e = VEC - 1; e >= 0; --e)
+            if (x[e] == top) first = e;
+        const int src = __ffs(__ballot_sync(0xFFFFFFFFu, cm == top)) - 1;   // lanes are in token order
+        w.best_i = __shfl_sync(0xFFFFFFFFu, vec * VEC + first, src & 31);
+    }
 }
 
-// What bounds it (bf16, B = 512, k = 8, V = 152064; 2.65 GB): the special-function unit (three exponentials a pair, 80 %
-// busy) and, in a long run, the board's power limit, so instructions and re-read bytes both cost time.  Against one vector
-// per thread and trip strided over the CTA: the warp-wide reference and the packed fp32 pairs take the maximum search, the
-// lane predicates and half the arithmetic instructions out of the loop (114.9 M warp instructions instead of 141.8 M on
-// B = 148), contiguous ranges make a range's pages and its second sweep its own, and six stages at two CTAs per SM keep a
-// third more of a pair on chip between the sweeps than four stages at three CTAs (3.17 GB read instead of 3.39 GB).  A
-// round of that size takes 630 us instead of 664 in a long run on one box; fp32, B = 1024, k = 5, V = 128256 1164 instead of
-// 1261; V = 262144, B = 40, k = 16 218 instead of 232.
+// A launch of short ranges is bound by the instructions it issues, and those that a warp spends once (950, seven trips' worth:
+// addresses, ends of ranges, maxima, merges) as much as those of its trips.  They are kept few: what is left of a range
+// beside whole groups goes through one rolled loop, indexes of maxima are kept in greedy rounds alone, quotients come by
+// multiplication and two sums share one tree.  B = 64, k = 5, V = 32000 11.4 -> 10.1 M warp instructions; us a round: V = 50257,
+// B = 96 53.3 -> 49.1, V = 50264, B = 192 ragged 59.8 -> 56.6, V = 152064, B = 4 23.1 -> 21.5, fp32, V = 32001, B = 8
+// 14.0 -> 12.7.
 //
 // CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
 // of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
 // order, so all hold the same normalisers; each sweeps its part again.
-template <int D, int THREADS, bool SHIFTED> constexpr uint32_t STAGED_SMEM = D * (THREADS * 32u + (SHIFTED ? THREADS / 32 * 32u : 0u));
-
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
@@ -276,7 +238,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     // 16-byte slots: [D][2 rows][THREADS]; SHIFTED: [D][NWARP][2 rows][33]
     extern __shared__ __align__(16) unsigned char stage_mem[];
-    __shared__ WarpRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
+    __shared__ PartRecord sh_rec[NREC];      // of every warp of the row pair, in trip order
     __shared__ MaxSum sh_redo[NREC];
     // The rows, the arms and what the last epilogue read of the scratch belong to the kernels before.  The epilogue may be
     // set up behind that wait only: what this kernel does not write, it reads before its own.
@@ -289,7 +251,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     const int unit = (int)blockIdx.x / CL;                        // the row (pair) of this CTA or cluster
     const int rank = CL > 1 ? (int)cluster_rank() : 0;
     const int first_bonus = BONUS_LAST ? p.batch * p.k : 0x7FFFFFFF;
-    const int b = BONUS_LAST ? (unit < first_bonus ? unit / p.k : unit - first_bonus) : unit / (p.k + 1);
+    const int b = BONUS_LAST ? (unit < first_bonus ? divide(unit, p.k, p.k_inverse) : unit - first_bonus) : divide(unit, p.k + 1, p.k1_inverse);
     const int kb = drafted(p.draft_len, b, p.k);
     const int j = BONUS_LAST ? (unit < first_bonus ? unit - b * p.k : kb) : unit - b * (p.k + 1);
     const int tid = threadIdx.x, lane = tid & 31;
@@ -307,7 +269,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     const int nvec = (p.V + VEC - 1) / VEC;
     const int trips_row = (nvec + 31) >> 5;
     const int part = rank * NWARP + warp;                         // this warp's part of the row's trips
-    const int g0 = segment_begin(trips_row, part, NREC), n_trip = segment_begin(trips_row, part + 1, NREC) - g0;
+    const int g0 = (unsigned)(trips_row * part) / NREC, n_trip = (unsigned)(trips_row * (part + 1)) / NREC - g0;   // segment_begin
     const int v0 = g0 * 32 + lane;                                // this lane's vector of trip 0
     // Copies are of UNIT bytes; a lane makes those of the units lane, lane + 32, .. of a trip.  SHIFTED: a row's units start
     // `lead` tokens in front of it (EXTRA: where they may, a trip needs one more).
@@ -341,16 +303,28 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         }
     };
     const bool a_room = ((size_t)b * (p.k + 1) + j) * p.V >= 16, d_room = ((size_t)b * p.k + j) * p.V >= 16;
-    auto copy_ragged = [&](int m, uint32_t dst, bool both) {
+    // A trip whose copies may not be whole: at the row's end, and (SHIFTED) at the start of a row with nothing in front of it.
+    auto copy_edge = [&](int m, uint32_t dst, bool both) {
+        if (SHIFTED) {
+            dst += put;
 #pragma unroll 1
-        for (int q = 0; q < (EXTRA && lane == 0 ? COPIES + 1 : COPIES); ++q) {
-            const int tok0 = ((g0 + m) * (512 / UNIT) + lane + 32 * q) * PER_UNIT;
-            copy_part(dst + q * (32u * UNIT), a4 + m * 512 + q * (32 * UNIT), a_row, tok0 - lead_a, a_room);
-            if (both) copy_part(dst + ROW_STRIDE + q * (32u * UNIT), d4 + m * 512 + q * (32 * UNIT), d_row, tok0 - lead_d, d_room);
+            for (int q = 0; q < (EXTRA && lane == 0 ? COPIES + 1 : COPIES); ++q) {
+                const int tok0 = ((g0 + m) * (512 / UNIT) + lane + 32 * q) * PER_UNIT;
+                copy_part(dst + q * (32u * UNIT), a4 + m * 512 + q * (32 * UNIT), a_row, tok0 - lead_a, a_room);
+                if (both) copy_part(dst + ROW_STRIDE + q * (32u * UNIT), d4 + m * 512 + q * (32 * UNIT), d_row, tok0 - lead_d, d_room);
+            }
+            __syncwarp();
+        } else if (v0 + 32 * m < nvec) {
+            cp_async16(dst, a4 + 512 * m);
+            if (both) cp_async16(dst + ROW_STRIDE, d4 + 512 * m);
+        } else {   // behind the row
+            fill_neg_inf<LT>(dst);
+            if (both) fill_neg_inf<LT>(dst + ROW_STRIDE);
         }
-        __syncwarp();
     };
+    const bool head = SHIFTED && EXTRA && g0 == 0 && !(a_room && d_room);   // trip 0 is such a trip
     auto copy_whole = [&](uint32_t dst, const char *a, const char *d, bool both) {
+        dst += put;
 #pragma unroll
         for (int q = 0; q < COPIES; ++q) {
             copy_unit(dst + q * (32u * UNIT), a + q * (32 * UNIT));
@@ -375,7 +349,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     };
     // This lane's tokens of a trip, from its slot (EXTRA: and the next one, behind a __syncwarp()).
     // EXTRA: three loads of 8 bytes, which halves of 8 bytes the tokens start in taken by the address: a third fewer selections
-    // than from two whole vectors (@@T@@).
+    // than from two whole vectors (V = 50257, B = 96 54.8 -> 53.4 us a round).
     auto fetch = [&](uint32_t src, int lead) {
         if (!EXTRA) return lds16(src);
         uint32_t w[6];
@@ -390,8 +364,6 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // reference that neither overflows nor underflows it, and sharing one spares the draft row its own maximum
     // search.  Whether the reference suited the draft row is checked after the sweep; if not, that row's statistics are
     // redone relative to its own maximum.
-    // a bonus row is read once: nothing of it is worth keeping in L2
-    const uint64_t drop = l2_policy_evict_first(), keep = pair ? l2_policy_evict_last() : drop;
     WarpSums<LT> w;
     w.a = w.b = 0ull;
     w.ref = 0.f;
@@ -401,43 +373,20 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     w.cmp = Logit<LT>::best_of(METASD_NEG_BIG);
     w.best_i = 0x7FFFFFFF;
     const uint64_t c2 = pack2(c);
-    // Requests below the kept share of the warp's range ask L2 to drop the line, the rest to keep it for sweep 2.
-    const int m_keep = n_trip - (int)((long long)n_trip * p.keep_permille / 1000);
     // BOTH: a row pair; else a bonus row.
+    uint32_t last_slot = slot0;   // of the warp's last trip
     auto sweep1 = [&](auto both_tag) {
         constexpr bool BOTH = decltype(both_tag)::value;
-        // One group of copies per trip, empty past the end: the group count stays in step with the trips.
-        auto request = [&](uint32_t dst, const char *a, const char *d, uint64_t pol) {
-            if (SHIFTED) {
-                copy_whole(dst, a, d, BOTH);
-            } else {
-                cp_async16(dst, a, pol);
-                if (BOTH) cp_async16(dst + ROW_STRIDE, d, pol);
-            }
+        // The copies of a trip that are all whole; a group of them per trip, empty past the end, so that the group count
+        // stays in step with the trips.
+        auto request = [&](uint32_t dst, const char *a, const char *d) {
+            copy_whole(dst, a, d, BOTH);
             cp_async_commit();
-        };
-        auto request_checked = [&](int m, uint32_t dst) {
-            if (SHIFTED) {
-                if (m < n_full && m + g0 > 0) {   // whole units: most of a short range is asked for here
-                    request(dst + put, a4 + 512 * m, d4 + 512 * m, drop);
-                    return;
-                }
-                if (m < n_trip) copy_ragged(m, dst + put, BOTH);
-                cp_async_commit();
-            } else if (m < lane_trips) {
-                request(dst, a4 + 512 * m, d4 + 512 * m, m >= m_keep ? keep : drop);
-            } else {
-                if (m < n_trip) {
-                    fill_neg_inf<LT>(dst);
-                    fill_neg_inf<LT>(dst + ROW_STRIDE);
-                }
-                cp_async_commit();
-            }
         };
         // Trip n, whose vectors have landed.
         auto consume = [&](int n, uint32_t src) {
             const uint4 ra = fetch(src, lead_a);
-            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT>(w, ra, v0 + 32 * n, c);
+            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT>(w, ra, v0 + 32 * n, c, p.greedy != 0);
             w.a = Logit<LT>::add_exp(w.a, ra, c2, w.nm);
             if (BOTH) w.b = Logit<LT>::add_exp(w.b, fetch(src + ROW_STRIDE, lead_d), c2, w.nm);
         };
@@ -452,8 +401,23 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
                 __syncwarp();
             }
         };
-#pragma unroll
-        for (int m = 0; m < D - 1; ++m) request_checked(m, slot0 + (uint32_t)m * STAGE_STRIDE);
+        const char *a_next = a4, *d_next = d4;
+        uint32_t dst = slot0;
+        auto request_checked = [&](int m) {
+            if (m < n_full && !(head && m == 0)) {
+                request(dst, a_next, d_next);
+            } else {
+                if (m < n_trip) copy_edge(m, dst, BOTH);
+                cp_async_commit();
+            }
+        };
+#pragma unroll 1
+        for (int m = 0; m < D - 1; ++m) {
+            request_checked(m);
+            a_next += 512;
+            d_next += 512;
+            dst += STAGE_STRIDE;
+        }
         // The first reference: the maximum of the warp's first trip.  Where the target's logits are all masked there, the
         // draft row's (or 0) stands in, so that the draft row's sum does not overflow.
         if (n_trip > 0) {
@@ -471,75 +435,89 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             w.nm = pack2(w.ref);
         }
         // Trip n asks for the trip D - 1 ahead, then works on its own vectors (slot n mod D).  Groups of D trips whose
-        // requests all lie inside the row carry no checks, and their slots and their L2 policy are constants (the boundary
-        // of the kept share is rounded down to a whole group: a few vectors more are kept).
+        // requests all lie inside the row carry no checks, and their slots are constants.
         int n = 0;
-        const char *a_next = a4 + 512 * (D - 1), *d_next = d4 + 512 * (D - 1);
-        auto group = [&](uint64_t pol) {
+        for (; n + 2 * D - 2 < n_full; n += D) {
 #pragma unroll
             for (int u = 0; u < D; ++u) {
                 meet();
-                request(slot0 + put + (uint32_t)((u + D - 1) % D) * STAGE_STRIDE, a_next + 512 * u, d_next + 512 * u, pol);
+                request(slot0 + (uint32_t)((u + D - 1) % D) * STAGE_STRIDE, a_next + 512 * u, d_next + 512 * u);
                 landed();
                 consume(n + u, slot0 + (uint32_t)u * STAGE_STRIDE);
             }
-            n += D;
             a_next += 512 * D;
             d_next += 512 * D;
-        };
-        if (!SHIFTED)
-            while (n + 2 * D - 2 < min(m_keep, n_full)) group(drop);
-        while (n + 2 * D - 2 < n_full) group(keep);
-        for (int slot = 0, ask = D - 1; n < n_trip; ++n) {
-            meet();
-            request_checked(n + D - 1, slot0 + (uint32_t)ask * STAGE_STRIDE);
-            landed();
-            if (SHIFTED && n >= n_full && n > 0) mask_ragged(n, slot0 + (uint32_t)slot * STAGE_STRIDE, BOTH);
-            consume(n, slot0 + (uint32_t)slot * STAGE_STRIDE);
-            ask = slot;
-            slot = slot + 1 == D ? 0 : slot + 1;
         }
+        // The rest trip by trip: few instructions, and few to be fetched where a range is short.
+        uint32_t src = slot0;
+#pragma unroll 1
+        for (int m = n + D - 1; n < n_trip; ++n, ++m) {
+            meet();
+            request_checked(m);
+            landed();
+            if (SHIFTED && n >= n_full && n > 0) mask_ragged(n, src, BOTH);
+            consume(n, src);
+            a_next += 512;
+            d_next += 512;
+            dst = src;
+            src = src == slot0 + (D - 1) * STAGE_STRIDE ? slot0 : src + STAGE_STRIDE;
+        }
+        last_slot = dst;
         cp_async_wait<0>();
     };
     if (pair) sweep1(std::true_type{});
     else sweep1(std::false_type{});
 
     // ---- the warps' records, merged by every warp for itself (no second barrier)
-    const float sum_aw = warp_sum_f(sum2(w.a)), sum_bw = warp_sum_f(sum2(w.b));
+    // Two sums over the lanes at once: the target row's end up in the lower half of the warp, the draft row's in the upper one.
+    const bool upper = lane & 16;
+    const float sum_w = half_warp_sums(sum2(w.a), sum2(w.b));
     if (CL > 1) {
         cluster_wait();   // every CTA of the cluster is running
-        if (lane < CL) {
-            const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane);
-            st_cluster(dst, __float_as_int(w.ref));          st_cluster(dst + 4, __float_as_int(sum_aw));
-            st_cluster(dst + 8, __float_as_int(sum_bw));    st_cluster(dst + 12, __float_as_int(w.best));
-            st_cluster(dst + 16, w.best_i);
+        if ((lane & 15) < CL) {
+            const uint32_t dst = map_to_rank(smem_addr(&sh_rec[part]), (uint32_t)lane & 15u);
+            if (upper) st_cluster(dst + 16, __float_as_int(sum_w));
+            else st_cluster4(dst, make_uint4(__float_as_uint(w.ref), __float_as_uint(sum_w), __float_as_uint(w.best), (uint32_t)w.best_i));
         }
         cluster_sync_all();
     } else {
-        if (lane == 0) sh_rec[warp] = WarpRecord{w.ref, sum_aw, sum_bw, w.best, w.best_i};
+        if (lane == 0) {
+            sh_rec[warp].ref = w.ref; sh_rec[warp].sum_a = sum_w; sh_rec[warp].best = w.best; sh_rec[warp].best_i = w.best_i;
+        }
+        if (lane == 16) sh_rec[warp].sum_b = sum_w;
         __syncthreads();
     }
     float ref_a = INFINITY, sum_a = 0.f, sum_b = 0.f;   // both sums end up relative to the target row's largest logit
     ArgMax rm = {-INFINITY, 0x7FFFFFFF};
+    // The lower half of the warp holds the target row's sums and the upper half the draft row's, NREC / 16 of them a lane
+    // (fewer: several times).
+    constexpr int HALF = NREC == 4 || NREC == 8 ? NREC : 16;
+    float part_ref[(NREC + 15) / 16], part_sum[(NREC + 15) / 16];
 #pragma unroll
-    for (int r0 = 0; r0 < NREC; r0 += 32)
-        if (NREC - r0 >= 32 || lane < NREC - r0) {
-            const WarpRecord r = sh_rec[r0 + lane];
+    for (int q = 0; q < (NREC + 15) / 16; ++q) {
+        const int i = 16 * q + (lane & (HALF - 1));
+        part_ref[q] = 0.f;
+        part_sum[q] = 0.f;
+        if (NREC % HALF == 0 || i < NREC) {
+            const PartRecord r = sh_rec[i];
+            part_ref[q] = r.ref;
+            part_sum[q] = upper ? r.sum_b : r.sum_a;
             if (r.best > METASD_NEG_BIG) ref_a = fminf(ref_a, r.ref);   // a part without a finite target logit has a stand-in
             rm = better(rm, ArgMax{r.best, r.best_i});
         }
+    }
     ref_a = -warp_max_f(-ref_a);
     if (!(ref_a < INFINITY)) ref_a = 0.f;
+    float merged = 0.f;
 #pragma unroll
-    for (int r0 = 0; r0 < NREC; r0 += 32)
-        if (NREC - r0 >= 32 || lane < NREC - r0) {
-            const WarpRecord r = sh_rec[r0 + lane];
-            const float d = ref_a - r.ref;   // above zero for stand-ins alone, whose sum_a is zero
-            sum_a = fmaf(r.sum_a, exp2i(fminf(d, 0.f)), sum_a);
-            sum_b = fmaf(r.sum_b, exp2i(d), sum_b);
-        }
-    sum_a = warp_sum_f(sum_a);
-    sum_b = warp_sum_f(sum_b);
+    for (int q = 0; q < (NREC + 15) / 16; ++q) {
+        const float d = ref_a - part_ref[q];   // above zero for stand-ins alone, whose sum_a is zero
+        merged = fmaf(part_sum[q], exp2_whole(upper ? d : fminf(d, 0.f)), merged);
+    }
+#pragma unroll
+    for (int o = HALF / 2; o > 0; o >>= 1) merged += __shfl_xor_sync(FULL, merged, o);
+    sum_a = __shfl_sync(FULL, merged, 0);
+    sum_b = __shfl_sync(FULL, merged, 16);
     {
         const float best = warp_max_f(rm.v);
         rm.i = __reduce_min_sync(FULL, rm.v == best ? rm.i : 0x7FFFFFFF);
@@ -571,7 +549,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             for (int e = 1; e < VEC; ++e) bm = fmaxf(bm, xb[e]);
             const float top = rintf(bm * c);
             if (top > own.m) {
-                own.s *= exp2i(own.m - top);
+                own.s *= exp2_whole(own.m - top);
                 own.m = top;
             }
 #pragma unroll
@@ -579,7 +557,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         }
         auto merge_warp = [](MaxSum v) {
             const float top = warp_max_f(v.m);
-            return MaxSum{top, warp_sum_f(v.s * exp2i(v.m - top))};
+            return MaxSum{top, warp_sum_f(v.s * exp2_whole(v.m - top))};
         };
         own = merge_warp(own);
         if (CL > 1) {
@@ -597,7 +575,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         for (int r = lane; r < NREC; r += 32) {
             const MaxSum q = sh_redo[r];
             const float top = fmaxf(rb.m, q.m);
-            rb = MaxSum{top, rb.s * exp2i(rb.m - top) + q.s * exp2i(q.m - top)};
+            rb = MaxSum{top, rb.s * exp2_whole(rb.m - top) + q.s * exp2_whole(q.m - top)};
         }
         rb = merge_warp(rb);
         ref_b = -rb.m;
@@ -623,7 +601,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     if (pair) {
         const float rho = sum_a / sum_b, whole = rintf(log2f(rho));
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
-        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(log2f(rho * exp2i(-whole)));
+        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(log2f(rho * exp2_whole(-whole)));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last).
@@ -635,42 +613,34 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             acc = Logit<LT>::add_exp_min(acc, fetch(src, lead_a), fetch(src + ROW_STRIDE, lead_d), c2, nma, nmb, lg);
             if (SHIFTED) __syncwarp();   // and has been read before its lane refills the slot
         };
-        auto refill = [&](uint32_t dst, int m, const char *a, const char *d) {
-            if (SHIFTED) {
-                if (m + g0 == 0) copy_ragged(0, dst + put, true);
-                else copy_whole(dst + put, a, d, true);
-            } else {
-                cp_async16(dst, a, drop);
-                cp_async16(dst + ROW_STRIDE, d, drop);
-            }
-        };
-        // the ragged top first, then whole groups downwards with constant slots
+        // Downwards, trip by trip; whole groups, whose refills are all real and whose slots are constants, where the range is long.
         int n = n_trip - 1;
-        for (int slot = n % D; n >= 0 && slot != D - 1; --n) {
-            const uint32_t src = slot0 + (uint32_t)slot * STAGE_STRIDE;
-            consume(src);
-            if (n >= D) refill(src, n - D, a4 + 512 * (n - D), d4 + 512 * (n - D));
-            cp_async_commit();
-            slot = slot == 0 ? D - 1 : slot - 1;
-        }
+        uint32_t src = last_slot;
         const char *a_next = a4 + 512 * (n - D), *d_next = d4 + 512 * (n - D);
-        for (; n >= D; n -= D) {   // n + 1 is a multiple of D and a whole group lies below: every refill is real
+#pragma unroll 1
+        while (n >= 0) {
+            if (src == slot0 + (D - 1) * STAGE_STRIDE) {
+                for (; n >= 2 * D - 1 + (head ? 1 : 0); n -= D) {
 #pragma unroll
-            for (int u = 0; u < D; ++u) {
-                const uint32_t src = slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE;
-                consume(src);
-                refill(src, n - u - D, a_next - 512 * u, d_next - 512 * u);
-                cp_async_commit();
+                    for (int u = 0; u < D; ++u) {
+                        consume(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
+                        copy_whole(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE, a_next - 512 * u, d_next - 512 * u, true);
+                        cp_async_commit();
+                    }
+                    a_next -= 512 * D;
+                    d_next -= 512 * D;
+                }
             }
-            a_next -= 512 * D;
-            d_next -= 512 * D;
-        }
-        if (n >= 0) {
-#pragma unroll
-            for (int u = 0; u < D; ++u) {
-                consume(slot0 + (uint32_t)(D - 1 - u) * STAGE_STRIDE);
-                cp_async_commit();
+            consume(src);
+            if (n >= D) {
+                if (head && n == D) copy_edge(0, src, true);
+                else copy_whole(src, a_next, d_next, true);
             }
+            cp_async_commit();
+            a_next -= 512;
+            d_next -= 512;
+            --n;
+            src = src == slot0 ? slot0 + (D - 1) * STAGE_STRIDE : src - STAGE_STRIDE;
         }
         cp_async_wait<0>();
         shared = sum2(acc);
@@ -678,59 +648,18 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     }
     // fp64 across lanes: a rounding here would move the draw by itself.  Tokens unlike a float64 evaluation's (all next
     // to an edge), of 49450 rejections at V = 32000: 28 with references per row and fp32 here, 20 with the warp's reference.
-    const double total = warp_sum((double)weight), total_min = warp_sum((double)shared);
-    if (lane == 0) {   // the warp's trips are part `part` of the row
-        const double scale = (double)(exp2i(fminf(ref_a - w.ref, 0.f)) / sum_a);
-        p.segments[row * NREC + part] = RowSegment{total * scale, total_min * scale};
+    const double total = half_warp_sums((double)weight, (double)shared);   // of the weights, and from lane 16 on of the shared mass
+    if ((lane & 15) == 0) {   // the warp's trips are part `part` of the row
+        const double scale = (double)(exp2_whole(fminf(ref_a - w.ref, 0.f)) / sum_a);
+        (&p.segments[row * NREC + part].weight)[upper] = total * scale;
     }
 }
-
-// Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it
-// in the stream drains, and wait (grid_dependency_wait) before they touch what that one does.
-template <typename... Params, typename... Args>
-static cudaError_t launch_kernel(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, int cluster, bool chained,
-                                 cudaStream_t stream, const Args &...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute at[2];
-    cfg.attrs = at;
-    if (chained) {
-        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
-    if (cluster > 1) {
-        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-        cudaLaunchAttribute &a = at[cfg.numAttrs++];
-        a.val.clusterDim.x = (unsigned)cluster; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-// Shared memory of an SM, of which every block takes 1 KB besides its own, and the most that a launch below asks for.
-constexpr unsigned SM_SMEM = 228 * 1024, STAGED_SMEM_MAX = 216 * 1024;
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm, cudaStream_t stream)
 {
-    // A launch of up to one wave wants its blocks spread evenly over the SMs: set up while the last epilogue still holds some of
-    // them, they would crowd on the others and stay there.  So such a launch is chained only where the last layer of blocks
-    // is nearly full (or, of clusters, which are placed within groups of SMs, where every one finds free SMs), and asks for
-    // the shared memory that keeps one block more than an even spread off an SM, and no more: what is left there, half an SM's
-    // where there is one block, is for the kernels of other streams.  Us a round, chained so / not, in blocks
-    // of 256 and 512 threads:
-    // 384 blocks (B = 64, k = 5, V = 32000) 22.8 / 24.6, 240 18.5 / 20.5, 144 (V = 128256) 28.1 / 28.7, 96 14.0 / 16.1;
-    // 320 blocks 22.2 / 20.5, 480 26.5 / 24.6; 32 clusters of 4 13.5 / 14.4, 36 21.8 / 19.8.  Several waves are always chained
-    // (B = 192, k = 8 ragged, V = 50264 61.9 / 69.8).
-    const unsigned ctas = units * CL, sms = (unsigned)n_sm, layers = (ctas + sms - 1) / sms, spare = layers * sms - ctas;
-    const bool one_wave = layers <= MINB;
-    const bool chained = !one_wave || ctas <= sms / 2 || (CL == 1 ? spare <= sms / 2 : layers == 1 && spare >= sms / 8);
-    constexpr unsigned needed = STAGED_SMEM<D, THREADS, SHIFTED>;   // the attribute that allows it, and more, was set by streaming_prepare
-    const unsigned smem = one_wave && chained ? std::max(needed, (SM_SMEM / (layers + 1) + 1023u) / 1024u * 1024u) : needed;
-    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, ctas, THREADS, smem, CL, chained, stream, p);
+    const StagedLaunch how = staged_launch(units, CL, MINB, STAGED_SMEM<D, THREADS, SHIFTED>, n_sm);
+    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, units * CL, THREADS, how.smem, CL, how.chained, stream, p);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -1152,41 +1081,37 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
 constexpr int DRAW_THREADS = 256, DRAW_THREADS_ROW = 512;
 
 // The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).  Those that
-// staged_shape() picks, by logit type, and those that a configuration can ask for.
+// staged_shape() picks, by logit type; a configuration can ask for METASD_STAGED_PINNED_SHAPES.
 #define METASD_STAGED_BF16_SHAPES(X) \
     X(128, 4, 12, true, 1) X(256, 4, 6, true, 1) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) \
     X(256, 6, 4, true, 2) X(128, 6, 6, true, 4)
 #define METASD_STAGED_FP32_SHAPES(X) \
     X(256, 4, 6, true, 1) X(256, 6, 4, true, 2) X(128, 6, 6, true, 4) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
-#define METASD_STAGED_PINNED_SHAPES(X) \
-    X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(1024, 6, 1, false, 1) X(1024, 4, 1, true, 1) X(768, 4, 2, true, 1) X(384, 4, 4, true, 1) \
-    X(512, 4, 3, true, 3) X(512, 4, 3, true, 2) X(768, 4, 2, true, 2)
 
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL>
-static cudaError_t prepare_staged(bool aligned)
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
+static cudaError_t prepare_staged()
 {
-    cudaError_t e = cudaSuccess;
-    if (aligned)
-        e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
-    if (e == cudaSuccess)   // a tensor may start off a 16-byte boundary whatever its rows' length
-        e = cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
-    return e;
+    return cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
 }
 
-// The pinned shape; threads == 0: every shape that staged_shape() may pick for rows of `warps` warps (0: for any row).
+// The pinned shape, whose aligned rows are the hinted kernel's; threads == 0: every shape that staged_shape() may pick for rows
+// of `warps` warps (0: for any row).  A tensor may start off a 16-byte boundary whatever its rows' length.
 template <typename LT>
 static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int warps, bool aligned)
 {
     if (threads) {
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C>(aligned);
+#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C, true>();
         METASD_STAGED_PINNED_SHAPES(X)
 #undef X
         return cudaErrorNotSupported;
     }
     cudaError_t e = cudaSuccess;
-#define X(T, D, M, BL, C) if (e == cudaSuccess && (warps == 0 || warps == T / 32 * C)) e = prepare_staged<LT, D, T, M, BL, C>(aligned);
+#define X(T, D, M, BL, C) \
+    if (e == cudaSuccess && (warps == 0 || warps == T / 32 * C)) { \
+        e = prepare_staged<LT, D, T, M, BL, C, true>(); \
+        if (e == cudaSuccess && aligned) e = prepare_staged<LT, D, T, M, BL, C, false>(); \
+    }
     if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
     else { METASD_STAGED_FP32_SHAPES(X) }
 #undef X
@@ -1196,11 +1121,15 @@ static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int wa
 template <typename LT>
 static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo, cudaStream_t stream)
 {
+    constexpr int dtype = sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32;
+    if (p.vector_ok && geo.hinted) return launch_row_stats_hinted(p, dtype, geo, stream);
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
 #define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
         return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, geo.n_sm, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
     if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
     else { METASD_STAGED_FP32_SHAPES(X) }
+#undef X
+#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) return launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
     METASD_STAGED_PINNED_SHAPES(X)
 #undef X
     return cudaErrorNotSupported;
@@ -1251,6 +1180,20 @@ static StagedShape staged_shape(int dtype, long long bytes, long long units, int
     }
 }
 
+// Whether L2 policies pay, which the hinted kernel has: where the row pairs in flight are more than L2 keeps between their sweeps
+// without them.  Us a round with and without, by MB in flight: bf16, 512/6/1 118: 138.6 and 136.6 (B = 256, k = 5, V = 100000), 152: 226 and
+// 223 (B = 256, k = 7, V = 128256), 180: 635 and 643 (B = 512, k = 8, V = 152064); 512/4/1 89: 462 and 451 (B = 1024, k = 8,
+// V = 50264), 113: 103.0 and 103.9, 142: 169 and 181 (B = 400, k = 5, V = 80000); 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
+// 76: 242 and 226 (256/6/4: B = 512, k = 4, V = 64000), 293 and 263 (256/6/2: B = 1024, k = 5, V = 32000), 95: 78.7 and 79.6, 114: 261 and 333
+// (128/6/8: B = 256, k = 5, V = 128256).  Short rows never come near it (128/4/1, 256/4/1).
+static bool hinted_pays(int dtype, long long bytes, long long units, const StagedShape &s, int n_sm)
+{
+    const bool fp32 = dtype == METASD_FP32;
+    if (s.threads < 512 && s.stages == 4) return false;
+    const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : s.stages == 4 ? 3 : 1024 / s.threads) / s.cluster;
+    return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.stages == 6 && s.cluster == 1 ? 165 : 115) * 1000000ll;
+}
+
 // The shape of a launch: what the configuration pinned, else by the size of the launch.
 static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units)
 {
@@ -1260,6 +1203,7 @@ static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab
         g.threads = s.threads;
         g.stages = s.stages;
         g.cluster = s.cluster;
+        g.hinted = hinted_pays(dtype, row_bytes(dtype, vocab), units, s, geo.n_sm);
     }
     return g;
 }
@@ -1299,6 +1243,7 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
     geo->stages = cfg.row_stages;
     geo->per_sm = 1;
     geo->cluster = 1;
+    geo->hinted = 0;
     if (cfg.row_cluster > 1 && geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;   // only the staged kernel has a cluster form
     if (geo->kernel == METASD_ROWS_PLAIN) {
         if (geo->threads && geo->threads != K1_THREADS) return cudaErrorNotSupported;
@@ -1318,8 +1263,10 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         if (!geo->threads) geo->threads = dtype == METASD_BF16 ? 512 : 1024;
         if (!geo->stages) geo->stages = dtype == METASD_BF16 && geo->threads == 512 ? 4 : 6;
         geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
+        geo->hinted = 1;
     }
     if ((e = dtype == METASD_BF16 ? prepare_small_kernels<__nv_bfloat16>() : prepare_small_kernels<float>()) != cudaSuccess) return e;
+    if ((e = hinted_prepare(dtype, geo->threads, geo->stages, geo->cluster)) != cudaSuccess) return e;
     const int warps = cfg.vocab > 0 ? row_warps(dtype, row_bytes(dtype, cfg.vocab)) : 0;
     const bool aligned = row_bytes(dtype, cfg.vocab) % 16 == 0;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, warps, aligned)
@@ -1333,6 +1280,8 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
     constexpr int dtype = sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32;
     const RowGeometry geo = resolve_geometry(context_geo, dtype, p.V, (long long)p.batch * (p.k + 1));
     p.n_seg = row_parts(geo, dtype, p.V);
+    p.k_inverse = inverse_of((uint32_t)p.k);
+    p.k1_inverse = inverse_of((uint32_t)p.k + 1u);
     if (geo.kernel == METASD_ROWS_STAGED) {
         e = launch_staged_t<LT>(p, geo, stream);
     } else if (!p.vector_ok) {

@@ -41,3 +41,9 @@ def test_results_do_not_depend_on_the_batch(dtype, V, B):
     for first, last in [(0, 1), (1, 13), (13, 60), (60, 200), (200, 400)]:
         for x, y in zip(whole, play(first, last)):
             assert torch.equal(x[first:last], y)
+
+
+@pytest.mark.parametrize("V", [80008, 152064])
+def test_results_do_not_depend_on_the_kernel_of_long_launches(V):
+    """1200 bf16 row pairs and bonus rows, more than L2 holds, which the kernel with L2 policies takes; 141 of them by the other."""
+    test_results_do_not_depend_on_the_batch("bf16", V, 400)
