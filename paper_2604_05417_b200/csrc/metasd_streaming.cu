@@ -1086,7 +1086,7 @@ constexpr int DRAW_THREADS = 256, DRAW_THREADS_ROW = 512;
     X(128, 4, 12, true, 1) X(256, 4, 6, true, 1) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) \
     X(256, 6, 4, true, 2) X(128, 6, 6, true, 4)
 #define METASD_STAGED_FP32_SHAPES(X) \
-    X(256, 4, 6, true, 1) X(256, 6, 4, true, 2) X(128, 6, 6, true, 4) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
+    X(256, 4, 6, true, 1) X(256, 6, 4, true, 1) X(512, 6, 2, true, 1) X(256, 6, 4, true, 2) X(128, 6, 6, true, 4) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
 
 template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
 static cudaError_t prepare_staged()
@@ -1158,6 +1158,9 @@ static int row_warps(int dtype, long long bytes)
 //     29.0, 64.3, 512/4/1 12.9, 13.3, 24.4, 28.1, 57.2.  V = 80000: 128/6/4 16.6 (72), 39.8 (384), 121 (1536), 256/6/2 16.5, 39.7, 112, 512/4/1
 //     19.3, 42.8, 110, 512/6/1 19.3, 41.6, 113.  V = 152064: 128/6/4 19.8 (36), 24.3 (72), 88.1 (576), 223 (1728), 256/6/2 22.5, 23.6, 85.9,
 //     215, 512/6/1 28.9, 29.4, 91.5, 218 (4608: 527, 256/6/2 590).
+//     V = 65000 512/4/1 162.5 (2400), 512/6/1 159.2; V = 80000 184.4 (2400) and 96.3 (1200), 181.0 and 90.9.
+//   fp32, 8 warps: V = 8000 256/4/1 24.0 (1280), 77.3 (5120), 256/6/1 24.6, 79.0; V = 16000 15.8 (320), 24.4 (640), 74.5 (2560), 146.5 (5120),
+//     16.5, 24.1, 67.9, 130.5.  16 warps, V = 32000: 256/6/2 33.3 (512), 54.2 (1024), 192.0 (4000), 512/6/1 32.4, 53.3, 185.9.
 //   fp32, 16 warps, V = 32000: 128/6/4 11.1 (32 units), 15.2 (128), 29.2 (384), 86.9 (1536), 256/6/2 11.8, 15.5, 28.1, 81.8.
 //   fp32, 32 warps: V = 64000: 128/6/8 11.8 (24 units), 50.8 (384), 180 (1728), 614 (6144), 256/6/4 12.1, 48.3, 157, 574, 1024/6/1
 //     17.5, 51.7, 168, 525; V = 128256: 15.8, 79.7, 292 and 1062, 16.0, 86.0, 302 and 1094, 26.5, 91.0, 302 and 1029.
@@ -1169,11 +1172,12 @@ static StagedShape staged_shape(int dtype, long long bytes, long long units, int
     const bool fp32 = dtype == METASD_FP32;
     switch (row_warps(dtype, bytes)) {
     case 4: return {128, 4, 1};
-    case 8: return {256, 4, 1};
+    case 8: return {256, fp32 && bytes >= 48 * 1000 && units > 4 * n_sm ? 6 : 4, 1};
     case 16:
         if (units * 4 <= n_sm || (units <= n_sm && bytes < 140 * 1000)) return {128, 6, 4};
-        if (fp32 || units <= (bytes < 100 * 1000 ? 3 : 7) * n_sm) return {256, 6, 2};
-        return bytes < 180 * 1000 ? StagedShape{512, 4, 1} : StagedShape{512, 6, 1};
+        if (fp32 ? bytes >= 150 * 1000 : units <= (bytes < 100 * 1000 ? 3 : 7) * n_sm) return {256, 6, 2};
+        if (fp32 && units <= 3 * n_sm) return {256, 6, 2};
+        return !fp32 && bytes < 120 * 1000 ? StagedShape{512, 4, 1} : StagedShape{512, 6, 1};
     default:
         if (units > 20 * n_sm) return {1024, 6, 1};
         return bytes >= 400 * 1000 || units <= n_sm ? StagedShape{128, 6, 8} : StagedShape{256, 6, 4};
