@@ -669,11 +669,19 @@ static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm
 template <typename LT, int VEC> struct RawVec { uint4 v; };
 template <typename LT> struct RawVec<LT, 1> { float v; };
 
+// A whole line comes to L2 at a piece's first vector, and stays in L1 for the search's next level.
+__device__ __forceinline__ uint4 ld_draw(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L2::128B.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 template <typename LT, int VEC>
 __device__ __forceinline__ RawVec<LT, VEC> load_raw(const LT *row, int i)
 {
     RawVec<LT, VEC> r;
-    if constexpr (VEC > 1) r.v = ld_stream(reinterpret_cast<const uint4 *>(row) + i);
+    if constexpr (VEC > 1) r.v = ld_draw(reinterpret_cast<const uint4 *>(row) + i);
     else r.v = Logit<LT>::scalar(row, i);
     return r;
 }
@@ -1075,10 +1083,13 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
 // -------------------------------------------------------------------------------------------
 // launchers
 // -------------------------------------------------------------------------------------------
-// Threads of an epilogue CTA besides its control warp.  Rows in one part (the plain and the bulk kernel) are walked whole, by
-// twice the threads where every sequence has an SM: B = 64, k = 4, V = 152064, plain 125 -> 107 us a round, bulk (whose rows are
-// not in L2) 169 -> 96, with the coalesced pieces of range_inverse_cdf; B = 300, k = 2, V = 128256 205 -> 196 and 256 -> 188.
-constexpr int DRAW_THREADS = 256, DRAW_THREADS_ROW = 512;
+// Threads of an epilogue CTA besides its control warp: twice as many where every sequence has an SM and what is walked, a part of
+// the row, is more than DRAW_PART_BYTES, 1024 vectors, of which 256 threads would read their pieces in two turns.  Us a round:
+// V = 152064, B = 4, k = 8 19.5 -> 18.3, V = 262144, B = 40, k = 16 182.3 -> 179.3.  Rows in one part (the plain and the bulk
+// kernel), with the coalesced pieces of range_inverse_cdf: B = 64, k = 4, V = 152064, plain 125 -> 107, bulk (whose rows are
+// not in L2) 169 -> 96; B = 300, k = 2, V = 128256 205 -> 196 and 256 -> 188.
+constexpr int DRAW_THREADS = 256, DRAW_THREADS_WIDE = 512;
+constexpr long long DRAW_PART_BYTES = 16 * 1024;
 
 // The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).  Those that
 // staged_shape() picks, by logit type; a configuration can ask for METASD_STAGED_PINNED_SHAPES.
@@ -1233,6 +1244,8 @@ static cudaError_t prepare_small_kernels()
     set((const void *)epilogue_kernel<LT, true, DRAW_THREADS, true>);
     set((const void *)epilogue_kernel<LT, true, DRAW_THREADS, false>);
     set((const void *)epilogue_kernel<LT, false, DRAW_THREADS, false>);
+    set((const void *)epilogue_kernel<LT, true, DRAW_THREADS_WIDE, false>);
+    set((const void *)epilogue_kernel<LT, false, DRAW_THREADS_WIDE, false>);
     set((const void *)select_kernel);
     return e;
 }
@@ -1297,11 +1310,11 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
     }
     if (e != cudaSuccess) return e;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const unsigned grid = (unsigned)p.batch, threads = DRAW_THREADS + 32, threads_row = DRAW_THREADS_ROW + 32;   // and the control warp
-    const bool row = p.n_seg <= 1 && p.batch <= geo.n_sm;
+    const unsigned grid = (unsigned)p.batch, threads = DRAW_THREADS + 32, threads_wide = DRAW_THREADS_WIDE + 32;   // and the control warp
+    const bool wide = p.batch <= geo.n_sm && (long long)p.V * (long long)sizeof(LT) > DRAW_PART_BYTES * p.n_seg;
     if (p.greedy) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, true>, grid, threads, 0, 1, true, stream, p);
-    else if (row && p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS_ROW, false>, grid, threads_row, 0, 1, true, stream, p);
-    else if (row) e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS_ROW, false>, grid, threads_row, 0, 1, true, stream, p);
+    else if (wide && p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS_WIDE, false>, grid, threads_wide, 0, 1, true, stream, p);
+    else if (wide) e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS_WIDE, false>, grid, threads_wide, 0, 1, true, stream, p);
     else if (p.vector_ok) e = launch_kernel(epilogue_kernel<LT, true, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
     else e = launch_kernel(epilogue_kernel<LT, false, DRAW_THREADS, false>, grid, threads, 0, 1, true, stream, p);
     *launches += 2;

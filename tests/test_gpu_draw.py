@@ -89,3 +89,12 @@ def test_sliding_windows_around_a_warp(window):
     wl = workload(B=6, N=3, k=2, V=512, sigmas=(0.3, 1.0, 2.5)).scaled(tau=window)
     c = run_lockstep(wl, rounds=70, bandit="swucb", table_mode=True, path=M.PATH_STREAMING)
     assert c["rounds"] == 70 and c["near_tie_arm"] == 0
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 131072), ("bf16", 131080), ("bf16", 151937), ("fp32", 131072), ("fp32", 131076), ("fp32", 140001)])
+def test_draws_on_both_sides_of_long_parts(dtype, V):
+    """Parts of up to 16 KB, which 256 threads walk, and longer ones, which 512 do where every sequence has an SM."""
+    from _harness import run_lockstep
+    wl = workload(B=4, N=2, k=2, V=V, sigmas=(0.4, 1.5)).scaled(dtype=dtype, temperature=0.8, order="shuffled")
+    c = run_lockstep(wl, rounds=4, seed=V % 83, path=M.PATH_STREAMING)
+    assert c["rounds"] == 4 and c["status"] == 0
