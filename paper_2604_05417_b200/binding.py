@@ -64,11 +64,12 @@ class MetasdError(RuntimeError):
 
 
 _lib = None
+_call = None   # the calls of a round without ctypes' cost (metasd_call.c), where that module is built
 
 
 def load_library(path: Optional[str] = None):
     """dlopen libmetasd.so and declare the signatures.  Raises if the library has not been built."""
-    global _lib
+    global _lib, _call
     if _lib is not None and path is None:
         return _lib
     path = path or LIB_PATH
@@ -102,7 +103,12 @@ def load_library(path: Optional[str] = None):
                                           C.c_uint32, vp, vp, vp, vp, vp]
     lib.metasd_strerror.argtypes = [C.c_int]
     lib.metasd_strerror.restype = C.c_char_p
+    lib.verify_noalloc_at = C.cast(lib.metasd_verify_noalloc, C.c_void_p).value
     if path == LIB_PATH:
+        try:
+            from . import _call
+        except ImportError:
+            pass
         _lib = lib
     return lib
 
@@ -178,11 +184,15 @@ class MetaSD:
         self.device = torch.device("cuda", device)
         self._ctx = C.c_void_p()
         _check(self.lib.metasd_init(C.byref(self._ctx), C.byref(cfg)), "metasd_init")
+        self._at = self._ctx.value
+        self._verify_at, self._select_at = (C.cast(fn, C.c_void_p).value for fn in (self.lib.metasd_verify, self.lib.metasd_select))
+        self._max_batch = max_batch
 
     def close(self):
         if getattr(self, "_ctx", None) is not None and self._ctx.value:
             self.lib.metasd_destroy(self._ctx)
             self._ctx = C.c_void_p()
+            self._at = None
 
     def __del__(self):
         try:
@@ -196,10 +206,16 @@ class MetaSD:
         _check(self.lib.metasd_reset(self._ctx, _ptr(seq_ids), n, _stream(self.device)), "metasd_reset")
 
     def select(self, batch: Optional[int] = None, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        batch = self.cfg.max_batch if batch is None else batch
+        batch = self._max_batch if batch is None else batch
         if out is None:
             out = torch.empty(batch, dtype=torch.int32, device=self.device)
-        _check(self.lib.metasd_select(self._ctx, batch, _ptr(out), _stream(self.device)), "metasd_select")
+        rc = NotImplemented
+        if _call is not None:
+            rc = _call.select(self._select_at, self._at, batch, out, _stream(self.device))
+        if rc is NotImplemented:
+            rc = self.lib.metasd_select(self._ctx, batch, _ptr(out), _stream(self.device))
+        if rc != OK:
+            raise MetasdError(rc, "metasd_select")
         return out
 
     def verify(self, target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor],
@@ -216,12 +232,19 @@ class MetaSD:
                                torch.empty(B, dtype=torch.float32, device=self.device))
         if want_diag and out.diag is None:
             out.diag = torch.zeros((B, k, 5), dtype=torch.float32, device=self.device)
-        rc = self.lib.metasd_verify(
-            self._ctx, B, k, _ptr(target_logits), _ptr(draft_logits), _ptr(drafter_table),
-            _ptr(draft_tokens), token_arm_stride, temperature, seed,
-            _ptr(out.accepted_len), _ptr(out.next_token), _ptr(out.reward), _ptr(out.diag),
-            _stream(self.device))
-        _check(rc, "metasd_verify")
+        rc = NotImplemented
+        if _call is not None:
+            rc = _call.verify(self._verify_at, self._at, B, k, target_logits, draft_logits, drafter_table, draft_tokens,
+                              token_arm_stride, temperature, seed, out.accepted_len, out.next_token, out.reward, out.diag,
+                              _stream(self.device))
+        if rc is NotImplemented:
+            rc = self.lib.metasd_verify(
+                self._ctx, B, k, _ptr(target_logits), _ptr(draft_logits), _ptr(drafter_table),
+                _ptr(draft_tokens), token_arm_stride, temperature, seed,
+                _ptr(out.accepted_len), _ptr(out.next_token), _ptr(out.reward), _ptr(out.diag),
+                _stream(self.device))
+        if rc != OK:
+            raise MetasdError(rc, "metasd_verify")
         return out
 
     def verify_host(self, target_logits: torch.Tensor, draft_logits: torch.Tensor,
@@ -280,7 +303,15 @@ def verify_noalloc(target_logits: torch.Tensor, draft_logits: torch.Tensor, draf
     library; the caller provides every buffer.  Returns the library's error code."""
     B, kp1, V = target_logits.shape
     dev = target_logits.device
-    return load_library().metasd_verify_noalloc(
+    lib = load_library()
+    if _call is not None:
+        rc = _call.verify_noalloc(
+            lib.verify_noalloc_at, B, kp1 - 1, V, DTYPES[target_logits.dtype], target_logits, draft_logits, draft_tokens,
+            temperature, reward_temperature, reward_kind, seed, sequence_base, round_, accepted_len, next_token, reward,
+            status, _stream(dev))
+        if rc is not NotImplemented:
+            return rc
+    return lib.metasd_verify_noalloc(
         B, kp1 - 1, V, DTYPES[target_logits.dtype], _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens),
         temperature, reward_temperature, reward_kind, seed,
         sequence_base, round_, _ptr(accepted_len), _ptr(next_token), _ptr(reward),
