@@ -1200,11 +1200,11 @@ static StagedShape staged_shape(int dtype, long long bytes, long long units, int
 // 223 (B = 256, k = 7, V = 128256), 180: 635 and 643 (B = 512, k = 8, V = 152064); 512/4/1 89: 462 and 451 (B = 1024, k = 8,
 // V = 50264), 113: 103.0 and 103.9, 142: 169 and 181 (B = 400, k = 5, V = 80000); 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
 // 76: 242 and 226 (256/6/4: B = 512, k = 4, V = 64000), 293 and 263 (256/6/2: B = 1024, k = 5, V = 32000), 95: 78.7 and 79.6, 114: 261 and 333
-// (128/6/8: B = 256, k = 5, V = 128256).  Short rows never come near it (128/4/1, 256/4/1).
+// (128/6/8: B = 256, k = 5, V = 128256).  Shapes of short rows are not built there.
 static bool hinted_pays(int dtype, long long bytes, long long units, const StagedShape &s, int n_sm)
 {
     const bool fp32 = dtype == METASD_FP32;
-    if (s.threads < 512 && s.stages == 4) return false;
+    if (!hinted_built(dtype, s.threads, s.stages, s.cluster)) return false;
     const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : s.stages == 4 ? 3 : 1024 / s.threads) / s.cluster;
     return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.stages == 6 && s.cluster == 1 ? 165 : 115) * 1000000ll;
 }

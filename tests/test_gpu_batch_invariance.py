@@ -43,7 +43,8 @@ def test_results_do_not_depend_on_the_batch(dtype, V, B):
             assert torch.equal(x[first:last], y)
 
 
-@pytest.mark.parametrize("V", [80008, 152064])
-def test_results_do_not_depend_on_the_kernel_of_long_launches(V):
-    """1200 bf16 row pairs and bonus rows, more than L2 holds, which the kernel with L2 policies takes; 141 of them by the other."""
-    test_results_do_not_depend_on_the_batch("bf16", V, 400)
+@pytest.mark.parametrize("dtype,V", [("bf16", 80008), ("bf16", 152064), ("fp32", 20400)])
+def test_results_do_not_depend_on_the_kernel_of_long_launches(dtype, V):
+    """1200 row pairs and bonus rows, more than L2 holds, which the kernel with L2 policies takes where it has their shape (fp32,
+    V = 20400: it has not); 141 of them by the other."""
+    test_results_do_not_depend_on_the_batch(dtype, V, 400)
