@@ -385,11 +385,11 @@ bool hinted_built(int dtype, int threads, int stages, int cluster)
 }
 
 template <typename LT>
-static cudaError_t prepare_t(int threads, int stages, int cluster)
+static cudaError_t prepare_t(int threads, int stages, int cluster, int warps)
 {
     cudaError_t e = cudaSuccess;
 #define X(T, D, M, BL, C) \
-    if (e == cudaSuccess && (threads == 0 || (threads == T && stages == D && cluster == C))) \
+    if (e == cudaSuccess && (threads == 0 ? warps == 0 || warps == T / 32 * C : threads == T && stages == D && cluster == C)) \
         e = cudaFuncSetAttribute(row_stats_hinted_kernel<LT, D, T, M, BL, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
     if constexpr (sizeof(LT) == 2) { METASD_HINTED_BF16_SHAPES(X) }
     else { METASD_HINTED_FP32_SHAPES(X) }
@@ -398,9 +398,9 @@ static cudaError_t prepare_t(int threads, int stages, int cluster)
     return e;
 }
 
-cudaError_t hinted_prepare(int dtype, int threads, int stages, int cluster)
+cudaError_t hinted_prepare(int dtype, int threads, int stages, int cluster, int warps)
 {
-    return dtype == METASD_BF16 ? prepare_t<__nv_bfloat16>(threads, stages, cluster) : prepare_t<float>(threads, stages, cluster);
+    return dtype == METASD_BF16 ? prepare_t<__nv_bfloat16>(threads, stages, cluster, warps) : prepare_t<float>(threads, stages, cluster, warps);
 }
 
 template <typename LT>

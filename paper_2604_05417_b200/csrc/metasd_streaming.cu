@@ -188,14 +188,17 @@ struct __align__(16) PartRecord {
 // A vector of the target row that holds a larger logit than any before it in the warp's range: rare (a warp's n-th trip
 // brings a new maximum with probability about 1/n), so the whole warp takes this branch together.  Where the largest logit
 // is, greedy rounds alone need to know.
-template <typename LT>
+template <typename LT, bool FIRST>   // FIRST: of the range; nothing has been added up
 __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int vec, float c, bool index)
 {
     constexpr int VEC = Logit<LT>::VEC;
     const float cm = Logit<LT>::max_of(raw), top = warp_max_f(cm);
     const bool first_finite = w.best == -INFINITY;   // the reference may still be a stand-in, on either side of `top`
     const float ref = -rintf(top * c);
-    if (ref < w.ref || first_finite) {
+    if (FIRST) {
+        w.ref = ref;
+        w.nm = pack2(ref);
+    } else if (ref < w.ref || first_finite) {
         const uint64_t shrink = pack2(exp2_whole(ref - w.ref));
         if (!first_finite) w.a = mul2(w.a, shrink);
         w.b = mul2(w.b, shrink);
@@ -223,10 +226,12 @@ __device__ __forceinline__ void new_best(WarpSums<LT> &w, const uint4 &raw, int 
 // B = 96 53.3 -> 49.1, V = 50264, B = 192 ragged 59.8 -> 56.6, V = 152064, B = 4 23.1 -> 21.5, fp32, V = 32001, B = 8
 // 14.0 -> 12.7.
 //
+// COMPACT: without the groups (compact_form).
+//
 // CL > 1: a thread-block cluster of CL CTAs shares one row (pair), every CTA a contiguous CL-th of its trips.  The warps
 // of all CTAs exchange their sweep-1 records through distributed shared memory and every warp merges them in the same
 // order, so all hold the same normalisers; each sweeps its part again.
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED, bool COMPACT>
 __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const VerifyParams p)
 {
     static_assert(D >= 2, "at least two stages");
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         // Trip n, whose vectors have landed.
         auto consume = [&](int n, uint32_t src) {
             const uint4 ra = fetch(src, lead_a);
-            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT>(w, ra, v0 + 32 * n, c, p.greedy != 0);
+            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) new_best<LT, false>(w, ra, v0 + 32 * n, c, p.greedy != 0);
             w.a = Logit<LT>::add_exp(w.a, ra, c2, w.nm);
             if (BOTH) w.b = Logit<LT>::add_exp(w.b, fetch(src + ROW_STRIDE, lead_d), c2, w.nm);
         };
@@ -426,18 +431,19 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
                 __syncwarp();
                 if (n_full <= 0) mask_ragged(0, slot0, BOTH);
             }
-            float top = warp_max_f(Logit<LT>::max_of(fetch(slot0, lead_a)));
-            if (!(top > METASD_NEG_BIG)) {
-                top = BOTH ? warp_max_f(Logit<LT>::max_of(fetch(slot0 + ROW_STRIDE, lead_d))) : 0.f;
-                if (!(top > METASD_NEG_BIG)) top = 0.f;
+            const uint4 ra = fetch(slot0, lead_a);
+            if (__any_sync(FULL, Logit<LT>::any_above(ra, w.cmp))) {
+                new_best<LT, true>(w, ra, v0, c, p.greedy != 0);
+            } else if (BOTH) {
+                const float top = warp_max_f(Logit<LT>::max_of(fetch(slot0 + ROW_STRIDE, lead_d)));
+                if (top > METASD_NEG_BIG) w.ref = -rintf(top * c);
+                w.nm = pack2(w.ref);
             }
-            w.ref = -rintf(top * c);
-            w.nm = pack2(w.ref);
         }
         // Trip n asks for the trip D - 1 ahead, then works on its own vectors (slot n mod D).  Groups of D trips whose
         // requests all lie inside the row carry no checks, and their slots are constants.
         int n = 0;
-        for (; n + 2 * D - 2 < n_full; n += D) {
+        for (; !COMPACT && n + 2 * D - 2 < n_full; n += D) {
 #pragma unroll
             for (int u = 0; u < D; ++u) {
                 meet();
@@ -503,7 +509,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
             part_ref[q] = r.ref;
             part_sum[q] = upper ? r.sum_b : r.sum_a;
             if (r.best > METASD_NEG_BIG) ref_a = fminf(ref_a, r.ref);   // a part without a finite target logit has a stand-in
-            rm = better(rm, ArgMax{r.best, r.best_i});
+            if (p.greedy) rm = better(rm, ArgMax{r.best, r.best_i});
         }
     }
     ref_a = -warp_max_f(-ref_a);
@@ -518,10 +524,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     for (int o = HALF / 2; o > 0; o >>= 1) merged += __shfl_xor_sync(FULL, merged, o);
     sum_a = __shfl_sync(FULL, merged, 0);
     sum_b = __shfl_sync(FULL, merged, 16);
-    {
+    if (p.greedy) {
         const float best = warp_max_f(rm.v);
         rm.i = __reduce_min_sync(FULL, rm.v == best ? rm.i : 0x7FFFFFFF);
-        rm.v = best;
     }
     float ref_b = ref_a;
     bool bad_b = false;
@@ -588,7 +593,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         RowStats r;
         r.ref_a = ref_a; r.sum_a = sum_a; r.ref_b = ref_b; r.sum_b = sum_b;
         r.argmax_a = rm.i;
-        const bool bad_a = !(sum_a > 0.f) || !(sum_a < INFINITY) || !(rm.v < INFINITY);
+        const bool bad_a = !(sum_a > 0.f) || !(sum_a < INFINITY);   // a +Inf logit makes the sum NaN: its own exponent is Inf - Inf
         r.flags = bad_a || bad_b ? METASD_STATUS_NONFINITE : 0u;
         p.stats[row] = r;
     }
@@ -599,9 +604,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // would be rounded at that size, and every term of the draft row scaled by the error, up to 7e-7).
     float weight = sum2(w.a), shared = 0.f;
     if (pair) {
-        const float rho = sum_a / sum_b, whole = rintf(log2f(rho));
+        // The logarithm's whole part: the exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2).
+        const int rho = __float_as_int(sum_a / sum_b), whole = (rho - 0x3F3504F3) >> 23;
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
-        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(log2f(rho * exp2_whole(-whole)));
+        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + (float)whole + (w.ref - ref_a)), lg = pack2(log2f(__int_as_float(rho - whole * (1 << 23))));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last).
@@ -619,7 +625,7 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         const char *a_next = a4 + 512 * (n - D), *d_next = d4 + 512 * (n - D);
 #pragma unroll 1
         while (n >= 0) {
-            if (src == slot0 + (D - 1) * STAGE_STRIDE) {
+            if (!COMPACT && src == slot0 + (D - 1) * STAGE_STRIDE) {
                 for (; n >= 2 * D - 1 + (head ? 1 : 0); n -= D) {
 #pragma unroll
                     for (int u = 0; u < D; ++u) {
@@ -655,11 +661,11 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     }
 }
 
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED, bool COMPACT>
 static cudaError_t launch_staged(const VerifyParams &p, unsigned units, int n_sm, cudaStream_t stream)
 {
     const StagedLaunch how = staged_launch(units, CL, MINB, STAGED_SMEM<D, THREADS, SHIFTED>, n_sm);
-    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>, units * CL, THREADS, how.smem, CL, how.chained, stream, p);
+    return launch_kernel(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED, COMPACT>, units * CL, THREADS, how.smem, CL, how.chained, stream, p);
 }
 
 // -------------------------------------------------------------------------------------------
@@ -1091,18 +1097,20 @@ __global__ void __launch_bounds__(DRAW_THREADS + 32, GREEDY ? 3 : DRAW_THREADS =
 constexpr int DRAW_THREADS = 256, DRAW_THREADS_WIDE = 512;
 constexpr long long DRAW_PART_BYTES = 16 * 1024;
 
-// The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row).  Those that
-// staged_shape() picks, by logit type; a configuration can ask for METASD_STAGED_PINNED_SHAPES.
+// The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row), and which forms of each
+// staged_shape() and compact_form() reach: aligned rows with and without groups of trips, SHIFTED ones with and without.  A
+// configuration can ask for METASD_STAGED_PINNED_SHAPES, of which these here are the SHIFTED ones, with groups.
 #define METASD_STAGED_BF16_SHAPES(X) \
-    X(128, 4, 12, true, 1) X(256, 4, 6, true, 1) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) \
-    X(256, 6, 4, true, 2) X(128, 6, 6, true, 4)
+    X(128, 4, 12, true, 1, 0, 1, 1, 0) X(256, 4, 6, true, 1, 0, 1, 1, 0) X(512, 6, 2, true, 1, 1, 1, 1, 1) X(512, 4, 3, true, 1, 0, 1, 1, 0) \
+    X(256, 6, 4, true, 2, 1, 1, 1, 1) X(128, 6, 6, true, 4, 1, 1, 1, 1)
 #define METASD_STAGED_FP32_SHAPES(X) \
-    X(256, 4, 6, true, 1) X(256, 6, 4, true, 1) X(512, 6, 2, true, 1) X(256, 6, 4, true, 2) X(128, 6, 6, true, 4) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
+    X(256, 4, 6, true, 1, 1, 1, 1, 0) X(256, 6, 4, true, 1, 1, 0, 1, 1) X(512, 6, 2, true, 1, 1, 1, 1, 1) X(256, 6, 4, true, 2, 1, 1, 1, 1) \
+    X(128, 6, 6, true, 4, 1, 1, 1, 1) X(1024, 6, 1, false, 1, 1, 0, 1, 0) X(256, 6, 4, true, 4, 1, 0, 1, 0) X(128, 6, 6, true, 8, 1, 0, 1, 0)
 
-template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED>
+template <typename LT, int D, int THREADS, int MINB, bool BONUS_LAST, int CL, bool SHIFTED, bool COMPACT>
 static cudaError_t prepare_staged()
 {
-    return cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED>,
+    return cudaFuncSetAttribute(row_stats_staged_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL, SHIFTED, COMPACT>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
 }
 
@@ -1112,16 +1120,18 @@ template <typename LT>
 static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int warps, bool aligned)
 {
     if (threads) {
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C, true>();
+#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C, true, false>();
         METASD_STAGED_PINNED_SHAPES(X)
 #undef X
         return cudaErrorNotSupported;
     }
     cudaError_t e = cudaSuccess;
-#define X(T, D, M, BL, C) \
-    if (e == cudaSuccess && (warps == 0 || warps == T / 32 * C)) { \
-        e = prepare_staged<LT, D, T, M, BL, C, true>(); \
-        if (e == cudaSuccess && aligned) e = prepare_staged<LT, D, T, M, BL, C, false>(); \
+#define X(T, D, M, BL, C, AG, AC, SG, SC) \
+    if (warps == 0 || warps == T / 32 * C) { \
+        if constexpr (AG) { if (e == cudaSuccess && aligned) e = prepare_staged<LT, D, T, M, BL, C, false, false>(); } \
+        if constexpr (AC) { if (e == cudaSuccess && aligned) e = prepare_staged<LT, D, T, M, BL, C, false, true>(); } \
+        if constexpr (SG) { if (e == cudaSuccess) e = prepare_staged<LT, D, T, M, BL, C, true, false>(); } \
+        if constexpr (SC) { if (e == cudaSuccess) e = prepare_staged<LT, D, T, M, BL, C, true, true>(); } \
     }
     if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
     else { METASD_STAGED_FP32_SHAPES(X) }
@@ -1129,24 +1139,48 @@ static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int wa
     return e;
 }
 
+static long long row_bytes(int dtype, int vocab) { return (long long)vocab * (dtype == METASD_BF16 ? 2 : 4); }
+
+// Whether a warp's trips all go through the rolled loops.  Groups of trips with constant slots issue a tenth fewer instructions, but
+// their code, three quarters of the kernel's, is fetched for it, and few warps wait for it: short ranges do without.  Us a round with
+// groups and without, by trips a warp: bf16 8: 10.5 and 9.4 (V = 8000, B = 1), 12.2 and 10.8 (B = 64), 63.1 and 61.4 (B = 1024); 10.1 and 9.6
+// (V = 32000, B = 1), 54.7 and 52.6 (B = 256); 12: 11.7 and 11.2 (V = 50264, B = 1), 62.2 and 61.0 (B = 200); 16: 35.5 and 33.2 (V = 64000,
+// B = 64); 20: 13.2 and 13.4 (V = 80000, B = 4), 40.1 and 38.8 (B = 64); 24: 14.1 and 14.9 (V = 100000, B = 4); 37: 20.5 and 23.7
+// (V = 152064, B = 4); fp32 8: 42.2 and 40.8 (V = 8000, B = 512); 16: 10.2 and 10.6 (V = 32000, B = 1), 24.2 and 23.5 (B = 64).  SHIFTED: 6 stages
+// 14.5 and 13.6 (V = 50257, B = 4), 13.5 and 12.5 (fp32, V = 32001, B = 8), 4 stages, at 40 registers, 15.9 and 18.7 (V = 16001, B = 64).
+static bool compact_form(int dtype, int vocab, bool aligned, const RowGeometry &geo)
+{
+    const long long trips = (row_bytes(dtype, vocab) + 511) / 512;
+    const int warps = geo.threads / 32 * geo.cluster;
+    if (!aligned) return geo.stages == 6 && warps <= 16 && trips <= 16 * warps;
+    return trips <= (dtype == METASD_FP32 ? 12 : 16) * warps;
+}
+
 template <typename LT>
-static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo, cudaStream_t stream)
+static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo, bool pinned, cudaStream_t stream)
 {
     constexpr int dtype = sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32;
     if (p.vector_ok && geo.hinted) return launch_row_stats_hinted(p, dtype, geo, stream);
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
-#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) \
-        return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false>(p, units, geo.n_sm, stream) : launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
+    if (pinned) {
+#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) return launch_staged<LT, D, T, M, BL, C, true, false>(p, units, geo.n_sm, stream);
+        METASD_STAGED_PINNED_SHAPES(X)
+#undef X
+        return cudaErrorNotSupported;
+    }
+    const bool compact = compact_form(dtype, p.V, p.vector_ok, geo);
+#define X(T, D, M, BL, C, AG, AC, SG, SC) \
+    if (geo.threads == T && geo.stages == D && geo.cluster == C) { \
+        if constexpr (AG) { if (p.vector_ok && !compact) return launch_staged<LT, D, T, M, BL, C, false, false>(p, units, geo.n_sm, stream); } \
+        if constexpr (AC) { if (p.vector_ok && compact) return launch_staged<LT, D, T, M, BL, C, false, true>(p, units, geo.n_sm, stream); } \
+        if constexpr (SG) { if (!p.vector_ok && !compact) return launch_staged<LT, D, T, M, BL, C, true, false>(p, units, geo.n_sm, stream); } \
+        if constexpr (SC) { if (!p.vector_ok && compact) return launch_staged<LT, D, T, M, BL, C, true, true>(p, units, geo.n_sm, stream); } \
+    }
     if constexpr (sizeof(LT) == 2) { METASD_STAGED_BF16_SHAPES(X) }
     else { METASD_STAGED_FP32_SHAPES(X) }
 #undef X
-#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) return launch_staged<LT, D, T, M, BL, C, true>(p, units, geo.n_sm, stream);
-    METASD_STAGED_PINNED_SHAPES(X)
-#undef X
     return cudaErrorNotSupported;
 }
-
-static long long row_bytes(int dtype, int vocab) { return (long long)vocab * (dtype == METASD_BF16 ? 2 : 4); }
 
 // Warps that share a row, by its length and type alone: which tokens a warp adds up, relative to what and in which order,
 // and the parts that a draw is made from, are then the same whatever else is in the launch, and a sequence's results do not
@@ -1183,7 +1217,7 @@ static StagedShape staged_shape(int dtype, long long bytes, long long units, int
     const bool fp32 = dtype == METASD_FP32;
     switch (row_warps(dtype, bytes)) {
     case 4: return {128, 4, 1};
-    case 8: return {256, fp32 && bytes >= 48 * 1000 && units > 4 * n_sm ? 6 : 4, 1};
+    case 8: return {256, fp32 && bytes > 48 * 1024 && units > 4 * n_sm ? 6 : 4, 1};
     case 16:
         if (units * 4 <= n_sm || (units <= n_sm && bytes < 140 * 1000)) return {128, 6, 4};
         if (fp32 ? bytes >= 150 * 1000 : units <= (bytes < 100 * 1000 ? 3 : 7) * n_sm) return {256, 6, 2};
@@ -1283,9 +1317,9 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         geo->hinted = 1;
     }
     if ((e = dtype == METASD_BF16 ? prepare_small_kernels<__nv_bfloat16>() : prepare_small_kernels<float>()) != cudaSuccess) return e;
-    if ((e = hinted_prepare(dtype, geo->threads, geo->stages, geo->cluster)) != cudaSuccess) return e;
     const int warps = cfg.vocab > 0 ? row_warps(dtype, row_bytes(dtype, cfg.vocab)) : 0;
     const bool aligned = row_bytes(dtype, cfg.vocab) % 16 == 0;
+    if (aligned && (e = hinted_prepare(dtype, geo->threads, geo->stages, geo->cluster, warps)) != cudaSuccess) return e;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, warps, aligned)
                                 : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, warps, aligned);
 }
@@ -1300,7 +1334,7 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
     p.k_inverse = inverse_of((uint32_t)p.k);
     p.k1_inverse = inverse_of((uint32_t)p.k + 1u);
     if (geo.kernel == METASD_ROWS_STAGED) {
-        e = launch_staged_t<LT>(p, geo, stream);
+        e = launch_staged_t<LT>(p, geo, context_geo.threads != 0, stream);
     } else if (!p.vector_ok) {
         row_stats_kernel<LT, false><<<dim3(p.k + 1, p.batch), K1_THREADS, 0, stream>>>(p);
     } else if (geo.kernel == METASD_ROWS_BULK) {

@@ -185,3 +185,13 @@ def test_alignment_of_rows_that_hardly_overlap(dtype, kernel):
         torch.testing.assert_close(res.reward.double(), want, rtol=1e-5, atol=0)
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 65536), ("bf16", 65544), ("bf16", 65519), ("bf16", 65553), ("fp32", 12288), ("fp32", 12292),
+                                     ("fp32", 24576), ("fp32", 24580), ("fp32", 32765), ("fp32", 32771)])
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+def test_ranges_on_both_sides_of_the_rolled_form(dtype, V, temperature):
+    """Ranges of 16 (fp32: 12) trips a warp, which go through rolled loops alone, and of one more."""
+    from _harness import run_lockstep
+    c = run_lockstep(workload(V=V, dtype=dtype, temperature=temperature), rounds=3, seed=V % 83, path=M.PATH_STREAMING)
+    assert c["rounds"] == 3 and c["status"] == 0
