@@ -482,6 +482,8 @@ __device__ __forceinline__ void cluster_sync_all()
 }
 // The two halves of that barrier on their own (every thread of every CTA of the cluster runs both, in this order).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// The arrival of a thread that has nothing to publish: no fence.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of the same shared-memory variable in the CTA of the given cluster rank.
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t local, uint32_t rank)

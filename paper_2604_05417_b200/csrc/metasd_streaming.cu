@@ -266,8 +266,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // (the same for every CTA of a cluster: none of them reaches a cluster barrier)
     if (j > kb || (BONUS_LAST && unit < first_bonus && j == kb)) return;
     const bool pair = j < kb;
-    // a peer's shared memory may be written once that peer is running: every CTA says so here and checks it after sweep 1
-    if (CL > 1) cluster_arrive();
+    // a peer's shared memory may be written once that peer is running: every CTA says so here, without a fence, and checks it
+    // after sweep 1 (with one: V = 32000, B = 1 11.1 us a round instead of 10.7, B = 64 23.0 instead of 22.65)
+    if (CL > 1) cluster_arrive_relaxed();
 
     const LT *a_row = reinterpret_cast<const LT *>(p.target) + ((size_t)b * (p.k + 1) + j) * p.V;
     const LT *d_row = pair ? draft_rows<LT>(p, b) + ((size_t)b * p.k + j) * p.V : a_row;
