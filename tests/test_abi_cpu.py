@@ -143,3 +143,20 @@ def test_current_stream_without_torchs_private_lookup(monkeypatch):
     assert asked == [torch.device("cpu"), torch.device("cuda", 3)]
     monkeypatch.setattr(M, "_raw_stream", lambda index: 100 + index)
     assert M._stream(torch.device("cuda", 3)) == 103
+
+
+def test_calls_of_a_round_convert_as_ctypes_does(lib):
+    """The extension module's calls: the library's own answers, NotImplemented for what it leaves to ctypes."""
+    if M._call is None:
+        pytest.skip("not built for this interpreter")
+    t = torch.zeros(3, dtype=torch.int32)
+    select, verify = (C.cast(fn, C.c_void_p).value for fn in (lib.metasd_select, lib.metasd_verify))
+    assert M._call.select(select, None, 2 ** 32 + 5, t, None) == lib.metasd_select(None, 5, M._ptr(t), None) == M.ERR_INVALID_ARGUMENT
+    assert M._call.select(select, None, 5.0, t, None) is NotImplemented
+    with pytest.raises(AttributeError):
+        M._call.select(select, None, 5, "not a tensor", None)
+    with pytest.raises(TypeError):
+        M._call.select(select, None, 5)
+    assert M._call.verify(verify, None, 1, 4, t, None, t, t, -1, 1, 2 ** 64 - 1, t, t, t, None, None) == M.ERR_INVALID_ARGUMENT
+    assert M._call.verify_noalloc(lib.verify_noalloc_at, 0, 1, 8, M.BF16, t, t, t, 1.0, 1.0, 0, 0, 0, 0, t, t, t, None, None) == M.ERR_INVALID_ARGUMENT
+    assert M._call.verify_noalloc(lib.verify_noalloc_at, 1, 1, 8, M.BF16, t, t, t, "1", 1.0, 0, 0, 0, 0, t, t, t, None, None) is NotImplemented
