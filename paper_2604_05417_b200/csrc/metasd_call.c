@@ -1,8 +1,9 @@
 /* The calls of a round as Python sees them, for the binding: argument conversion and the call, nothing else.
  *
  * The functions are those of libmetasd.so (include/metasd.h), whose addresses come with every call.  Conversions are ctypes'
- * own for the same signatures (whole numbers are cut to their width, None is a null pointer), except that a tensor's
- * data_ptr() is called here.  Arguments of other types are left to ctypes (NotImplemented), which says what is wrong with them.
+ * own for the same signatures (whole numbers are cut to their width, None is a null pointer), and a tensor's data_ptr() is
+ * called here as the binding does for ctypes: a number in a tensor's place is refused, with the module and without.  Arguments
+ * of other types are left to ctypes (NotImplemented), which says what is wrong with them.
  * The interpreter lock is released around the call, as ctypes does.
  *
  * What it is for: a round of a few sequences is as long as its host calls.  One sequence, V = 32000, verify and select: ctypes'
@@ -17,20 +18,23 @@
 static PyObject *data_ptr_name;
 
 /* 1: done; 0: not a type handled here; -1: an exception is set. */
-static int as_pointer(PyObject *o, void **out)
+static int as_address(PyObject *o, void **out)
+{
+    if (o != Py_None && !PyLong_CheckExact(o)) return 0;
+    *out = o == Py_None ? NULL : (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
+    return 1;
+}
+
+/* What has no data_ptr(), a number for one, is an AttributeError. */
+static int as_tensor(PyObject *o, void **out)
 {
     if (o == Py_None) {
         *out = NULL;
         return 1;
     }
-    if (PyLong_CheckExact(o)) {
-        *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
-        return 1;
-    }
     PyObject *at = PyObject_CallMethodNoArgs(o, data_ptr_name);
     if (!at) return -1;
-    const int ok = PyLong_CheckExact(at);
-    if (ok) *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(at);
+    const int ok = as_address(at, out);
     Py_DECREF(at);
     return ok;
 }
@@ -53,11 +57,13 @@ static int as_float(PyObject *o, float *out)
 
 #define MOST 20
 
-/* Converts the arguments by their kinds: p pointer, i whole number, f float.  Returns as as_pointer does. */
+/* Converts the arguments by their kinds: a address (of a function, a context or a stream), t tensor, i whole number, f float.
+ * Returns as as_address does. */
 static int convert(const char *kinds, PyObject *const *args, Py_ssize_t n, void **p, uint64_t *i, float *f)
 {
     for (Py_ssize_t a = 0; a < n; ++a) {
-        const int r = kinds[a] == 'p' ? as_pointer(args[a], p + a) : kinds[a] == 'i' ? as_bits(args[a], i + a) : as_float(args[a], f + a);
+        const int r = kinds[a] == 't' ? as_tensor(args[a], p + a) : kinds[a] == 'a' ? as_address(args[a], p + a) :
+                      kinds[a] == 'i' ? as_bits(args[a], i + a) : as_float(args[a], f + a);
         if (r != 1) return r;
     }
     return 1;
@@ -78,7 +84,7 @@ static int convert(const char *kinds, PyObject *const *args, Py_ssize_t n, void 
 
 static PyObject *call_verify(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
-    CONVERTED("ppiippppifippppp");
+    CONVERTED("aaiittttifitttta");
     int (*verify)(void *, int32_t, int32_t, const void *, const void *, const void *, const int32_t *, int64_t, float, uint64_t,
                   int32_t *, int32_t *, float *, metasd_diag *, void *) = p[0];
     Py_BEGIN_ALLOW_THREADS
@@ -90,7 +96,7 @@ static PyObject *call_verify(PyObject *self, PyObject *const *args, Py_ssize_t n
 
 static PyObject *call_select(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
-    CONVERTED("ppipp");
+    CONVERTED("aaita");
     int (*select)(void *, int32_t, int32_t *, void *) = p[0];
     Py_BEGIN_ALLOW_THREADS
     rc = select(p[1], (int32_t)i[2], p[3], p[4]);
@@ -100,7 +106,7 @@ static PyObject *call_select(PyObject *self, PyObject *const *args, Py_ssize_t n
 
 static PyObject *call_verify_noalloc(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
-    CONVERTED("piiiipppffiiiippppp");
+    CONVERTED("aiiiitttffiiiitttta");
     int (*verify)(int32_t, int32_t, int32_t, int32_t, const void *, const void *, const int32_t *, float, float, int32_t, uint64_t,
                   uint32_t, uint32_t, int32_t *, int32_t *, float *, uint32_t *, void *) = p[0];
     Py_BEGIN_ALLOW_THREADS

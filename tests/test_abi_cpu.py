@@ -160,3 +160,41 @@ def test_calls_of_a_round_convert_as_ctypes_does(lib):
     assert M._call.verify(verify, None, 1, 4, t, None, t, t, -1, 1, 2 ** 64 - 1, t, t, t, None, None) == M.ERR_INVALID_ARGUMENT
     assert M._call.verify_noalloc(lib.verify_noalloc_at, 0, 1, 8, M.BF16, t, t, t, 1.0, 1.0, 0, 0, 0, 0, t, t, t, None, None) == M.ERR_INVALID_ARGUMENT
     assert M._call.verify_noalloc(lib.verify_noalloc_at, 1, 1, 8, M.BF16, t, t, t, "1", 1.0, 0, 0, 0, 0, t, t, t, None, None) is NotImplemented
+
+
+def test_calls_of_a_round_refuse_numbers_where_tensors_are_due(lib, monkeypatch):
+    """A plain integer is an address where the binding passes one (function, context, stream) and nowhere else, with the
+    extension module and without it."""
+    t = torch.zeros((1, 2, 8))
+    numbers = (12345, 0, True)
+
+    def noalloc(**kw):
+        call = dict(draft_logits=t, draft_tokens=t, accepted_len=t, next_token=t, reward=t, status=t)
+        call.update(kw)
+        # no sequences: the library itself refuses the call before it looks at any address
+        return M.verify_noalloc(torch.zeros((0, 2, 8)), call["draft_logits"], call["draft_tokens"], 1.0, 1, 0, call["accepted_len"],
+                                call["next_token"], call["reward"], status=call["status"])
+
+    monkeypatch.setattr(M, "_stream", lambda device: 0)
+    for module in {M._call, None}:
+        monkeypatch.setattr(M, "_call", module)
+        assert noalloc() == M.ERR_INVALID_ARGUMENT
+        for name in ("draft_logits", "draft_tokens", "accepted_len", "next_token", "reward", "status"):
+            for number in numbers:
+                with pytest.raises(AttributeError):
+                    noalloc(**{name: number})
+    if M._call is None:
+        return
+    monkeypatch.undo()
+    select, verify = (C.cast(fn, C.c_void_p).value for fn in (lib.metasd_select, lib.metasd_verify))
+    good = [verify, None, 1, 4, t, t, t, t, 0, 1.0, 1, t, t, t, t, 0]
+    assert M._call.verify(*good) == M.ERR_INVALID_ARGUMENT      # no context
+    for at in (4, 5, 6, 7, 11, 12, 13, 14):
+        for number in numbers:
+            with pytest.raises(AttributeError):
+                M._call.verify(*(good[:at] + [number] + good[at + 1:]))
+    with pytest.raises(AttributeError):
+        M._call.select(select, None, 1, 12345, 0)
+    # and a tensor is no address
+    assert M._call.select(select, t, 1, t, 0) is NotImplemented
+    assert M._call.select(select, None, 1, t, t) is NotImplemented
