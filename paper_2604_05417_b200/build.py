@@ -10,7 +10,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmetasd.so")
-CALL, CALL_SOURCE = os.path.join(HERE, "_call.so"), os.path.join(CSRC, "metasd_call.c")   # the binding's calls
+# the binding's calls, under a name that other interpreters do not load
+CALL, CALL_SOURCE = os.path.join(HERE, "_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so")), os.path.join(CSRC, "metasd_call.c")
 SOURCES = ["metasd_api.cu", "metasd_streaming.cu", "metasd_hinted.cu", "metasd_bulk.cu", "metasd_fused.cu", "metasd_noalloc.cu"]
 HEADERS = ["metasd_internal.h", "metasd_device.cuh", "metasd_staged.cuh", os.path.join(ROOT, "include", "metasd.h")]
 
@@ -24,15 +25,25 @@ def _stale() -> bool:
 
 
 def build_call(force: bool = False) -> bool:
-    """Compile the binding's calls for this interpreter; False where its headers are missing (the binding then uses ctypes)."""
-    include = sysconfig.get_paths()["include"]
-    if not os.path.exists(os.path.join(include, "Python.h")):
+    """Compile the binding's calls for this interpreter; False where its headers or a compiler are missing (the binding then uses
+    ctypes)."""
+    include, header = sysconfig.get_paths()["include"], os.path.join(ROOT, "include", "metasd.h")
+    untagged = os.path.join(os.path.dirname(CALL), "_call.so")   # an earlier build's, which any interpreter would load
+    if untagged != CALL and os.path.exists(untagged):
+        os.unlink(untagged)
+    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= max(os.path.getmtime(f) for f in (CALL_SOURCE, header)):
+        return True
+    tmp = CALL + ".tmp.%d" % os.getpid()
+    try:
+        if not os.path.exists(os.path.join(include, "Python.h")):
+            raise FileNotFoundError(include)
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-Werror=int-conversion", "-Werror=incompatible-pointer-types",
+                               "-shared", "-fPIC", "-I", include, "-I", os.path.dirname(header), CALL_SOURCE, "-o", tmp])
+    except FileNotFoundError:
+        if os.path.exists(CALL):
+            os.unlink(CALL)   # not what the sources say any more
         return False
-    if force or not os.path.exists(CALL) or os.path.getmtime(CALL_SOURCE) > os.path.getmtime(CALL):
-        tmp = CALL + ".tmp.%d" % os.getpid()
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", include,
-                               "-I", os.path.join(ROOT, "include"), CALL_SOURCE, "-o", tmp])
-        os.replace(tmp, CALL)
+    os.replace(tmp, CALL)
     return True
 
 

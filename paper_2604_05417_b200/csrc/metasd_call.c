@@ -85,8 +85,7 @@ static int convert(const char *kinds, PyObject *const *args, Py_ssize_t n, void 
 static PyObject *call_verify(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
     CONVERTED("aaiittttifitttta");
-    int (*verify)(void *, int32_t, int32_t, const void *, const void *, const void *, const int32_t *, int64_t, float, uint64_t,
-                  int32_t *, int32_t *, float *, metasd_diag *, void *) = p[0];
+    __typeof__(&metasd_verify) verify = p[0];   /* as the header declares it: the arguments are checked */
     Py_BEGIN_ALLOW_THREADS
     rc = verify(p[1], (int32_t)i[2], (int32_t)i[3], p[4], p[5], p[6], p[7], (int64_t)i[8], f[9], i[10], p[11], p[12], p[13], p[14],
                 p[15]);
@@ -97,7 +96,7 @@ static PyObject *call_verify(PyObject *self, PyObject *const *args, Py_ssize_t n
 static PyObject *call_select(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
     CONVERTED("aaita");
-    int (*select)(void *, int32_t, int32_t *, void *) = p[0];
+    __typeof__(&metasd_select) select = p[0];
     Py_BEGIN_ALLOW_THREADS
     rc = select(p[1], (int32_t)i[2], p[3], p[4]);
     Py_END_ALLOW_THREADS
@@ -107,8 +106,7 @@ static PyObject *call_select(PyObject *self, PyObject *const *args, Py_ssize_t n
 static PyObject *call_verify_noalloc(PyObject *self, PyObject *const *args, Py_ssize_t n)
 {
     CONVERTED("aiiiitttffiiiitttta");
-    int (*verify)(int32_t, int32_t, int32_t, int32_t, const void *, const void *, const int32_t *, float, float, int32_t, uint64_t,
-                  uint32_t, uint32_t, int32_t *, int32_t *, float *, uint32_t *, void *) = p[0];
+    __typeof__(&metasd_verify_noalloc) verify = p[0];
     Py_BEGIN_ALLOW_THREADS
     rc = verify((int32_t)i[1], (int32_t)i[2], (int32_t)i[3], (int32_t)i[4], p[5], p[6], p[7], f[8], f[9], (int32_t)i[10], i[11],
                 (uint32_t)i[12], (uint32_t)i[13], p[14], p[15], p[16], p[17], p[18]);

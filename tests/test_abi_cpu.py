@@ -3,6 +3,7 @@ arguments on the host, and fails loudly (no fallback) when there is no CUDA devi
 import ctypes as C
 import os
 import re
+import subprocess
 
 import pytest
 import torch
@@ -198,3 +199,35 @@ def test_calls_of_a_round_refuse_numbers_where_tensors_are_due(lib, monkeypatch)
     # and a tensor is no address
     assert M._call.select(select, t, 1, t, 0) is NotImplemented
     assert M._call.select(select, None, 1, t, t) is NotImplemented
+
+
+def test_the_extension_module_is_built_for_this_interpreter_from_what_is_there(monkeypatch, tmp_path):
+    """The file's name carries the interpreter's tag, a change of the C ABI's header compiles it anew, a declaration that the
+    module does not agree with fails to compile, and without a compiler the binding is left to ctypes."""
+    import shutil
+    import sysconfig
+    if not os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h")):
+        pytest.skip("no headers of this interpreter")
+    assert B.CALL.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    header = tmp_path / "include" / "metasd.h"
+    header.parent.mkdir()
+    shutil.copy(os.path.join(ROOT, "include", "metasd.h"), header)
+    monkeypatch.setattr(B, "ROOT", str(tmp_path))
+    monkeypatch.setattr(B, "CALL", str(tmp_path / os.path.basename(B.CALL)))
+    untagged = tmp_path / "_call.so"      # as earlier builds named it: any interpreter would load it
+    untagged.write_bytes(b"")
+    assert B.build_call() and os.path.exists(B.CALL) and not untagged.exists()
+    built = os.path.getmtime(B.CALL)
+    assert B.build_call() and os.path.getmtime(B.CALL) == built
+    os.utime(header, (built + 10, built + 10))
+    os.utime(B.CALL, (built - 10, built - 10))
+    assert B.build_call() and os.path.getmtime(B.CALL) > built - 10
+    text = header.read_text()
+    changed = text.replace("int metasd_select(metasd_ctx *ctx, int32_t batch,", "int metasd_select(metasd_ctx *ctx, double batch_share, int32_t batch,")
+    assert changed != text
+    header.write_text(changed)
+    with pytest.raises(subprocess.CalledProcessError):
+        B.build_call(force=True)
+    header.write_text(text)
+    monkeypatch.setenv("CC", str(tmp_path / "no_such_compiler"))
+    assert B.build_call(force=True) is False
