@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "libmetasd.so")
 # the binding's calls, under a name that other interpreters do not load
 CALL, CALL_SOURCE = os.path.join(HERE, "_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so")), os.path.join(CSRC, "metasd_call.c")
 SOURCES = ["metasd_api.cu", "metasd_streaming.cu", "metasd_hinted.cu", "metasd_bulk.cu", "metasd_fused.cu", "metasd_noalloc.cu"]
-HEADERS = ["metasd_internal.h", "metasd_device.cuh", "metasd_staged.cuh", os.path.join(ROOT, "include", "metasd.h")]
+HEADERS = ["metasd_internal.h", "metasd_device.cuh", "metasd_shapes.h", "metasd_staged.cuh", os.path.join(ROOT, "include", "metasd.h")]
 
 
 def _stale() -> bool:

@@ -371,19 +371,6 @@ static cudaError_t launch(const VerifyParams &p, unsigned units, int n_sm, cudaS
     return launch_kernel(row_stats_hinted_kernel<LT, D, THREADS, MINB, BONUS_LAST, CL>, units * CL, THREADS, how.smem, CL, how.chained, stream, p);
 }
 
-// The built shapes, as in metasd_streaming.cu: those that its rule may pick (hinted_built), and those that a configuration can ask for.
-#define METASD_HINTED_BF16_SHAPES(X) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(256, 6, 4, true, 2)
-#define METASD_HINTED_FP32_SHAPES(X) X(256, 6, 4, true, 2) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
-
-bool hinted_built(int dtype, int threads, int stages, int cluster)
-{
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return true;
-    if (dtype == METASD_BF16) { METASD_HINTED_BF16_SHAPES(X) }
-    else { METASD_HINTED_FP32_SHAPES(X) }
-#undef X
-    return false;
-}
-
 template <typename LT>
 static cudaError_t prepare_t(int threads, int stages, int cluster, int warps)
 {

@@ -96,7 +96,6 @@ int row_parts(const RowGeometry &geo, int dtype, int vocab);   // parts of a row
 cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, RowGeometry *geo);
 cudaError_t launch_streaming(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream, uint64_t *launches);
 // the staged kernel with L2 policies (metasd_hinted.cu); threads == 0: every shape that may be picked for rows of `warps` warps (0: any)
-bool hinted_built(int dtype, int threads, int stages, int cluster);
 cudaError_t hinted_prepare(int dtype, int threads, int stages, int cluster, int warps);
 cudaError_t launch_row_stats_hinted(const VerifyParams &p, int dtype, const RowGeometry &geo, cudaStream_t stream);
 cudaError_t bulk_prepare(int dtype, RowGeometry *geo);

@@ -1,0 +1,69 @@
+"""The rules that pick a row-statistics kernel and its shape (csrc/metasd_shapes.h) against the tables of what is built, on the
+host: the header compiled by itself, every row length and launch size of a wide range put through it."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_2604_05417_b200 import binding as M
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SMS = 148
+
+SHIM = r"""
+#include "metasd_shapes.h"
+using namespace metasd;
+
+// Which form of which kernel takes a launch, as launch_staged_t() decides; form 0: aligned, groups; 1: aligned, compact; 2: shifted,
+// groups; 3: shifted, compact; 4: the hinted kernel.  Returns whether it is built.
+extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligned, int *threads, int *stages, int *cluster, int *form)
+{
+    const long long bytes = row_bytes(dtype, vocab);
+    const StagedShape s = staged_shape(dtype, bytes, units, n_sm);
+    *threads = s.threads; *stages = s.stages; *cluster = s.cluster;
+    if (s.threads / 32 * s.cluster != row_warps(dtype, bytes)) return 0;
+    if (aligned && hinted_pays(dtype, bytes, units, s, n_sm)) {
+        *form = 4;
+        return hinted_built(dtype, s.threads, s.stages, s.cluster);
+    }
+    const int f = *form = (aligned ? 0 : 2) + compact_form(dtype, vocab, aligned, s);
+#define X(T, D, MINB, BL, CL, AG, AC, SG, SC) \
+    if (s.threads == T && s.stages == D && s.cluster == CL) return f == 0 ? AG : f == 1 ? AC : f == 2 ? SG : SC;
+    if (dtype == METASD_BF16) { METASD_STAGED_BF16_SHAPES(X) }
+    else { METASD_STAGED_FP32_SHAPES(X) }
+#undef X
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("shapes")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O1", "-Wall", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                           "-I", os.path.join(ROOT, "paper_2604_05417_b200", "csrc"), str(d / "shim.cpp"), "-o", str(d / "shim.so")])
+    return C.CDLL(str(d / "shim.so"))
+
+
+def route(rules, dtype, V, units, aligned=None):
+    """(threads, stages, CTAs per row, form) of a launch, and whether that is built."""
+    t, s, c, f = (C.c_int() for _ in range(4))
+    aligned = V % (8 if dtype == M.BF16 else 4) == 0 if aligned is None else aligned
+    built = rules.route(dtype, V, C.c_longlong(units), SMS, int(aligned), C.byref(t), C.byref(s), C.byref(c), C.byref(f))
+    return (t.value, s.value, c.value, f.value), built
+
+
+@pytest.mark.parametrize("dtype", [M.BF16, M.FP32])
+def test_every_shape_and_form_that_a_launch_may_pick_is_built(rules, dtype):
+    lengths = sorted({max(1, round(1.09 ** i) * 8 + d) for i in range(140) for d in (0, 1, 4)})
+    units = sorted({max(2, round(1.15 ** i) + d) for i in range(87) for d in (0, 1)})
+    taken = set()
+    for V in lengths:
+        for u in units:
+            for aligned in ((True, False) if V % 8 == 0 else (False,)):     # a tensor may start off a boundary whatever its rows' length
+                how, built = route(rules, dtype, V, u, aligned)
+                assert built, (V, u, aligned, how)
+                taken.add(how)
+    assert len(taken) > 12
