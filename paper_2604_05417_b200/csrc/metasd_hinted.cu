@@ -307,9 +307,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_hinted_kernel(const V
     // would be rounded at that size, and every term of the draft row scaled by the error, up to 7e-7).
     float weight = sum2(w.a), shared = 0.f;
     if (pair) {
-        const float rho = sum_a / sum_b, whole = rintf(log2f(rho));
+        const float rho = sum_a / sum_b, whole = whole_log2(rho);
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
-        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(log2f(rho * exp2i(-whole)));
+        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(rest_log2(rho, whole));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last).

@@ -605,10 +605,10 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     // would be rounded at that size, and every term of the draft row scaled by the error, up to 7e-7).
     float weight = sum2(w.a), shared = 0.f;
     if (pair) {
-        // The logarithm's whole part: the exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2).
-        const int rho = __float_as_int(sum_a / sum_b), whole = (rho - 0x3F3504F3) >> 23;
+        float whole, rest;
+        split_log2(sum_a / sum_b, whole, rest);
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
-        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + (float)whole + (w.ref - ref_a)), lg = pack2(log2f(__int_as_float(rho - whole * (1 << 23))));
+        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(rest);
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last).

@@ -48,3 +48,47 @@ def test_results_do_not_depend_on_the_kernel_of_long_launches(dtype, V):
     """1200 row pairs and bonus rows, more than L2 holds, which the kernel with L2 policies takes where it has their shape (fp32,
     V = 20400: it has not); 141 of them by the other."""
     test_results_do_not_depend_on_the_batch(dtype, V, 400)
+
+
+@pytest.mark.parametrize("dtype,V,few", [("bf16", 152064, 80), ("fp32", 128256, 40)])
+@pytest.mark.parametrize("octave", [0, 4])
+def test_rows_whose_sums_are_a_power_of_two_times_the_square_root_of_two_apart(dtype, V, few, octave):
+    """Where log2(sum_a / sum_b) lies half way between two whole numbers, both row-statistics kernels must take the same one: the
+    rounding of the draft row's exponents follows it.  400 rows whose ratio, 1.4142135 (1 + d) 2^octave with d in -3e-7 .. 3e-7,
+    meets every fp32 number there; 800 row pairs and bonus rows in a launch, and `few` sequences at a time."""
+    B, T = 400, 0.9
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(4)
+    low = -rng.integers(39, 512, size=20000 >> octave) / 64.0
+    low = torch.from_numpy(low).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    S = float(torch.exp2(low.double() * float(np.float32(1.4426950408889634 / T))).sum())
+    ones = np.arange(20000 >> octave, 45000 >> octave)
+    pairs = []
+    for d in np.linspace(-3e-7, 3e-7, B):
+        want = 1.41421354 * 2 ** octave * (1.0 + d)
+        n = np.rint(want * (ones + S))
+        i = int(np.argmin(np.abs(n / (ones + S) / want - 1.0)))
+        pairs.append((int(n[i]), int(ones[i])))
+    target = torch.full((B, 2, V), float("-inf"), dtype=low.dtype, device=dev)
+    draft = torch.full((B, 1, V), float("-inf"), dtype=low.dtype, device=dev)
+    for b, (n, m) in enumerate(pairs):
+        target[b, :, :n] = 0.0
+        draft[b, 0, 75000:75000 + m] = 0.0
+    draft[:, 0, :low.numel()] = low.to(dev)
+    tokens = torch.zeros((B, 1), dtype=torch.int32, device=dev)
+
+    def play(first, last):
+        msd = M.MetaSD(last - first, 1, 1, V, dtype=dtype, sequence_base=first)
+        res = msd.verify(target[first:last], draft[first:last], tokens[first:last], T, 31, want_diag=True)
+        torch.cuda.synchronize()
+        assert msd.last_status() == 0
+        reward = torch.from_numpy(np.array(M.parse_state(msd.state_export(), last - first, 1, msd.cfg.window)["stat_a"]))   # fp64
+        msd.close()
+        return [res.accepted_len, res.next_token, res.diag, reward]
+
+    whole = play(0, B)
+    differ = torch.zeros(B, dtype=torch.bool)
+    for first in range(0, B, few):
+        for x, y in zip(whole, play(first, first + few)):
+            differ[first:first + few] |= (x[first:first + few].cpu() != y.cpu()).reshape(few, -1).any(1)
+    assert int(differ.sum()) == 0
