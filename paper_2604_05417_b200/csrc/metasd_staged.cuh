@@ -48,22 +48,14 @@ template <typename LT> struct WarpSums {
     int32_t best_i;
 };
 
-// log2(rho) as a whole number and what is left.  Both kernels must split it the same way: the draft row's exponents are rounded with
-// the whole part added, and which kernel takes a row depends on the size of its launch.
+// log2(rho) as a whole number and what is left.  Kernels that may take the same row, by the size of its launch, must split it the
+// same way: the draft row's exponents are rounded with the whole part added.
 __device__ __forceinline__ float whole_log2(float rho) { return rintf(log2f(rho)); }
 __device__ __forceinline__ float rest_log2(float rho, float whole) { return log2f(rho * exp2i(-whole)); }
-// The same with one logarithm: the whole part is the exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2), and not
-// always whole_log2's where log2(m) is next to +-1/2 (some 5 numbers an octave).  |log2(rho)| is below 128 and log2f within 2e-5 of it.
-__device__ __forceinline__ void split_log2(float rho, float &whole, float &rest)
-{
-    const int bits = __float_as_int(rho), e = (bits - 0x3F3504F3) >> 23;
-    whole = (float)e;
-    rest = log2f(__int_as_float(bits - e * (1 << 23)));
-    if (fabsf(rest) > 0.4999f) {
-        whole = whole_log2(rho);
-        rest = rest_log2(rho, whole);
-    }
-}
+// The same in fewer instructions: the exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2).  Of some 5 numbers an octave,
+// next to 2^n sqrt(2), another whole part than whole_log2's.
+__device__ __forceinline__ int whole_exponent(float rho) { return (__float_as_int(rho) - 0x3F3504F3) >> 23; }
+__device__ __forceinline__ float rest_exponent(float rho, int whole) { return log2f(__int_as_float(__float_as_int(rho) - whole * (1 << 23))); }
 
 // Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it
 // in the stream drains, and wait (grid_dependency_wait) before they touch what that one does.

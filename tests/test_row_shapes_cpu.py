@@ -24,8 +24,8 @@ extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligne
     *threads = s.threads; *stages = s.stages; *cluster = s.cluster;
     if (s.threads / 32 * s.cluster != row_warps(dtype, bytes)) return 0;
     if (aligned && hinted_pays(dtype, bytes, units, s, n_sm)) {
-        *form = 4;
-        return hinted_built(dtype, s.threads, s.stages, s.cluster);
+        *form = 4;      // of the staged kernel's forms, the aligned one in groups alone splits logarithms as the hinted kernel does
+        return hinted_built(dtype, s.threads, s.stages, s.cluster) && !compact_form(dtype, vocab, true, s);
     }
     const int f = *form = (aligned ? 0 : 2) + compact_form(dtype, vocab, aligned, s);
 #define X(T, D, MINB, BL, CL, AG, AC, SG, SC) \
