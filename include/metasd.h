@@ -130,8 +130,10 @@ typedef struct metasd_config {
     int32_t row_kernel;         /* metasd_row_kernel */
     int32_t row_threads;        /* threads per CTA of the row-statistics kernel; only the built shapes are accepted */
     int32_t row_stages;         /* depth of its shared-memory staging; only the built shapes are accepted */
-    int32_t keep_permille;      /* share (its end, in 1/1000) of every row that the first sweep asks L2 to keep for the
-                                   second, in launches of more rows than L2 holds; 0 = default, negative = keep nothing */
+    int32_t keep_permille;      /* share (its end, in 1/1000) of every row that the first sweep asks L2 to keep for the second: of the
+                                   plain kernel's 16-byte aligned rows and, of the staged kernel's, in launches of more rows than L2
+                                   holds and in a pinned shape; 0 = default, negative = keep nothing (the staged kernel: no L2
+                                   policies at all) */
     int32_t fused_cluster;      /* METASD_PATH_FUSED: CTAs per cluster (0 = the smallest that fits) */
     int32_t fused_threads;      /* METASD_PATH_FUSED: threads per CTA (0 = chosen from the slice length) */
     int32_t wait_poll_limit;    /* polls after which a device-side wait on an asynchronous copy gives up and sets

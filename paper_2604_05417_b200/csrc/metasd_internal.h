@@ -50,7 +50,7 @@ struct RowGeometry {
     int32_t per_sm;     // CTAs per SM the shape is built for
     int32_t n_sm;       // SMs of the device (persistent kernels size their grid with it)
     int32_t cluster;    // CTAs that share one row pair (1: none)
-    int32_t hinted;     // aligned rows by the staged kernel with L2 policies
+    int32_t hinted;     // staged kernel: a launch's aligned rows are the hinted kernel's; in a context's geometry: they may be
 };
 
 struct VerifyParams {

@@ -44,7 +44,7 @@ inline StagedLaunch staged_launch(unsigned units, unsigned cluster, unsigned per
 
 // The built shapes of the staged kernel: (threads, stages, CTAs per SM, bonus rows last, CTAs per row), and which forms of each
 // staged_shape() and compact_form() reach: aligned rows with and without groups of trips, SHIFTED ones with and without.  A
-// configuration can ask for METASD_STAGED_PINNED_SHAPES, of which these here are the SHIFTED ones, with groups.
+// configuration can ask for METASD_STAGED_PINNED_SHAPES, which are built with groups.
 #define METASD_STAGED_BF16_SHAPES(X) \
     X(128, 4, 12, true, 1, 0, 1, 1, 0) X(256, 4, 6, true, 1, 0, 1, 1, 0) X(512, 6, 2, true, 1, 1, 1, 1, 1) X(512, 4, 3, true, 1, 0, 1, 1, 0) \
     X(256, 6, 4, true, 2, 1, 1, 1, 1) X(128, 6, 6, true, 4, 1, 1, 1, 1)
@@ -126,6 +126,13 @@ inline bool hinted_pays(int dtype, long long bytes, long long units, const Stage
     if (!hinted_built(dtype, s.threads, s.stages, s.cluster)) return false;
     const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : s.stages == 4 ? 3 : 1024 / s.threads) / s.cluster;
     return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.stages == 6 && s.cluster == 1 ? 165 : 115) * 1000000ll;
+}
+
+// Whether the hinted kernel takes a launch's aligned rows: where its policies pay, and in a pinned shape, unless the configuration
+// asks for none.
+inline bool hinted_takes(bool policies, bool pinned, int dtype, long long bytes, long long units, const StagedShape &s, int n_sm)
+{
+    return policies && (pinned || hinted_pays(dtype, bytes, units, s, n_sm));
 }
 
 // Whether a warp's trips all go through the rolled loops.  Groups of trips with constant slots issue a tenth fewer instructions, but

@@ -517,7 +517,8 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
     if (!(ref_a < INFINITY)) ref_a = 0.f;
     float merged = 0.f;
 #pragma unroll
-    for (int q = 0; q < (NREC + 15) / 16; ++q) {
+    for (int i = 0; i < (NREC + 15) / 16; ++i) {
+        const int q = NREC == 48 ? i * 2 % 3 : i;   // the hinted kernel's order, which holds two records a lane there
         const float d = ref_a - part_ref[q];   // above zero for stand-ins alone, whose sum_a is zero
         merged = fmaf(part_sum[q], exp2_whole(upper ? d : fminf(d, 0.f)), merged);
     }
@@ -1108,13 +1109,16 @@ static cudaError_t prepare_staged()
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, STAGED_SMEM_MAX);
 }
 
-// The pinned shape, whose aligned rows are the hinted kernel's; threads == 0: every shape that staged_shape() may pick for rows
-// of `warps` warps (0: for any row).  A tensor may start off a 16-byte boundary whatever its rows' length.
+// The pinned shape; threads == 0: every shape that staged_shape() may pick for rows of `warps` warps (0: for any row)  A tensor may start off a 16-byte boundary whatever its rows' length.
 template <typename LT>
 static cudaError_t prepare_staged_t(int threads, int stages, int cluster, int warps, bool aligned)
 {
     if (threads) {
-#define X(T, D, M, BL, C) if (threads == T && stages == D && cluster == C) return prepare_staged<LT, D, T, M, BL, C, true, false>();
+#define X(T, D, M, BL, C) \
+    if (threads == T && stages == D && cluster == C) { \
+        const cudaError_t e = aligned ? prepare_staged<LT, D, T, M, BL, C, false, false>() : cudaSuccess; \
+        return e != cudaSuccess ? e : prepare_staged<LT, D, T, M, BL, C, true, false>(); \
+    }
         METASD_STAGED_PINNED_SHAPES(X)
 #undef X
         return cudaErrorNotSupported;
@@ -1140,7 +1144,10 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
     if (p.vector_ok && geo.hinted) return launch_row_stats_hinted(p, dtype, geo, stream);
     const unsigned units = (unsigned)p.batch * (unsigned)(p.k + 1);
     if (pinned) {
-#define X(T, D, M, BL, C) if (geo.threads == T && geo.stages == D && geo.cluster == C) return launch_staged<LT, D, T, M, BL, C, true, false>(p, units, geo.n_sm, stream);
+#define X(T, D, M, BL, C) \
+    if (geo.threads == T && geo.stages == D && geo.cluster == C) \
+        return p.vector_ok ? launch_staged<LT, D, T, M, BL, C, false, false>(p, units, geo.n_sm, stream) \
+                           : launch_staged<LT, D, T, M, BL, C, true, false>(p, units, geo.n_sm, stream);
         METASD_STAGED_PINNED_SHAPES(X)
 #undef X
         return cudaErrorNotSupported;
@@ -1168,7 +1175,7 @@ static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab
         g.threads = s.threads;
         g.stages = s.stages;
         g.cluster = s.cluster;
-        g.hinted = hinted_pays(dtype, row_bytes(dtype, vocab), units, s, geo.n_sm);
+        g.hinted = hinted_takes(geo.hinted, false, dtype, row_bytes(dtype, vocab), units, s, geo.n_sm);
     }
     return g;
 }
@@ -1210,7 +1217,7 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
     geo->stages = cfg.row_stages;
     geo->per_sm = 1;
     geo->cluster = 1;
-    geo->hinted = 0;
+    geo->hinted = geo->kernel == METASD_ROWS_STAGED && cfg.keep_permille >= 0;
     if (cfg.row_cluster > 1 && geo->kernel != METASD_ROWS_STAGED) return cudaErrorNotSupported;   // only the staged kernel has a cluster form
     if (geo->kernel == METASD_ROWS_PLAIN) {
         if (geo->threads && geo->threads != K1_THREADS) return cudaErrorNotSupported;
@@ -1230,12 +1237,11 @@ cudaError_t streaming_prepare(int device, int dtype, const metasd_config &cfg, R
         if (!geo->threads) geo->threads = dtype == METASD_BF16 ? 512 : 1024;
         if (!geo->stages) geo->stages = dtype == METASD_BF16 && geo->threads == 512 ? 4 : 6;
         geo->cluster = cfg.row_cluster > 1 ? cfg.row_cluster : 1;
-        geo->hinted = 1;
     }
     if ((e = dtype == METASD_BF16 ? prepare_small_kernels<__nv_bfloat16>() : prepare_small_kernels<float>()) != cudaSuccess) return e;
     const int warps = cfg.vocab > 0 ? row_warps(dtype, row_bytes(dtype, cfg.vocab)) : 0;
     const bool aligned = row_bytes(dtype, cfg.vocab) % 16 == 0;
-    if (aligned && (e = hinted_prepare(dtype, geo->threads, geo->stages, geo->cluster, warps)) != cudaSuccess) return e;
+    if (aligned && geo->hinted && (e = hinted_prepare(dtype, geo->threads, geo->stages, geo->cluster, warps)) != cudaSuccess) return e;
     return dtype == METASD_BF16 ? prepare_staged_t<__nv_bfloat16>(geo->threads, geo->stages, geo->cluster, warps, aligned)
                                 : prepare_staged_t<float>(geo->threads, geo->stages, geo->cluster, warps, aligned);
 }

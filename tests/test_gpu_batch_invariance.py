@@ -92,3 +92,31 @@ def test_rows_whose_sums_are_a_power_of_two_times_the_square_root_of_two_apart(d
         for x, y in zip(whole, play(first, first + few)):
             differ[first:first + few] |= (x[first:first + few].cpu() != y.cpu()).reshape(few, -1).any(1)
     assert int(differ.sum()) == 0
+
+
+PINNED = [(512, 6, 1), (512, 4, 1), (1024, 6, 1), (1024, 4, 1), (768, 4, 1), (384, 4, 1), (512, 4, 3), (512, 4, 2), (768, 4, 2)]
+
+
+@pytest.mark.parametrize("dtype,V,B,shape", [("bf16", 152064, 400, None), ("bf16", 262144, 100, None), ("fp32", 80000, 1000, None)] +
+                         [(dtype, V, 7, shape) for shape in PINNED for dtype, V in (("bf16", 50264), ("fp32", 33000))])
+def test_results_do_not_depend_on_l2_policies(dtype, V, B, shape):
+    """keep_permille < 0: aligned rows of long launches and of pinned shapes by the staged kernel, which has no policies, instead of
+    the hinted one.  Bit for bit."""
+    k, N = 2, 2
+    wl = Workload("t", B=B, N=N, k=k, V=V, rounds=1, temperature=0.9, dtype=dtype, bandit="ucb", sigmas=(0.4, 1.5))
+    rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=V % 89).table_round(0)
+    table = M.pointer_table(rd["drafts"])
+    tuning = {} if shape is None else dict(row_kernel=M.ROWS_STAGED, row_threads=shape[0], row_stages=shape[1], row_cluster=shape[2])
+    results = []
+    for keep in (0, -1):
+        msd = M.MetaSD(B, N, k, V, dtype=dtype, keep_permille=keep, **tuning)
+        out = []
+        for T in (0.9, 0.0):
+            res = msd.verify(rd["target"], None, rd["tokens"], T, 31, drafter_table=table, token_arm_stride=B * k, want_diag=True)
+            out += [res.accepted_len, res.next_token, res.reward, res.diag, msd.select()]
+        assert msd.last_status() == 0
+        out.append(torch.from_numpy(np.array(M.parse_state(msd.state_export(), B, N, msd.cfg.window)["stat_a"])))
+        msd.close()
+        results.append(out)
+    for x, y in zip(*results):
+        assert torch.equal(x, y)

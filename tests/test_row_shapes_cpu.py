@@ -17,13 +17,13 @@ using namespace metasd;
 
 // Which form of which kernel takes a launch, as launch_staged_t() decides; form 0: aligned, groups; 1: aligned, compact; 2: shifted,
 // groups; 3: shifted, compact; 4: the hinted kernel.  Returns whether it is built.
-extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligned, int *threads, int *stages, int *cluster, int *form)
+extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligned, int policies, int *threads, int *stages, int *cluster, int *form)
 {
     const long long bytes = row_bytes(dtype, vocab);
     const StagedShape s = staged_shape(dtype, bytes, units, n_sm);
     *threads = s.threads; *stages = s.stages; *cluster = s.cluster;
     if (s.threads / 32 * s.cluster != row_warps(dtype, bytes)) return 0;
-    if (aligned && hinted_pays(dtype, bytes, units, s, n_sm)) {
+    if (aligned && hinted_takes(policies, false, dtype, bytes, units, s, n_sm)) {
         *form = 4;      // of the staged kernel's forms, the aligned one in groups alone splits logarithms as the hinted kernel does
         return hinted_built(dtype, s.threads, s.stages, s.cluster) && !compact_form(dtype, vocab, true, s);
     }
@@ -35,6 +35,8 @@ extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligne
 #undef X
     return 0;
 }
+
+extern "C" int pinned_takes(int policies) { return hinted_takes(policies, true, METASD_BF16, 2048, 2, StagedShape{384, 4, 1}, 148); }
 """
 
 
@@ -47,11 +49,11 @@ def rules(tmp_path_factory):
     return C.CDLL(str(d / "shim.so"))
 
 
-def route(rules, dtype, V, units, aligned=None):
+def route(rules, dtype, V, units, aligned=None, policies=True):
     """(threads, stages, CTAs per row, form) of a launch, and whether that is built."""
     t, s, c, f = (C.c_int() for _ in range(4))
     aligned = V % (8 if dtype == M.BF16 else 4) == 0 if aligned is None else aligned
-    built = rules.route(dtype, V, C.c_longlong(units), SMS, int(aligned), C.byref(t), C.byref(s), C.byref(c), C.byref(f))
+    built = rules.route(dtype, V, C.c_longlong(units), SMS, int(aligned), int(policies), C.byref(t), C.byref(s), C.byref(c), C.byref(f))
     return (t.value, s.value, c.value, f.value), built
 
 
@@ -66,4 +68,13 @@ def test_every_shape_and_form_that_a_launch_may_pick_is_built(rules, dtype):
                 how, built = route(rules, dtype, V, u, aligned)
                 assert built, (V, u, aligned, how)
                 taken.add(how)
+                if how[3] == 4:      # without policies: the same shape by the staged kernel
+                    plain, built = route(rules, dtype, V, u, aligned, policies=False)
+                    assert built and plain == how[:3] + (0,), (V, u, plain)
     assert len(taken) > 12
+
+
+def test_a_configuration_without_policies_keeps_every_launch_off_the_hinted_kernel(rules):
+    assert (rules.pinned_takes(1), rules.pinned_takes(0)) == (1, 0)
+    for dtype, V, units in [(M.BF16, 152064, 4608), (M.FP32, 128256, 6144), (M.BF16, 262144, 680)]:
+        assert route(rules, dtype, V, units)[0][3] == 4 and route(rules, dtype, V, units, policies=False)[0][3] == 0
