@@ -29,8 +29,9 @@ inline StagedLaunch staged_launch(unsigned units, unsigned cluster, unsigned per
     // A launch of up to one wave wants its blocks spread evenly over the SMs: set up while the last epilogue still holds some of
     // them, they would crowd on the others and stay there.  So such a launch is chained only where the last layer of blocks
     // is nearly full (or, of clusters, which are placed within groups of SMs, where every one finds free SMs), and asks for
-    // the shared memory that keeps one block more than an even spread off an SM, and no more: what is left there, half an SM's
-    // where there is one block, is for the kernels of other streams.  Us a round, chained so / not, in blocks
+    // the shared memory that keeps one block more than an even spread off an SM, in whole KB: what is left there, half an SM's
+    // where there is one block, is for the kernels of other streams.  (Of a spread of 12 blocks of 128 threads the last finds no room
+    // either, which is the faster: B = 290, k = 5, V = 8000 23.2 us a round, with room for it 24.5.)  Us a round, chained so / not, in blocks
     // of 256 and 512 threads:
     // 384 blocks (B = 64, k = 5, V = 32000) 22.8 / 24.6, 240 18.5 / 20.5, 144 (V = 128256) 28.1 / 28.7, 96 14.0 / 16.1;
     // 320 blocks 22.2 / 20.5, 480 26.5 / 24.6; 32 clusters of 4 13.5 / 14.4, 36 21.8 / 19.8.  Several waves are always chained
@@ -53,7 +54,7 @@ inline StagedLaunch staged_launch(unsigned units, unsigned cluster, unsigned per
     X(128, 6, 6, true, 4, 1, 1, 1, 1) X(1024, 6, 1, false, 1, 1, 0, 1, 0) X(256, 6, 4, true, 4, 1, 0, 1, 0) X(128, 6, 6, true, 8, 1, 0, 1, 0)
 
 // The shapes of the hinted kernel that hinted_pays() may pick, besides those that a configuration can ask for.
-#define METASD_HINTED_BF16_SHAPES(X) X(512, 6, 2, true, 1) X(512, 4, 3, true, 1) X(256, 6, 4, true, 2)
+#define METASD_HINTED_BF16_SHAPES(X) X(512, 6, 2, true, 1) X(256, 6, 4, true, 2)
 #define METASD_HINTED_FP32_SHAPES(X) X(256, 6, 4, true, 2) X(1024, 6, 1, false, 1) X(256, 6, 4, true, 4) X(128, 6, 6, true, 8)
 
 inline bool hinted_built(int dtype, int threads, int stages, int cluster)
@@ -116,16 +117,15 @@ inline StagedShape staged_shape(int dtype, long long bytes, long long units, int
 
 // Whether L2 policies pay, which the hinted kernel has: where the row pairs in flight are more than L2 keeps between their sweeps
 // without them.  Us a round with and without, by MB in flight: bf16, 512/6/1 118: 138.6 and 136.6 (B = 256, k = 5, V = 100000), 152: 226 and
-// 223 (B = 256, k = 7, V = 128256), 180: 635 and 643 (B = 512, k = 8, V = 152064); 512/4/1 89: 462 and 451 (B = 1024, k = 8,
-// V = 50264), 113: 103.0 and 103.9, 142: 169 and 181 (B = 400, k = 5, V = 80000); 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
+// 223 (B = 256, k = 7, V = 128256), 180: 635 and 643 (B = 512, k = 8, V = 152064); 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
 // 76: 242 and 226 (256/6/4: B = 512, k = 4, V = 64000), 293 and 263 (256/6/2: B = 1024, k = 5, V = 32000), 95: 78.7 and 79.6, 114: 261 and 333
 // (128/6/8: B = 256, k = 5, V = 128256).  Shapes of short rows are not built there.
 inline bool hinted_pays(int dtype, long long bytes, long long units, const StagedShape &s, int n_sm)
 {
     const bool fp32 = dtype == METASD_FP32;
     if (!hinted_built(dtype, s.threads, s.stages, s.cluster)) return false;
-    const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : s.stages == 4 ? 3 : 1024 / s.threads) / s.cluster;
-    return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.stages == 6 && s.cluster == 1 ? 165 : 115) * 1000000ll;
+    const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : 1024 / s.threads) / s.cluster;
+    return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.cluster == 1 ? 165 : 115) * 1000000ll;
 }
 
 // Whether the hinted kernel takes a launch's aligned rows: where its policies pay, and in a pinned shape, unless the configuration
