@@ -11,13 +11,21 @@ from paper_2604_05417_b200.workloads import RoundGenerator, Workload
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,V,B", [("bf16", 4096, 400), ("bf16", 4101, 400), ("bf16", 20001, 400), ("bf16", 32000, 400),
-                                       ("bf16", 50257, 400), ("bf16", 50264, 400), ("bf16", 80008, 400), ("bf16", 100003, 400),
-                                       ("bf16", 131072, 400), ("fp32", 4096, 400), ("fp32", 4099, 400), ("fp32", 32000, 400),
-                                       ("fp32", 32001, 400), ("fp32", 64008, 400), ("fp32", 64009, 400), ("fp32", 110000, 400),
-                                       ("fp32", 64003, 1000)])
+# 1200 (3000) row pairs and bonus rows in one launch
+BATCHES = [("bf16", 4096, 400), ("bf16", 4101, 400), ("bf16", 20001, 400), ("bf16", 32000, 400),
+           ("bf16", 50257, 400), ("bf16", 50264, 400), ("bf16", 80008, 400), ("bf16", 100003, 400),
+           ("bf16", 131072, 400), ("fp32", 4096, 400), ("fp32", 4099, 400), ("fp32", 32000, 400),
+           ("fp32", 32001, 400), ("fp32", 64008, 400), ("fp32", 64009, 400), ("fp32", 110000, 400),
+           ("fp32", 64003, 1000)]
+# every shape of the hinted kernel, against launches by the staged one: bf16 512/6/1 and 256/6/2, fp32 256/6/2, 256/6/4 and 1024/6/1 (128/6/8:
+# V = 110000 above); and short fp32 rows, whose shape the hinted kernel is not built in
+LONG_LAUNCHES = [("bf16", 152064, 400), ("fp32", 20400, 400), ("fp32", 48000, 400), ("fp32", 80000, 400), ("fp32", 80000, 1000)]
+PARTS = [(0, 1), (1, 13), (13, 60), (60, 200), (200, 400)]
+
+
+@pytest.mark.parametrize("dtype,V,B", BATCHES)
 def test_results_do_not_depend_on_the_batch(dtype, V, B):
-    """1200 (3000) row pairs and bonus rows in one launch; 3, 36, 141, 420 and 600 of them in launches of their own."""
+    """All sequences in one launch; 3, 36, 141, 420 and 600 row pairs and bonus rows in launches of their own."""
     k, N = 2, 2
     wl = Workload("t", B=B, N=N, k=k, V=V, rounds=1, temperature=0.9, dtype=dtype, bandit="ucb", sigmas=(0.4, 1.5))
     rd = RoundGenerator(wl, device=torch.device("cuda", 0), seed=V % 89).table_round(0)
@@ -38,16 +46,16 @@ def test_results_do_not_depend_on_the_batch(dtype, V, B):
         return out + [torch.from_numpy(np.array(state[n])) for n in ("stat_a", "stat_b")]
 
     whole = play(0, B)
-    for first, last in [(0, 1), (1, 13), (13, 60), (60, 200), (200, 400)]:
+    for first, last in PARTS:
         for x, y in zip(whole, play(first, last)):
             assert torch.equal(x[first:last], y)
 
 
-@pytest.mark.parametrize("dtype,V", [("bf16", 80008), ("bf16", 152064), ("fp32", 20400)])
-def test_results_do_not_depend_on_the_kernel_of_long_launches(dtype, V):
-    """1200 row pairs and bonus rows, more than L2 holds, which the kernel with L2 policies takes where it has their shape (fp32,
-    V = 20400: it has not); 141 of them by the other."""
-    test_results_do_not_depend_on_the_batch(dtype, V, 400)
+@pytest.mark.parametrize("dtype,V,B", LONG_LAUNCHES)
+def test_results_do_not_depend_on_the_kernel_of_long_launches(dtype, V, B):
+    """More row pairs in flight than L2 holds, which the hinted kernel takes, against launches of few by the staged one (which kernel
+    takes which: test_row_shapes_cpu.py)."""
+    test_results_do_not_depend_on_the_batch(dtype, V, B)
 
 
 @pytest.mark.parametrize("dtype,V,few", [("bf16", 152064, 80), ("fp32", 128256, 40)])

@@ -10,6 +10,15 @@ from paper_2604_05417_b200.workloads import RoundGenerator, Workload
 
 pytestmark = pytest.mark.gpu
 
+# Launches of a few rows are the staged kernel's.  Long launches are the hinted kernel's (csrc/metasd_hinted.cu), which has a text of its
+# own: these are the shapes it takes the largest ones in, and pinned it takes aligned rows of any launch.
+KERNELS = ["auto", "pinned"]
+PINNED = {"bf16": dict(row_kernel=M.ROWS_STAGED, row_threads=512, row_stages=6), "fp32": dict(row_kernel=M.ROWS_STAGED, row_threads=1024, row_stages=6)}
+
+
+def shape(kernel, dtype):
+    return PINNED[dtype] if kernel == "pinned" else {}
+
 
 def workload(**kw):
     d = dict(name="t", B=3, N=2, k=2, V=1024, rounds=2, temperature=1.0, dtype="bf16", bandit="ucb", sigmas=(0.5, 2.0))
@@ -19,15 +28,17 @@ def workload(**kw):
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [8, 248, 256, 264, 4088, 4096, 4104, 6 * 4096, 6 * 4096 + 8, 11 * 4096, 12 * 4096 - 8, 12 * 4096 + 264])
-def test_row_lengths_at_the_edges_of_trips_and_groups(dtype, V):
+@pytest.mark.parametrize("kernel", KERNELS)
+def test_row_lengths_at_the_edges_of_trips_and_groups(dtype, V, kernel):
     from _harness import run_lockstep
-    c = run_lockstep(workload(V=V, dtype=dtype), rounds=3, seed=V % 83, path=M.PATH_STREAMING)
+    c = run_lockstep(workload(V=V, dtype=dtype), rounds=3, seed=V % 83, path=M.PATH_STREAMING, **shape(kernel, dtype))
     assert c["rounds"] == 3 and c["status"] == 0
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("shift", [0.0, 120.0, -120.0])
-def test_masked_stretches_cover_whole_warps(dtype, shift):
+@pytest.mark.parametrize("kernel", KERNELS)
+def test_masked_stretches_cover_whole_warps(dtype, shift, kernel):
     """Target and / or draft logits of whole ranges of the vocabulary are -inf, the draft row on another scale."""
     from _harness import make_pair, compare_round
     V = 3 * 4096 + 40
@@ -42,7 +53,7 @@ def test_masked_stretches_cover_whole_warps(dtype, shift):
     draft[3, :, : V - 9] = ninf
     target[4, :, 3:] = ninf
     draft[4, :, : V // 3] = ninf
-    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING, **shape(kernel, dtype))
     try:
         res = gpu.verify(target, draft, rd["tokens"], 1.0, 3, want_diag=True)
         out = orc.verify(target, draft, rd["tokens"].cpu().numpy(), 1.0, 3)
@@ -55,7 +66,8 @@ def test_masked_stretches_cover_whole_warps(dtype, shift):
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [3 * 4096 + 40, 3 * 4096 + 41])
 @pytest.mark.parametrize("T", [1.0, 2.0])
-def test_masks_of_the_types_lowest_value(dtype, V, T):
+@pytest.mark.parametrize("kernel", KERNELS)
+def test_masks_of_the_types_lowest_value(dtype, V, T, kernel):
     """Masks written as torch.finfo(dtype).min (and as -1e38) over stretches that hold the first trips of some warps: they
     weigh nothing, as -inf does, although their product with log2(e) / T leaves the range of fp32."""
     from _harness import make_pair, compare_round
@@ -70,7 +82,7 @@ def test_masks_of_the_types_lowest_value(dtype, V, T):
     draft[3, :, : V - 9] = low
     target[4, :, 3:] = -1e38
     draft[4, :, : V // 3] = low
-    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING, **shape(kernel, dtype))
     try:
         res = gpu.verify(target, draft, rd["tokens"], T, 3, want_diag=True)
         out = orc.verify(target, draft, rd["tokens"].cpu().numpy(), T, 3)
@@ -82,7 +94,8 @@ def test_masks_of_the_types_lowest_value(dtype, V, T):
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
 @pytest.mark.parametrize("V", [4096, 4099])
-def test_draft_sums_next_to_the_end_of_the_fp32_range(dtype, V):
+@pytest.mark.parametrize("kernel", KERNELS)
+def test_draft_sums_next_to_the_end_of_the_fp32_range(dtype, V, kernel):
     """Draft rows whose sum, relative to the target row's maximum (0 here), is 2^99 .. 2^128: 2^127.6 is a finite fp32
     number, and its inverse's whole exponent, 128, is not one that an fp32 power of two can have."""
     from _harness import make_pair, compare_round
@@ -96,7 +109,7 @@ def test_draft_sums_next_to_the_end_of_the_fp32_range(dtype, V):
         draft[b, :, 0], draft[b, :, 5] = low, high
     target, draft = (x.to({"bf16": torch.bfloat16, "fp32": torch.float32}[dtype]) for x in (target, draft))
     tokens = torch.zeros((8, 2), dtype=torch.int32, device=dev)
-    gpu, orc = make_pair(wl, path=M.PATH_STREAMING)
+    gpu, orc = make_pair(wl, path=M.PATH_STREAMING, **shape(kernel, dtype))
     try:
         res = gpu.verify(target, draft, tokens, 1.0, 3, want_diag=True)
         out = orc.verify(target, draft, tokens.cpu().numpy(), 1.0, 3)
@@ -163,7 +176,7 @@ def test_every_shape_that_a_launch_size_selects(dtype, V, B, k):
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp32"])
-@pytest.mark.parametrize("kernel", [M.ROWS_AUTO, M.ROWS_PLAIN, M.ROWS_BULK])
+@pytest.mark.parametrize("kernel", [M.ROWS_AUTO, M.ROWS_PLAIN, M.ROWS_BULK, "pinned"])
 def test_alignment_of_rows_that_hardly_overlap(dtype, kernel):
     """Target and draft mass in different halves of the vocabulary: the alignment 1 - d_TV is a small sum of positive terms,
     each a 2^-22 exponential of an fp32 exponent of up to 130 (off by 2^-18 at most) over an fp32 normaliser, never a
@@ -176,7 +189,7 @@ def test_alignment_of_rows_that_hardly_overlap(dtype, kernel):
     target[..., V // 2:] -= gap
     draft[..., : V // 2] -= gap
     target, draft = target.to(rd["target"].dtype), draft.to(rd["draft"].dtype)
-    gpu = M.MetaSD(B, 1, 1, V, dtype=dtype, path=M.PATH_STREAMING, row_kernel=kernel)
+    gpu = M.MetaSD(B, 1, 1, V, dtype=dtype, path=M.PATH_STREAMING, **(shape(kernel, dtype) or dict(row_kernel=kernel)))
     try:
         res = gpu.verify(target, draft, rd["tokens"], 1.0, 3, want_diag=True)
         p, q = (torch.softmax(x[:, 0].double(), -1) for x in (target, draft))

@@ -74,6 +74,23 @@ def test_every_shape_and_form_that_a_launch_may_pick_is_built(rules, dtype):
     assert len(taken) > 12
 
 
+def test_the_batch_tests_reach_every_shape_of_the_hinted_kernel(rules):
+    """Which launches of tests/test_gpu_batch_invariance.py are the hinted kernel's; each of its shapes meets the staged kernel's."""
+    import test_gpu_batch_invariance as T
+    met = set()
+    for dtype, V, B in T.BATCHES + T.LONG_LAUNCHES:
+        code = M.DTYPES[dtype]
+        hows = [route(rules, code, V, 3 * n)[0] for n in [B] + [last - first for first, last in T.PARTS]]
+        assert hows[1][3] != 4                      # a sequence on its own: the staged kernel
+        met |= {(dtype,) + how[:3] for how in hows if how[3] == 4}
+        if (dtype, V, B) in T.LONG_LAUNCHES:
+            assert (hows[0][3] == 4) == (V != 20400)
+    assert met == {("bf16", 512, 6, 1), ("bf16", 256, 6, 2), ("fp32", 256, 6, 2), ("fp32", 256, 6, 4), ("fp32", 1024, 6, 1), ("fp32", 128, 6, 8)}
+    # and so do both sides of the test of square roots of two
+    for code, V, few in ((M.BF16, 152064, 80), (M.FP32, 128256, 40)):
+        assert route(rules, code, V, 800)[0][3] == 4 and route(rules, code, V, 2 * few)[0][3] == 0
+
+
 def test_a_configuration_without_policies_keeps_every_launch_off_the_hinted_kernel(rules):
     assert (rules.pinned_takes(1), rules.pinned_takes(0)) == (1, 0)
     for dtype, V, units in [(M.BF16, 152064, 4608), (M.FP32, 128256, 6144), (M.BF16, 262144, 680)]:
