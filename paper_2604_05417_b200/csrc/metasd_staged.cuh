@@ -52,9 +52,10 @@ template <typename LT> struct WarpSums {
 // same way: the draft row's exponents are rounded with the whole part added.
 __device__ __forceinline__ float whole_log2(float rho) { return rintf(log2f(rho)); }
 __device__ __forceinline__ float rest_log2(float rho, float whole) { return log2f(rho * exp2i(-whole)); }
-// The same in fewer instructions: the exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2).  Of some 5 numbers an octave,
-// next to 2^n sqrt(2), another whole part than whole_log2's.
+// The exponent of rho = 2^whole m with m next to one, sqrt(1/2) .. sqrt(2), in fewer instructions.  Of some 5 numbers an octave, next to
+// 2^n sqrt(2), another whole part than whole_log2's.
 __device__ __forceinline__ int whole_exponent(float rho) { return (__float_as_int(rho) - 0x3F3504F3) >> 23; }
+// rest_log2's value (rho finite, both powers of two in range).
 __device__ __forceinline__ float rest_exponent(float rho, int whole) { return log2f(__int_as_float(__float_as_int(rho) - whole * (1 << 23))); }
 
 // Launches a kernel.  CHAINED, with programmatic stream serialisation: its blocks may be set up while the kernel before it

@@ -609,10 +609,9 @@ __global__ void __launch_bounds__(THREADS, MINB) row_stats_staged_kernel(const V
         // Aligned rows in groups are those that the hinted kernel may take in a larger launch.  (All forms its way: V = 32000, B = 1 9.35 ->
         // 9.48 us a round, V = 50257, B = 96 45.9 -> 46.1.)
         const float rho = sum_a / sum_b;
-        const float whole = SHIFTED || COMPACT ? (float)whole_exponent(rho) : whole_log2(rho);
-        const float rest = SHIFTED || COMPACT ? rest_exponent(rho, whole_exponent(rho)) : rest_log2(rho, whole);
+        const int whole = SHIFTED || COMPACT ? whole_exponent(rho) : (int)whole_log2(rho);
         // The warp's own reference again: where p < q both sweeps then add the same numbers, which leave nothing behind.
-        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + whole + (w.ref - ref_a)), lg = pack2(rest);
+        const uint64_t nma = pack2(w.ref), nmb = pack2(ref_b + (float)whole + (w.ref - ref_a)), lg = pack2(rest_exponent(rho, whole));
         uint64_t acc = 0ull;
         // A trip of sweep 2 from its slot; the slot is then refilled with the trip D further down (inside the row for
         // every lane: the ragged trips are the row's last).
