@@ -116,8 +116,10 @@ inline StagedShape staged_shape(int dtype, long long bytes, long long units, int
 }
 
 // Whether L2 policies pay, which the hinted kernel has: where the row pairs in flight are more than L2 keeps between their sweeps
-// without them.  Us a round with and without, by MB in flight: bf16, 512/6/1 118: 138.6 and 136.6 (B = 256, k = 5, V = 100000), 152: 226 and
-// 223 (B = 256, k = 7, V = 128256), 180: 635 and 643 (B = 512, k = 8, V = 152064); 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
+// without them.  Us a round with and without, by MB in flight: bf16, 512/6/1, B = 256, k = 7, at full clock 107: 166.2 and 166.2 (V = 90000),
+// 118: 180.2 and 180.0 (V = 100000), 133: 196.4 and 200.1 (V = 112000), 152: 219.9 and 230.3 (V = 128256), 158: 237 and 248 (V = 133512), and
+// under the power cap of a long run, where fewer instructions count, 133: 217.8 and 217.4, 152: 250.6 and 248.3 (8 drafters' rows by the
+// table), 158: 274 and 278: the line is the capped runs'; 256/6/2 152: 86.7 and 90.6, 180: 86.2 and 94.0; fp32
 // 76: 242 and 226 (256/6/4: B = 512, k = 4, V = 64000), 293 and 263 (256/6/2: B = 1024, k = 5, V = 32000), 95: 78.7 and 79.6, 114: 261 and 333
 // (128/6/8: B = 256, k = 5, V = 128256).  Shapes of short rows are not built there.
 inline bool hinted_pays(int dtype, long long bytes, long long units, const StagedShape &s, int n_sm)
@@ -125,7 +127,7 @@ inline bool hinted_pays(int dtype, long long bytes, long long units, const Stage
     const bool fp32 = dtype == METASD_FP32;
     if (!hinted_built(dtype, s.threads, s.stages, s.cluster)) return false;
     const long long resident = (long long)n_sm * (s.threads == 128 ? 6 : 1024 / s.threads) / s.cluster;
-    return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.cluster == 1 ? 165 : 115) * 1000000ll;
+    return std::min(units, resident) * 2 * bytes > (fp32 ? 90 : s.cluster == 1 ? 154 : 115) * 1000000ll;
 }
 
 // Whether the hinted kernel takes a launch's aligned rows: where its policies pay, and in a pinned shape, unless the configuration

@@ -91,6 +91,14 @@ def test_the_batch_tests_reach_every_shape_of_the_hinted_kernel(rules):
         assert route(rules, code, V, 800)[0][3] == 4 and route(rules, code, V, 2 * few)[0][3] == 0
 
 
+@pytest.mark.parametrize("dtype,V,units,how", [
+    # policies pay from 154 MB in flight on in the shape of the longest bf16 launches
+    (M.BF16, 128256, 2048, (512, 6, 1, 0)), (M.BF16, 131192, 2870, (512, 6, 1, 4)), (M.BF16, 133512, 3892, (512, 6, 1, 4))])
+def test_launches_either_side_of_a_line(rules, dtype, V, units, how):
+    """Kernel and shape where both sides of a rule's line were measured (the figures stand at the rules)."""
+    assert route(rules, dtype, V, units)[0] == how
+
+
 def test_a_configuration_without_policies_keeps_every_launch_off_the_hinted_kernel(rules):
     assert (rules.pinned_takes(1), rules.pinned_takes(0)) == (1, 0)
     for dtype, V, units in [(M.BF16, 152064, 4608), (M.FP32, 128256, 6144), (M.BF16, 262144, 680)]:
