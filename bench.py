@@ -383,7 +383,9 @@ def main():
                 # the same over the first timed steps only: before the power cap pulls the SM clock down
                 "first_40_steps": {"kernel_ms": statistics.mean(step_ms[:40]),
                                    "frac": bytes_round / (statistics.mean(step_ms[:40]) * 1e-3) / 1e9 / peak},
-                "note": "duration = CUDA events around select+verify of one step (%s path, %s row kernel)" % (path_name, row_kernel)}
+                "note": "duration = CUDA events around select+verify of one step (%s path, %s row kernel%s)" % (
+                    path_name, row_kernel, ", the form with L2 policies where more rows are in flight than L2 holds"
+                    if row_kernel == "staged" and args.keep_permille >= 0 else "")}
     if sustained is not None:
         ms = sustained["kernel_ms"]
         roofline["sustained"] = {"steps": sustained["steps"], "kernel_ms": ms, "frac": bytes_round / (ms * 1e-3) / 1e9 / peak,

@@ -50,7 +50,7 @@ inline StagedLaunch staged_launch(unsigned units, unsigned cluster, unsigned per
     X(128, 4, 12, true, 1, 0, 1, 1, 0) X(256, 4, 6, true, 1, 0, 1, 1, 0) X(512, 6, 2, true, 1, 1, 1, 1, 1) X(512, 4, 3, true, 1, 0, 1, 1, 0) \
     X(256, 6, 4, true, 2, 1, 1, 1, 1) X(128, 6, 6, true, 4, 1, 1, 1, 1)
 #define METASD_STAGED_FP32_SHAPES(X) \
-    X(256, 4, 6, true, 1, 1, 1, 1, 0) X(256, 6, 4, true, 1, 1, 0, 1, 1) X(512, 6, 2, true, 1, 1, 1, 1, 1) X(256, 6, 4, true, 2, 1, 1, 1, 1) \
+    X(256, 4, 6, true, 1, 1, 1, 1, 0) X(256, 6, 4, true, 1, 1, 0, 1, 1) X(512, 6, 2, true, 1, 1, 1, 0, 0) X(256, 6, 4, true, 2, 1, 1, 1, 1) \
     X(128, 6, 6, true, 4, 1, 1, 1, 1) X(1024, 6, 1, false, 1, 1, 0, 1, 0) X(256, 6, 4, true, 4, 1, 0, 1, 0) X(128, 6, 6, true, 8, 1, 0, 1, 0)
 
 // The shapes of the hinted kernel that hinted_pays() may pick, besides those that a configuration can ask for.
@@ -92,13 +92,15 @@ inline int row_warps(int dtype, long long bytes)
 //     V = 65000 512/4/1 162.5 (2400), 512/6/1 159.2; V = 80000 184.4 (2400) and 96.3 (1200), 181.0 and 90.9.
 //   fp32, 8 warps: V = 8000 256/4/1 24.0 (1280), 77.3 (5120), 256/6/1 24.6, 79.0; V = 16000 15.8 (320), 24.4 (640), 74.5 (2560), 146.5 (5120),
 //     16.5, 24.1, 67.9, 130.5.  16 warps, V = 32000: 256/6/2 33.3 (512), 54.2 (1024), 192.0 (4000), 512/6/1 32.4, 53.3, 185.9.
+//     Rows off 16-byte boundaries, 16 warps: V = 23367 256/6/2 33.3 (462), 55.5 (945), 113.4 (2100), 216 (4200), 512/6/1 35.2, 60.5, 121.2, 229;
+//     V = 35911 83.8 (945), 175.3 (2100), 340 (4200), 89.7, 184.1, 354.
 //   fp32, 16 warps, V = 32000: 128/6/4 11.1 (32 units), 15.2 (128), 29.2 (384), 86.9 (1536), 256/6/2 11.8, 15.5, 28.1, 81.8.
 //   fp32, 32 warps: V = 64000: 128/6/8 11.8 (24 units), 50.8 (384), 180 (1728), 614 (6144), 256/6/4 12.1, 48.3, 157, 574, 1024/6/1
 //     17.5, 51.7, 168, 525; V = 128256: 15.8, 79.7, 292 and 1062, 16.0, 86.0, 302 and 1094, 26.5, 91.0, 302 and 1029.
 struct StagedShape {
     int threads, stages, cluster;
 };
-inline StagedShape staged_shape(int dtype, long long bytes, long long units, int n_sm)
+inline StagedShape staged_shape(int dtype, long long bytes, long long units, bool aligned, int n_sm)
 {
     const bool fp32 = dtype == METASD_FP32;
     switch (row_warps(dtype, bytes)) {
@@ -107,7 +109,7 @@ inline StagedShape staged_shape(int dtype, long long bytes, long long units, int
     case 16:
         if (units * 4 <= n_sm || (units <= n_sm && bytes < 140 * 1000)) return {128, 6, 4};
         if (fp32 ? bytes >= 150 * 1000 : units <= (bytes < 100 * 1000 ? 3 : 7) * n_sm) return {256, 6, 2};
-        if (fp32 && units <= 3 * n_sm) return {256, 6, 2};
+        if (fp32 && (units <= 3 * n_sm || !aligned)) return {256, 6, 2};
         return !fp32 && bytes < 120 * 1000 ? StagedShape{512, 4, 1} : StagedShape{512, 6, 1};
     default:
         if (units > 20 * n_sm) return {1024, 6, 1};

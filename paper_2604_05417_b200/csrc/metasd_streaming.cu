@@ -1166,11 +1166,11 @@ static cudaError_t launch_staged_t(const VerifyParams &p, const RowGeometry &geo
 }
 
 // The shape of a launch: what the configuration pinned, else by the size of the launch.
-static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units)
+static RowGeometry resolve_geometry(const RowGeometry &geo, int dtype, int vocab, long long units, bool aligned)
 {
     RowGeometry g = geo;
     if (g.kernel == METASD_ROWS_STAGED && g.threads == 0) {
-        const StagedShape s = staged_shape(dtype, row_bytes(dtype, vocab), units, geo.n_sm);
+        const StagedShape s = staged_shape(dtype, row_bytes(dtype, vocab), units, aligned, geo.n_sm);
         g.threads = s.threads;
         g.stages = s.stages;
         g.cluster = s.cluster;
@@ -1250,7 +1250,7 @@ static cudaError_t launch_streaming_t(VerifyParams p, const RowGeometry &context
 {
     cudaError_t e = cudaSuccess;
     constexpr int dtype = sizeof(LT) == 2 ? METASD_BF16 : METASD_FP32;
-    const RowGeometry geo = resolve_geometry(context_geo, dtype, p.V, (long long)p.batch * (p.k + 1));
+    const RowGeometry geo = resolve_geometry(context_geo, dtype, p.V, (long long)p.batch * (p.k + 1), p.vector_ok);
     p.n_seg = row_parts(geo, dtype, p.V);
     p.k_inverse = inverse_of((uint32_t)p.k);
     p.k1_inverse = inverse_of((uint32_t)p.k + 1u);

@@ -20,7 +20,7 @@ using namespace metasd;
 extern "C" int route(int dtype, int vocab, long long units, int n_sm, int aligned, int policies, int *threads, int *stages, int *cluster, int *form)
 {
     const long long bytes = row_bytes(dtype, vocab);
-    const StagedShape s = staged_shape(dtype, bytes, units, n_sm);
+    const StagedShape s = staged_shape(dtype, bytes, units, aligned, n_sm);
     *threads = s.threads; *stages = s.stages; *cluster = s.cluster;
     if (s.threads / 32 * s.cluster != row_warps(dtype, bytes)) return 0;
     if (aligned && hinted_takes(policies, false, dtype, bytes, units, s, n_sm)) {
@@ -93,7 +93,9 @@ def test_the_batch_tests_reach_every_shape_of_the_hinted_kernel(rules):
 
 @pytest.mark.parametrize("dtype,V,units,how", [
     # policies pay from 154 MB in flight on in the shape of the longest bf16 launches
-    (M.BF16, 128256, 2048, (512, 6, 1, 0)), (M.BF16, 131192, 2870, (512, 6, 1, 4)), (M.BF16, 133512, 3892, (512, 6, 1, 4))])
+    (M.BF16, 128256, 2048, (512, 6, 1, 0)), (M.BF16, 131192, 2870, (512, 6, 1, 4)), (M.BF16, 133512, 3892, (512, 6, 1, 4)),
+    # many fp32 rows: in one CTA each where they are aligned, else in two
+    (M.FP32, 32000, 4000, (512, 6, 1, 0)), (M.FP32, 32001, 4000, (256, 6, 2, 3)), (M.FP32, 35911, 2100, (256, 6, 2, 2))])
 def test_launches_either_side_of_a_line(rules, dtype, V, units, how):
     """Kernel and shape where both sides of a rule's line were measured (the figures stand at the rules)."""
     assert route(rules, dtype, V, units)[0] == how
